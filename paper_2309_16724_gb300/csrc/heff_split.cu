@@ -50,38 +50,63 @@ void stream_end(OpStream& os, cudaStream_t s);
 
 namespace {
 
-using sp::Item;
 using sp::Job;
 constexpr int kSentinel = -100000;
 constexpr int kSub = sp::kSub;
+constexpr int kGroupBlocks = 2;                  // left blocks of an exponent group (on average)
+constexpr int kWinSteps = sp::kChunkSteps;       // 16-K steps of one T' CTA (a whole number of exponent groups)
+constexpr int kWinOct = 2 * kWinSteps;           // 8-K pieces of it
 
-struct SlabDesc {        // one FP64 source matrix -> slab (rows = slab rows, K = cols)
+// One block placed in a stacked operand (a slab whose rows or K run over
+// several blocks): FP64 source block -> rows row0.., K k0.. of the stack
+struct SlabDesc {
   int64_t src_off;       // element offset in the FP64 source, -1 = identity
-  int64_t slab_off;      // byte offset in the slab arena
+  int64_t slab_off;      // byte offset of the stack's slab
   int32_t rows, cols, ld;
-  int32_t exp_off;       // row exponent array offset (own exponents or rho of the sector)
-  int32_t shift_idx;     // index into the delta array (-1: no shift)
-  int32_t own_off;       // offset of the block's own row exponents (A side), -1 otherwise
-  int32_t pad0, pad1;
+  int32_t row0, k0;      // place in the stack (k0 a multiple of 8)
+  int32_t R, kst;        // the stack's rows and 16-K steps
+  int32_t noct;          // 8-K pieces to write (the last block of a stack also fills up to 16)
+  int32_t exp_off;       // offset of the row exponents of the block's rows ...
+  int32_t exp_ld;        // ... of the stack's first exponent group; stride to the next
+  int32_t gst;           // K steps of an exponent group (0: one group)
+  int32_t pad;
 };
 struct Unit { int32_t desc, tr, ks, pad; };
 
-struct Source {          // float-float matrix whose columns feed T' (K2 B operand)
-  int64_t off;           // element offset in Th/Tl (sel 0) or psi_ff (sel 1)
-  int32_t rows, cols, sel, cexp_off;
-  int32_t ld;            // column stride (T rows rounded up to 4: 16-byte aligned columns; psi block rows),
-                         // or the row stride of a row-major T (its columns rounded up to 4)
-  int32_t rowmajor;      // 1: T stored row-major (written by transposed K1 jobs)
-};
+// One product of the T' sum: T'(w, f) = sum over the tasks with left block w
+// and output block f of v_t T_u
 struct TPTask {
-  int32_t src;           // Source index (chunk-local)
-  int32_t gcol;          // gamma offset of the output block
-  int32_t aid;           // A slab descriptor (its delta is folded into v)
-  int32_t pad;
-  double v;              // sector-value table entry
-  int64_t tp_off;        // byte offset of the T' slab in the chunk buffer
+  int64_t off;           // element (0, 0) of the task's T block in Th / Tl, or of its psi block
+  int32_t ld;            // column stride, or row stride of a row-major T
+  int32_t flags;         // kFromPsi, kRowMajor
+  float vh, vl;          // v_t (float-float)
 };
-struct TPUnit { int32_t task, tr, ks, pad; };
+constexpr int32_t kFromPsi = 1, kRowMajor = 2;
+// the K axis of one left sector's operand: 8-K piece -> (left block w, first row k within it, valid rows)
+struct Oct { int32_t w, k, nk, pad; };
+// one left output sector of a term chunk: F_a (all psi blocks with left
+// sector a side by side: contiguous in psi) += [A_1 A_2 ..] [T'_1; T'_2; ..]
+struct Stack {
+  int64_t tp_off;        // byte offset of the T' slab in the chunk buffer
+  int64_t tab_off;       // CSR offsets of its (w, f) task lists
+  int64_t grp_off;       // offset of its per-(group, column) exponents
+  int32_t oct_off, noct; // its 8-K pieces (2 kst)
+  int32_t nf, N, Npad;   // output blocks, their columns, columns padded to whole 128-column tiles
+  int32_t col0;          // first column in the column map and in gamma
+  int32_t kst, ngrp;     // 16-K steps, exponent groups (= drain chunks)
+  int32_t gst;           // 16-K steps of a group (divides kWinSteps)
+  int32_t desc0;         // slab descriptor of its first left block
+  int32_t m, mpad;       // rows of the left blocks, padded to whole 128-row tiles
+  int64_t ax_off;        // offset of its per-(group, row) exponents
+};
+struct Col { int32_t f, c; };            // stack column -> output block (within the sector), its column
+struct TPUnit { int32_t st, win, tile, pad; };  // one CTA of the T' kernel (a window, 32 columns) or of winexp_kernel (a group, 32 rows)
+struct MaxUnit { int64_t off; int32_t n, npad, ngrp, out0, tile, pad; };  // one CTA of groupmax_kernel
+// a K2 tile whose K was split over several jobs: F += the partial tiles in order
+struct SplitTile {
+  int64_t out_off;
+  int32_t rows, cols, ld, lstride, slot0, nslot;
+};
 
 // Small-task class: tasks whose four dimensions (m, k1, k2, n) are all at
 // most kSmallDim run in FP64 on CUDA cores instead of the split tensor path
@@ -102,8 +127,10 @@ struct SmallOut {               // an output block with small tasks
 struct SmallSeg { int32_t t0, t1; };  // a segment's tasks (one output block)
 
 struct SChunk {
-  int64_t k1_j0, k1_j1, src0, src1, tp0, tp1, tpu0, tpu1, k2_j0, k2_j1;
-  int64_t sau0, sau1, sdu0, sdu1;  // out-of-core: the chunk's slicing units (A side, D side)
+  int64_t k1_j0, k1_j1, k2_j0, k2_j1;
+  int64_t st0, st1, tpu0, tpu1, gu0, gu1, sp0, sp1;  // stacks, T' units, gamma units, split tiles
+  int64_t au0, au1, du0, du1;      // their slicing units
+  int64_t ax0, ax1, dr0, dr1;      // exponent units: (stack, group, rows) of A, (block, rows) of D
   double k1_flops, k2_flops;
 };
 
@@ -117,51 +144,52 @@ struct SplitState {
   SmallSeg* d_small_seg = nullptr;
   double* d_small_part = nullptr;  // kSmallDim^2 doubles per segment
   int sk = 2;  // 16-K steps per pipeline stage (a tile-shape parameter of the split GEMM)
-  // slabs
+  // stacked operand slabs
   unsigned char *dA = nullptr, *dD = nullptr, *dE = nullptr, *dTP = nullptr;
   int64_t a_bytes = 0, d_bytes = 0, e_bytes = 0, tp_bytes = 0;
   std::vector<SlabDesc> adesc, ddesc, edesc;
-  std::vector<Unit> aunit, dunit, eunit;
+  std::vector<Unit> aunit, dunit;  // slicing units: (block, 128-row tile, 16-K step)
+  std::vector<Unit> drow, erow;           // row units: (block, kRowTile rows)
+  std::vector<TPUnit> axu;                // exponent units of A: (stack, group, kRowTile rows)
+  std::vector<MaxUnit> amu, gu;           // group maxima of A (once) and of T' (per chunk)
   SlabDesc *d_adesc = nullptr, *d_ddesc = nullptr, *d_edesc = nullptr;
-  Unit *d_aunit = nullptr, *d_dunit = nullptr, *d_eunit = nullptr;
+  Unit *d_aunit = nullptr, *d_dunit = nullptr;
+  Unit *d_drow = nullptr, *d_erow = nullptr;
+  TPUnit* d_axu = nullptr;
+  MaxUnit *d_amu = nullptr, *d_gu = nullptr;
   // exponents
-  int *d_rho = nullptr, *d_aown = nullptr, *d_delta = nullptr, *d_zeta = nullptr, *d_eps = nullptr;
-  int *d_gamma = nullptr, *d_cexp = nullptr;
-  int64_t n_rho = 0, n_aown = 0, n_zeta = 0, n_eps = 0, n_gamma = 0, n_cexp = 0;
+  // A: per (group, row) exponents, their maxima rho per (stack, row) and the
+  // drain exponents; T': the same of one chunk (grp, gamma, scale); E, D: eps, zeta
+  int *d_ax = nullptr, *d_rho = nullptr, *d_zeta = nullptr, *d_eps = nullptr, *d_gamma = nullptr, *d_grp = nullptr;
+  uint8_t *d_ascale = nullptr, *d_scale = nullptr;
+  int64_t n_ax = 0, n_rho = 0, n_zeta = 0, n_eps = 0, n_gamma = 0, n_grp = 0;
   // float-float buffers
   float *dTh = nullptr, *dTl = nullptr, *dPh = nullptr, *dPl = nullptr;
   int64_t t_elems = 0;
   // plan
   std::vector<SChunk> chunks;
   std::vector<Job> k1j, k2j;
-  std::vector<Item> k1i, k2i;
-  std::vector<Source> src;
   std::vector<TPTask> tpt;
+  std::vector<int32_t> tab;
+  std::vector<Oct> oct;
+  std::vector<Stack> stk;
+  std::vector<Col> col;
   std::vector<TPUnit> tpu;
+  std::vector<SplitTile> spt;
   Job *d_k1j = nullptr, *d_k2j = nullptr;
-  Item *d_k1i = nullptr, *d_k2i = nullptr;
-  Source* d_src = nullptr;
   TPTask* d_tpt = nullptr;
+  int32_t* d_tab = nullptr;
+  Oct* d_oct = nullptr;
+  Stack* d_stk = nullptr;
+  Col* d_col = nullptr;
   TPUnit* d_tpu = nullptr;
+  SplitTile* d_spt = nullptr;
+  double* d_part = nullptr;      // partial tiles of the split K2 jobs (kRows x kCols doubles each)
+  int64_t n_part = 0;
   int* d_status = nullptr;
-  int* d_counter = nullptr;
-  int* d_phi = nullptr;          // per TP task: phi_t
-  uint8_t* d_scale = nullptr;    // per (task, column) biased drain exponents of one chunk
-  int64_t* d_scoff = nullptr;    // per TP task: offset into d_scale (chunk-local)
-  std::vector<int64_t> scoff;
-  int64_t n_scale = 0;
+  int* d_counter = nullptr;      // job counters: two per term chunk
   int n_sms = 148;
   int spin = int(sp::kSpinLimit);  // polls of each work-loop mbarrier wait of the split GEMM
-  // out-of-core operators: the operator slabs of one chunk are cut per H.psi
-  // from the chunk's FP64 blocks (resident or in its device slot) into a
-  // chunk workspace; the identity slabs stay
-  std::vector<SlabDesc> sdesc;   // per-chunk slicing descriptors (A and D sides)
-  std::vector<Unit> sunit;
-  SlabDesc* d_sdesc = nullptr;
-  Unit* d_sunit = nullptr;
-  std::vector<Unit> resunit_a, resunit_d;  // units of the resident blocks (exponents at prepare)
-  Unit *d_resunit_a = nullptr, *d_resunit_d = nullptr;
-  int64_t ident_u0 = 0;          // first unit of the identity descriptors in aunit
 };
 
 // ------------------------------------------------------------------ device helpers
@@ -180,95 +208,97 @@ __device__ __forceinline__ int exp_of_f(float x) {
 
 // x * 2^e: one multiply by the power of two when that is a normal number (the
 // same correctly rounded result as ldexp), ldexp otherwise
-__device__ __forceinline__ float scale2f(float x, int e) {
-  return (e >= -126 && e <= 127) ? x * __int_as_float((127 + e) << 23) : ldexpf(x, e);
-}
 __device__ __forceinline__ double scale2(double x, int e) {
   return (e >= -1022 && e <= 1023) ? x * __longlong_as_double((long long)(1023 + e) << 52) : ldexp(x, e);
 }
 
-// row exponents of FP64 source matrices: one CTA (128 threads) per (desc, row tile)
-__global__ void rowexp_kernel(const SlabDesc* __restrict__ descs, const Unit* __restrict__ units,
-                              const double* __restrict__ src, int* __restrict__ out, int use_own) {
+// row exponents of FP64 source blocks: one CTA of 32 x 8 threads per (block,
+// kRowTile rows), the eight thread rows share the columns of a row
+constexpr int kRowTile = 32;
+__global__ void __launch_bounds__(256) rowexp_kernel(const SlabDesc* __restrict__ descs, const Unit* __restrict__ units,
+                                                     const double* __restrict__ src, int* __restrict__ out) {
+  __shared__ double sm[8][kRowTile];
   const Unit u = units[blockIdx.x];
-  if (u.ks != 0) return;  // one unit per row tile does the work
   const SlabDesc d = descs[u.desc];
-  const int r = u.tr * 128 + threadIdx.x;
-  if (r >= d.rows) return;
-  int e = kSentinel;
-  if (d.src_off < 0) {
-    e = 1;  // identity row: max |x| = 1 < 2^1
-  } else {
-    double m = 0.0;
-    for (int c = 0; c < d.cols; ++c) m = fmax(m, fabs(src[d.src_off + r + int64_t(c) * d.ld]));
-    e = exp_of(m);
+  const int lane = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const int r = u.tr * kRowTile + lane;
+  double m = 0.0;
+  if (r < d.rows) {
+    const double* p = src + d.src_off + r;
+#pragma unroll 4
+    for (int c = ty; c < d.cols; c += 8) m = fmax(m, fabs(p[int64_t(c) * d.ld]));
   }
-  out[(use_own ? d.own_off : d.exp_off) + r] = e;
+  sm[ty][lane] = m;
+  __syncthreads();
+  if (ty != 0 || r >= d.rows) return;
+#pragma unroll
+  for (int q = 1; q < 8; ++q) m = fmax(m, sm[q][lane]);
+  out[d.exp_off + r] = exp_of(m);
 }
 
-// rho(a', r) = max over blocks of own exponents
-__global__ void rho_kernel(const SlabDesc* __restrict__ descs, const Unit* __restrict__ units,
-                           const int* __restrict__ own, int* __restrict__ rho) {
-  const Unit u = units[blockIdx.x];
-  if (u.ks != 0) return;
-  const SlabDesc d = descs[u.desc];
-  const int r = u.tr * 128 + threadIdx.x;
-  if (r >= d.rows) return;
-  atomicMax(&rho[d.exp_off + r], own[d.own_off + r]);
+// row exponents of the stacked left blocks, one per (group, row): one
+// CTA of 32 x 8 threads per (stack, group, kRowTile rows), one thread row per
+// K of an 8-K piece.  (One exponent per row for all blocks of a sector was
+// measured to cost about 4 bits: the diagonal ramp of the block Hamiltonian
+// sets it for most rows.)
+__global__ void __launch_bounds__(256) winexp_kernel(const TPUnit* __restrict__ units, const Stack* __restrict__ stacks,
+                                                     const Oct* __restrict__ octs, const SlabDesc* __restrict__ descs,
+                                                     const double* __restrict__ src, int* __restrict__ out) {
+  __shared__ double sm[8][kRowTile];
+  const TPUnit u = units[blockIdx.x];
+  const Stack s = stacks[u.st];
+  const int lane = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const int r = u.tile * kRowTile + lane;
+  double m = 0.0;
+  if (r < s.m)
+    for (int o = u.win * 2 * s.gst; o < min((u.win + 1) * 2 * s.gst, s.noct); ++o) {
+      const Oct k = octs[s.oct_off + o];
+      if (k.w < 0 || ty >= k.nk) continue;
+      const SlabDesc d = descs[s.desc0 + k.w];
+      m = fmax(m, d.src_off < 0 ? (r == k.k + ty ? 1.0 : 0.0) : fabs(src[d.src_off + r + int64_t(k.k + ty) * d.ld]));
+    }
+  sm[ty][lane] = m;
+  __syncthreads();
+  if (ty != 0 || r >= s.m) return;
+#pragma unroll
+  for (int q = 1; q < 8; ++q) m = fmax(m, sm[q][lane]);
+  out[s.ax_off + int64_t(u.win) * s.mpad + r] = exp_of(m);
 }
 
-// delta_b = min over non-zero rows of (rho - own)
-__global__ void delta_kernel(const SlabDesc* __restrict__ descs, const Unit* __restrict__ units,
-                             const int* __restrict__ own, const int* __restrict__ rho, int* __restrict__ delta) {
-  const Unit u = units[blockIdx.x];
-  if (u.ks != 0) return;
-  const SlabDesc d = descs[u.desc];
-  const int r = u.tr * 128 + threadIdx.x;
-  if (r >= d.rows) return;
-  const int e = own[d.own_off + r];
-  if (e == kSentinel) return;
-  atomicMin(&delta[d.shift_idx], rho[d.exp_off + r] - e);
-}
-
-__global__ void delta_fix_kernel(int* __restrict__ delta, int n) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n && delta[i] == INT_MAX) delta[i] = 0;
-}
-
-// slab of FP64 matrices (compact layout, split_gemm.cuh): one CTA of 128
-// threads per (desc, row tile, K step); thread = one slab row, 16 K elements =
-// 2 core-matrix columns; rows past the stored ones write nothing
+// slices of FP64 blocks into their stack's slab (compact layout,
+// split_gemm.cuh): one CTA of 128 threads per (block, 128-row tile, 16-K
+// step); thread = one block row, 16 K elements = two 16-byte pieces per
+// slice.  Any row offset and any K offset that is a multiple of 8 keeps the
+// pieces whole
 __global__ void slab_fp64_kernel(const SlabDesc* __restrict__ descs, const Unit* __restrict__ units,
                                  const double* __restrict__ src, const int* __restrict__ rexp,
-                                 const int* __restrict__ delta, unsigned char* __restrict__ slab, int S) {
+                                 unsigned char* __restrict__ slab, int S) {
   const Unit u = units[blockIdx.x];
   const SlabDesc d = descs[u.desc];
-  const int t = threadIdx.x;
-  const int r = u.tr * 128 + t;
-  const int kst = (d.cols + sp::kKS - 1) / sp::kKS;
-  const int trows = sp::tile_rows(d.rows, u.tr);
-  if (t >= trows) return;
-  unsigned char* base = slab + d.slab_off + sp::slab_pos(d.rows, kst, S, u.tr, u.ks, 0);
-  int sigma = 0;
-  if (r < d.rows) {
-    sigma = rexp[d.exp_off + r];
-    if (d.shift_idx >= 0) sigma -= delta[d.shift_idx];
-    if (sigma < -1000) sigma = 0;
-  }
-  const int mi = t >> 3, rr = t & 7;
+  const int r = u.tr * 128 + threadIdx.x;
+  if (r >= d.rows) return;
+  const int row = d.row0 + r, tr = row >> 7, t = row & 127;
+  const int trows = sp::tile_rows(d.R, tr);
+  unsigned char* tile = slab + d.slab_off + sp::slab_pos(d.R, d.kst, S, tr, 0, 0) + (t >> 3) * 256 + (t & 7) * 16;
 #pragma unroll
   for (int kg = 0; kg < 2; ++kg) {
+    const int o = 2 * u.ks + kg;  // 8-K piece of the block
+    if (o >= d.noct) break;
+    const int ko = (d.k0 >> 3) + o;  // 8-K piece of the stack
+    int sigma = rexp[d.exp_off + r + (d.gst ? int64_t(ko / (2 * d.gst)) * d.exp_ld : 0)];
+    if (sigma < -1000) sigma = 0;
     double y[8];
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
-      const int k = u.ks * sp::kKS + kg * 8 + q;
+      const int k = o * 8 + q;
       double x = 0.0;
-      if (r < d.rows && k < d.cols) {
+      if (k < d.cols) {
         if (d.src_off < 0) x = (r == k) ? 1.0 : 0.0;
         else x = src[d.src_off + r + int64_t(k) * d.ld];
       }
       y[q] = scale2(x, sp::kLead - sigma);  // |y| < 2^kLead
     }
+    unsigned char* base = tile + int64_t(ko >> 1) * S * trows * 32 + (ko & 1) * 128;
     float si = 1.f;  // 2^-8i
     for (int i = 0; i < S; ++i, si *= 0x1p-8f) {
       __align__(16) __nv_bfloat16 v[8];
@@ -278,262 +308,257 @@ __global__ void slab_fp64_kernel(const SlabDesc* __restrict__ descs, const Unit*
         y[q] = (y[q] - qi) * 256.0;
         v[q] = __float2bfloat16_rn((float)qi * si);
       }
-      *(uint4*)(base + int64_t(i) * trows * 32 + (mi * 2 + kg) * 128 + rr * 16) = *(const uint4*)v;
+      *(uint4*)(base + int64_t(i) * trows * 32) = *(const uint4*)v;
     }
   }
 }
 
-__global__ void psi_ff_kernel(const double* __restrict__ x, float* __restrict__ h, float* __restrict__ l, int64_t n) {
-  const int64_t stride = int64_t(gridDim.x) * blockDim.x;
-  for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += stride) {
-    const double v = x[i];
-    const float a = (float)v;
-    h[i] = a;
-    l[i] = (float)(v - (double)a);
-  }
-}
-
-// column exponents of the float-float sources: one CTA per source.  T
-// written by K1 has 16-byte aligned columns (column-major, rows padded to a
-// multiple of 4) or rows (row-major, columns padded), so both read it with
-// 16-byte loads: column-major, each warp takes two columns at a time and its
-// lanes four rows each; row-major, each thread takes four neighbouring
-// columns and walks the rows.  Elements past the valid rows / columns are
-// read (they lie inside the padding) but not used.  psi sources (unpadded)
-// keep a warp per column with one float per lane.
-__global__ void cexp_kernel(const Source* __restrict__ src, const float* __restrict__ Th,
-                            const float* __restrict__ Ph, int* __restrict__ cexp) {
-  const Source s = src[blockIdx.x];
-  const int lane = threadIdx.x & 31, nw = blockDim.x >> 5, warp = threadIdx.x >> 5;
-  const float* base = (s.sel ? Ph : Th) + s.off;
-  if (s.rowmajor) {
-    for (int c4 = 4 * threadIdx.x; c4 < s.cols; c4 += 4 * blockDim.x) {
-      float m0 = 0.f, m1 = 0.f, m2 = 0.f, m3 = 0.f;
-#pragma unroll 4
-      for (int r = 0; r < s.rows; ++r) {
-        const float4 v = *reinterpret_cast<const float4*>(base + int64_t(r) * s.ld + c4);
-        m0 = fmaxf(m0, fabsf(v.x));
-        m1 = fmaxf(m1, fabsf(v.y));
-        m2 = fmaxf(m2, fabsf(v.z));
-        m3 = fmaxf(m3, fabsf(v.w));
-      }
-      cexp[s.cexp_off + c4] = exp_of_f(m0);
-      if (c4 + 1 < s.cols) cexp[s.cexp_off + c4 + 1] = exp_of_f(m1);
-      if (c4 + 2 < s.cols) cexp[s.cexp_off + c4 + 2] = exp_of_f(m2);
-      if (c4 + 3 < s.cols) cexp[s.cexp_off + c4 + 3] = exp_of_f(m3);
-    }
-    return;
-  }
-  if (s.sel == 0) {
-    for (int c = 2 * warp; c < s.cols; c += 2 * nw) {
-      const bool two = c + 1 < s.cols;
-      const float* h0 = base + int64_t(c) * s.ld;
-      const float* h1 = h0 + s.ld;
-      float m0 = 0.f, m1 = 0.f;
-      for (int r = 4 * lane; r < s.rows; r += 128) {
-        const float4 v0 = *reinterpret_cast<const float4*>(h0 + r);
-        const float4 v1 = two ? *reinterpret_cast<const float4*>(h1 + r) : make_float4(0.f, 0.f, 0.f, 0.f);
-        const int left = s.rows - r;  // valid rows from r on (>= 1)
-        m0 = fmaxf(m0, fabsf(v0.x));
-        m1 = fmaxf(m1, fabsf(v1.x));
-        if (left > 1) {
-          m0 = fmaxf(m0, fabsf(v0.y));
-          m1 = fmaxf(m1, fabsf(v1.y));
-        }
-        if (left > 2) {
-          m0 = fmaxf(m0, fabsf(v0.z));
-          m1 = fmaxf(m1, fabsf(v1.z));
-        }
-        if (left > 3) {
-          m0 = fmaxf(m0, fabsf(v0.w));
-          m1 = fmaxf(m1, fabsf(v1.w));
-        }
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        m0 = fmaxf(m0, __shfl_xor_sync(0xffffffffu, m0, o));
-        m1 = fmaxf(m1, __shfl_xor_sync(0xffffffffu, m1, o));
-      }
-      if (lane == 0) {
-        cexp[s.cexp_off + c] = exp_of_f(m0);
-        if (two) cexp[s.cexp_off + c + 1] = exp_of_f(m1);
-      }
-    }
-    return;
-  }
-  for (int c = warp; c < s.cols; c += nw) {
-    const float* h = base + int64_t(c) * s.ld;
-    float m = 0.f;
-    for (int r = lane; r < s.rows; r += 32) m = fmaxf(m, fabsf(h[r]));
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if (lane == 0) cexp[s.cexp_off + c] = exp_of_f(m);
-  }
-}
-
-__global__ void fill_kernel(int* __restrict__ p, int64_t n, int v) {
-  const int64_t stride = int64_t(gridDim.x) * blockDim.x;
-  for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += stride) p[i] = v;
-}
-
-// gamma(f, c) = max over tasks of vexp + cexp(c): one CTA per task, threads over columns
-// reference column exponents of the output blocks (max over their tasks)
-// and each task's own exponent phi_t = exponent(v_t 2^-delta)
-__global__ void gamma_kernel(const TPTask* __restrict__ tasks, const Source* __restrict__ src,
-                             const int* __restrict__ cexp, const int* __restrict__ delta, int* __restrict__ gamma,
-                             int* __restrict__ phi) {
-  const TPTask t = tasks[blockIdx.x];
-  const Source s = src[t.src];
-  const int vexp = t.v == 0.0 ? kSentinel : exp_of(t.v) - delta[t.aid];
-  if (threadIdx.x == 0) phi[blockIdx.x] = vexp;
-  if (t.v == 0.0) return;
-  for (int c = threadIdx.x; c < s.cols; c += blockDim.x) {
-    const int ce = cexp[s.cexp_off + c];
-    if (ce == kSentinel) continue;
-    atomicMax(&gamma[t.gcol + c], vexp + ce);
-  }
-}
-
-// per-(task, column) drain exponents d = phi_t + cexp(c) - gamma(c) <= 0 (the
-// factor is 2^d), stored biased as 127 + d (the FP32 exponent field of 2^d);
-// 0 (factor 0) for empty columns, for d below -126 and for the padding up to
-// the next multiple of 128 columns
-__global__ void scale_kernel(const TPTask* __restrict__ tasks, const Source* __restrict__ src,
-                             const int* __restrict__ cexp, const int* __restrict__ gamma,
-                             const int* __restrict__ phi, const int64_t* __restrict__ sc_off, uint8_t* __restrict__ scale) {
-  const TPTask t = tasks[blockIdx.x];
-  const Source s = src[t.src];
-  const int ph = phi[blockIdx.x];
-  uint8_t* out = scale + sc_off[blockIdx.x];
-  const int padded = (s.cols + 127) & ~127;
-  for (int c = threadIdx.x; c < padded; c += blockDim.x) {
-    int d = -127;
-    if (c < s.cols && ph > -1000) {
-      const int ce = cexp[s.cexp_off + c];
-      if (ce > -1000) d = max(-127, ph + ce - gamma[t.gcol + c]);
-    }
-    out[c] = d <= -127 ? 0 : (uint8_t)(127 + d);
-  }
-}
-
-// T' slab of one task: rows = columns of its source (the output columns),
-// K = rows of the source, cut relative to the task's own column exponents
-__global__ void slab_tprime_kernel(const TPTask* __restrict__ tasks, const TPUnit* __restrict__ units,
-                                   const Source* __restrict__ src, const float* __restrict__ Th,
-                                   const float* __restrict__ Tl, const float* __restrict__ Ph,
-                                   const float* __restrict__ Pl, const int* __restrict__ cexp,
-                                   const int* __restrict__ phi, const int* __restrict__ delta,
-                                   unsigned char* __restrict__ slab, int S) {
-  const TPUnit u = units[blockIdx.x];
-  const TPTask t = tasks[u.task];
-  const int ph_t = phi[u.task];
-  const double vs = ldexp(t.v, -delta[t.aid]);
-  const float vh = (float)vs, vl = (float)(vs - (double)vh);
-  const Source s = src[t.src];
-  const int tt = threadIdx.x;
-  const int c = u.tr * 128 + tt;  // slab row = source column
-  const int kst = (s.rows + sp::kKS - 1) / sp::kKS;
-  const int trows = sp::tile_rows(s.cols, u.tr);
-  if (tt >= trows) return;
-  unsigned char* base = slab + t.tp_off + sp::slab_pos(s.cols, kst, S, u.tr, u.ks, 0);
-  const float* H = s.sel ? Ph : Th;
-  const float* Lo = s.sel ? Pl : Tl;
-  int sc = 0;  // the task's own column exponent: |v 2^-delta T[:, c]| < 2^sc
-  if (c < s.cols) {
-    const int ce = cexp[s.cexp_off + c];
-    sc = (ce < -1000 || ph_t < -1000) ? 0 : ph_t + ce;
-  }
-  // the 16 K values of column c: T columns are 16-byte aligned (stride a
-  // multiple of 4), so four 16-byte loads per array; rows past the column's
-  // end read padding or the next column and are set to zero
-  float av[16], bv[16];
-  const int k0 = u.ks * sp::kKS;
-#pragma unroll
-  for (int q = 0; q < 16; ++q) av[q] = bv[q] = 0.f;
-  if (c < s.cols && s.rowmajor) {
-    // row-major T: element (k0 + q, c) at (k0 + q) * ld + c; neighbouring
-    // lanes read neighbouring columns
-#pragma unroll
-    for (int q = 0; q < 16; ++q)
-      if (k0 + q < s.rows) {
-        const int64_t o = s.off + int64_t(k0 + q) * s.ld + c;
-        av[q] = H[o];
-        bv[q] = Lo[o];
-      }
-  } else if (c < s.cols) {
-    const int64_t o = s.off + k0 + int64_t(c) * s.ld;
-    if (!s.sel) {
-#pragma unroll
-      for (int v = 0; v < 4; ++v) {
-        const float4 x = reinterpret_cast<const float4*>(H + o)[v];
-        const float4 y = reinterpret_cast<const float4*>(Lo + o)[v];
-        av[4 * v] = x.x, av[4 * v + 1] = x.y, av[4 * v + 2] = x.z, av[4 * v + 3] = x.w;
-        bv[4 * v] = y.x, bv[4 * v + 1] = y.y, bv[4 * v + 2] = y.z, bv[4 * v + 3] = y.w;
-      }
-#pragma unroll
-      for (int q = 0; q < 16; ++q)
-        if (k0 + q >= s.rows) av[q] = bv[q] = 0.f;
-    } else {
-#pragma unroll
-      for (int q = 0; q < 16; ++q)
-        if (k0 + q < s.rows) {
-          av[q] = H[o + q];
-          bv[q] = Lo[o + q];
-        }
-    }
-  }
-  const int mi = tt >> 3, rr = tt & 7;
-  // the same IEEE operations as the scalar form, on packed FP32 pairs (two
-  // K values per instruction): rint by the 1.5 * 2^23 shift (|x| <= 2^8 + 1
-  // here), the power-of-two scaling as one multiply while the factor is a
-  // normal number, differences as fma(b, -1, a)
-  const int es = sp::kLead - sc;
-  const bool fast = es >= -126 && es <= 127;
-  const float fac = fast ? __int_as_float((127 + es) << 23) : 1.f;
-  const float2 nvh = make_float2(-vh, -vh), vh2 = make_float2(vh, vh), vl2 = make_float2(vl, vl);
-  const float2 nf2 = make_float2(-fac, -fac), f2 = make_float2(fac, fac), m1 = make_float2(-1.f, -1.f);
-  const float2 mg = make_float2(12582912.f, 12582912.f), c256 = make_float2(256.f, 256.f);
-#pragma unroll
-  for (int kg = 0; kg < 2; ++kg) {
-    float2 ph[4], pl[4];
+// eight float-float values (four packed pairs) scaled by 2^es to |x| <
+// 2^kLead and cut into S slices: 16 bytes each at base + i * stride.  rint by
+// the 1.5 * 2^23 shift (|x| <= 2^8 + 1 here); every difference is exact
+__device__ __forceinline__ void cut_oct(float2 (&h)[4], float2 (&l)[4], int es, unsigned char* base, int64_t stride,
+                                        int S) {
+  const float2 m1 = make_float2(-1.f, -1.f), mg = make_float2(12582912.f, 12582912.f), c256 = make_float2(256.f, 256.f);
+  if (es >= -126 && es <= 127) {
+    const float fac = __int_as_float((127 + es) << 23);
+    const float2 f2 = make_float2(fac, fac);
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      const int q = kg * 8 + 2 * j;
-      const float2 a = make_float2(av[q], av[q + 1]), b = make_float2(bv[q], bv[q + 1]);
-      // (a + b) * (vh + vl) in float-float: pn = -RN(a vh), e = a vh - RN(a vh) + a vl + b vh
-      const float2 pn = __fmul2_rn(a, nvh);
-      float2 e = __ffma2_rn(a, vh2, pn);
-      e = __ffma2_rn(a, vl2, e);
-      e = __ffma2_rn(b, vh2, e);
-      // scale to |x| < 2^kLead (exact power of two)
-      float2 h, l;
-      if (fast) {
-        h = __fmul2_rn(pn, nf2);
-        l = __fmul2_rn(e, f2);
-      } else {
-        h = make_float2(ldexpf(-pn.x, es), ldexpf(-pn.y, es));
-        l = make_float2(ldexpf(e.x, es), ldexpf(e.y, es));
-      }
-      const float2 hs = __fadd2_rn(h, l);
-      pl[j] = __ffma2_rn(__ffma2_rn(h, m1, hs), m1, l);  // l - (hs - h)
-      ph[j] = hs;
+      h[j] = __fmul2_rn(h[j], f2);
+      l[j] = __fmul2_rn(l[j], f2);
     }
-    float2 si = make_float2(1.f, 1.f);  // 2^-8i
-    for (int i = 0; i < S; ++i, si = __fmul2_rn(si, make_float2(0x1p-8f, 0x1p-8f))) {
-      uint4 w;
-      uint32_t* wv = &w.x;
+  } else {
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const float2 qi = __ffma2_rn(mg, m1, __fadd2_rn(ph[j], mg));  // rint(ph)
-        const float2 rh = __ffma2_rn(qi, m1, ph[j]);                 // ph - qi, exact
-        const float2 hs = __fadd2_rn(rh, pl[j]);
-        pl[j] = __fmul2_rn(__ffma2_rn(__ffma2_rn(rh, m1, hs), m1, pl[j]), c256);  // (pl - (hs - rh)) * 256
-        ph[j] = __fmul2_rn(hs, c256);
-        const __nv_bfloat162 v2 = __float22bfloat162_rn(__fmul2_rn(qi, si));
-        wv[j] = *reinterpret_cast<const uint32_t*>(&v2);
-      }
-      *(uint4*)(base + int64_t(i) * trows * 32 + (mi * 2 + kg) * 128 + rr * 16) = w;
+    for (int j = 0; j < 4; ++j) {
+      h[j] = make_float2(ldexpf(h[j].x, es), ldexpf(h[j].y, es));
+      l[j] = make_float2(ldexpf(l[j].x, es), ldexpf(l[j].y, es));
     }
+  }
+  float2 si = make_float2(1.f, 1.f);  // 2^-8i
+  for (int i = 0; i < S; ++i, si = __fmul2_rn(si, make_float2(0x1p-8f, 0x1p-8f))) {
+    uint4 w;
+    uint32_t* wv = &w.x;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const float2 qi = __ffma2_rn(mg, m1, __fadd2_rn(h[j], mg));  // rint(h)
+      const float2 rh = __ffma2_rn(qi, m1, h[j]);                 // h - qi, exact
+      const float2 hs = __fadd2_rn(rh, l[j]);
+      l[j] = __fmul2_rn(__ffma2_rn(__ffma2_rn(rh, m1, hs), m1, l[j]), c256);  // (l - (hs - rh)) * 256
+      h[j] = __fmul2_rn(hs, c256);
+      const __nv_bfloat162 v2 = __float22bfloat162_rn(__fmul2_rn(qi, si));
+      wv[j] = *reinterpret_cast<const uint32_t*>(&v2);
+    }
+    *(uint4*)(base + int64_t(i) * stride) = w;
+  }
+}
+
+// psi, once per H.psi: the float-float copy (read by T' for tasks without a
+// right operator), the row exponents and the slabs of its stacks in one
+// kernel; one CTA of 32 x 8 threads per (block, kRowTile rows).  psi is read
+// once in FP64; the cut reads the CTA's own float-float values back from L2
+// and runs in FP32 (an FP64 cut of the same slabs took 280 us instead of 60
+// at L = 32, D = 2048: GB300's FP64 rate is 1/64 of FP32's)
+__global__ void __launch_bounds__(256) psi_slab_kernel(const SlabDesc* __restrict__ descs, const Unit* __restrict__ units,
+                                                       const double* __restrict__ psi, float* Ph, float* Pl,
+                                                       int* __restrict__ eps, unsigned char* __restrict__ slab, int S) {
+  __shared__ float sm[8][kRowTile];
+  const Unit u = units[blockIdx.x];
+  const SlabDesc d = descs[u.desc];
+  const int lane = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const int r = u.tr * kRowTile + lane;
+  float m = 0.f;
+  if (r < d.rows) {
+#pragma unroll 4
+    for (int c = ty; c < d.cols; c += 8) {
+      const int64_t i = d.src_off + r + int64_t(c) * d.ld;
+      const double v = psi[i];
+      const float a = (float)v;
+      Ph[i] = a;
+      Pl[i] = (float)(v - (double)a);
+      m = fmaxf(m, fabsf(a));
+    }
+  }
+  sm[ty][lane] = m;
+  __syncthreads();  // (also orders the float-float copy before its reads below)
+  if (r >= d.rows) return;
+#pragma unroll
+  for (int q = 0; q < 8; ++q) m = fmaxf(m, sm[q][lane]);
+  const int e = exp_of_f(m);
+  if (ty == 0) eps[d.exp_off + r] = e;
+  const int row = d.row0 + r, tr = row >> 7, tt = row & 127, trows = sp::tile_rows(d.R, tr);
+  unsigned char* tile = slab + d.slab_off + sp::slab_pos(d.R, d.kst, S, tr, 0, 0) + (tt >> 3) * 256 + (tt & 7) * 16;
+  for (int o = ty; o < d.noct; o += 8) {
+    float2 h[4], l[4];
+    float* hv = &h[0].x;
+    float* lv = &l[0].x;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int c = o * 8 + q;
+      const int64_t i = d.src_off + r + int64_t(c) * d.ld;
+      hv[q] = c < d.cols ? Ph[i] : 0.f;
+      lv[q] = c < d.cols ? Pl[i] : 0.f;
+    }
+    cut_oct(h, l, sp::kLead - (e < -1000 ? 0 : e), tile + int64_t(o >> 1) * S * trows * 32 + (o & 1) * 128, trows * 32, S);
+  }
+}
+
+// eight consecutive rows k.. of column c of a task's T (or psi) block; rows
+// past nk are zero.  Column-major T has 16-byte aligned pieces (row offsets
+// and strides are multiples of 4): rows past the block's end are read (they
+// lie inside the buffer) and dropped.  Row-major T: neighbouring lanes read
+// neighbouring columns.  psi blocks are unpadded.
+__device__ __forceinline__ void load_oct(const TPTask& t, const float* __restrict__ T, const float* __restrict__ P,
+                                         int k, int c, int nk, float (&x)[8]) {
+  if (t.flags == 0) {
+    const float4* p = reinterpret_cast<const float4*>(T + t.off + k + int64_t(c) * t.ld);
+    const float4 a = p[0], b = nk > 4 ? p[1] : make_float4(0.f, 0.f, 0.f, 0.f);
+    x[0] = a.x, x[1] = a.y, x[2] = a.z, x[3] = a.w, x[4] = b.x, x[5] = b.y, x[6] = b.z, x[7] = b.w;
+#pragma unroll
+    for (int q = 1; q < 8; ++q)
+      if (q >= nk) x[q] = 0.f;
+  } else {
+    const bool rm = (t.flags & kRowMajor) != 0;
+    const float* p = ((t.flags & kFromPsi) ? P : T) + t.off + (rm ? int64_t(k) * t.ld + c : k + int64_t(c) * t.ld);
+    const int64_t step = rm ? t.ld : 1;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) x[q] = q < nk ? p[q * step] : 0.f;
+  }
+}
+
+// h + l += v T of one task, eight K: (a + b) * (vh + vl) in float-float, added
+// with TwoSum
+__device__ __forceinline__ void add_task(const TPTask& t, const float (&av)[8], const float (&bv)[8], float2 (&h)[4],
+                                         float2 (&l)[4]) {
+  const float2 m1 = make_float2(-1.f, -1.f);
+  const float2 vh2 = make_float2(t.vh, t.vh), nvh = make_float2(-t.vh, -t.vh), vl2 = make_float2(t.vl, t.vl);
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const float2 a = make_float2(av[2 * j], av[2 * j + 1]), b = make_float2(bv[2 * j], bv[2 * j + 1]);
+    const float2 pn = __fmul2_rn(a, nvh);               // -RN(a vh)
+    float2 e = __ffma2_rn(a, vh2, pn);
+    e = __ffma2_rn(a, vl2, e);
+    e = __ffma2_rn(b, vh2, e);
+    const float2 h0 = h[j];
+    const float2 hs = __ffma2_rn(pn, m1, h0);           // RN(h0 + p)
+    const float2 nb = __ffma2_rn(hs, m1, h0);           // -(hs - h0)
+    const float2 a1 = __ffma2_rn(__fadd2_rn(hs, nb), m1, h0);
+    const float2 b1 = __ffma2_rn(pn, m1, nb);
+    l[j] = __fadd2_rn(l[j], __fadd2_rn(e, __fadd2_rn(a1, b1)));
+    h[j] = hs;
+  }
+}
+
+// T' slab of one (sector, 192-K window, 32 columns): lane = output column,
+// each of the 12 warps one 16-K step of the window (two 8-K pieces).  The
+// tasks that share the left block and the output block are summed here (T' =
+// sum_t v_t T_t), so K2 runs once per (left block, output block) instead of
+// once per task (1.7 to 3 times fewer flops).  The float-float sums stay in
+// registers until the group's column exponents are known (one exchange
+// through shared memory), so T is read once, in whole 32-byte sectors (row
+// offsets and strides are multiples of 8).
+constexpr int kTPWarps = kWinSteps;
+__global__ void __launch_bounds__(32 * kTPWarps, 2)
+    tprime_kernel(const TPUnit* __restrict__ units, const Stack* __restrict__ stacks, const Col* __restrict__ cols,
+                  const Oct* __restrict__ octs, const int32_t* __restrict__ tab, const TPTask* __restrict__ tasks,
+                  const float* __restrict__ Th, const float* __restrict__ Tl, const float* __restrict__ Ph,
+                  const float* __restrict__ Pl, int* __restrict__ grp, unsigned char* __restrict__ slab, int S) {
+  __shared__ float sm[kTPWarps][32];
+  const TPUnit u = units[blockIdx.x];
+  const Stack& s = stacks[u.st];
+  const int lane = threadIdx.x & 31, wq = threadIdx.x >> 5;
+  const int N = s.N, nf = s.nf, noct = s.noct;
+  const int c = u.tile * 32 + lane, o = u.win * kWinOct + 2 * wq;
+  float2 h[2][4], l[2][4];
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) h[i][j] = l[i][j] = make_float2(0.f, 0.f);
+  if (c < N && o < noct) {  // (noct is even)
+    const Col cm = cols[s.col0 + c];
+    const int32_t* tb = tab + s.tab_off + cm.f;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const Oct k = octs[s.oct_off + o + i];
+      if (k.w < 0) continue;  // (the fill of a stack's last piece)
+      const int t1 = tb[int64_t(k.w) * nf + 1];
+      for (int t = tb[int64_t(k.w) * nf]; t < t1; ++t) {
+        const TPTask tk = tasks[t];
+        float av[8], bv[8];
+        load_oct(tk, Th, Ph, k.k, cm.c, k.nk, av);
+        load_oct(tk, Tl, Pl, k.k, cm.c, k.nk, bv);
+        add_task(tk, av, bv, h[i], l[i]);
+      }
+    }
+  }
+  // normalise, and the column's exponent over its group: |T'(:, c)| < 2^ce
+  const float2 m1 = make_float2(-1.f, -1.f);
+  float m = 0.f;
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const float2 hs = __fadd2_rn(h[i][j], l[i][j]);
+      l[i][j] = __ffma2_rn(__ffma2_rn(h[i][j], m1, hs), m1, l[i][j]);  // l - (hs - h)
+      h[i][j] = hs;
+      m = fmaxf(m, fmaxf(fabsf(hs.x), fabsf(hs.y)));
+    }
+  sm[wq][lane] = m;
+  __syncthreads();
+  if (c >= N) return;
+  if (o >= noct) return;
+  const int gst = s.gst, w0 = wq / gst * gst;  // the warps of this step's exponent group
+  for (int q = w0; q < w0 + gst; ++q) m = fmaxf(m, sm[q][lane]);
+  const int ce = exp_of_f(m);
+  if (wq == w0) grp[s.grp_off + int64_t((u.win * kWinSteps + w0) / gst) * s.Npad + c] = ce;
+  const int trows = sp::tile_rows(N, c >> 7), tt = c & 127, es = sp::kLead - (ce < -1000 ? 0 : ce);
+  unsigned char* base = slab + s.tp_off + sp::slab_pos(N, s.kst, S, c >> 7, o >> 1, 0) + (tt >> 3) * 256 + (tt & 7) * 16;
+  cut_oct(h[0], l[0], es, base, trows * 32, S);
+  cut_oct(h[1], l[1], es, base + 128, trows * 32, S);
+}
+
+// group maxima: out(x) = max over the groups of the exponents of row (or
+// column) x, and the drain exponents d = own(group, x) - out(x) <= 0 (the factor is
+// 2^d), stored biased as 127 + d (the FP32 exponent field of 2^d); 0 (factor
+// 0) for zero rows, for d below -126 and for the padding up to the next
+// multiple of 128.  One CTA of 128 x 4 threads per (stack, 128 rows).
+__global__ void __launch_bounds__(512) groupmax_kernel(const MaxUnit* __restrict__ units, const int* __restrict__ grp,
+                                                       int* __restrict__ out, uint8_t* __restrict__ scale) {
+  __shared__ int sm[4][128];
+  const MaxUnit u = units[blockIdx.x];
+  const int tt = threadIdx.x & 127, ty = threadIdx.x >> 7, c = u.tile * 128 + tt;
+  const int* g = grp + u.off + c;
+  int m = kSentinel;
+  if (c < u.n) {
+#pragma unroll 8
+    for (int q = ty; q < u.ngrp; q += 4) m = max(m, g[int64_t(q) * u.npad]);
+  }
+  sm[ty][tt] = m;
+  __syncthreads();
+  m = max(max(sm[0][tt], sm[1][tt]), max(sm[2][tt], sm[3][tt]));
+  if (ty == 0 && c < u.n) out[u.out0 + c] = m;
+  uint8_t* sc = scale + u.off + c;
+#pragma unroll 8
+  for (int q = ty; q < u.ngrp; q += 4) {
+    int d = -127;
+    if (c < u.n) {
+      const int e = g[int64_t(q) * u.npad];
+      if (e > -1000) d = max(-127, e - m);
+    }
+    sc[int64_t(q) * u.npad] = d <= -127 ? 0 : (uint8_t)(127 + d);
+  }
+}
+
+// F += the partial tiles of the K2 tiles whose K was split, in K order; one
+// CTA per (tile, 16 TMEM columns)
+__global__ void __launch_bounds__(256) part_reduce_kernel(const SplitTile* __restrict__ tiles,
+                                                          const double* __restrict__ part, double* __restrict__ F) {
+  const SplitTile t = tiles[blockIdx.x];
+  const int p = threadIdx.x & 127;
+  if (p >= t.rows) return;
+  for (int q = blockIdx.y * 16 + (threadIdx.x >> 7); q < min(t.cols, int(blockIdx.y) * 16 + 16); q += 2) {
+    double x = 0.0;
+    for (int i = 0; i < t.nslot; ++i) x += part[(int64_t(t.slot0 + i) * sp::kCols + q) * sp::kRows + p];
+    F[t.out_off + (t.lstride ? int64_t(p) * t.ld + q : p + int64_t(q) * t.ld)] += x;
   }
 }
 
@@ -644,52 +669,44 @@ int dput(T** p, const std::vector<T>& h, std::string& err) {
 }
 
 // bytes of a compact slab (split_gemm.cuh): full 128-row tiles and a last tile of its rows rounded up to 16
-int64_t slab_bytes(int rows, int cols, int S) {
+int64_t slab_bytes(int rows, int kst, int S) {
   const int nt = (rows + 127) / 128;
   if (nt == 0) return 0;
-  return (int64_t(nt - 1) * kSub + sp::tile_rows(rows, nt - 1) * 32) * ((cols + sp::kKS - 1) / sp::kKS) * S;
+  return (int64_t(nt - 1) * kSub + sp::tile_rows(rows, nt - 1) * 32) * kst * S;
 }
 
-void add_units(std::vector<Unit>& u, int desc, int rows, int cols) {
-  for (int tr = 0; tr < (rows + 127) / 128; ++tr)
-    for (int ks = 0; ks < (cols + sp::kKS - 1) / sp::kKS; ++ks) u.push_back(Unit{desc, tr, ks, 0});
+void add_units(std::vector<Unit>& u, int desc, const SlabDesc& d) {
+  for (int tr = 0; tr < (d.rows + 127) / 128; ++tr)
+    for (int ks = 0; ks < (d.noct + 1) / 2; ++ks) u.push_back(Unit{desc, tr, ks, 0});
 }
 
-// MMA N of job column tile tc (kCols wide) of a block with `cols` columns
+// MMA N of job column tile tc (kCols wide) of an operand with `cols` rows
 int32_t nmma_of(int cols, int tc) {
   const int rem = std::min(sp::kCols, cols - tc * sp::kCols);
   return int32_t((rem + 15) / 16 * 16);
 }
 
-// byte offset of job column tile tc (kCols = 128 wide) in a compact B slab: its row tile
-int64_t btile_off(int tc, int kst, int S) { return int64_t(tc) * kst * S * kSub; }
+// byte offset of 128-row tile t of a compact slab
+int64_t tile_off(int t, int kst, int S) { return int64_t(t) * kst * S * kSub; }
 
-// Modelled cost of one orientation of a tile product: the M side has Mr rows
-// (128-row tiles, every MMA has M = 128), the N side Nr rows (tiles of kCols,
-// MMA N = the valid extent rounded up to 16); steps / chunks are the 16-K
-// steps and drain chunks summed over the items.  Measured on GB300: an MMA
-// (M = 128, K = 16) takes about max(N / 2, 32 + N / 4) cycles (48 at N = 64,
-// 64 at N = 128), and a drain exposes about 23 cycles per column.
+// Modelled cost (cycles) of one tile column of N MMA columns: measured on
+// GB300, an MMA (M = 128, K = 16) takes about max(N / 2, 32 + N / 4) cycles
+// (48 at N = 64, 64 at N = 128), and a drain exposes about 23 cycles per column
+double tile_cost(double nm, double steps, double chunks, int S) {
+  return S * (S + 1) / 2.0 * std::max(nm / 2.0, 32.0 + nm / 4.0) * steps + 23.0 * nm * chunks;
+}
+// ... and of one orientation of a product: the M side has Mr rows (128-row
+// tiles, every MMA has M = 128), the N side Nr rows (tiles of kCols, MMA N =
+// the valid extent rounded up to 16)
 double orient_cost(int Mr, int Nr, double steps, double chunks, int S) {
-  const double pairs = S * (S + 1) / 2.0;
   double per = 0.0;
-  for (int tc = 0; tc < (Nr + sp::kCols - 1) / sp::kCols; ++tc) {
-    const double nm = nmma_of(Nr, tc);
-    per += pairs * std::max(nm / 2.0, 32.0 + nm / 4.0) * steps + 23.0 * nm * chunks;
-  }
+  for (int tc = 0; tc < (Nr + sp::kCols - 1) / sp::kCols; ++tc) per += tile_cost(nmma_of(Nr, tc), steps, chunks, S);
   return per * ((Mr + 127) / 128);
 }
 
-int exp_host(double x) {
-  if (x == 0.0) return kSentinel;
-  int e;
-  std::frexp(x, &e);
-  return e;
-}
-
 // the stripe GEMM instantiated for each mode and slice count
-using GemmFn = void (*)(const sp::Job*, int, const sp::Item*, const unsigned char*, const unsigned char*, const int*,
-                        const int*, int, float*, float*, double*, int*, int*, sp::TaskScale, int, int);
+using GemmFn = void (*)(const sp::Job*, int, const unsigned char*, const unsigned char*, const int*, const int*, int,
+                        float*, float*, double*, double*, int*, int*, const uint8_t*, const uint8_t*, int, int);
 GemmFn gemm_fn(int mode, int S) {
   static const GemmFn t[2][sp::kMaxS - 1] = {
       {sp::split_gemm_kernel<sp::MODE_T, 2>, sp::split_gemm_kernel<sp::MODE_T, 3>, sp::split_gemm_kernel<sp::MODE_T, 4>,
@@ -699,23 +716,37 @@ GemmFn gemm_fn(int mode, int S) {
   return t[mode == sp::MODE_F ? 1 : 0][S - 2];
 }
 
-void launch_gemm(int mode, cudaStream_t s, SplitState* st, const Job* jobs, int njobs, const Item* items,
-                 const unsigned char* A, const unsigned char* B, const int* rexp, const int* cexp, float* Th,
-                 float* Tl, double* F, sp::TaskScale ts) {
+void launch_gemm(int mode, cudaStream_t s, SplitState* st, const Job* jobs, int njobs, int* counter,
+                 const unsigned char* A, const unsigned char* B, const int* rexp, const int* cexp, double* F) {
   if (njobs <= 0) return;
   // only the stages in use: the rest of the SM's 256 KB stays L1 (the drain's
-  // spills and the job / item / exponent loads; launching with the maximum
-  // measured 17 % slower K2)
+  // spills and the job / exponent loads; launching with the maximum measured
+  // 17 % slower K2)
   const int smem = sp::stages_of(st->S, st->sk) * sp::stage_bytes_of(st->S, st->sk) + 1024;
   const int grid = std::min(njobs, st->n_sms);
-  cudaMemsetAsync(st->d_counter, 0, sizeof(int), s);
-  gemm_fn(mode, st->S)<<<grid, sp::kThreads, smem, s>>>(jobs, njobs, items, A, B, rexp, cexp, 2 * sp::kLead, Th, Tl, F,
-                                                        st->d_status, st->d_counter, ts, st->sk, st->spin);
+  gemm_fn(mode, st->S)<<<grid, sp::kThreads, smem, s>>>(jobs, njobs, A, B, rexp, cexp, 2 * sp::kLead, st->dTh, st->dTl,
+                                                        F, st->d_part, st->d_status, counter, st->d_ascale,
+                                                        st->d_scale, st->sk, st->spin);
 }
 
 }  // namespace
 
 
+// Plan of the split path.  Every product of a term chunk is one tile of a
+// large "stacked" product:
+//
+//  * K1, per right input sector b: T_b = E_b D_b^T, E_b the psi blocks with
+//    right sector b above one another, D_b the right operator blocks with
+//    input sector b above one another (K = dim b).  At qc16 sizes (sectors of
+//    1 to 129) one product per (D, E) pair filled 16 % of its 128 x 128 MMA
+//    tiles; the stacks fill them, and 91 % of their (D, E) pairs are needed
+//    (tiles without a needed pair are left out).
+//  * T': for each (left block A, output block f) the sum of its tasks' v T.
+//  * K2, per left output sector a: the psi blocks of a lie side by side in
+//    psi, one column-major matrix F_a, and F_a += [A_1 A_2 ..] [T'_1; T'_2; ..]
+//    with the left blocks of output sector a side by side along K (each
+//    padded to 8).  Drain chunks = exponent groups are equal pieces of this K
+//    axis, however many blocks they span.
 int split_prepare(su2_env* env, int S, std::string& err) {
   env->info.split_slices = S;
   env->info.split_stage_k = 2;
@@ -740,93 +771,29 @@ int split_prepare(su2_env* env, int S, std::string& err) {
   }
   st->d_status = env->ctx->d_status;
   if (env->spin_limit > 0) st->spin = env->spin_limit;
-  if (int rc0 = dalloc(&st->d_counter, 1, err)) return rc0;
   const auto& B = env->blocks;
   const auto& ls = env->lsec;
+  const auto& rs = env->rsec;
   const auto& L = env->L;
   const auto& R = env->R;
-  const int nLb = int(L.blocks.size());
-  // ---------------------------------------------------------- A side
-  std::vector<int64_t> rho_off(ls.size());
-  int64_t acc = 0;
-  for (size_t a = 0; a < ls.size(); ++a) {
-    rho_off[a] = acc;
-    acc += ls[a].dim;
-  }
-  st->n_rho = acc;
-  const bool ooc = env->os.on;  // out-of-core operators: block slabs live in a per-chunk workspace
-  int64_t own = 0, ab = 0;
-  for (int bi = 0; bi < nLb; ++bi) {
-    const OpBlock& ob = L.blocks[bi];
-    st->adesc.push_back(SlabDesc{ob.off, ooc ? -1 : ab, ob.rows, ob.cols, ob.rows, int32_t(rho_off[ob.qo]), bi,
-                                 int32_t(own), 0, 0});
-    own += ob.rows;
-    if (!ooc) ab += slab_bytes(ob.rows, ob.cols, S);
-  }
-  for (size_t a = 0; a < ls.size(); ++a) {
-    const int d = ls[a].dim;
-    st->adesc.push_back(
-        SlabDesc{-1, ab, d, d, d, int32_t(rho_off[a]), int32_t(nLb + a), int32_t(own), 0, 0});
-    own += d;
-    ab += slab_bytes(d, d, S);
-  }
-  st->n_aown = own;
-  st->a_bytes = ab;
-  for (size_t i = 0; i < st->adesc.size(); ++i) {
-    if (int(i) == nLb) st->ident_u0 = int64_t(st->aunit.size());
-    add_units(st->aunit, int(i), st->adesc[i].rows, st->adesc[i].cols);
-  }
-  if (nLb == int(st->adesc.size())) st->ident_u0 = int64_t(st->aunit.size());
-  // ---------------------------------------------------------- D side
-  int64_t zoff = 0, db = 0;
-  std::vector<int64_t> zeta_off(R.blocks.size());
-  for (size_t bi = 0; bi < R.blocks.size(); ++bi) {
-    const OpBlock& ob = R.blocks[bi];
-    zeta_off[bi] = zoff;
-    st->ddesc.push_back(SlabDesc{ob.off, ooc ? -1 : db, ob.rows, ob.cols, ob.rows, int32_t(zoff), -1, -1, 0, 0});
-    zoff += ob.rows;
-    if (!ooc) db += slab_bytes(ob.rows, ob.cols, S);
-  }
-  st->n_zeta = zoff;
-  st->d_bytes = db;
-  for (size_t i = 0; i < st->ddesc.size(); ++i) add_units(st->dunit, int(i), st->ddesc[i].rows, st->ddesc[i].cols);
-  // ---------------------------------------------------------- E side (psi blocks)
-  int64_t eoff = 0, eb = 0;
-  std::vector<int64_t> eps_off(B.size()), e_slab(B.size());
-  for (size_t e = 0; e < B.size(); ++e) {
-    eps_off[e] = eoff;
-    e_slab[e] = eb;
-    st->edesc.push_back(SlabDesc{B[e].offset, eb, B[e].rows, B[e].cols, B[e].rows, int32_t(eoff), -1, -1, 0, 0});
-    eoff += B[e].rows;
-    eb += slab_bytes(B[e].rows, B[e].cols, S);
-  }
-  st->n_eps = eoff;
-  st->e_bytes = eb;
-  for (size_t i = 0; i < st->edesc.size(); ++i) add_units(st->eunit, int(i), st->edesc[i].rows, st->edesc[i].cols);
-  // gamma offsets per psi block (output columns)
-  std::vector<int64_t> goff(B.size());
-  int64_t gacc = 0;
-  for (size_t f = 0; f < B.size(); ++f) {
-    goff[f] = gacc;
-    gacc += B[f].cols;
-  }
-  st->n_gamma = gacc;
-  if (st->n_rho >= INT32_MAX || st->n_zeta >= INT32_MAX || st->n_eps >= INT32_MAX || st->n_gamma >= INT32_MAX) {
-    err = "exponent tables too large";
-    return SU2_EINVAL;
-  }
-  // ---------------------------------------------------------- chunk plan
+  const int nB = int(B.size()), nl = int(ls.size()), nr = int(rs.size());
+  const int nLb = int(L.blocks.size()), nRb = int(R.blocks.size());
   const int nterms = int(env->table.terms.size());
-  std::vector<std::vector<int64_t>> by_term(nterms);
-  // small-task class, in task order (sorted by output block)
+  const int64_t nt = int64_t(env->tasks.size());
+  const bool ooc = env->os.on;  // out-of-core operators: the slabs of a chunk are cut per H.psi into a workspace
   auto is_small = [&](const Task& t) {
     const Block& Fb = B[t.f];
     const Block& Eb = B[t.e];
     return std::max(std::max(Fb.rows, Fb.cols), std::max(Eb.rows, Eb.cols)) <= kSmallDim;
   };
-  for (int64_t i = 0; i < int64_t(env->tasks.size()); ++i) {
+  // ---------------------------------------------------------- small-task class, in task order (sorted by output block)
+  std::vector<int64_t> big;  // the other tasks
+  for (int64_t i = 0; i < nt; ++i) {
     const Task& t = env->tasks[i];
-    if (!is_small(t)) continue;
+    if (!is_small(t)) {
+      big.push_back(i);
+      continue;
+    }
     const Block& Fb = B[t.f];
     const Block& Eb = B[t.e];
     const int32_t ti = int32_t(st->small.size());
@@ -843,254 +810,428 @@ int split_prepare(su2_env* env, int S, std::string& err) {
                                   t.dblk >= 0 ? R.blocks[t.dblk].off : -1, Fb.rows, Eb.rows, Eb.cols, Fb.cols, t.v});
     st->small_seg.back().t1 = ti + 1;
   }
-  for (int64_t i = 0; i < int64_t(env->tasks.size()); ++i)
-    if (!is_small(env->tasks[i])) by_term[env->tasks[i].term].push_back(i);
-  int64_t budget = env->split_budget;
-  if (budget <= 0) {  // default: a quarter of the free device memory, at most 16 GiB
-    size_t fr = 0, tot = 0;
-    cudaMemGetInfo(&fr, &tot);
-    budget = std::min<int64_t>(int64_t(16) << 30, std::max<int64_t>(int64_t(fr) / 4, int64_t(1) << 30));
-  }
-  std::vector<int> starts{0};
-  if (ooc) {
-    starts = env->os.starts;
-  } else {
-    int64_t bytes = 0;
-    std::unordered_map<uint64_t, char> seen;
-    for (int ti = 0; ti < nterms; ++ti) {
-      int64_t add = 0;
-      std::unordered_map<uint64_t, char> mine;
-      for (int64_t i : by_term[ti]) {
-        const Task& t = env->tasks[i];
-        const Block& E = B[t.e];
-        const int n = B[t.f].cols;
-        add += slab_bytes(n, E.rows, S);
-        if (t.dblk >= 0) {
-          const uint64_t key = (uint64_t(uint32_t(t.dblk)) << 32) | uint32_t(t.e);
-          if (!seen.count(key) && !mine.count(key)) {
-            mine[key] = 1;
-            add += 8 * int64_t(E.rows) * n;
-          }
-        }
-      }
-      if (bytes > 0 && bytes + add > budget) {
-        starts.push_back(ti);
-        seen.clear();
-        bytes = 0;
-      }
-      for (auto& kv : mine) seen.insert(kv);
-      bytes += add;
+  // ---------------------------------------------------------- psi by left sector (F) and by right sector (E)
+  std::vector<int> f_first(size_t(nl), -1), f_num(size_t(nl), 0), f_cols(size_t(nl), 0), f_loc(size_t(nB), 0);
+  std::vector<int> f_col0(size_t(nl), 0);
+  for (int e = 0; e < nB; ++e) {
+    const int a = B[e].a;
+    if (f_first[a] < 0) {
+      f_first[a] = e;
+      f_col0[a] = int(st->col.size());
     }
-    starts.push_back(nterms);
+    // (the canonical block order keeps the blocks of a left sector together)
+    if (e != f_first[a] + f_num[a] || B[e].offset != B[f_first[a]].offset + int64_t(f_cols[a]) * B[e].rows) {
+      err = "split plan: the psi blocks of a left sector are not contiguous";
+      return SU2_EINVAL;
+    }
+    f_loc[e] = f_num[a]++;
+    f_cols[a] += B[e].cols;
+    for (int c = 0; c < B[e].cols; ++c) st->col.push_back(Col{f_loc[e], c});
   }
-  int64_t max_t = 0, max_tp = 0, max_cexp = 0, max_as = 0, max_ds = 0;
-  const int64_t nt = int64_t(env->tasks.size());
-  if (ooc) {  // units of the resident blocks: their exponents are taken once, at prepare
-    for (size_t i = 0; i < size_t(nLb); ++i)
-      if (L.blocks[i].off < env->os.prefix) add_units(st->resunit_a, int(i), st->adesc[i].rows, st->adesc[i].cols);
-    for (size_t i = st->ident_u0; i < st->aunit.size(); ++i) st->resunit_a.push_back(st->aunit[i]);
-    for (size_t i = 0; i < R.blocks.size(); ++i)
-      if (R.blocks[i].off < env->os.prefix) add_units(st->resunit_d, int(i), st->ddesc[i].rows, st->ddesc[i].cols);
+  st->n_gamma = int64_t(st->col.size());
+  std::vector<int> e_row0(size_t(nB), 0), e_rows(size_t(nr), 0);
+  std::vector<std::vector<int>> e_of(static_cast<size_t>(nr));
+  for (int e = 0; e < nB; ++e) {
+    e_row0[e] = e_rows[B[e].b];
+    e_rows[B[e].b] += (B[e].rows + 7) & ~7;  // T rows of a block start at a multiple of 8 (whole 32-byte sectors)
+    e_of[B[e].b].push_back(e);
   }
-  for (size_t c = 0; c + 1 < starts.size(); ++c) {
-    const int t0 = starts[c], t1 = starts[c + 1];
-    SChunk ch{};
-    // out-of-core: the chunk's operator blocks, sliced into the chunk
-    // workspace (A blocks after the identity slabs) from their device place
-    // for this chunk
-    std::unordered_map<int, int64_t> aloc, dloc;
-    if (ooc) {
-      ch.sau0 = ch.sdu0 = 0;
-      std::vector<Unit> ua, ud;
-      int64_t ab_c = ab, db_c = 0;
-      for (int ti = t0; ti < t1; ++ti)
+  std::vector<int64_t> eps_off(static_cast<size_t>(nr)), e_slab(static_cast<size_t>(nr));
+  for (int b = 0; b < nr; ++b) {
+    const int kst = (rs[b].dim + sp::kKS - 1) / sp::kKS;
+    eps_off[b] = st->n_eps;
+    e_slab[b] = st->e_bytes;
+    for (int e : e_of[b]) {
+      const int id = int(st->edesc.size());
+      st->edesc.push_back(SlabDesc{B[e].offset, e_slab[b], B[e].rows, B[e].cols, B[e].rows, e_row0[e], 0, e_rows[b], kst,
+                                   2 * kst, int32_t(eps_off[b] + e_row0[e]), 0, 0, 0});
+      for (int tr = 0; tr < (B[e].rows + kRowTile - 1) / kRowTile; ++tr) st->erow.push_back(Unit{id, tr, 0, 0});
+    }
+    st->n_eps += e_rows[b];
+    st->e_bytes += slab_bytes(e_rows[b], kst, S);
+  }
+  if (st->n_eps >= INT32_MAX || st->n_gamma >= INT32_MAX) {
+    err = "exponent tables too large";
+    return SU2_EINVAL;
+  }
+  // the identity of left sector a is left block nLb + a
+  auto a_id = [&](const Task& t) { return t.ablk >= 0 ? t.ablk : nLb + B[t.e].a; };
+  auto a_out = [&](int id) { return id < nLb ? L.blocks[id].qo : id - nLb; };
+  auto a_cols = [&](int id) { return id < nLb ? L.blocks[id].cols : ls[id - nLb].dim; };
+  auto d_in = [&](int d) { return R.blocks[d].qi; };
+  // ---------------------------------------------------------- term chunks
+  // consecutive terms in the order of their left operators' first use (the
+  // tasks of one left operator share their A blocks, and are merged within a
+  // chunk), until T (float-float) and the T' slabs of the chunk reach the
+  // budget; out-of-core: the planner's ranges of terms
+  std::vector<int> chunk_of(size_t(std::max(nterms, 1)), 0);
+  int nch = 1;
+  if (ooc) {
+    nch = int(env->os.starts.size()) - 1;
+    for (int c = 0; c < nch; ++c)
+      for (int ti = env->os.starts[c]; ti < env->os.starts[c + 1]; ++ti) chunk_of[ti] = c;
+  } else {
+    int64_t budget = env->split_budget;
+    if (budget <= 0) {  // default: a quarter of the free device memory, at most 16 GiB
+      size_t fr = 0, tot = 0;
+      cudaMemGetInfo(&fr, &tot);
+      budget = std::min<int64_t>(int64_t(16) << 30, std::max<int64_t>(int64_t(fr) / 4, int64_t(1) << 30));
+    }
+    std::vector<int> order;
+    {
+      std::unordered_map<int, int> rank;
+      std::vector<std::pair<int, int>> key;
+      for (int ti = 0; ti < nterms; ++ti)
+        key.push_back({rank.emplace(env->table.terms[ti].A, int(rank.size())).first->second, ti});
+      std::sort(key.begin(), key.end());
+      for (const auto& k : key) order.push_back(k.second);
+    }
+    std::vector<std::vector<int64_t>> by_term(static_cast<size_t>(nterms));
+    for (int64_t i : big) by_term[env->tasks[i].term].push_back(i);
+    std::vector<int> a_seen(size_t(nLb) + nl, -1), d_seen(size_t(std::max(nRb, 1)), -1);
+    int cur = 0;
+    int64_t bytes = 0;
+    for (int ti : order) {
+      auto add_of = [&]() {
+        int64_t add = 0;
         for (int64_t i : by_term[ti]) {
           const Task& t = env->tasks[i];
-          if (t.ablk >= 0 && !aloc.count(t.ablk)) {
-            SlabDesc d = st->adesc[t.ablk];
-            d.src_off = env->os.dev_off(L.blocks[t.ablk].off, int(c));
-            d.slab_off = ab_c;
-            aloc[t.ablk] = ab_c;
-            ab_c += slab_bytes(d.rows, d.cols, S);
-            st->sdesc.push_back(d);
-            add_units(ua, int(st->sdesc.size()) - 1, d.rows, d.cols);
+          const int id = a_id(t);
+          if (a_seen[id] != cur) {
+            a_seen[id] = cur;
+            add += int64_t((a_cols(id) + 7) & ~7) * f_cols[a_out(id)] * 2 * S;
           }
-          if (t.dblk >= 0 && !dloc.count(t.dblk)) {
-            SlabDesc d = st->ddesc[t.dblk];
-            d.src_off = env->os.dev_off(R.blocks[t.dblk].off, int(c));
-            d.slab_off = db_c;
-            dloc[t.dblk] = db_c;
-            db_c += slab_bytes(d.rows, d.cols, S);
-            st->sdesc.push_back(d);
-            add_units(ud, int(st->sdesc.size()) - 1, d.rows, d.cols);
+          if (t.dblk >= 0 && d_seen[t.dblk] != cur) {
+            d_seen[t.dblk] = cur;
+            add += 8 * int64_t(R.blocks[t.dblk].rows) * e_rows[d_in(t.dblk)];
           }
         }
-      ch.sau0 = int64_t(st->sunit.size());
-      st->sunit.insert(st->sunit.end(), ua.begin(), ua.end());
-      ch.sau1 = ch.sdu0 = int64_t(st->sunit.size());
-      st->sunit.insert(st->sunit.end(), ud.begin(), ud.end());
-      ch.sdu1 = int64_t(st->sunit.size());
-      max_as = std::max(max_as, ab_c);
-      max_ds = std::max(max_ds, db_c);
+        return add;
+      };
+      int64_t add = add_of();
+      if (bytes > 0 && bytes + add > budget) {
+        cur += 1;
+        bytes = 0;
+        add = add_of();
+      }
+      chunk_of[ti] = cur;
+      bytes += add;
     }
-    auto aslab = [&](int aid) -> int64_t { return (ooc && aid < nLb) ? aloc.at(aid) : st->adesc[aid].slab_off; };
-    auto dslab = [&](int dblk) -> int64_t { return ooc ? dloc.at(dblk) : st->ddesc[dblk].slab_off; };
+    nch = cur + 1;
+  }
+  std::vector<std::vector<int64_t>> chunk_tasks(static_cast<size_t>(nch));
+  for (int64_t i : big) chunk_tasks[chunk_of[env->tasks[i].term]].push_back(i);
+  // ---------------------------------------------------------- per chunk
+  int64_t max_t = 0, max_tp = 0, max_as = 0, max_ds = 0;
+  std::vector<int> a_w(size_t(nLb) + nl, -1), a_stamp(size_t(nLb) + nl, -1), d_row(size_t(std::max(nRb, 1)), 0),
+      d_stamp(size_t(std::max(nRb, 1)), -1), d_loc(size_t(std::max(nRb, 1)), 0);
+  for (int c = 0; c < nch; ++c) {
+    const auto& mine = chunk_tasks[c];
+    SChunk ch{};
     ch.k1_j0 = int64_t(st->k1j.size());
-    ch.src0 = int64_t(st->src.size());
-    ch.tp0 = int64_t(st->tpt.size());
-    ch.tpu0 = int64_t(st->tpu.size());
     ch.k2_j0 = int64_t(st->k2j.size());
-    std::unordered_map<uint64_t, int> umap;  // (dblk, e) -> source index (chunk-local)
-    std::unordered_map<int, int> pmap;       // e -> psi source index
-    int64_t tsz = 0, csz = 0, tpsz = 0, scsz = 0;
+    ch.st0 = int64_t(st->stk.size());
+    ch.tpu0 = int64_t(st->tpu.size());
+    ch.gu0 = int64_t(st->gu.size());
+    ch.sp0 = int64_t(st->spt.size());
+    ch.au0 = int64_t(st->aunit.size());
+    ch.du0 = int64_t(st->dunit.size());
+    ch.ax0 = int64_t(st->axu.size());
+    ch.dr0 = int64_t(st->drow.size());
+    int64_t a_pos = ooc ? 0 : st->a_bytes, d_pos = ooc ? 0 : st->d_bytes, tsz = 0, tpsz = 0, grpsz = 0;
+    // the chunk's left blocks by output sector and right blocks by input sector
+    std::vector<std::vector<int>> a_of(static_cast<size_t>(nl)), d_of(static_cast<size_t>(nr));
+    for (int64_t i : mine) {
+      const Task& t = env->tasks[i];
+      const int id = a_id(t);
+      if (a_stamp[id] != c) {
+        a_stamp[id] = c;
+        a_of[a_out(id)].push_back(id);
+      }
+      if (t.dblk >= 0 && d_stamp[t.dblk] != c) {
+        d_stamp[t.dblk] = c;
+        d_of[d_in(t.dblk)].push_back(t.dblk);
+      }
+    }
+    for (auto& v : a_of) std::sort(v.begin(), v.end());
+    for (auto& v : d_of) std::sort(v.begin(), v.end());
+    // ---- K1: one stacked product per right input sector
+    std::vector<int64_t> t_off(size_t(nr), -1), d_slab(size_t(nr), 0), zeta_off(size_t(nr), 0);
+    std::vector<int> ldT(size_t(nr), 0), d_rows(size_t(nr), 0), t_rm(size_t(nr), 0);
+    for (int b = 0; b < nr; ++b) {
+      if (d_of[b].empty()) continue;
+      const int kst = (rs[b].dim + sp::kKS - 1) / sp::kKS;
+      for (size_t q = 0; q < d_of[b].size(); ++q) {
+        const int d = d_of[b][q];
+        d_row[d] = d_rows[b];
+        d_loc[d] = int(q);
+        d_rows[b] += R.blocks[d].rows;
+      }
+      zeta_off[b] = st->n_zeta;
+      d_slab[b] = d_pos;
+      for (int d : d_of[b]) {
+        const OpBlock& ob = R.blocks[d];
+        const int id = int(st->ddesc.size());
+        st->ddesc.push_back(SlabDesc{ooc ? env->os.dev_off(ob.off, c) : ob.off, d_pos, ob.rows, ob.cols, ob.rows, d_row[d], 0,
+                                     d_rows[b], kst, 2 * kst, int32_t(zeta_off[b] + d_row[d]), 0, 0, 0});
+        add_units(st->dunit, id, st->ddesc.back());
+        for (int tr = 0; tr < (ob.rows + kRowTile - 1) / kRowTile; ++tr) st->drow.push_back(Unit{id, tr, 0, 0});
+      }
+      st->n_zeta += d_rows[b];
+      d_pos += slab_bytes(d_rows[b], kst, S);
+      const double nch2 = (kst + sp::kChunkSteps - 1) / sp::kChunkSteps;
+      // M along the psi rows (T column-major) or, transposed, along the right
+      // blocks' rows (T row-major, so that the lanes of a warp still write
+      // neighbouring elements), whichever the cost model prefers
+      t_rm[b] = orient_cost(d_rows[b], e_rows[b], kst, nch2, S) < orient_cost(e_rows[b], d_rows[b], kst, nch2, S);
+      ldT[b] = ((t_rm[b] ? d_rows[b] : e_rows[b]) + 7) & ~7;
+      t_off[b] = tsz;
+      tsz += int64_t(ldT[b]) * (t_rm[b] ? e_rows[b] : d_rows[b]);
+    }
+    // needed (E, D) pairs
+    std::vector<std::vector<char>> need(static_cast<size_t>(nr));
+    std::vector<int> e_loc(static_cast<size_t>(nB));
+    for (int b = 0; b < nr; ++b) {
+      need[b].assign(e_of[b].size() * d_of[b].size(), 0);
+      for (size_t q = 0; q < e_of[b].size(); ++q) e_loc[e_of[b][q]] = int(q);
+    }
+    for (int64_t i : mine) {
+      const Task& t = env->tasks[i];
+      if (t.dblk < 0) continue;
+      const int b = B[t.e].b;
+      char& x = need[b][size_t(e_loc[t.e]) * d_of[b].size() + d_loc[t.dblk]];
+      if (!x) ch.k1_flops += 2.0 * B[t.e].rows * B[t.e].cols * R.blocks[t.dblk].rows;
+      x = 1;
+    }
     std::vector<Job> k1jobs;
-    std::vector<int> k1cost;
-    auto src_for = [&](const Task& t) -> int {
-      const Block& E = B[t.e];
-      if (t.dblk < 0) {
-        auto it = pmap.find(t.e);
-        if (it != pmap.end()) return it->second;
-        const int id = int(st->src.size() - ch.src0);
-        st->src.push_back(Source{E.offset, E.rows, E.cols, 1, int32_t(csz), E.rows, 0});
-        csz += E.cols;
-        pmap[t.e] = id;
-        return id;
-      }
-      const uint64_t key = (uint64_t(uint32_t(t.dblk)) << 32) | uint32_t(t.e);
-      auto it = umap.find(key);
-      if (it != umap.end()) return it->second;
-      const OpBlock& Db = R.blocks[t.dblk];
-      const int k1 = E.rows, k2 = E.cols, n = Db.rows;
-      const int id = int(st->src.size() - ch.src0);
-      const int kst2 = (k2 + sp::kKS - 1) / sp::kKS;
-      const double nch2 = (kst2 + sp::kChunkSteps - 1) / sp::kChunkSteps;
-      // T = E D^T with M along the rows of T (E rows; T column-major) or,
-      // transposed, along its columns (D rows; T row-major, so that the
-      // lanes of a warp still write neighbouring elements), whichever the
-      // cost model prefers
-      const bool trans = orient_cost(n, k1, kst2, nch2, S) < orient_cost(k1, n, kst2, nch2, S);
-      const int ldT = trans ? (n + 3) & ~3 : (k1 + 3) & ~3;
-      st->src.push_back(Source{tsz, k1, n, 0, int32_t(csz), ldT, trans ? 1 : 0});
-      csz += n;
-      umap[key] = id;
-      const int mr = trans ? n : k1, nr = trans ? k1 : n;
-      const int64_t mslab = trans ? dslab(t.dblk) : st->edesc[t.e].slab_off;
-      const int64_t nslab = trans ? st->edesc[t.e].slab_off : dslab(t.dblk);
-      // the N tiles of one M tile are neighbouring jobs (they share the M-side tile)
-      for (int tr = 0; tr < (mr + 127) / 128; ++tr)
-        for (int tc = 0; tc < (nr + sp::kCols - 1) / sp::kCols; ++tc) {
-          const int ii = int(st->k1i.size());
-          st->k1i.push_back(Item{mslab + int64_t(tr) * kst2 * S * kSub, nslab + btile_off(tc, kst2, S), kst2, 0, -1});
-          k1jobs.push_back(Job{tsz, mr, nr, ldT, tr, tc, ii, ii + 1, int32_t(eps_off[t.e]),
-                               int32_t(zeta_off[t.dblk]), kst2, nmma_of(nr, tc), trans ? sp::kJobTrans : 0});
-          k1cost.push_back(kst2);
-        }
-      ch.k1_flops += 2.0 * k1 * k2 * n;
-      tsz += int64_t(ldT) * (trans ? k1 : n);
-      return id;
-    };
-    // K2 jobs grouped by output block
-    std::vector<Job> k2jobs;
-    std::vector<int64_t> k2cost;
-    int64_t i = 0;
-    while (i < nt) {
-      const int f = env->tasks[i].f;
-      int64_t j = i;
-      std::vector<int64_t> mine;
-      for (; j < nt && env->tasks[j].f == f; ++j) {
-        const Task& t = env->tasks[j];
-        if (t.term >= t0 && t.term < t1 && !is_small(t)) mine.push_back(j);
-      }
-      i = j;
-      if (mine.empty()) continue;
-      const Block& Fb = B[f];
-      std::vector<int> aid(mine.size());
-      std::vector<int64_t> tp(mine.size());
-      std::vector<int> kst(mine.size());
-      std::vector<int> tid(mine.size());
-      std::vector<int64_t> sco(mine.size());
-      for (size_t q = 0; q < mine.size(); ++q) {
-        const Task& t = env->tasks[mine[q]];
-        const Block& E = B[t.e];
-        const int s = src_for(t);
-        aid[q] = t.ablk >= 0 ? t.ablk : nLb + B[t.e].a;
-        tp[q] = tpsz;
-        kst[q] = (E.rows + sp::kKS - 1) / sp::kKS;
-        const int task_id = int(st->tpt.size() - ch.tp0);
-        tid[q] = task_id;
-        st->tpt.push_back(TPTask{s, int32_t(goff[f]), aid[q], 0, t.v, tpsz});
-        sco[q] = scsz;
-        st->scoff.push_back(scsz);
-        scsz += (Fb.cols + 127) & ~127;  // whole 128-column tiles (16-byte aligned drain loads)
-        for (int tr = 0; tr < (Fb.cols + 127) / 128; ++tr)
-          for (int ks = 0; ks < kst[q]; ++ks) st->tpu.push_back(TPUnit{task_id, tr, ks, 0});
-        tpsz += slab_bytes(Fb.cols, E.rows, S);
-        if (t.ablk >= 0) ch.k2_flops += 2.0 * Fb.rows * E.rows * Fb.cols;
-      }
-      // F_f += A T' with M along the rows of F_f (A rows) or, transposed,
-      // along its columns (T' rows), whichever the cost model prefers for the
-      // block's items
-      double steps = 0.0, chunks = 0.0;
-      for (size_t q = 0; q < mine.size(); ++q) {
-        steps += kst[q];
-        chunks += (kst[q] + sp::kChunkSteps - 1) / sp::kChunkSteps;
-      }
-      const bool trans = orient_cost(Fb.cols, Fb.rows, steps, chunks, S) < orient_cost(Fb.rows, Fb.cols, steps, chunks, S);
-      const int mr = trans ? Fb.cols : Fb.rows, nr = trans ? Fb.rows : Fb.cols;
-      // the N tiles of one M tile are neighbouring jobs (they share the M-side tiles)
-      for (int tr = 0; tr < (mr + 127) / 128; ++tr)
-        for (int tc = 0; tc < (nr + sp::kCols - 1) / sp::kCols; ++tc) {
-          const int i0 = int(st->k2i.size());
-          int tot = 0;
-          for (size_t q = 0; q < mine.size(); ++q) {
-            const int64_t aoff = aslab(aid[q]) + int64_t(trans ? tc : tr) * kst[q] * S * kSub;
-            const int64_t toff = tp[q] + btile_off(trans ? tr : tc, kst[q], S);
-            st->k2i.push_back(Item{trans ? toff : aoff, trans ? aoff : toff, kst[q], 0, sco[q]});
-            tot += kst[q];
+    std::vector<double> k1cost;
+    for (int b = 0; b < nr; ++b) {
+      if (d_of[b].empty()) continue;
+      const int kst = (rs[b].dim + sp::kKS - 1) / sp::kKS;
+      const int nte = (e_rows[b] + 127) / 128, ntd = (d_rows[b] + 127) / 128;
+      std::vector<char> tile(size_t(nte) * ntd, 0);
+      for (size_t q = 0; q < e_of[b].size(); ++q)
+        for (size_t u = 0; u < d_of[b].size(); ++u)
+          if (need[b][q * d_of[b].size() + u]) {
+            const int e = e_of[b][q], d = d_of[b][u];
+            for (int te = e_row0[e] / 128; te <= (e_row0[e] + B[e].rows - 1) / 128; ++te)
+              for (int td = d_row[d] / 128; td <= (d_row[d] + R.blocks[d].rows - 1) / 128; ++td)
+                tile[size_t(te) * ntd + td] = 1;
           }
-          k2jobs.push_back(Job{Fb.offset, mr, nr, Fb.rows, tr, tc, i0, int(st->k2i.size()),
-                               int32_t(rho_off[Fb.a]), int32_t(goff[f]), tot, nmma_of(nr, tc),
-                               trans ? (sp::kJobTrans | sp::kJobLaneStride) : 0});
-          k2cost.push_back(tot);
+      const bool tr = t_rm[b] != 0;
+      const int mr = tr ? d_rows[b] : e_rows[b], nrw = tr ? e_rows[b] : d_rows[b];
+      const int64_t ms = tr ? d_slab[b] : e_slab[b], ns = tr ? e_slab[b] : d_slab[b];
+      // the N tiles of one M tile are neighbouring jobs (they share the M-side tile)
+      for (int tm = 0; tm < (tr ? ntd : nte); ++tm)
+        for (int tn = 0; tn < (tr ? nte : ntd); ++tn) {
+          if (!tile[tr ? size_t(tn) * ntd + tm : size_t(tm) * ntd + tn]) continue;
+          k1jobs.push_back(Job{t_off[b], ms + tile_off(tm, kst, S), ns + tile_off(tn, kst, S), 0, 0, mr, nrw, ldT[b], tm, tn,
+                               int32_t(eps_off[b]), int32_t(zeta_off[b]), kst, sp::kChunkSteps, nmma_of(nrw, tn),
+                               tr ? sp::kJobTrans : 0, 0, 0, 0});
+          k1cost.push_back(tile_cost(nmma_of(nrw, tn), kst, (kst + sp::kChunkSteps - 1) / sp::kChunkSteps, S));
         }
     }
+    // ---- T' and K2: one stacked product per left output sector
+    std::vector<std::vector<int64_t>> t_of(static_cast<size_t>(nl));
+    for (int64_t i : mine) t_of[B[env->tasks[i].f].a].push_back(i);
+    std::vector<Job> k2jobs;
+    std::vector<double> k2cost;
+    struct Tile { Job j; double cost; int ngrp, trans, m_rows, n_rows; };
+    std::vector<Tile> tiles;
+    for (int a = 0; a < nl; ++a) {
+      if (t_of[a].empty()) continue;
+      Stack s{};
+      const int m = ls[a].dim, nf = f_num[a], N = f_cols[a], nw = int(a_of[a].size());
+      s.nf = nf;
+      s.N = N;
+      s.Npad = (N + 127) & ~127;
+      s.col0 = f_col0[a];
+      s.oct_off = int32_t(st->oct.size());
+      int K8 = 0;
+      for (int w = 0; w < nw; ++w) K8 += (a_cols(a_of[a][w]) + 7) / 8;
+      s.kst = (K8 + 1) / 2;
+      s.noct = 2 * s.kst;
+      // exponent groups (drain chunks) of about two blocks, at most 192 K:
+      // the blocks of a group share one exponent per row, and a group of a
+      // dozen small blocks was measured to double the error of H.psi (L = 12,
+      // D = 100)
+      s.gst = kWinSteps;
+      for (int g : {2, 3, 4, 6})
+        if (16 * g * nw >= kGroupBlocks * 8 * K8) {
+          s.gst = g;
+          break;
+        }
+      s.ngrp = (s.kst + s.gst - 1) / s.gst;
+      s.m = m;
+      s.mpad = (m + 127) & ~127;
+      s.desc0 = int32_t(st->adesc.size());
+      s.ax_off = st->n_ax;
+      st->n_ax += int64_t(s.ngrp) * s.mpad;
+      const int32_t rho_off = int32_t(st->n_rho);
+      st->n_rho += m;
+      int ko = 0;
+      const int64_t aslab = a_pos;
+      for (int w = 0; w < nw; ++w) {
+        const int id = a_of[a][w], k = a_cols(id), no = (k + 7) / 8;
+        a_w[id] = w;
+        const int64_t src = id >= nLb ? -1 : ooc ? env->os.dev_off(L.blocks[id].off, c) : L.blocks[id].off;
+        const int did = int(st->adesc.size());
+        st->adesc.push_back(SlabDesc{src, aslab, m, k, m, 0, 8 * ko, m, s.kst, no + (w + 1 == nw ? s.noct - K8 : 0),
+                                     int32_t(s.ax_off), s.mpad, s.gst, 0});
+        add_units(st->aunit, did, st->adesc.back());
+        for (int q = 0; q < no; ++q) st->oct.push_back(Oct{w, 8 * q, std::min(8, k - 8 * q), 0});
+        ko += no;
+      }
+      if (K8 < s.noct) st->oct.push_back(Oct{-1, 0, 0, 0});
+      a_pos += slab_bytes(m, s.kst, S);
+      s.tp_off = tpsz;
+      tpsz += slab_bytes(N, s.kst, S);
+      s.grp_off = grpsz;
+      grpsz += int64_t(s.ngrp) * s.Npad;
+      s.tab_off = int64_t(st->tab.size());
+      // task lists by (left block, output block), in task order
+      std::vector<int32_t> cnt(size_t(nw) * nf + 1, 0);
+      for (int64_t i : t_of[a]) cnt[size_t(a_w[a_id(env->tasks[i])]) * nf + f_loc[env->tasks[i].f] + 1] += 1;
+      for (size_t q = 0; q + 1 < cnt.size(); ++q) {
+        if (cnt[q + 1] > 0) {
+          const int id = a_of[a][q / nf];
+          if (id < nLb) ch.k2_flops += 2.0 * m * a_cols(id) * B[f_first[a] + int(q % nf)].cols;
+        }
+        cnt[q + 1] += cnt[q];
+      }
+      const int64_t base = int64_t(st->tpt.size());
+      if (base + int64_t(t_of[a].size()) >= INT32_MAX) {
+        err = "split plan too large";
+        return SU2_EINVAL;
+      }
+      st->tpt.resize(size_t(base) + t_of[a].size());
+      std::vector<int32_t> fill(cnt.begin(), cnt.end() - 1);
+      for (int64_t i : t_of[a]) {
+        const Task& t = env->tasks[i];
+        const int id = a_id(t);
+        const size_t at = size_t(base) + fill[size_t(a_w[id]) * nf + f_loc[t.f]]++;
+        TPTask& tp = st->tpt[at];
+        tp.vh = float(t.v);
+        tp.vl = float(t.v - double(tp.vh));
+        if (t.dblk < 0) {
+          tp.off = B[t.e].offset;
+          tp.ld = B[t.e].rows;
+          tp.flags = kFromPsi;
+        } else {
+          const int b = B[t.e].b;
+          tp.ld = ldT[b];
+          tp.flags = t_rm[b] ? kRowMajor : 0;
+          tp.off = t_off[b] + (t_rm[b] ? int64_t(e_row0[t.e]) * ldT[b] + d_row[t.dblk]
+                                       : int64_t(d_row[t.dblk]) * ldT[b] + e_row0[t.e]);
+        }
+      }
+      for (size_t q = 0; q < cnt.size(); ++q) st->tab.push_back(int32_t(base + cnt[q]));
+      // 128-column tiles with a task (the others add nothing)
+      std::vector<char> live(size_t((N + 127) / 128), 0);
+      {
+        std::vector<char> fl(size_t(nf), 0);
+        for (int64_t i : t_of[a]) fl[f_loc[env->tasks[i].f]] = 1;
+        for (int q = 0; q < N; ++q)
+          if (fl[st->col[size_t(s.col0) + q].f]) live[q / 128] = 1;
+      }
+      const int sid = int(st->stk.size() - ch.st0);
+      st->stk.push_back(s);
+      for (int tl = 0; tl < int(live.size()); ++tl)
+        if (live[tl]) {
+          st->gu.push_back(MaxUnit{s.grp_off, N, s.Npad, s.ngrp, s.col0, tl, 0});
+          for (int g = 0; g < (s.kst + kWinSteps - 1) / kWinSteps; ++g)
+            for (int q = 4 * tl; q < std::min(4 * tl + 4, (N + 31) / 32); ++q) st->tpu.push_back(TPUnit{sid, g, q, 0});
+        }
+      for (int q = 0; q < s.mpad / 128; ++q) st->amu.push_back(MaxUnit{s.ax_off, m, s.mpad, s.ngrp, rho_off, q, 0});
+      for (int g = 0; g < s.ngrp; ++g)
+        for (int q = 0; q < (m + kRowTile - 1) / kRowTile; ++q) st->axu.push_back(TPUnit{int32_t(st->stk.size()) - 1, g, q, 0});
+      // M along the rows of F_a or, transposed, along its columns (T' rows),
+      // whichever the cost model prefers
+      const bool tr = orient_cost(N, m, s.kst, s.ngrp, S) < orient_cost(m, N, s.kst, s.ngrp, S);
+      const int mr = tr ? N : m, nrw = tr ? m : N;
+      for (int tm = 0; tm < (mr + 127) / 128; ++tm)
+        for (int tn = 0; tn < (nrw + 127) / 128; ++tn) {
+          if (!live[tr ? tm : tn]) continue;
+          const int64_t ms = (tr ? s.tp_off : aslab) + tile_off(tm, s.kst, S), ns = (tr ? aslab : s.tp_off) + tile_off(tn, s.kst, S);
+          Job j{B[f_first[a]].offset, ms, ns, tr ? s.grp_off : s.ax_off, tr ? s.ax_off : s.grp_off, mr, nrw, m, tm, tn,
+                rho_off, s.col0, s.kst, s.gst, nmma_of(nrw, tn), tr ? (sp::kJobTrans | sp::kJobLaneStride) : 0,
+                tr ? s.Npad : s.mpad, tr ? s.mpad : s.Npad, 0};
+          tiles.push_back(Tile{j, tile_cost(j.nmma, s.kst, s.ngrp, S), s.ngrp, tr, mr, nrw});
+        }
+    }
+    // K split: F_a's K axis runs over every left block of the sector, so one
+    // tile can hold most of a small window's work.  Tiles above a quarter of
+    // an SM's share are cut into runs of whole groups (at least 24 steps), whose
+    // partial tiles a second kernel adds in K order.
+    double total = 0.0;
+    for (const Tile& t : tiles) total += t.cost;
+    const double share = total / (4.0 * st->n_sms);
+    int64_t slots = 0;
+    for (const Tile& t : tiles) {
+      const int parts = std::max(1, std::min(int(std::ceil(t.cost / std::max(share, 1.0))), t.j.nst / 24));
+      const int arows = sp::tile_rows(t.m_rows, t.j.tr);
+      if (parts > 1)
+        st->spt.push_back(SplitTile{t.j.out_off + (t.trans ? int64_t(t.j.tr) * 128 * t.j.ld + t.j.tc * 128
+                                                           : int64_t(t.j.tc) * 128 * t.j.ld + t.j.tr * 128),
+                                    std::min(128, t.m_rows - t.j.tr * 128), std::min(128, t.n_rows - t.j.tc * 128), t.j.ld,
+                                    t.trans, int32_t(slots), parts});
+      for (int p = 0; p < parts; ++p) {
+        const int g0 = int(int64_t(t.ngrp) * p / parts), g1 = int(int64_t(t.ngrp) * (p + 1) / parts);
+        Job j = t.j;
+        j.m_off += int64_t(g0) * j.gst * S * arows * 32;
+        j.n_off += int64_t(g0) * j.gst * S * j.nmma * 32;
+        j.msc += int64_t(g0) * j.msc_ld;
+        j.nsc += int64_t(g0) * j.nsc_ld;
+        j.nst = std::min(t.j.nst, g1 * j.gst) - g0 * j.gst;
+        if (parts > 1) {
+          j.flags |= sp::kJobPartial;
+          j.out_off = slots++ * (int64_t(sp::kRows) * sp::kCols);
+        }
+        k2jobs.push_back(j);
+        k2cost.push_back(t.cost * (g1 - g0) / t.ngrp);
+      }
+    }
+    st->n_part = std::max(st->n_part, slots);
     // LPT order
-    std::vector<int> o1(k1jobs.size());
-    for (size_t q = 0; q < o1.size(); ++q) o1[q] = int(q);
-    std::stable_sort(o1.begin(), o1.end(), [&](int a, int b) { return k1cost[a] > k1cost[b]; });
-    for (int q : o1) st->k1j.push_back(k1jobs[q]);
-    std::vector<int> o2(k2jobs.size());
-    for (size_t q = 0; q < o2.size(); ++q) o2[q] = int(q);
-    std::stable_sort(o2.begin(), o2.end(), [&](int a, int b) { return k2cost[a] > k2cost[b]; });
-    for (int q : o2) st->k2j.push_back(k2jobs[q]);
-    // T' units of the tasks that read the same source tile run next to each
-    // other (the second read of the T tile then hits L2)
-    std::stable_sort(st->tpu.begin() + ch.tpu0, st->tpu.end(), [&](const TPUnit& x, const TPUnit& y) {
-      const int sx = st->tpt[ch.tp0 + x.task].src, sy = st->tpt[ch.tp0 + y.task].src;
-      if (sx != sy) return sx < sy;
-      if (x.tr != y.tr) return x.tr < y.tr;
-      return x.ks < y.ks;
-    });
+    auto lpt = [](std::vector<Job>& jobs, const std::vector<double>& cost, std::vector<Job>& out) {
+      std::vector<int> o(jobs.size());
+      for (size_t q = 0; q < o.size(); ++q) o[q] = int(q);
+      std::stable_sort(o.begin(), o.end(), [&](int x, int y) { return cost[x] > cost[y]; });
+      for (int q : o) out.push_back(jobs[q]);
+    };
+    lpt(k1jobs, k1cost, st->k1j);
+    lpt(k2jobs, k2cost, st->k2j);
     ch.k1_j1 = int64_t(st->k1j.size());
-    ch.src1 = int64_t(st->src.size());
-    ch.tp1 = int64_t(st->tpt.size());
-    ch.tpu1 = int64_t(st->tpu.size());
     ch.k2_j1 = int64_t(st->k2j.size());
+    ch.st1 = int64_t(st->stk.size());
+    ch.tpu1 = int64_t(st->tpu.size());
+    ch.gu1 = int64_t(st->gu.size());
+    ch.sp1 = int64_t(st->spt.size());
+    ch.au1 = int64_t(st->aunit.size());
+    ch.du1 = int64_t(st->dunit.size());
+    ch.ax1 = int64_t(st->axu.size());
+    ch.dr1 = int64_t(st->drow.size());
     st->chunks.push_back(ch);
+    if (ooc) {
+      max_as = std::max(max_as, a_pos);
+      max_ds = std::max(max_ds, d_pos);
+    } else {
+      st->a_bytes = a_pos;
+      st->d_bytes = d_pos;
+    }
     max_t = std::max(max_t, tsz);
     max_tp = std::max(max_tp, tpsz);
-    max_cexp = std::max(max_cexp, csz);
-    st->n_scale = std::max(st->n_scale, scsz);
+    st->n_grp = std::max(st->n_grp, grpsz);
   }
-  if (int64_t(st->k2i.size()) >= INT32_MAX || int64_t(st->k1i.size()) >= INT32_MAX) {
+  if (st->n_zeta >= INT32_MAX || st->n_ax >= INT32_MAX || int64_t(st->oct.size()) >= INT32_MAX || int64_t(st->adesc.size()) >= INT32_MAX ||
+      int64_t(st->ddesc.size()) >= INT32_MAX) {
     err = "split plan too large";
     return SU2_EINVAL;
   }
   st->t_elems = max_t;
   st->tp_bytes = max_tp;
-  st->n_cexp = max_cexp;
   if (ooc) {
-    st->a_bytes = std::max(max_as, ab);  // identity slabs, then the largest chunk's A slabs
+    st->a_bytes = max_as;
     st->d_bytes = max_ds;
   }
   // ---------------------------------------------------------- device memory
@@ -1099,102 +1240,91 @@ int split_prepare(su2_env* env, int S, std::string& err) {
   if (!rc2) rc2 = dalloc(&st->dD, size_t(st->d_bytes), err);
   if (!rc2) rc2 = dalloc(&st->dE, size_t(st->e_bytes), err);
   if (!rc2) rc2 = dalloc(&st->dTP, size_t(std::max<int64_t>(st->tp_bytes, 16)), err);
-  // + 16: the 16-byte loads of a T' unit may run up to 16 K past its source's last column
   if (!rc2) rc2 = dalloc(&st->dTh, size_t(st->t_elems + 16), err);
   if (!rc2) rc2 = dalloc(&st->dTl, size_t(st->t_elems + 16), err);
   if (!rc2) rc2 = dalloc(&st->dPh, size_t(env->psi_len), err);
   if (!rc2) rc2 = dalloc(&st->dPl, size_t(env->psi_len), err);
   if (!rc2) rc2 = dalloc(&st->d_rho, size_t(st->n_rho), err);
-  if (!rc2) rc2 = dalloc(&st->d_aown, size_t(st->n_aown), err);
-  if (!rc2) rc2 = dalloc(&st->d_delta, st->adesc.size(), err);
+  if (!rc2) rc2 = dalloc(&st->d_ax, size_t(st->n_ax), err);
+  if (!rc2) rc2 = dalloc(&st->d_ascale, size_t(st->n_ax), err);
   if (!rc2) rc2 = dalloc(&st->d_zeta, size_t(st->n_zeta), err);
   if (!rc2) rc2 = dalloc(&st->d_eps, size_t(st->n_eps), err);
   if (!rc2) rc2 = dalloc(&st->d_gamma, size_t(st->n_gamma), err);
-  if (!rc2) rc2 = dalloc(&st->d_cexp, size_t(std::max<int64_t>(st->n_cexp, 1)), err);
+  if (!rc2) rc2 = dalloc(&st->d_grp, size_t(st->n_grp), err);
+  if (!rc2) rc2 = dalloc(&st->d_scale, size_t(st->n_grp), err);
+  if (!rc2) rc2 = dalloc(&st->d_part, size_t(st->n_part) * sp::kRows * sp::kCols, err);
+  if (!rc2) rc2 = dalloc(&st->d_counter, 2 * st->chunks.size(), err);
   if (!rc2) rc2 = dput(&st->d_adesc, st->adesc, err);
   if (!rc2) rc2 = dput(&st->d_ddesc, st->ddesc, err);
   if (!rc2) rc2 = dput(&st->d_edesc, st->edesc, err);
   if (!rc2) rc2 = dput(&st->d_aunit, st->aunit, err);
   if (!rc2) rc2 = dput(&st->d_dunit, st->dunit, err);
-  if (!rc2) rc2 = dput(&st->d_eunit, st->eunit, err);
+  if (!rc2) rc2 = dput(&st->d_axu, st->axu, err);
+  if (!rc2) rc2 = dput(&st->d_amu, st->amu, err);
+  if (!rc2) rc2 = dput(&st->d_drow, st->drow, err);
+  if (!rc2) rc2 = dput(&st->d_erow, st->erow, err);
   if (!rc2) rc2 = dput(&st->d_k1j, st->k1j, err);
   if (!rc2) rc2 = dput(&st->d_k2j, st->k2j, err);
-  if (!rc2) rc2 = dput(&st->d_k1i, st->k1i, err);
-  if (!rc2) rc2 = dput(&st->d_k2i, st->k2i, err);
-  if (!rc2) rc2 = dput(&st->d_src, st->src, err);
   if (!rc2) rc2 = dput(&st->d_tpt, st->tpt, err);
+  if (!rc2) rc2 = dput(&st->d_tab, st->tab, err);
+  if (!rc2) rc2 = dput(&st->d_oct, st->oct, err);
+  if (!rc2) rc2 = dput(&st->d_stk, st->stk, err);
+  if (!rc2) rc2 = dput(&st->d_col, st->col, err);
   if (!rc2) rc2 = dput(&st->d_tpu, st->tpu, err);
-  if (!rc2) rc2 = dalloc(&st->d_phi, std::max<size_t>(st->tpt.size(), 1), err);
-  if (!rc2) rc2 = dalloc(&st->d_scale, size_t(std::max<int64_t>(st->n_scale, 1)), err);
-  if (!rc2) rc2 = dput(&st->d_scoff, st->scoff, err);
+  if (!rc2) rc2 = dput(&st->d_gu, st->gu, err);
+  if (!rc2) rc2 = dput(&st->d_spt, st->spt, err);
   if (!rc2) rc2 = dput(&st->d_small, st->small, err);
   if (!rc2) rc2 = dput(&st->d_small_out, st->small_out, err);
   if (!rc2) rc2 = dput(&st->d_small_seg, st->small_seg, err);
   if (!rc2) rc2 = dalloc(&st->d_small_part, std::max<size_t>(st->small_seg.size(), 1) * kSmallDim * kSmallDim, err);
-  if (!rc2 && ooc) rc2 = dput(&st->d_sdesc, st->sdesc, err);
-  if (!rc2 && ooc) rc2 = dput(&st->d_sunit, st->sunit, err);
-  if (!rc2 && ooc) rc2 = dput(&st->d_resunit_a, st->resunit_a, err);
-  if (!rc2 && ooc) rc2 = dput(&st->d_resunit_d, st->resunit_d, err);
   if (rc2) return rc2;
-  // ---------------------------------------------------------- operator slabs (once per site)
+  // ---------------------------------------------------------- operator exponents and slabs (once per site)
   cudaStream_t s = env->ctx->stream;
-  const int na = int(st->aunit.size()), nd = int(st->dunit.size());
-  fill_kernel<<<256, 256, 0, s>>>(st->d_rho, st->n_rho, kSentinel);
-  fill_kernel<<<64, 256, 0, s>>>(st->d_delta, int64_t(st->adesc.size()), INT_MAX);
-  if (ooc) {
-    // exponents of every block, as in the resident case: the resident blocks
-    // (and the identities) in place, then each chunk's blocks with its
-    // streamed range in slot c % 2; then rho, delta and the identity slabs
+  // stack rows that pad a block (psi stacks) or a tile are never written
+  cudaMemsetAsync(st->dE, 0, size_t(st->e_bytes), s);
+  cudaMemsetAsync(st->d_eps, 0, size_t(st->n_eps) * sizeof(int), s);
+  // row exponents of the operator stacks; out-of-core: chunk by chunk with its
+  // streamed range in slot c % 2
+  for (int c = 0; c < nch && !rc2; ++c) {
+    const SChunk& ch = st->chunks[c];
     OpStream& os = env->os;
-    fill_kernel<<<256, 256, 0, s>>>(st->d_aown, st->n_aown, kSentinel);
-    if (!st->resunit_a.empty())
-      rowexp_kernel<<<unsigned(st->resunit_a.size()), 128, 0, s>>>(st->d_adesc, st->d_resunit_a, os.dbuf, st->d_aown, 1);
-    if (!st->resunit_d.empty())
-      rowexp_kernel<<<unsigned(st->resunit_d.size()), 128, 0, s>>>(st->d_ddesc, st->d_resunit_d, os.dbuf, st->d_zeta, 0);
-    for (size_t c = 0; c < st->chunks.size(); ++c) {
-      const SChunk& ch = st->chunks[c];
-      const int64_t n = os.he[c] - os.hs[c];
-      if (n > 0 &&
-          cudaMemcpyAsync(os.dbuf + os.prefix + int64_t(c & 1) * os.slot, os.host + (os.hs[c] - os.prefix),
-                          size_t(n) * sizeof(double), cudaMemcpyHostToDevice, s) != cudaSuccess) {
-        err = "out-of-core operators: copy failed";
-        return SU2_ECUDA;
-      }
-      if (ch.sau1 > ch.sau0)
-        rowexp_kernel<<<unsigned(ch.sau1 - ch.sau0), 128, 0, s>>>(st->d_sdesc, st->d_sunit + ch.sau0, os.dbuf,
-                                                                   st->d_aown, 1);
-      if (ch.sdu1 > ch.sdu0)
-        rowexp_kernel<<<unsigned(ch.sdu1 - ch.sdu0), 128, 0, s>>>(st->d_sdesc, st->d_sunit + ch.sdu0, os.dbuf,
-                                                                   st->d_zeta, 0);
+    if (ooc && os.he[c] > os.hs[c] &&
+        cudaMemcpyAsync(os.dbuf + os.prefix + int64_t(c & 1) * os.slot, os.host + (os.hs[c] - os.prefix),
+                        size_t(os.he[c] - os.hs[c]) * sizeof(double), cudaMemcpyHostToDevice, s) != cudaSuccess) {
+      err = "out-of-core operators: copy failed";
+      rc2 = SU2_ECUDA;
+      break;
     }
-    if (na) {
-      rho_kernel<<<na, 128, 0, s>>>(st->d_adesc, st->d_aunit, st->d_aown, st->d_rho);
-      delta_kernel<<<na, 128, 0, s>>>(st->d_adesc, st->d_aunit, st->d_aown, st->d_rho, st->d_delta);
-      delta_fix_kernel<<<int((st->adesc.size() + 255) / 256), 256, 0, s>>>(st->d_delta, int(st->adesc.size()));
-      const int64_t ni = int64_t(na) - st->ident_u0;
-      if (ni > 0)
-        slab_fp64_kernel<<<unsigned(ni), 128, 0, s>>>(st->d_adesc, st->d_aunit + st->ident_u0, os.dbuf, st->d_rho,
-                                                       st->d_delta, st->dA, S);
-    }
-  } else if (na) {
-    rowexp_kernel<<<na, 128, 0, s>>>(st->d_adesc, st->d_aunit, env->dL, st->d_aown, 1);
-    rho_kernel<<<na, 128, 0, s>>>(st->d_adesc, st->d_aunit, st->d_aown, st->d_rho);
-    delta_kernel<<<na, 128, 0, s>>>(st->d_adesc, st->d_aunit, st->d_aown, st->d_rho, st->d_delta);
-    delta_fix_kernel<<<int((st->adesc.size() + 255) / 256), 256, 0, s>>>(st->d_delta, int(st->adesc.size()));
-    slab_fp64_kernel<<<na, 128, 0, s>>>(st->d_adesc, st->d_aunit, env->dL, st->d_rho, st->d_delta, st->dA, S);
+    if (ch.ax1 > ch.ax0)
+      winexp_kernel<<<unsigned(ch.ax1 - ch.ax0), 256, 0, s>>>(st->d_axu + ch.ax0, st->d_stk, st->d_oct, st->d_adesc,
+                                                               env->dL, st->d_ax);
+    if (ch.dr1 > ch.dr0)
+      rowexp_kernel<<<unsigned(ch.dr1 - ch.dr0), 256, 0, s>>>(st->d_ddesc, st->d_drow + ch.dr0, env->dR, st->d_zeta);
   }
-  if (nd && !ooc) {
-    rowexp_kernel<<<nd, 128, 0, s>>>(st->d_ddesc, st->d_dunit, env->dR, st->d_zeta, 0);
-    slab_fp64_kernel<<<nd, 128, 0, s>>>(st->d_ddesc, st->d_dunit, env->dR, st->d_zeta, st->d_delta, st->dD, S);
+  if (!st->amu.empty())
+    groupmax_kernel<<<unsigned(st->amu.size()), 512, 0, s>>>(st->d_amu, st->d_ax, st->d_rho, st->d_ascale);
+  if (!ooc) {
+    if (!st->aunit.empty())
+      slab_fp64_kernel<<<unsigned(st->aunit.size()), 128, 0, s>>>(st->d_adesc, st->d_aunit, env->dL, st->d_ax,
+                                                                   st->dA, S);
+    if (!st->dunit.empty())
+      slab_fp64_kernel<<<unsigned(st->dunit.size()), 128, 0, s>>>(st->d_ddesc, st->d_dunit, env->dR, st->d_zeta,
+                                                                   st->dD, S);
   }
   {
     const cudaError_t e1 = cudaGetLastError();
     const cudaError_t e2 = cudaStreamSynchronize(s);
-    if (e1 != cudaSuccess || e2 != cudaSuccess) {
+    if (!rc2 && (e1 != cudaSuccess || e2 != cudaSuccess)) {
       err = std::string("split-precision operator slabs failed: ") + cudaGetErrorString(e1 != cudaSuccess ? e1 : e2);
       return SU2_ECUDA;
     }
   }
+  if (rc2) return rc2;
+  // the host keeps what an H.psi launches with; the rest lives on the device
+  st->adesc = {}; st->ddesc = {}; st->edesc = {};
+  st->aunit = {}; st->dunit = {}; st->drow = {}; st->axu = {}; st->amu = {};
+  st->k1j = {}; st->k2j = {}; st->tpt = {}; st->tab = {}; st->oct = {}; st->stk = {}; st->col = {};
+  st->tpu = {}; st->gu = {}; st->spt = {}; st->small = {};
   return SU2_OK;
 }
 
@@ -1216,16 +1346,16 @@ int split_apply(su2_env* env, const double* psi, double* F, std::string& err) {
   cudaStream_t s = env->ctx->stream;
   Profiler& pf = env->prof;
   const int S = st->S;
-  const int ne = int(st->eunit.size());
+  const bool any = !st->chunks.empty() && (st->chunks.size() > 1 || st->chunks[0].st1 > st->chunks[0].st0);
   SPLIT_CHECK("before");
-  pf.count(ne ? 3 : 1);
   int slot = pf.begin(s, 2, 0.0);
-  psi_ff_kernel<<<1024, 256, 0, s>>>(psi, st->dPh, st->dPl, env->psi_len);
-  if (ne) {
-    rowexp_kernel<<<ne, 128, 0, s>>>(st->d_edesc, st->d_eunit, psi, st->d_eps, 0);
-    slab_fp64_kernel<<<ne, 128, 0, s>>>(st->d_edesc, st->d_eunit, psi, st->d_eps, st->d_delta, st->dE, S);
-  }
   cudaMemsetAsync(F, 0, size_t(env->psi_len) * sizeof(double), s);
+  if (any) {  // (an environment of small tasks only needs no slabs)
+    pf.count(1);
+    cudaMemsetAsync(st->d_counter, 0, 2 * st->chunks.size() * sizeof(int), s);
+    psi_slab_kernel<<<unsigned(st->erow.size()), 256, 0, s>>>(st->d_edesc, st->d_erow, psi, st->dPh, st->dPl, st->d_eps,
+                                                              st->dE, S);
+  }
   pf.end(s, slot);
   SPLIT_CHECK("psi slabs");
   const double npairs = S * (S + 1) / 2.0;
@@ -1237,49 +1367,37 @@ int split_apply(su2_env* env, const double* psi, double* F, std::string& err) {
       // the chunk's operator slabs, cut as soon as its blocks are on the
       // device; its slot is then free for the copy of chunk ci + 2
       stream_wait(env->os, int(ci), s);
-      pf.count(int(c.sau1 > c.sau0) + int(c.sdu1 > c.sdu0));
+      pf.count(int(c.au1 > c.au0) + int(c.du1 > c.du0));
       slot = pf.begin(s, 2, 0.0);
-      if (c.sau1 > c.sau0)
-        slab_fp64_kernel<<<unsigned(c.sau1 - c.sau0), 128, 0, s>>>(st->d_sdesc, st->d_sunit + c.sau0, env->os.dbuf,
-                                                                    st->d_rho, st->d_delta, st->dA, S);
-      if (c.sdu1 > c.sdu0)
-        slab_fp64_kernel<<<unsigned(c.sdu1 - c.sdu0), 128, 0, s>>>(st->d_sdesc, st->d_sunit + c.sdu0, env->os.dbuf,
-                                                                    st->d_zeta, st->d_delta, st->dD, S);
+      if (c.au1 > c.au0)
+        slab_fp64_kernel<<<unsigned(c.au1 - c.au0), 128, 0, s>>>(st->d_adesc, st->d_aunit + c.au0, env->os.dbuf,
+                                                                  st->d_ax, st->dA, S);
+      if (c.du1 > c.du0)
+        slab_fp64_kernel<<<unsigned(c.du1 - c.du0), 128, 0, s>>>(st->d_ddesc, st->d_dunit + c.du0, env->os.dbuf,
+                                                                  st->d_zeta, st->dD, S);
       pf.end(s, slot);
       stream_release(env->os, int(ci), s);
       SPLIT_CHECK("operator slabs of the chunk");
     }
-    pf.count(int(c.k1_j1 > c.k1_j0) + int(c.k2_j1 > c.k2_j0) + 5);
+    if (c.st1 == c.st0) continue;  // small tasks only
+    pf.count(int(c.k1_j1 > c.k1_j0) + int(c.k2_j1 > c.k2_j0) + 2 + int(c.sp1 > c.sp0));
     slot = pf.begin(s, 3, c.k1_flops * npairs);
-    launch_gemm(sp::MODE_T, s, st, st->d_k1j + c.k1_j0, int(c.k1_j1 - c.k1_j0), st->d_k1i, st->dE, st->dD, st->d_eps,
-                st->d_zeta, st->dTh, st->dTl, nullptr, sp::TaskScale{nullptr});
+    launch_gemm(sp::MODE_T, s, st, st->d_k1j + c.k1_j0, int(c.k1_j1 - c.k1_j0), st->d_counter + 2 * ci, st->dE, st->dD,
+                st->d_eps, st->d_zeta, nullptr);
     pf.end(s, slot);
     SPLIT_CHECK("K1 split GEMM");
     slot = pf.begin(s, 2, 0.0);
-    const int nsrc = int(c.src1 - c.src0);
-    if (nsrc > 0) cexp_kernel<<<unsigned(nsrc), 256, 0, s>>>(st->d_src + c.src0, st->dTh, st->dPh, st->d_cexp);
-    SPLIT_CHECK("column exponents");
-    fill_kernel<<<256, 256, 0, s>>>(st->d_gamma, st->n_gamma, kSentinel);
-    const int ntp = int(c.tp1 - c.tp0);
-    if (ntp)
-      gamma_kernel<<<ntp, 128, 0, s>>>(st->d_tpt + c.tp0, st->d_src + c.src0, st->d_cexp, st->d_delta, st->d_gamma,
-                                       st->d_phi + c.tp0);
-    if (ntp)
-      scale_kernel<<<ntp, 128, 0, s>>>(st->d_tpt + c.tp0, st->d_src + c.src0, st->d_cexp, st->d_gamma,
-                                       st->d_phi + c.tp0, st->d_scoff + c.tp0, st->d_scale);
-    const int64_t nu = c.tpu1 - c.tpu0;
-    if (nu) {
-      // units of this chunk refer to chunk-local task indices
-      slab_tprime_kernel<<<unsigned(nu), 128, 0, s>>>(st->d_tpt + c.tp0, st->d_tpu + c.tpu0, st->d_src + c.src0,
-                                                      st->dTh, st->dTl, st->dPh, st->dPl, st->d_cexp,
-                                                      st->d_phi + c.tp0, st->d_delta, st->dTP, S);
-    }
+    tprime_kernel<<<unsigned(c.tpu1 - c.tpu0), 32 * kTPWarps, 0, s>>>(st->d_tpu + c.tpu0, st->d_stk + c.st0, st->d_col, st->d_oct,
+                                                            st->d_tab, st->d_tpt, st->dTh, st->dTl, st->dPh, st->dPl,
+                                                            st->d_grp, st->dTP, S);
+    groupmax_kernel<<<unsigned(c.gu1 - c.gu0), 512, 0, s>>>(st->d_gu + c.gu0, st->d_grp, st->d_gamma, st->d_scale);
     pf.end(s, slot);
     SPLIT_CHECK("T' slabs");
     slot = pf.begin(s, 4, c.k2_flops * npairs);
-    launch_gemm(sp::MODE_F, s, st, st->d_k2j + c.k2_j0, int(c.k2_j1 - c.k2_j0), st->d_k2i, st->dA, st->dTP,
-                st->d_rho, st->d_gamma, nullptr, nullptr, F,
-                sp::TaskScale{st->d_scale});
+    launch_gemm(sp::MODE_F, s, st, st->d_k2j + c.k2_j0, int(c.k2_j1 - c.k2_j0), st->d_counter + 2 * ci + 1, st->dA,
+                st->dTP, st->d_rho, st->d_gamma, F);
+    if (c.sp1 > c.sp0)
+      part_reduce_kernel<<<dim3(unsigned(c.sp1 - c.sp0), sp::kCols / 16), 256, 0, s>>>(st->d_spt + c.sp0, st->d_part, F);
     pf.end(s, slot);
     SPLIT_CHECK("K2 split GEMM");
   }
@@ -1407,11 +1525,10 @@ void split_free(su2_env* env) {
   auto* st = static_cast<SplitState*>(env->split);
   if (!st) return;
   void* ps[] = {st->dA, st->dD, st->dE, st->dTP, st->d_adesc, st->d_ddesc, st->d_edesc, st->d_aunit, st->d_dunit,
-                st->d_eunit, st->d_rho, st->d_aown, st->d_delta, st->d_zeta, st->d_eps, st->d_gamma, st->d_cexp,
-                st->dTh, st->dTl, st->dPh, st->dPl, st->d_k1j, st->d_k2j, st->d_k1i, st->d_k2i, st->d_src,
-                st->d_tpt, st->d_tpu, st->d_counter, st->d_phi,
-                st->d_scale, st->d_scoff, st->d_small, st->d_small_out, st->d_small_seg, st->d_small_part,
-                st->d_sdesc, st->d_sunit, st->d_resunit_a, st->d_resunit_d};
+                st->d_drow, st->d_erow, st->d_axu, st->d_amu, st->d_gu, st->d_ax, st->d_ascale, st->d_rho, st->d_zeta,
+                st->d_eps, st->d_gamma, st->d_grp, st->dTh, st->dTl, st->dPh, st->dPl, st->d_k1j, st->d_k2j, st->d_tpt,
+                st->d_tab, st->d_oct, st->d_stk, st->d_col, st->d_tpu, st->d_spt, st->d_part, st->d_counter,
+                st->d_scale, st->d_small, st->d_small_out, st->d_small_seg, st->d_small_part};
   for (void* p : ps) cudaFree(p);
   delete st;
   env->split = nullptr;

@@ -10,9 +10,9 @@
 // q_i * 2^-8i where q_i are the integers peeled from x * 2^(8 - sigma_row)
 // (|x| < 2^sigma_row): |q_0| <= 256, |q_i| <= 128.
 //
-// One job = one 128 x 128 output tile and a list of items (A slab, B slab,
-// K steps); all items of a job share the row and column scales, so the
-// K-concatenated stripe sum_items A_item . B_item^T accumulates in TMEM
+// One job = one 128 x 128 output tile of a stacked product (several operator
+// blocks side by side along rows or K, heff_split.cu) and its whole K, or a
+// run of it; the K axis accumulates in TMEM
 // without a separate reduction (the stripe product of Sec. III.A).  Slice
 // pairs (i, j), i + j < S, go to four FP32 TMEM accumulators of 128 columns
 // (all 512) by level l = min(i + j, 3).  Levels 0, 1 and 2 hold integer
@@ -21,15 +21,14 @@
 // exact whatever rounding the tensor core applies when it adds into the
 // accumulator (it truncates: a shared tail accumulator of many pairs would
 // collect a biased error of order #adds * 2^-23 of its size); level 3 carries
-// the 2^-24-weighted tail.  A chunk is up to 192 K of one item; after it the
+// the 2^-24-weighted tail.  A chunk is up to 192 K; after it the
 // drain warps fold the four levels into a float-float register accumulator
-// (K2: scaled by the item's per-column factor, so every task keeps its own
-// S*8 bits), and the first MMA of the next chunk into each level overwrites
-// it.  The chunk enters as the exact pair (x0 + r, (y1 - r) + y2 + y3), with
-// r = rint(y1): level 0 is an integer of at most 192 * 2^16 and level 1 stays
-// below 2^16, so x0 + r is an integer below 2^24 and y1 - r is at most 1/2.
-// The job's first chunk becomes the accumulator; later ones are added with
-// TwoSum and renormalised.  At the end of the job they write the tile (K1:
+// (K2: scaled by the chunk's per-row and per-column factors, so every chunk
+// keeps its own S*8 bits), and the first MMA of the next chunk into each level overwrites
+// it.  The chunk enters as the pair (s, (y1 - (s - x0)) + y2 + y3) with
+// s = RN(x0 + y1), exact in levels 0 and 1.  The job's first chunk becomes
+// the accumulator; later ones are added with TwoSum, the pair renormalised
+// every fourth chunk.  At the end of the job they write the tile (K1:
 // normalised float-float T; K2: F += FP64).
 //
 // Warp roles (576 threads): warp 0, one lane: job fetcher (dynamic schedule:
@@ -104,42 +103,37 @@ constexpr int kDrainWarps = 16;
 constexpr int kThreads = 64 + 32 * kDrainWarps;  // producer + MMA + drain warps
 constexpr long kSpinLimit = 1L << 26;
 
-struct Item {
-  int64_t a_off, b_off;  // byte offsets of the item's A / B row tiles in their compact slabs
-  int32_t nst;           // K stages of 16
-  int32_t pad;
-  int64_t sc_off;        // MODE_F: offset of the item's per-column drain exponents (a multiple of 128), -1 otherwise
-};
-// MODE_F: task t's B slab is cut relative to its own column exponents; the
-// drain multiplies each chunk of t by 2^d, d = own(col) - gamma(col) in
-// [-126, 0] (an exact power of two, <= 1), before adding it to the tile
-// accumulator.  dexp[sc_off + col] holds the biased exponent 127 + d, the
-// exponent field of the FP32 number 2^d, or 0 (the factor 0) for a column
-// that is zero.  The per-task vector is padded to whole 128-column tiles.
-struct TaskScale {
-  const uint8_t* dexp;
-};
-// A job computes an M x N tile of the product; the MMA's M side (TMEM
-// lanes) comes from the items' a_off slabs and its N side (TMEM columns) from
-// the b_off slabs.  Without kJobTrans the M side runs along the output
-// block's rows; with it the tile is computed transposed (M along the output
-// columns, N along its rows) and the A and B slab arrays swap roles.  The
-// host picks per output block the orientation with the smaller modelled cost
-// (M is always 128 rows; N is the valid extent rounded up to 16).  The
-// element of lane p and TMEM column q is written at out_off + p + q * ld, or
-// with kJobLaneStride at out_off + p * ld + q (a transposed tile of a
-// column-major block; a transposed tile of a row-major block needs no flag).
+// A job computes an M x N tile of a product, or (kJobPartial) a run of its K;
+// the MMA's M side (TMEM lanes) comes from the slab at m_off and its N side
+// (TMEM columns) from the slab at n_off.  Without kJobTrans the M side runs
+// along the rows of the output and its slab is Aslab; with it the tile is
+// computed transposed (M along the output columns, N along its rows) and the
+// two slab arrays swap roles.  The host picks the orientation with the
+// smaller modelled cost (M is always 128 rows; N is the valid extent rounded
+// up to 16).  The element of lane p and TMEM column q is written at out_off +
+// p + q * ld, or with kJobLaneStride at out_off + p * ld + q (a transposed
+// tile of a column-major matrix; a transposed tile of a row-major one needs
+// no flag).
+// MODE_F: both operands are cut relative to row exponents of their own for
+// every chunk of K (a chunk holds several operator blocks of different size).  The drain multiplies each chunk by 2^(dm + dn), dm = own(group, lane)
+// - rexp(lane) and dn likewise for the column, both in [-126, 0], before
+// adding it to the tile accumulator.  scale[off + chunk * ld + index] holds
+// the biased exponent 127 + d, the exponent field of the FP32 number 2^d, or 0
+// (the factor 0) for a row that is zero; ld is a multiple of 128.
 constexpr int32_t kJobTrans = 1;
 constexpr int32_t kJobLaneStride = 2;
+constexpr int32_t kJobPartial = 4;  // MODE_F: store the tile at part + out_off (kRows x kCols, lanes contiguous)
 struct Job {
-  int64_t out_off;       // element offset of the output block (column-major, leading dimension ld)
-  int32_t rows, cols;    // valid extent along M and along N (the block's rows and columns, swapped if transposed)
-  int32_t ld, tr, tc;    // leading dimension of the block; tile indices along M (kRows) and N (kCols)
-  int32_t i0, i1;        // items
-  int32_t rsc, csc;      // offsets of the exponent arrays of the block's rows / columns
-  int32_t nst;           // total K stages of all items
+  int64_t out_off;       // element offset of the output matrix (leading dimension ld)
+  int64_t m_off, n_off;  // byte offsets of the first M-side / N-side sub-tile (row tile and K start)
+  int64_t msc, nsc;      // MODE_F: drain exponents of the job's first chunk, M side and N side
+  int32_t rows, cols;    // valid extent of the output along M and along N (swapped if transposed)
+  int32_t ld, tr, tc;    // leading dimension; tile indices along M (kRows) and N (kCols)
+  int32_t rsc, csc;      // offsets of the exponent arrays of the output's rows / columns
+  int32_t nst, gst;      // K steps of 16; steps of a drain chunk (at most kChunkSteps)
   int32_t nmma;          // MMA N of this tile: the valid N extent rounded up to 16 (<= kCols)
-  int32_t flags;         // kJobTrans, kJobLaneStride
+  int32_t flags;         // kJobTrans, kJobLaneStride, kJobPartial
+  int32_t msc_ld, nsc_ld, pad;
 };
 
 enum { MODE_T = 0, MODE_F = 1 };
@@ -301,11 +295,6 @@ __device__ __forceinline__ void tmem_ld_levels<8>(uint32_t a, float (&x)[32]) {
 // single packed instruction with no separate negation
 __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
-__device__ __forceinline__ void two_sum2(float2 a, float2 b, float2& s, float2& e) {
-  s = add2(a, b);
-  const float2 bb = sub2(s, a);
-  e = add2(sub2(a, sub2(s, bb)), sub2(b, bb));
-}
 // x * 2^k: one multiply by the power of two built from its exponent field
 // while 2^k is a normal number (the correctly rounded product, as ldexp
 // gives), ldexp otherwise
@@ -321,11 +310,12 @@ __device__ __forceinline__ double ldexp_d(double x, int k) {
 
 template <int MODE, int S>
 __global__ void __launch_bounds__(kThreads, 1)
-    split_gemm_kernel(const Job* __restrict__ jobs, int njobs, const Item* __restrict__ items,
-                      const unsigned char* __restrict__ Aslab, const unsigned char* __restrict__ Bslab,
-                      const int* __restrict__ rexp, const int* __restrict__ cexp, int shift,
-                      float* __restrict__ Th, float* __restrict__ Tl, double* __restrict__ F, int* __restrict__ status,
-                      int* __restrict__ job_counter, TaskScale ts, int sk, int spin) {
+    split_gemm_kernel(const Job* __restrict__ jobs, int njobs, const unsigned char* __restrict__ Aslab,
+                      const unsigned char* __restrict__ Bslab, const int* __restrict__ rexp,
+                      const int* __restrict__ cexp, int shift, float* __restrict__ Th, float* __restrict__ Tl,
+                      double* __restrict__ F, double* __restrict__ part, int* __restrict__ status,
+                      int* __restrict__ job_counter, const uint8_t* __restrict__ ascale,
+                      const uint8_t* __restrict__ bscale, int sk, int spin) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   const int stage_bytes = stage_bytes_of(S, sk);
@@ -396,43 +386,41 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int arows = tile_rows(jb.rows, jb.tr);
         const int abytes = arows * 32, bbytes = jb.nmma * 32;  // stored bytes of one A / B sub-tile
         const uint32_t nmeta = ((uint32_t)(jb.nmma >> 4) << 8) | ((uint32_t)(arows >> 4) << 12);
-        for (int it = jb.i0; it < jb.i1 && ok; ++it) {
-          const Item item = items[it];
-          const int nstage = (item.nst + sk - 1) / sk;
-          for (int ks = 0; ks < nstage; ++ks) {
-            if (!mbar_wait(smem_u32(&empty_bar[st]), ph ^ 1, &abort_flag, spin)) {
-              ok = false;
-              break;
-            }
-            const int k16 = ks * sk;  // first 16-K step of the stage within the item
-            const int nk = min(sk, item.nst - k16);
-            uint32_t m = nmeta | ((uint32_t)nk << 4);
-            if (k16 % kChunkSteps == 0) m |= kMetaFirst;
-            if ((k16 + sk) % kChunkSteps == 0 || ks == nstage - 1) m |= kMetaLast;
-            stage_meta[st] = m;
-            const uint32_t fb = smem_u32(&full_bar[st]);
-            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(fb),
-                         "r"(nk * S * (abytes + bbytes))
-                         : "memory");
-            // the nk steps x S slices of A, then of B, are contiguous in their slabs
-            const uint32_t dst = smem_u32(smem + st * stage_bytes);
-            const unsigned char* srcA = mslab + item.a_off + (int64_t)k16 * S * abytes;
-            const unsigned char* srcB = nslab + item.b_off + (int64_t)k16 * S * bbytes;
-            asm volatile(
-                "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
-                "l"(srcA), "r"(nk * S * abytes), "r"(fb)
-                : "memory");
-            asm volatile(
-                "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                    dst + sk * S * kSub),
-                "l"(srcB), "r"(nk * S * bbytes), "r"(fb)
-                : "memory");
-            ++nissued;
-            if (++st == NS) {
-              st = 0;
-              ph ^= 1;
-            }
+        const int gst = jb.gst;  // K steps of a chunk; a stage never crosses a chunk's end
+        for (int k16 = 0, kc = 0; k16 < jb.nst;) {
+          if (!mbar_wait(smem_u32(&empty_bar[st]), ph ^ 1, &abort_flag, spin)) {
+            ok = false;
+            break;
           }
+          const int nk = min(sk, min(jb.nst - k16, gst - kc));
+          uint32_t m = nmeta | ((uint32_t)nk << 4);
+          if (kc == 0) m |= kMetaFirst;
+          if (kc + nk == gst || k16 + nk == jb.nst) m |= kMetaLast;
+          stage_meta[st] = m;
+          const uint32_t fb = smem_u32(&full_bar[st]);
+          asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(fb),
+                       "r"(nk * S * (abytes + bbytes))
+                       : "memory");
+          // the nk steps x S slices of A, then of B, are contiguous in their slabs
+          const uint32_t dst = smem_u32(smem + st * stage_bytes);
+          const unsigned char* srcA = mslab + jb.m_off + (int64_t)k16 * S * abytes;
+          const unsigned char* srcB = nslab + jb.n_off + (int64_t)k16 * S * bbytes;
+          asm volatile(
+              "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+              "l"(srcA), "r"(nk * S * abytes), "r"(fb)
+              : "memory");
+          asm volatile(
+              "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                  dst + sk * S * kSub),
+              "l"(srcB), "r"(nk * S * bbytes), "r"(fb)
+              : "memory");
+          ++nissued;
+          if (++st == NS) {
+            st = 0;
+            ph ^= 1;
+          }
+          k16 += nk;
+          kc = kc + nk == gst ? 0 : kc + nk;
         }
       }
       // end marker for the MMA issuer: a stage without data
@@ -557,6 +545,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         lo2[c] = make_float2(0.f, 0.f);
       }
       bool first = true;
+      uint32_t nren = 0;  // chunks folded into this job's accumulator
       // the 16 drain warps split the job's nmma columns evenly: nmma / 4 (a
       // multiple of 4, at most kDrainCols) per lane-quarter warp, so a narrow
       // tile drains in proportionally less time
@@ -566,40 +555,44 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int ng = w / kGroup;  // column groups of this warp
       const int c0 = jb.tc * kCols + cgrp * w;
       const uint32_t lane_addr = lane_base + cgrp * w;
-      const int i1 = jb.i1;
       const bool trans = (jb.flags & kJobTrans) != 0;
       const int p = jb.tr * kRows + row;  // this lane's index along M
-      for (int it = jb.i0; it < i1 && ok; ++it) {
-        const Item item = items[it];
-        // MODE_F: the item's drain exponents (one per output column), fetched
-        // before the chunk wait.  Output columns along N: the same for every
-        // lane, so lane v holds word v (bytes = columns 4v .. 4v + 3) and the
-        // group loop broadcasts it.  Transposed: the lane's own column, its
-        // byte replicated into all four positions.
-        uint32_t dxl = 0u;
-        if (MODE == MODE_F) {
-          if (trans) {
-            dxl = (uint32_t)__ldg(ts.dexp + item.sc_off + p) * 0x01010101u;
-          } else {
-            const uint32_t* dw = reinterpret_cast<const uint32_t*>(ts.dexp + item.sc_off + c0);
-            if (lane < ng) dxl = __ldg(dw + lane);
-          }
-        }
-        const int nch = (item.nst + kChunkSteps - 1) / kChunkSteps;
+      const int nch = (jb.nst + jb.gst - 1) / jb.gst;
+      {
+        // MODE_F: the chunk's drain exponents, fetched before the chunk wait:
+        // the lane's own (M side, one byte), and the columns' (N side), the
+        // same for every lane, so lane v holds word v (bytes = columns 4v ..
+        // 4v + 3) and the group loop broadcasts it
+        const uint8_t* mp = MODE == MODE_F ? (trans ? bscale : ascale) + jb.msc + p : nullptr;
+        const uint8_t* np = MODE == MODE_F ? (trans ? ascale : bscale) + jb.nsc + c0 + 4 * min(lane, ng - 1) : nullptr;
+        const int64_t mld = jb.msc_ld, nld = jb.nsc_ld;
         for (int ch = 0; ch < nch; ++ch) {
+          uint32_t dxl = 0u;
+          float fm = 1.f;
+          if (MODE == MODE_F) {
+            fm = __uint_as_float((uint32_t)__ldg(mp) << 23);
+            dxl = __ldg(reinterpret_cast<const uint32_t*>(np));
+            mp += mld;
+            np += nld;
+          }
           const uint32_t buf = chunk % kNumBuf;
           if (!warp_wait(smem_u32(&accf_bar[buf]), (chunk / kNumBuf) & 1, &abort_flag, spin)) {
             ok = false;
             break;
           }
           asm volatile("tcgen05.fence::after_thread_sync;");
+          // every fourth chunk the pair is renormalised (|lo| <= ulp(hi) / 2):
+          // in between lo gathers at most four chunks' remainders, whose own
+          // rounding stays below 2^-45 of the leading part
+          const bool renorm = (nren & 3u) == 3u;
+          ++nren;
 #pragma unroll
           for (int g = 0; g < kNG; ++g) {
             if (g >= ng) break;
             const uint32_t a = lane_addr + buf * kBufCols + g * kGroup;
             float x[4 * kGroup];  // levels 0..3, kGroup columns each
             tmem_ld_levels<kGroup>(a, x);
-            const uint32_t dxg = MODE == MODE_F ? __shfl_sync(0xffffffffu, dxl, trans ? lane : g) : 0u;
+            const uint32_t dxg = MODE == MODE_F ? __shfl_sync(0xffffffffu, dxl, g) : 0u;
             if (g == ng - 1) {
               // the warp's last TMEM read of this chunk has completed: hand
               // the buffer back before the arithmetic on the last group
@@ -616,36 +609,46 @@ __global__ void __launch_bounds__(kThreads, 1)
               const float2 y1 = nlev > 1 ? make_float2(x[kGroup + c], x[kGroup + c + 1]) : z;
               const float2 y2 = nlev > 2 ? make_float2(x[2 * kGroup + c], x[2 * kGroup + c + 1]) : z;
               const float2 y3 = nlev > 3 ? make_float2(x[3 * kGroup + c], x[3 * kGroup + c + 1]) : z;
-              // x0 + y1 split exactly without TwoSum: level 0 is an integer
-              // with |x0| <= 192 * 256 * 256 (slice 0 of each operand is an
-              // integer of magnitude <= 256), level 1 a multiple of 2^-8 with
-              // |y1| <= 192 * 2 * 256 * 128 * 2^-8 < 2^22, so r = rint(y1) (by
-              // the 1.5 * 2^23 shift), s = x0 + r (an integer < 2^24) and
-              // e = y1 - r (|e| <= 1/2) are all exact and s + e = x0 + y1
-              const float2 mg = make_float2(12582912.f, 12582912.f);
-              const float2 r = sub2(add2(y1, mg), mg);
-              float2 sc = add2(x0, r);
-              float2 t = add2(sub2(y1, r), add2(y2, y3));
+              // x0 + y1 as an exact pair in three operations: level 0 is an
+              // integer with |x0| <= 192 * 256 * 256 < 2^24 and level 1 a
+              // multiple of 2^-8 with |y1| <= 192 * 2 * 256 * 128 * 2^-8 <
+              // 2^16.  s = RN(x0 + y1); s - x0 is a multiple of 2^-8 not above
+              // |y1| + ulp(s) / 2 <= 2^16, hence exact in 24 bits whichever
+              // operand is larger, and so is e = y1 - (s - x0)
+              const float2 sc = add2(x0, y1);
+              const float2 t = add2(sub2(y1, sub2(sc, x0)), add2(y2, y3));
+              // 2^(dm + dn) of columns k and k + 1: the biased exponent byte
+              // moved to the FP32 exponent field (byte 3 of a word, shifted
+              // right once), times the lane's factor.  The scaling rides in the FMAs below: the product with
+              // a power of two is exact, so RN(s f + h) is the sum of the
+              // scaled chunk with one rounding
+              float2 f2 = make_float2(1.f, 1.f);
               if (MODE == MODE_F) {
-                // 2^d of columns k and k + 1: the biased exponent byte moved
-                // to the FP32 exponent field (byte 3 of a word, shifted right
-                // once); the scaling of both parts is exact
                 const uint32_t b0 = __byte_perm(dxg, 0u, 0x0444u | ((uint32_t)c << 12)) >> 1;
                 const uint32_t b1 = __byte_perm(dxg, 0u, 0x0444u | ((uint32_t)(c + 1) << 12)) >> 1;
-                const float2 f2 = make_float2(__uint_as_float(b0), __uint_as_float(b1));
-                sc = __fmul2_rn(sc, f2);
-                t = __fmul2_rn(t, f2);
+                f2 = __fmul2_rn(make_float2(__uint_as_float(b0), __uint_as_float(b1)), make_float2(fm, fm));
               }
               if (first) {  // the accumulator is zero: it becomes the chunk (sc, t)
-                hi2[k >> 1] = sc;
-                lo2[k >> 1] = t;
-              } else {  // TwoSum into the leading part, the rest into the trailing part, renormalise
-                float2 h, e2;
-                two_sum2(hi2[k >> 1], sc, h, e2);
-                const float2 l = add2(lo2[k >> 1], add2(e2, t));
-                const float2 hs = add2(h, l);
-                lo2[k >> 1] = sub2(l, sub2(hs, h));
-                hi2[k >> 1] = hs;
+                hi2[k >> 1] = MODE == MODE_F ? __fmul2_rn(sc, f2) : sc;
+                lo2[k >> 1] = MODE == MODE_F ? __fmul2_rn(t, f2) : t;
+              } else {
+                // TwoSum of the leading part and the scaled chunk; what it
+                // leaves and the chunk's tail go into the trailing part
+                const float2 h0 = hi2[k >> 1];
+                const float2 h = MODE == MODE_F ? __ffma2_rn(sc, f2, h0) : add2(h0, sc);
+                const float2 nb = sub2(h0, h);  // -(h - h0)
+                const float2 ea = sub2(h0, add2(h, nb));
+                const float2 eb = MODE == MODE_F ? __ffma2_rn(sc, f2, nb) : add2(sc, nb);
+                const float2 lt = MODE == MODE_F ? __ffma2_rn(t, f2, lo2[k >> 1]) : add2(t, lo2[k >> 1]);
+                const float2 l = add2(lt, add2(ea, eb));
+                if (renorm) {
+                  const float2 hs = add2(h, l);
+                  lo2[k >> 1] = sub2(l, sub2(hs, h));
+                  hi2[k >> 1] = hs;
+                } else {
+                  hi2[k >> 1] = h;
+                  lo2[k >> 1] = l;
+                }
               }
             }
           }
@@ -667,8 +670,10 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int ep = trans ? cexp[jb.csc + p] : rexp[jb.rsc + p];
         const int* const eq = trans ? rexp + jb.rsc : cexp + jb.csc;
         const bool lstride = (jb.flags & kJobLaneStride) != 0;
-        const int64_t obase = jb.out_off + (lstride ? (int64_t)p * jld : (int64_t)p);
-        const int64_t ostep = lstride ? 1 : jld;
+        const bool partial = MODE == MODE_F && (jb.flags & kJobPartial) != 0;
+        const int64_t obase = partial ? jb.out_off + row - (int64_t)jb.tc * kCols * kRows
+                                      : jb.out_off + (lstride ? (int64_t)p * jld : (int64_t)p);
+        const int64_t ostep = partial ? kRows : lstride ? 1 : jld;
 #pragma unroll
         for (int c = 0; c < kDrainCols; ++c) {
           if (c >= w) break;
@@ -687,9 +692,11 @@ __global__ void __launch_bounds__(kThreads, 1)
               Th[o] = ldexp_f(hs, ex);
               Tl[o] = ldexp_f(ls, ex);
             } else {
-              F[o] += ldexp_d((double)((c & 1) ? hi2[c >> 1].y : hi2[c >> 1].x) +
-                                (double)((c & 1) ? lo2[c >> 1].y : lo2[c >> 1].x),
-                            ex);
+              const double v = ldexp_d((double)((c & 1) ? hi2[c >> 1].y : hi2[c >> 1].x) +
+                                           (double)((c & 1) ? lo2[c >> 1].y : lo2[c >> 1].x),
+                                       ex);
+              if (partial) part[o] = v;
+              else F[o] += v;
             }
           }
         }

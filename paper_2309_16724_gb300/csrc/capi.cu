@@ -264,97 +264,199 @@ static int build_plan(su2_env* env, const su2_sectors* S, int64_t budget) {
   }
   double flops = 0.0;
   int64_t max_t = 0, nk1 = 0;
+  Plan64& P = env->p64;
+  const int64_t nt = int64_t(tasks.size());
+  const int nB = int(blocks.size()), nLb = int(env->L.blocks.size());
+  // psi blocks of one left sector lie side by side (canonical block order):
+  // one column-major matrix of dim(a) rows
+  const int nl = int(S->left.size());
+  std::vector<int> f_first(size_t(nl), -1), f_num(size_t(nl), 0), f_cols(size_t(nl), 0), f_col0(size_t(nl), 0),
+      f_loc(size_t(nB), 0);
+  for (int f = 0; f < nB; ++f) {
+    const int a = blocks[f].a;
+    if (f_first[a] < 0) {
+      f_first[a] = f;
+      f_col0[a] = int(P.col.size());
+    }
+    if (f != f_first[a] + f_num[a] || blocks[f].offset != blocks[f_first[a]].offset + int64_t(f_cols[a]) * blocks[f].rows)
+      return fail(env->ctx, SU2_EINVAL, "the psi blocks of a left sector are not contiguous");
+    f_loc[f] = f_num[a]++;
+    f_cols[a] += blocks[f].cols;
+    for (int c = 0; c < blocks[f].cols; ++c) P.col.push_back(P64Col{f_loc[f], c});
+  }
+  int n_sms = 148;
+  if (env->device >= 0) cudaDeviceGetAttribute(&n_sms, cudaDevAttrMultiProcessorCount, env->device);
+  std::vector<int> w_stamp(size_t(nLb) + 1, -1), w_of(size_t(nLb) + 1, 0);
+  int stamp = 0;
   for (size_t c = 0; c + 1 < starts.size(); ++c) {
     const int t0 = starts[c], t1 = starts[c + 1];
-    Chunk ch{int64_t(env->k1.size()), 0, int64_t(env->k2.size()), 0, 0.0, 0.0};
+    Chunk64 ch{int64_t(P.k1.size()), 0, int64_t(P.k2.size()), 0, int64_t(P.tile.size()), 0, 0.0, 0.0};
     std::unordered_map<uint64_t, int64_t> toff;  // key -> offset in T buffer
     int64_t tsz = 0;
-    // K1 uniques in term order
+    // K1: the distinct (right block, input block) pairs in term order, then by input block
+    std::vector<std::vector<P64Ent>> by_in(static_cast<size_t>(nB));
     for (int ti = t0; ti < t1; ++ti)
       for (int64_t i : by_term[ti]) {
         const Task& t = tasks[i];
         if (t.dblk < 0) continue;
         const uint64_t key = (uint64_t(uint32_t(t.dblk)) << 32) | uint32_t(t.e);
-        if (toff.count(key)) continue;
+        if (!toff.emplace(key, tsz).second) continue;
         const Block& E = blocks[t.e];
         const OpBlock& D = env->R.blocks[t.dblk];
-        toff[key] = tsz;
-        const int k1 = E.rows, k2 = E.cols, n = D.rows;
-        for (int tc = 0; tc < (n + kTile - 1) / kTile; ++tc)
-          for (int tr = 0; tr < (k1 + kTile - 1) / kTile; ++tr)
-            env->k1.push_back(K1Job{E.offset, env->os.on ? env->os.dev_off(D.off, int(c)) : D.off, tsz, k1, k2, n,
-                                    tr, tc, 0});
-        flops += 2.0 * k1 * k2 * n;
-        ch.k1_flops += 2.0 * k1 * k2 * n;
+        by_in[t.e].push_back(P64Ent{env->os.on ? env->os.dev_off(D.off, int(c)) : D.off, tsz, D.rows, 0});
+        flops += 2.0 * E.rows * E.cols * D.rows;
+        ch.k1_flops += 2.0 * E.rows * E.cols * D.rows;
         ++nk1;
-        tsz += (int64_t(k1) * n + 1) & ~int64_t(1);
+        tsz += (int64_t(E.rows) * D.rows + 1) & ~int64_t(1);
       }
-    max_t = std::max(max_t, tsz);
-    ch.k1_end = int64_t(env->k1.size());
-    // K2: tasks of the chunk in (f, term, e) order, grouped by f
-    std::vector<K2Job> jobs;
-    std::vector<double> cost;
-    int64_t i = 0;
-    const int64_t nt = int64_t(tasks.size());
-    while (i < nt) {
-      const int f = tasks[i].f;
-      int64_t j = i;
-      const int64_t tb = int64_t(env->k2t.size());
-      double c2 = 0.0;
-      for (; j < nt && tasks[j].f == f; ++j) {
-        const Task& t = tasks[j];
-        if (t.term < t0 || t.term >= t1) continue;
-        const Block& E = blocks[t.e];
-        const Block& F = blocks[t.f];
-        K2Task k;
-        k.k1 = E.rows;
-        k.v = t.v;
-        k.flags = 0;
-        if (t.ablk < 0) {
-          k.flags |= K2_A_IDENTITY;
-          k.a_off = -1;
-          c2 += 1.0;
-        } else {
-          k.a_off = env->os.on ? env->os.dev_off(env->L.blocks[t.ablk].off, int(c)) : env->L.blocks[t.ablk].off;
-          flops += 2.0 * F.rows * E.rows * F.cols;
-          ch.k2_flops += 2.0 * F.rows * E.rows * F.cols;
-          c2 += E.rows;
-        }
-        if (t.dblk < 0) {
-          k.flags |= K2_B_FROM_PSI;
-          k.b_off = E.offset;
-        } else {
-          k.b_off = toff.at((uint64_t(uint32_t(t.dblk)) << 32) | uint32_t(t.e));
-        }
-        env->k2t.push_back(k);
+    for (int e = 0; e < nB; ++e) {
+      if (by_in[e].empty()) continue;
+      P64In in{blocks[e].offset, blocks[e].rows, blocks[e].cols, int32_t(P.ent.size()), 0, 0, 0};
+      int64_t ncol = 0;
+      for (P64Ent& x : by_in[e]) {
+        x.col0 = int32_t(ncol);
+        ncol += x.n;
+        P.ent.push_back(x);
       }
-      const int64_t te = int64_t(env->k2t.size());
-      if (te > tb) {
-        const Block& F = blocks[f];
-        for (int tc = 0; tc < (F.cols + kTile - 1) / kTile; ++tc)
-          for (int tr = 0; tr < (F.rows + kTile - 1) / kTile; ++tr) {
-            jobs.push_back(K2Job{F.offset, F.rows, F.cols, tr, tc, int32_t(tb), int32_t(te)});
-            cost.push_back(c2);
-          }
+      if (ncol >= INT32_MAX || int64_t(P.ent.size()) >= INT32_MAX) return fail(env->ctx, SU2_EINVAL, "task table too large");
+      in.ent1 = int32_t(P.ent.size());
+      in.ncol = int32_t(ncol);
+      int at = in.ent0;
+      for (int tc = 0; tc < (in.ncol + kTile - 1) / kTile; ++tc) {
+        while (at + 1 < in.ent1 && P.ent[at + 1].col0 <= tc * kTile) ++at;
+        for (int tr = 0; tr < (in.k1 + kTile - 1) / kTile; ++tr) P.k1.push_back(P64K1{int32_t(P.in.size()), at, tr, tc});
       }
-      i = j;
+      P.in.push_back(in);
     }
-    std::vector<int64_t> ord(jobs.size());
-    for (size_t q = 0; q < ord.size(); ++q) ord[q] = int64_t(q);
-    std::stable_sort(ord.begin(), ord.end(), [&](int64_t a, int64_t b) { return cost[a] > cost[b]; });
-    for (int64_t q : ord) env->k2.push_back(jobs[q]);
-    ch.k2_end = int64_t(env->k2.size());
-    env->chunks.push_back(ch);
+    max_t = std::max(max_t, tsz);
+    ch.k1_end = int64_t(P.k1.size());
+    // longest first (K1 tiles: their K)
+    std::stable_sort(P.k1.begin() + ch.k1_begin, P.k1.end(),
+                     [&](const P64K1& x, const P64K1& y) { return P.in[x.in].k2 > P.in[y.in].k2; });
+    // K2: one stack per left output sector
+    struct Tile { P64K2 j; double cost; int steps; };
+    std::vector<Tile> tiles;
+    double total = 0.0;
+    int64_t i = 0;
+    while (i < nt) {
+      const int a = blocks[tasks[i].f].a;
+      std::vector<int64_t> mine;
+      for (; i < nt && blocks[tasks[i].f].a == a; ++i)
+        if (tasks[i].term >= t0 && tasks[i].term < t1) mine.push_back(i);
+      if (mine.empty()) continue;
+      P64Stack s{};
+      s.m = S->left[a].dim;
+      s.nf = f_num[a];
+      s.N = f_cols[a];
+      s.col0 = f_col0[a];
+      s.f_off = blocks[f_first[a]].offset;
+      s.left0 = int32_t(P.left.size());
+      s.step0 = int32_t(P.step.size());
+      s.tab_off = int64_t(P.tab.size());
+      // its left blocks along K (the identity last)
+      std::vector<int> ws;
+      for (int64_t q : mine) {
+        const int id = tasks[q].ablk < 0 ? nLb : tasks[q].ablk;
+        if (w_stamp[id] != stamp) {
+          w_stamp[id] = stamp;
+          ws.push_back(id);
+        }
+      }
+      ++stamp;
+      std::sort(ws.begin(), ws.end());
+      const int nw = int(ws.size());
+      int64_t K = 0;
+      for (int w = 0; w < nw; ++w) {
+        w_of[ws[w]] = w;
+        const bool id = ws[w] == nLb;
+        P.left.push_back(P64Left{id ? -1 : env->os.on ? env->os.dev_off(env->L.blocks[ws[w]].off, int(c)) : env->L.blocks[ws[w]].off,
+                                 int32_t(K), 0});
+        K += id ? s.m : env->L.blocks[ws[w]].cols;
+      }
+      P.left.push_back(P64Left{-1, int32_t(K), 0});
+      if (K >= INT32_MAX || int64_t(P.left.size()) >= INT32_MAX || int64_t(P.task.size() + mine.size()) >= INT32_MAX)
+        return fail(env->ctx, SU2_EINVAL, "task table too large");
+      s.K = int32_t(K);
+      const int nsteps = int((K + 15) / 16);
+      for (int st = 0, w = 0; st < nsteps; ++st) {
+        while (P.left[size_t(s.left0) + w + 1].k0 <= 16 * st) ++w;
+        P.step.push_back(w);
+      }
+      // task lists by (left block, output block), in task order
+      std::vector<int32_t> cnt(size_t(nw) * s.nf + 1, 0);
+      auto cell = [&](const Task& t) { return size_t(w_of[t.ablk < 0 ? nLb : t.ablk]) * s.nf + f_loc[t.f]; };
+      std::vector<char> live(size_t(s.nf), 0);
+      for (int64_t q : mine) {
+        const Task& t = tasks[q];
+        cnt[cell(t) + 1] += 1;
+        live[f_loc[t.f]] = 1;
+        // the counted flops of H.psi are those of the sector-task-table
+        if (t.ablk >= 0) flops += 2.0 * s.m * blocks[t.e].rows * blocks[t.f].cols;
+      }
+      const int32_t base = int32_t(P.task.size());
+      for (size_t q = 0; q + 1 < cnt.size(); ++q) {
+        if (cnt[q + 1] > 0 && ws[q / s.nf] != nLb)
+          ch.k2_flops += 2.0 * s.m * env->L.blocks[ws[q / s.nf]].cols * blocks[f_first[a] + int(q % s.nf)].cols;
+        cnt[q + 1] += cnt[q];
+      }
+      for (int32_t x : cnt) P.tab.push_back(base + x);
+      P.task.resize(size_t(base) + mine.size());
+      for (int64_t q : mine) {
+        const Task& t = tasks[q];
+        P64Task& k = P.task[size_t(base) + cnt[cell(t)]++];
+        k.v = t.v;
+        k.ld = blocks[t.e].rows;
+        k.psi = t.dblk < 0;
+        k.off = k.psi ? blocks[t.e].offset : toff.at((uint64_t(uint32_t(t.dblk)) << 32) | uint32_t(t.e));
+      }
+      // tiles with a task; modelled cycles of a K step: its DFMAs at two lanes
+      // per SM and clock, and about 1500 cycles to fill it
+      for (int tc = 0; tc < (s.N + kTile - 1) / kTile; ++tc) {
+        bool any = false;
+        for (int q = tc * kTile; q < std::min(s.N, (tc + 1) * kTile) && !any; ++q) any = live[P.col[size_t(s.col0) + q].f];
+        if (!any) continue;
+        for (int tr = 0; tr < (s.m + kTile - 1) / kTile; ++tr) {
+          const double rows = std::min(kTile, s.m - tr * kTile), cls = (std::min(kTile, s.N - tc * kTile) + 15) / 16 * 16;
+          const double cost = nsteps * (8.0 * rows * cls + 1500.0);
+          tiles.push_back(Tile{P64K2{int32_t(P.stack.size()), tr, tc, 0, nsteps, -1}, cost, nsteps});
+          total += cost;
+        }
+      }
+      P.stack.push_back(s);
+    }
+    // K split: tiles above an eighth of an SM's share run as several jobs of at
+    // least four K steps, summed afterwards in K order
+    const double share = std::max(1.0, total / (8.0 * n_sms));
+    std::vector<std::pair<double, P64K2>> jobs;
+    int64_t slots = 0;
+    for (const Tile& t : tiles) {
+      const int parts = std::max(1, std::min(int(std::min(1e6, std::ceil(t.cost / share))), t.steps / 4));
+      const P64Stack& s = P.stack[t.j.st];
+      if (parts > 1)
+        P.tile.push_back(P64Tile{s.f_off + t.j.tr * kTile + int64_t(t.j.tc) * kTile * s.m, std::min(kTile, s.m - t.j.tr * kTile),
+                                 std::min(kTile, s.N - t.j.tc * kTile), s.m, int32_t(slots), parts, 0});
+      for (int q = 0; q < parts; ++q) {
+        P64K2 j = t.j;
+        j.s0 = int(int64_t(t.steps) * q / parts);
+        j.s1 = int(int64_t(t.steps) * (q + 1) / parts);
+        if (parts > 1) j.slot = int32_t(slots++);
+        jobs.push_back({t.cost * (j.s1 - j.s0) / t.steps, j});
+      }
+    }
+    P.n_part = std::max(P.n_part, slots);
+    std::stable_sort(jobs.begin(), jobs.end(), [](const std::pair<double, P64K2>& x, const std::pair<double, P64K2>& y) { return x.first > y.first; });
+    for (const auto& q : jobs) P.k2.push_back(q.second);
+    ch.k2_end = int64_t(P.k2.size());
+    ch.sp_end = int64_t(P.tile.size());
+    P.chunks.push_back(ch);
   }
-  if (int64_t(env->k2t.size()) >= (int64_t(1) << 31)) return fail(env->ctx, SU2_EINVAL, "task table too large");
   env->t_elems = max_t;
   env->info.t_chunk_bytes = max_t * int64_t(sizeof(double));
   env->info.flops_su2 = flops;
   env->info.n_k1 = nk1;
-  env->info.n_chunks = int64_t(env->chunks.size());
+  env->info.n_chunks = int64_t(env->p64.chunks.size());
   // diagonal: tasks with e == f, grouped by f
   int64_t i = 0;
-  const int64_t nt = int64_t(tasks.size());
   while (i < nt) {
     const int f = tasks[i].f;
     const int64_t tb = int64_t(env->dt.size());
@@ -376,7 +478,10 @@ static int build_plan(su2_env* env, const su2_sectors* S, int64_t budget) {
       env->dt.push_back(d);
     }
     const int64_t te = int64_t(env->dt.size());
-    if (te > tb) env->dj.push_back(DiagJob{blocks[f].offset, blocks[f].rows, blocks[f].cols, int32_t(tb), int32_t(te)});
+    if (te > tb)
+      for (int tc = 0; tc < (blocks[f].cols + kTile - 1) / kTile; ++tc)
+        for (int tr = 0; tr < (blocks[f].rows + kTile - 1) / kTile; ++tr)
+          env->dj.push_back(DiagJob{blocks[f].offset, blocks[f].rows, blocks[f].cols, tr, tc, int32_t(tb), int32_t(te)});
   }
   return SU2_OK;
 }
@@ -392,9 +497,9 @@ static void env_free_device(su2_env* e) {
   cudaFree(e->dL);
   cudaFree(e->dR);
   cudaFree(e->dT);
-  cudaFree(e->dk1);
-  cudaFree(e->dk2);
-  cudaFree(e->dk2t);
+  const Plan64& p = e->p64;
+  void* pd[] = {p.d_ent, p.d_in, p.d_k1, p.d_left, p.d_step, p.d_tab, p.d_task, p.d_col, p.d_stack, p.d_k2, p.d_tile, p.d_part};
+  for (void* x : pd) cudaFree(x);
   cudaFree(e->ddj);
   cudaFree(e->ddt);
   cudaFree(e->d_in_scratch);
@@ -535,9 +640,19 @@ static int finish_env(su2_ctx* ctx, su2_env* env, const su2_sectors* S, const su
       }
     }
     if (!rc) rc = dev_alloc(ctx, &env->dT, size_t(std::max<int64_t>(env->t_elems, 2)));
-    if (!rc) rc = upload(ctx, &env->dk1, env->k1);
-    if (!rc) rc = upload(ctx, &env->dk2, env->k2);
-    if (!rc) rc = upload(ctx, &env->dk2t, env->k2t);
+    Plan64& p = env->p64;
+    if (!rc) rc = upload(ctx, &p.d_ent, p.ent);
+    if (!rc) rc = upload(ctx, &p.d_in, p.in);
+    if (!rc) rc = upload(ctx, &p.d_k1, p.k1);
+    if (!rc) rc = upload(ctx, &p.d_left, p.left);
+    if (!rc) rc = upload(ctx, &p.d_step, p.step);
+    if (!rc) rc = upload(ctx, &p.d_tab, p.tab);
+    if (!rc) rc = upload(ctx, &p.d_task, p.task);
+    if (!rc) rc = upload(ctx, &p.d_col, p.col);
+    if (!rc) rc = upload(ctx, &p.d_stack, p.stack);
+    if (!rc) rc = upload(ctx, &p.d_k2, p.k2);
+    if (!rc) rc = upload(ctx, &p.d_tile, p.tile);
+    if (!rc) rc = dev_alloc(ctx, &p.d_part, size_t(std::max<int64_t>(p.n_part, 1)) * kTile * kTile);
     if (!rc) rc = upload(ctx, &env->ddj, env->dj);
     if (!rc) rc = upload(ctx, &env->ddt, env->dt);
     if (!rc && opts && (opts->prepare_split || opts->autotune)) {
@@ -713,10 +828,9 @@ int su2_apply_heff(su2_ctx* ctx, const su2_env* env_c, const double* psi_in, dou
   if (prec != SU2_FP64) return fail(ctx, SU2_EINVAL, "unknown precision");
   CUDA_TRY(ctx, cudaMemsetAsync(psi_out, 0, size_t(n) * sizeof(double), ctx->stream));
   if (env->os.on) stream_begin(env->os, ctx->stream);
-  for (size_t ci = 0; ci < env->chunks.size(); ++ci) {
+  for (size_t ci = 0; ci < env->p64.chunks.size(); ++ci) {
     if (env->os.on) stream_wait(env->os, int(ci), ctx->stream);
-    launch_heff_fp64(ctx->stream, env->dL, env->dR, psi_in, psi_out, env->dT, env->dk1, env->dk2, env->dk2t,
-                     env->chunks[ci], n, &env->prof);
+    launch_stack_fp64(ctx->stream, env->p64, env->p64.chunks[ci], env->dL, env->dR, psi_in, psi_out, env->dT, &env->prof);
     if (env->os.on) stream_release(env->os, int(ci), ctx->stream);
   }
   if (env->os.on) stream_end(env->os, ctx->stream);

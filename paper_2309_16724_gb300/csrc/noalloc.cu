@@ -92,9 +92,8 @@ extern "C" int su2_apply_heff_static_scratch(su2_ctx* ctx, const su2_env* env, c
     return SU2_ECUDA;
   }
   su2::Profiler off;  // no event recording on this path
-  for (const su2::Chunk& c : env->chunks)
-    su2::launch_heff_fp64(ctx->stream, env->dL, env->dR, psi_in_dev, psi_out_dev, scratch, env->dk1, env->dk2,
-                          env->dk2t, c, n, &off);
+  for (const su2::Chunk64& c : env->p64.chunks)
+    su2::launch_stack_fp64(ctx->stream, env->p64, c, env->dL, env->dR, psi_in_dev, psi_out_dev, scratch, &off);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
     ctx->err = std::string("launch: ") + cudaGetErrorString(e);

@@ -7,10 +7,56 @@
 
 #include "su2_internal.h"
 
-// FP64 path: 64x64 output tiles.
+// FP64 products: 64x64 output tiles.
 namespace su2 {
 constexpr int kTile = 64;
 
+// ---- FP64 H.psi: stacked products (heff_fp64.cu)
+// K1: the T(k1 x n) = E(k1 x k2) . D(n x k2)^T of one input block and all the
+// right operator blocks its tasks read, side by side
+struct P64Ent { int64_t d_off, t_off; int32_t n, col0; };  // one right block: its columns start at col0
+struct P64In { int64_t e_off; int32_t k1, k2, ent0, ent1, ncol, pad; };
+struct P64K1 { int32_t in, ent, tr, tc; };                 // one tile; ent: the entry that holds its first column
+// K2: F of all output blocks with one left sector (contiguous in psi: m x N)
+// += [A_1 A_2 ..] [T'_1; T'_2; ..], T'(w, f) = sum_t v_t T_t over the tasks of
+// left block w and output block f
+struct P64Left { int64_t a_off; int32_t k0, pad; };        // A block (-1: identity), its first K
+struct P64Task { int64_t off; double v; int32_t ld, psi; };
+struct P64Col { int32_t f, c; };
+struct P64Stack { int64_t f_off, tab_off; int32_t left0, step0, nf, N, m, K, col0, pad; };
+struct P64K2 { int32_t st, tr, tc, s0, s1, slot; };        // K steps [s0, s1) of one tile; slot >= 0: a partial tile
+struct P64Tile { int64_t f_off; int32_t rows, cols, ld, slot0, nslot, pad; };
+struct Chunk64 {
+  int64_t k1_begin, k1_end, k2_begin, k2_end, sp_begin, sp_end;
+  double k1_flops, k2_flops;
+};
+struct Plan64 {
+  std::vector<Chunk64> chunks;
+  std::vector<P64Ent> ent;
+  std::vector<P64In> in;
+  std::vector<P64K1> k1;
+  std::vector<P64Left> left;
+  std::vector<int32_t> step, tab;
+  std::vector<P64Task> task;
+  std::vector<P64Col> col;
+  std::vector<P64Stack> stack;
+  std::vector<P64K2> k2;
+  std::vector<P64Tile> tile;
+  int64_t n_part = 0;  // partial tiles of a chunk (the most of any chunk)
+  P64Ent* d_ent = nullptr;
+  P64In* d_in = nullptr;
+  P64K1* d_k1 = nullptr;
+  P64Left* d_left = nullptr;
+  int32_t *d_step = nullptr, *d_tab = nullptr;
+  P64Task* d_task = nullptr;
+  P64Col* d_col = nullptr;
+  P64Stack* d_stack = nullptr;
+  P64K2* d_k2 = nullptr;
+  P64Tile* d_tile = nullptr;
+  double* d_part = nullptr;
+};
+
+// ---- FP64 products of the renormalisation (renorm.cu)
 // K1: T(k1 x n) = E(k1 x k2) . D(n x k2)^T for one deduplicated
 // (right operator block, input block) pair, one 64x64 tile of T.
 struct K1Job {
@@ -30,9 +76,9 @@ struct K2Task {
   int32_t k1, flags;
   double v;       // sector-value table entry
 };
-struct DiagJob {  // one output block of the diagonal, its diagonal tasks [t0, t1)
+struct DiagJob {  // one 64 x 64 tile of a block of the diagonal, its diagonal tasks [t0, t1)
   int64_t f_off;
-  int32_t m, n, t0, t1;
+  int32_t m, n, tr, tc, t0, t1;
 };
 struct DiagTask {
   int64_t a_off, d_off;  // -1: identity
@@ -102,6 +148,9 @@ constexpr int kSmallDim = 16;
 void launch_heff_fp64(cudaStream_t s, const double* L, const double* R, const double* psi, double* F, double* T,
                       const K1Job* k1, const K2Job* k2, const K2Task* tasks, const Chunk& c, int64_t psi_len,
                       Profiler* prof);
+// one term chunk of the FP64 H.psi: F += its terms (T: the chunk's intermediates)
+void launch_stack_fp64(cudaStream_t s, const Plan64& p, const Chunk64& c, const double* L, const double* R,
+                       const double* psi, double* F, double* T, Profiler* prof);
 void launch_diag(cudaStream_t s, const double* L, const double* R, double* d, const DiagJob* jobs, int64_t njobs,
                  const DiagTask* tasks, int64_t psi_len);
 }  // namespace su2
@@ -171,19 +220,12 @@ struct su2_env {
   std::vector<su2::Sector> lsec, rsec;
   int64_t split_budget = 0;
   int spin_limit = 0;  // polls of each work-loop wait of the split GEMM (0: the kernel's default)
-  // FP64 plan
-  std::vector<su2::Chunk> chunks;
-  std::vector<su2::K1Job> k1;
-  std::vector<su2::K2Job> k2;
-  std::vector<su2::K2Task> k2t;
+  su2::Plan64 p64;  // FP64 plan
   std::vector<su2::DiagJob> dj;
   std::vector<su2::DiagTask> dt;
   int64_t t_elems = 0;  // T buffer size (doubles)
   // device copies
   double *dL = nullptr, *dR = nullptr, *dT = nullptr;
-  su2::K1Job* dk1 = nullptr;
-  su2::K2Job* dk2 = nullptr;
-  su2::K2Task* dk2t = nullptr;
   su2::DiagJob* ddj = nullptr;
   su2::DiagTask* ddt = nullptr;
   double *d_in_scratch = nullptr, *d_out_scratch = nullptr;  // for host-buffer calls

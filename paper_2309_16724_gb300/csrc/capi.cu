@@ -424,9 +424,10 @@ static int build_plan(su2_env* env, const su2_sectors* S, int64_t budget) {
       }
       P.stack.push_back(s);
     }
-    // K split: tiles above an eighth of an SM's share run as several jobs of at
-    // least four K steps, summed afterwards in K order
-    const double share = std::max(1.0, total / (8.0 * n_sms));
+    // K split: tiles above a sixteenth of an SM's share run as several jobs of at
+    // least four K steps, summed afterwards in K order (two or three CTAs share
+    // an SM, so a job takes a sixth of the whole)
+    const double share = std::max(1.0, total / (16.0 * n_sms));
     std::vector<std::pair<double, P64K2>> jobs;
     int64_t slots = 0;
     for (const Tile& t : tiles) {

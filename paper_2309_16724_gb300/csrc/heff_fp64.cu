@@ -118,31 +118,43 @@ __global__ void __launch_bounds__(NT) k2_fp64(const K2Job* __restrict__ jobs, co
 
 // ------------------------------------------------------------------ stacked H.psi
 // acc(row, col) += sum_kk A(kk, row) B(kk, col), thread (tx, ty) owning rows
-// ty + 16 i and columns tx + 16 j, j < NJ; row slots i with on[i] only
-template <int NJ>
+// ty + 16 i, i < NI, and columns tx + 16 j, j < NJ.  NI is uniform in a warp
+// (two rows of ty) and NJ in the CTA, and both are template parameters: a
+// DFMA that is predicated off for a whole warp still takes its slot in the
+// FP64 pipe (measured: 91 % busy at 54 % useful lanes)
+template <int NI, int NJ>
 __device__ __forceinline__ void fma_step(double (&acc)[4][4], const double (*sA)[kTile], const double (*sB)[kTile],
-                                         const bool (&on)[4], int tx, int ty, int kend) {
+                                         int tx, int ty, int kend) {
 #pragma unroll 4
   for (int kk = 0; kk < kend; ++kk) {
     double b[NJ];
 #pragma unroll
     for (int j = 0; j < NJ; ++j) b[j] = sB[kk][tx + 16 * j];
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
-      if (on[i]) {
-        const double a = sA[kk][ty + 16 * i];
+    for (int i = 0; i < NI; ++i) {
+      const double a = sA[kk][ty + 16 * i];
 #pragma unroll
-        for (int j = 0; j < NJ; ++j) acc[i][j] = fma(a, b[j], acc[i][j]);
-      }
+      for (int j = 0; j < NJ; ++j) acc[i][j] = fma(a, b[j], acc[i][j]);
+    }
   }
 }
-__device__ __forceinline__ void fma_tile(double (&acc)[4][4], const double (*sA)[kTile], const double (*sB)[kTile],
-                                         const bool (&on)[4], int tx, int ty, int kend, int nj) {
-  if (nj == 4) fma_step<4>(acc, sA, sB, on, tx, ty, kend);
-  else if (nj == 3) fma_step<3>(acc, sA, sB, on, tx, ty, kend);
-  else if (nj == 2) fma_step<2>(acc, sA, sB, on, tx, ty, kend);
-  else fma_step<1>(acc, sA, sB, on, tx, ty, kend);
+template <int NJ>
+__device__ __forceinline__ void fma_rows(double (&acc)[4][4], const double (*sA)[kTile], const double (*sB)[kTile],
+                                         int tx, int ty, int kend, int ni) {
+  if (ni == 4) fma_step<4, NJ>(acc, sA, sB, tx, ty, kend);
+  else if (ni == 3) fma_step<3, NJ>(acc, sA, sB, tx, ty, kend);
+  else if (ni == 2) fma_step<2, NJ>(acc, sA, sB, tx, ty, kend);
+  else if (ni == 1) fma_step<1, NJ>(acc, sA, sB, tx, ty, kend);
 }
+__device__ __forceinline__ void fma_tile(double (&acc)[4][4], const double (*sA)[kTile], const double (*sB)[kTile],
+                                         int tx, int ty, int kend, int ni, int nj) {
+  if (nj == 4) fma_rows<4>(acc, sA, sB, tx, ty, kend, ni);
+  else if (nj == 3) fma_rows<3>(acc, sA, sB, tx, ty, kend, ni);
+  else if (nj == 2) fma_rows<2>(acc, sA, sB, tx, ty, kend, ni);
+  else fma_rows<1>(acc, sA, sB, tx, ty, kend, ni);
+}
+// row slots of this warp below `rows` (its lower row is ty & ~1)
+__device__ __forceinline__ int row_slots(int ty, int rows) { return max(0, min(4, (rows - (ty & ~1) + 15) >> 4)); }
 
 // the entry of [lo, hi) that holds column c (col0 ascending, col0[lo] <= c)
 __device__ __forceinline__ int find_ent(const P64Ent* __restrict__ ents, int lo, int hi, int c) {
@@ -185,7 +197,7 @@ __global__ void __launch_bounds__(NT, 2) k1_stack(const P64K1* __restrict__ jobs
   bool on[4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) on[i] = r0 + ty + 16 * i < p.k1;
-  const int nj = (min(kTile, p.ncol - c0) + 15) / 16;
+  const int ni = row_slots(ty, p.k1 - r0), nj = (min(kTile, p.ncol - c0) + 15) / 16;
   load(0);
   for (int k0 = 0; k0 < p.k2; k0 += TK) {
 #pragma unroll
@@ -195,7 +207,7 @@ __global__ void __launch_bounds__(NT, 2) k1_stack(const P64K1* __restrict__ jobs
     }
     __syncthreads();
     if (k0 + TK < p.k2) load(k0 + TK);
-    fma_tile(acc, sA, sB, on, tx, ty, min(TK, p.k2 - k0), nj);
+    fma_tile(acc, sA, sB, tx, ty, min(TK, p.k2 - k0), ni, nj);
     __syncthreads();
   }
 #pragma unroll
@@ -280,7 +292,7 @@ __global__ void __launch_bounds__(NT, 2) k2_stack(const P64K2* __restrict__ jobs
   bool on[4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) on[i] = r0 + ty + 16 * i < s.m;
-  const int nj = (min(kTile, s.N - c0) + 15) / 16;
+  const int ni = row_slots(ty, s.m - r0), nj = (min(kTile, s.N - c0) + 15) / 16;
   fill_meta(j.s0);
   fill_meta(j.s0 + 1);
   __syncthreads();
@@ -294,7 +306,7 @@ __global__ void __launch_bounds__(NT, 2) k2_stack(const P64K2* __restrict__ jobs
     __syncthreads();  // (every thread has used meta[st & 1])
     fill_meta(st + 2);
     if (st + 1 < j.s1) load(st + 1);
-    fma_tile(acc, sA, sB, on, tx, ty, min(TK, s.K - st * TK), nj);
+    fma_tile(acc, sA, sB, tx, ty, min(TK, s.K - st * TK), ni, nj);
     __syncthreads();
   }
 #pragma unroll
@@ -351,7 +363,7 @@ __global__ void __launch_bounds__(NT, 2) diag_kernel(const DiagJob* __restrict__
   bool on[4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) on[i] = r0 + ty + 16 * i < j.m;
-  const int nj = (min(kTile, j.n - c0) + 15) / 16;
+  const int ni = row_slots(ty, j.m - r0), nj = (min(kTile, j.n - c0) + 15) / 16;
   load(j.t0);
   for (int t = j.t0; t < j.t1; t += TK) {
 #pragma unroll
@@ -361,7 +373,7 @@ __global__ void __launch_bounds__(NT, 2) diag_kernel(const DiagJob* __restrict__
     }
     __syncthreads();
     if (t + TK < j.t1) load(t + TK);
-    fma_tile(acc, sA, sB, on, tx, ty, min(TK, j.t1 - t), nj);
+    fma_tile(acc, sA, sB, tx, ty, min(TK, j.t1 - t), ni, nj);
     __syncthreads();
   }
 #pragma unroll

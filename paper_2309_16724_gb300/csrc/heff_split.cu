@@ -111,9 +111,12 @@ struct SplitTile {
 // Small-task class: tasks whose four dimensions (m, k1, k2, n) are all at
 // most kSmallDim run in FP64 on CUDA cores instead of the split tensor path
 // (no slabs, no MMA tile padding, no drain chunk).  One warp per segment of
-// up to kSmallSeg tasks of one output block writes a partial block; a second
-// pass adds each block's partials into F in segment order (deterministic).
-constexpr int kSmallSeg = 32;
+// tasks of one output block (sorted by left block) writes a partial block; a
+// second pass adds each block's partials into F in a fixed order
+// (deterministic).  A segment's length makes one wave of kSmallWarps warps per
+// SM out of all tasks, between 4 and 32: 32 for all left two CTAs per SM at L =
+// 12, D = 100 and took 335 us there
+constexpr int kSmallWarps = 16;
 struct SmallTask {
   int64_t e_off, a_off, d_off;  // psi block, left / right operator block (-1: identity)
   int32_t m, k1, k2, n;
@@ -563,15 +566,18 @@ __global__ void __launch_bounds__(256) part_reduce_kernel(const SplitTile* __res
 }
 
 // FP64 partials of the small-task class: warp w sums v A E D^T over the
-// tasks of segment w, in task order (T = E D^T, k1 x n, then A T, m x n; the
-// operands staged in shared memory), and writes the m x n partial to
-// part[w * kSmallDim^2 ...]; lane l owns the elements l, l + 32, ...
+// tasks of segment w: T = sum_t v_t E D^T (k1 x n) over neighbouring tasks with
+// the same left block, then A T (m x n); the partial goes to part[w *
+// kSmallDim^2 ...].  Lane l owns the elements l, l + 32, ..., eight
+// independent DFMA chains, and loads the next task's operands into registers
+// while it computes
+constexpr int kSmallElems = kSmallDim * kSmallDim / 32;  // elements of a lane
 __global__ void __launch_bounds__(128) small_tasks_kernel(const SmallSeg* __restrict__ segs, int nseg,
                                                           const SmallTask* __restrict__ tasks,
                                                           const double* __restrict__ psi,
                                                           const double* __restrict__ Lop,
                                                           const double* __restrict__ Rop, double* __restrict__ part) {
-  constexpr int kD = kSmallDim * kSmallDim;
+  constexpr int kD = kSmallDim * kSmallDim, kQ = kSmallElems;
   __shared__ double sm[4][4][kD];  // per warp: E, D, A, T
   const int wl = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int w = blockIdx.x * 4 + wl;
@@ -581,63 +587,117 @@ __global__ void __launch_bounds__(128) small_tasks_kernel(const SmallSeg* __rest
   double* A = sm[wl][2];
   double* T = sm[wl][3];
   const SmallSeg g = segs[w];
-  double acc[kD / 32];
+  double acc[kQ], ts[kQ], pe[kQ], pd[kQ];
 #pragma unroll
-  for (int q = 0; q < kD / 32; ++q) acc[q] = 0.0;
+  for (int q = 0; q < kQ; ++q) acc[q] = ts[q] = pe[q] = pd[q] = 0.0;
+  auto fetch = [&](const SmallTask& t) {
+#pragma unroll
+    for (int q = 0; q < kQ; ++q) {
+      const int i = lane + 32 * q;
+      if (i < t.k1 * t.k2) pe[q] = psi[t.e_off + i];
+      if (t.d_off >= 0 && i < t.n * t.k2) pd[q] = Rop[t.d_off + i];
+    }
+  };
+  SmallTask t = tasks[g.t0];
+  fetch(t);
+  bool fresh = true;  // the first task of its left block
   for (int ti = g.t0; ti < g.t1; ++ti) {
-    const SmallTask t = tasks[ti];
-    for (int i = lane; i < t.k1 * t.k2; i += 32) E[i] = psi[t.e_off + i];
-    if (t.d_off >= 0)
-      for (int i = lane; i < t.n * t.k2; i += 32) D[i] = Rop[t.d_off + i];
-    if (t.a_off >= 0)
+    const int nE = t.k1 * t.k2, nD = t.n * t.k2, nT = t.k1 * t.n;
+#pragma unroll
+    for (int q = 0; q < kQ; ++q) {
+      const int i = lane + 32 * q;
+      if (i < nE) E[i] = pe[q];
+      if (t.d_off >= 0 && i < nD) D[i] = pd[q];
+    }
+    if (fresh && t.a_off >= 0)
       for (int i = lane; i < t.m * t.k1; i += 32) A[i] = Lop[t.a_off + i];
     __syncwarp();
-    // T = E D^T (identity D: T = E)
-    for (int i = lane; i < t.k1 * t.n; i += 32) {
-      const int r = i % t.k1, c = i / t.k1;
-      double x = 0.0;
-      if (t.d_off >= 0) {
-        for (int k = 0; k < t.k2; ++k) x = fma(E[r + k * t.k1], D[c + k * t.n], x);
-      } else {
-        x = E[i];
-      }
-      T[i] = x;
-    }
-    __syncwarp();
-    // += v A T (identity A: += v T)
+    const SmallTask nx = tasks[min(ti + 1, g.t1 - 1)];
+    if (ti + 1 < g.t1) fetch(nx);
+    // element i of T: row i % k1, column i / k1 (i < 256, k1 <= 16: the reciprocal is exact)
+    const int inv = (65536 + t.k1 - 1) / t.k1;
+    int ro[kQ], co[kQ];
+    double x[kQ];
 #pragma unroll
-    for (int q = 0; q < kD / 32; ++q) {
+    for (int q = 0; q < kQ; ++q) {
       const int i = lane + 32 * q;
-      if (i < t.m * t.n) {
-        const int r = i % t.m, c = i / t.m;
-        double x = 0.0;
-        if (t.a_off >= 0) {
-          for (int k = 0; k < t.k1; ++k) x = fma(A[r + k * t.m], T[k + c * t.k1], x);
-        } else {
-          x = T[r + c * t.k1];
-        }
-        acc[q] = fma(t.v, x, acc[q]);
-      }
+      co[q] = (i * inv) >> 16;
+      ro[q] = i - co[q] * t.k1;
+      x[q] = 0.0;
     }
+    const int nq = (nT + 31) >> 5;
+    if (t.d_off >= 0) {
+      for (int k = 0; k < t.k2; ++k) {
+        const double* Ek = E + k * t.k1;
+        const double* Dk = D + k * t.n;
+#pragma unroll
+        for (int q = 0; q < kQ; ++q) {
+          if (q >= nq) break;
+          if (co[q] < t.n) x[q] = fma(Ek[ro[q]], Dk[co[q]], x[q]);
+        }
+      }
+    } else {  // identity D: T = E
+#pragma unroll
+      for (int q = 0; q < kQ; ++q)
+        if (lane + 32 * q < nT) x[q] = E[lane + 32 * q];
+    }
+#pragma unroll
+    for (int q = 0; q < kQ; ++q) ts[q] = fma(t.v, x[q], ts[q]);
+    const bool last = ti + 1 == g.t1 || nx.a_off != t.a_off || nx.k1 != t.k1;
+    if (last) {  // acc += A T (identity A: += T)
+      if (t.a_off < 0) {
+#pragma unroll
+        for (int q = 0; q < kQ; ++q) acc[q] += ts[q];
+      } else {
+#pragma unroll
+        for (int q = 0; q < kQ; ++q)
+          if (lane + 32 * q < nT) T[lane + 32 * q] = ts[q];
+        __syncwarp();
+        const int invm = (65536 + t.m - 1) / t.m, nF = t.m * t.n, nqf = (nF + 31) >> 5;
+#pragma unroll
+        for (int q = 0; q < kQ; ++q) {
+          const int i = lane + 32 * q;
+          co[q] = (i * invm) >> 16;
+          ro[q] = i - co[q] * t.m;
+          co[q] = min(co[q], t.n - 1) * t.k1;
+        }
+        for (int k = 0; k < t.k1; ++k) {
+          const double* Ak = A + k * t.m;
+#pragma unroll
+          for (int q = 0; q < kQ; ++q) {
+            if (q >= nqf) break;
+            acc[q] = fma(Ak[ro[q]], T[co[q] + k], acc[q]);
+          }
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < kQ; ++q) ts[q] = 0.0;
+    }
+    fresh = last;
+    t = nx;
     __syncwarp();
   }
 #pragma unroll
-  for (int q = 0; q < kD / 32; ++q) part[int64_t(w) * kD + lane + 32 * q] = acc[q];
+  for (int q = 0; q < kQ; ++q) part[int64_t(w) * kD + lane + 32 * q] = acc[q];
 }
 
-// F += the partials of each output block's segments, in segment order: one
-// warp per output block
-__global__ void small_reduce_kernel(const SmallOut* __restrict__ outs, int nout, const double* __restrict__ part,
-                                    double* __restrict__ F) {
+// F += the partials of each output block's segments: one CTA per output block,
+// four threads per element (every fourth segment each), added in that order
+__global__ void __launch_bounds__(4 * kSmallDim * kSmallDim) small_reduce_kernel(const SmallOut* __restrict__ outs,
+                                                                                 const double* __restrict__ part,
+                                                                                 double* __restrict__ F) {
   constexpr int kD = kSmallDim * kSmallDim;
-  const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (w >= nout) return;
-  const SmallOut o = outs[w];
-  for (int i = lane; i < o.m * o.n; i += 32) {
-    double x = 0.0;
-    for (int sg = o.s0; sg < o.s1; ++sg) x += part[int64_t(sg) * kD + i];
-    F[o.f_off + i] += x;
+  __shared__ double sm[4][kD];
+  const SmallOut o = outs[blockIdx.x];
+  const int i = threadIdx.x & (kD - 1), g = threadIdx.x / kD;
+  double x = 0.0;
+  if (i < o.m * o.n) {
+#pragma unroll 4
+    for (int sg = o.s0 + g; sg < o.s1; sg += 4) x += part[int64_t(sg) * kD + i];
   }
+  sm[g][i] = x;
+  __syncthreads();
+  if (g == 0 && i < o.m * o.n) F[o.f_off + i] += (sm[0][i] + sm[1][i]) + (sm[2][i] + sm[3][i]);
 }
 
 template <class T>
@@ -786,14 +846,16 @@ int split_prepare(su2_env* env, int S, std::string& err) {
     const Block& Eb = B[t.e];
     return std::max(std::max(Fb.rows, Fb.cols), std::max(Eb.rows, Eb.cols)) <= kSmallDim;
   };
-  // ---------------------------------------------------------- small-task class, in task order (sorted by output block)
-  std::vector<int64_t> big;  // the other tasks
-  for (int64_t i = 0; i < nt; ++i) {
+  // ---------------------------------------------------------- small-task class, by output block and left block
+  std::vector<int64_t> big, few;  // the other tasks; the small ones
+  for (int64_t i = 0; i < nt; ++i) (is_small(env->tasks[i]) ? few : big).push_back(i);
+  std::stable_sort(few.begin(), few.end(), [&](int64_t x, int64_t y) {
+    const Task &p = env->tasks[x], &q = env->tasks[y];
+    return p.f != q.f ? p.f < q.f : p.ablk < q.ablk;
+  });
+  const int64_t seg_len = std::max<int64_t>(4, std::min<int64_t>(32, (int64_t(few.size()) + st->n_sms * kSmallWarps - 1) / (st->n_sms * kSmallWarps)));
+  for (int64_t i : few) {
     const Task& t = env->tasks[i];
-    if (!is_small(t)) {
-      big.push_back(i);
-      continue;
-    }
     const Block& Fb = B[t.f];
     const Block& Eb = B[t.e];
     const int32_t ti = int32_t(st->small.size());
@@ -802,7 +864,7 @@ int split_prepare(su2_env* env, int S, std::string& err) {
       st->small_out.push_back(SmallOut{Fb.offset, Fb.rows, Fb.cols, sg, sg});
     }
     SmallOut& so = st->small_out.back();
-    if (so.s1 == so.s0 || st->small_seg.back().t1 - st->small_seg.back().t0 == kSmallSeg) {
+    if (so.s1 == so.s0 || st->small_seg.back().t1 - st->small_seg.back().t0 == seg_len) {
       st->small_seg.push_back(SmallSeg{ti, ti});
       so.s1 += 1;
     }
@@ -1409,7 +1471,7 @@ int split_apply(su2_env* env, const double* psi, double* F, std::string& err) {
     const int nseg = int(st->small_seg.size()), nout = int(st->small_out.size());
     small_tasks_kernel<<<unsigned((nseg + 3) / 4), 128, 0, s>>>(st->d_small_seg, nseg, st->d_small, psi, env->dL,
                                                                  env->dR, st->d_small_part);
-    small_reduce_kernel<<<unsigned((nout + 3) / 4), 128, 0, s>>>(st->d_small_out, nout, st->d_small_part, F);
+    small_reduce_kernel<<<unsigned(nout), 4 * kSmallDim * kSmallDim, 0, s>>>(st->d_small_out, st->d_small_part, F);
     pf.end(s, slot);
     SPLIT_CHECK("small tasks");
   }

@@ -15,18 +15,20 @@
 
 namespace su2 {
 int dav_grid(int64_t n);
-void dav_multidot(cudaStream_t, const double*, int64_t, int, const double*, int64_t, double*, double*, double,
+void dav_multidot(cudaStream_t, const double*, int64_t, int, const double*, int64_t, double*, double*,
+                  const int* dn = nullptr);
+void dav_ortho(cudaStream_t, const double*, int64_t, int, const double*, int64_t, bool, double*, double*, double*,
+               const int* dn = nullptr);
+void dav_ritz(cudaStream_t, const double*, const double*, int64_t, int, const double*, const double*, const double*,
+              int64_t, double*, double*, double*, double*, const int* dn = nullptr);
+void dav_rayleigh(cudaStream_t, double*, int, int, const double*, int64_t, double*, double*, int*,
                   const int* dn = nullptr);
 void dav_combine(cudaStream_t, const double*, const double*, int64_t, int, const double*, int64_t, double*, double*,
                  const int* dn = nullptr);
-void dav_subtract(cudaStream_t, const double*, int64_t, int, const double*, int64_t, double*, const int* dn = nullptr);
 void dav_residual(cudaStream_t, const double*, const double*, const double*, int64_t, double*);
-void dav_precond(cudaStream_t, const double*, const double*, const double*, int64_t, double*);
 void dav_scale(cudaStream_t, double*, const double*, const double*, int64_t);
-void dav_jacobi(cudaStream_t, const double*, int, int, double*, double*, int*, const int* dn = nullptr);
 void dav_absmax(cudaStream_t, const double*, int64_t, double*, int64_t*, int*);
 void dav_diag_set(cudaStream_t, double*, int, int, const double*);
-void dav_copy_col(cudaStream_t, double*, int, int, const double*, int, const int* dn = nullptr);
 void dav_newest(cudaStream_t, double*, int64_t, const int*, double*, int);
 void dav_restart(cudaStream_t, double*, double*, int64_t, const double*, int, double*, const double*, int, int, int*,
                  double*);
@@ -919,7 +921,7 @@ struct su2_dav {
   const su2_env* env = nullptr;
   su2_dav_opts o{};
   int64_t n = 0;
-  double *V = nullptr, *AV = nullptr, *x = nullptr, *ax = nullptr, *r = nullptr, *t = nullptr, *tmp = nullptr,
+  double *V = nullptr, *AV = nullptr, *x = nullptr, *t = nullptr, *tmp = nullptr,
          *diag = nullptr;
   double *Hsub = nullptr, *Y = nullptr, *w = nullptr, *h = nullptr, *partial = nullptr, *scal = nullptr;
   int64_t* pidx = nullptr;
@@ -948,7 +950,7 @@ static void dav_free(su2_dav* d) {
   cudaFree(d->d_nsub);
   cudaFree(d->w_in);
   cudaFree(d->w_out);
-  double* ps[] = {d->V, d->AV, d->x, d->ax, d->r, d->t, d->tmp, d->diag, d->Hsub, d->Y, d->w, d->h, d->partial, d->scal};
+  double* ps[] = {d->V, d->AV, d->x, d->t, d->tmp, d->diag, d->Hsub, d->Y, d->w, d->h, d->partial, d->scal};
   for (double* p : ps) cudaFree(p);
   cudaFree(d->pidx);
   if (d->host) cudaFreeHost(d->host);
@@ -1000,8 +1002,6 @@ int su2_davidson_create(su2_ctx* ctx, const su2_env* env, const double* psi0, co
   rc = dev_alloc(ctx, &d->V, size_t(ms) * n);
   if (!rc) rc = dev_alloc(ctx, &d->AV, size_t(ms) * n);
   if (!rc) rc = dev_alloc(ctx, &d->x, size_t(n));
-  if (!rc) rc = dev_alloc(ctx, &d->ax, size_t(n));
-  if (!rc) rc = dev_alloc(ctx, &d->r, size_t(n));
   if (!rc) rc = dev_alloc(ctx, &d->t, size_t(n));
   if (!rc) rc = dev_alloc(ctx, &d->tmp, size_t(2 * d->o.keep) * n);
   if (!rc) rc = dev_alloc(ctx, &d->diag, size_t(n));
@@ -1035,7 +1035,7 @@ int su2_davidson_create(su2_ctx* ctx, const su2_env* env, const double* psi0, co
     return rc;
   }
   // V0 = psi0 / ||psi0||
-  dav_multidot(s, psi0, n, 1, psi0, n, d->partial, d->scal, 1.0);
+  dav_multidot(s, psi0, n, 1, psi0, n, d->partial, d->scal);
   dav_scale(s, d->V, psi0, d->scal, n);
   cudaMemsetAsync(d->Hsub, 0, 32 * 32 * sizeof(double), s);
   d->nsub = 1;
@@ -1062,19 +1062,13 @@ static int dav_record_iteration(su2_ctx* ctx, su2_dav* d, cudaStream_t s) {
   int rc = su2_apply_heff(ctx, d->env, d->w_in, d->w_out, d->o.prec);
   if (rc) return rc;
   dav_newest(s, d->AV, n, d->d_nsub, d->w_out, 1);
-  dav_multidot(s, d->V, n, 0, d->w_out, n, d->partial, d->h, 1.0, d->d_nsub);
-  dav_copy_col(s, d->Hsub, ld, 0, d->h, 0, d->d_nsub);
-  dav_jacobi(s, d->Hsub, ld, 0, d->w, d->Y, ctx->d_status, d->d_nsub);
-  dav_combine(s, d->V, d->AV, n, 0, d->Y, n, d->x, d->ax, d->d_nsub);
-  dav_residual(s, d->x, d->ax, d->w, n, d->r);
-  dav_multidot(s, d->r, n, 1, d->r, n, d->partial, d->scal, 1.0);
-  dav_precond(s, d->r, d->diag, d->w, n, d->t);
+  dav_multidot(s, d->V, n, 0, d->w_out, n, d->partial, nullptr, d->d_nsub);
+  dav_rayleigh(s, d->Hsub, ld, 0, d->partial, n, d->w, d->Y, ctx->d_status, d->d_nsub);
+  dav_ritz(s, d->V, d->AV, n, 0, d->Y, d->w, d->diag, n, d->x, d->t, d->partial, d->scal, d->d_nsub);
   dav_restart(s, d->V, d->AV, n, d->Y, ld, d->Hsub, d->w, d->o.keep, d->o.max_sub, d->d_nsub, d->tmp);
-  for (int pass = 0; pass < 2; ++pass) {
-    dav_multidot(s, d->V, n, 0, d->t, n, d->partial, d->h, 1.0, d->d_nsub);
-    dav_subtract(s, d->V, n, 0, d->h, n, d->t, d->d_nsub);
-  }
-  dav_multidot(s, d->t, n, 1, d->t, n, d->partial, d->scal + 1, 1.0);
+  dav_multidot(s, d->V, n, 0, d->t, n, d->partial, d->h, d->d_nsub);
+  dav_ortho(s, d->V, n, 0, d->h, n, false, d->t, d->partial, d->h, d->d_nsub);
+  dav_ortho(s, d->V, n, 0, d->h, n, true, d->t, d->partial, d->scal + 1, d->d_nsub);
   dav_append(s, d->V, n, d->d_nsub, d->t, d->scal + 1);
   cudaMemcpyAsync(d->host, d->w, sizeof(double), cudaMemcpyDeviceToHost, s);
   cudaMemcpyAsync(d->host + 1, d->scal, 2 * sizeof(double), cudaMemcpyDeviceToHost, s);
@@ -1146,12 +1140,9 @@ int su2_davidson_step(su2_ctx* ctx, su2_dav* d, double* theta, double* resnorm) 
   const int j = d->nsub - 1;  // newest vector
   rc = su2_apply_heff(ctx, d->env, d->V + int64_t(j) * n, d->AV + int64_t(j) * n, d->o.prec);
   if (rc) return rc;
-  dav_multidot(s, d->V, n, d->nsub, d->AV + int64_t(j) * n, n, d->partial, d->h, 1.0);
-  dav_copy_col(s, d->Hsub, ld, j, d->h, d->nsub);
-  dav_jacobi(s, d->Hsub, ld, d->nsub, d->w, d->Y, ctx->d_status);
-  dav_combine(s, d->V, d->AV, n, d->nsub, d->Y, n, d->x, d->ax);
-  dav_residual(s, d->x, d->ax, d->w, n, d->r);
-  dav_multidot(s, d->r, n, 1, d->r, n, d->partial, d->scal, 1.0);
+  dav_multidot(s, d->V, n, d->nsub, d->AV + int64_t(j) * n, n, d->partial, nullptr);
+  dav_rayleigh(s, d->Hsub, ld, d->nsub, d->partial, n, d->w, d->Y, ctx->d_status);
+  dav_ritz(s, d->V, d->AV, n, d->nsub, d->Y, d->w, d->diag, n, d->x, d->t, d->partial, d->scal);
   CUDA_TRY(ctx, cudaMemcpyAsync(d->host, d->w, sizeof(double), cudaMemcpyDeviceToHost, s));
   CUDA_TRY(ctx, cudaMemcpyAsync(d->host + 1, d->scal, sizeof(double), cudaMemcpyDeviceToHost, s));
   CUDA_TRY(ctx, cudaStreamSynchronize(s));
@@ -1166,7 +1157,6 @@ int su2_davidson_step(su2_ctx* ctx, su2_dav* d, double* theta, double* resnorm) 
     d->converged = true;
     return SU2_OK;
   }
-  dav_precond(s, d->r, d->diag, d->w, n, d->t);
   if (d->nsub >= ms) {  // restart on the lowest Ritz vectors
     const int keep = d->o.keep;
     for (int q = 0; q < keep; ++q)
@@ -1181,11 +1171,10 @@ int su2_davidson_step(su2_ctx* ctx, su2_dav* d, double* theta, double* resnorm) 
     dav_diag_set(s, d->Hsub, ld, keep, d->w);
     d->nsub = keep;
   }
-  for (int pass = 0; pass < 2; ++pass) {  // classical Gram-Schmidt, twice
-    dav_multidot(s, d->V, n, d->nsub, d->t, n, d->partial, d->h, 1.0);
-    dav_subtract(s, d->V, n, d->nsub, d->h, n, d->t);
-  }
-  dav_multidot(s, d->t, n, 1, d->t, n, d->partial, d->scal, 1.0);
+  // classical Gram-Schmidt, twice
+  dav_multidot(s, d->V, n, d->nsub, d->t, n, d->partial, d->h);
+  dav_ortho(s, d->V, n, d->nsub, d->h, n, false, d->t, d->partial, d->h);
+  dav_ortho(s, d->V, n, d->nsub, d->h, n, true, d->t, d->partial, d->scal);
   CUDA_TRY(ctx, cudaMemcpyAsync(d->host + 2, d->scal, sizeof(double), cudaMemcpyDeviceToHost, s));
   CUDA_TRY(ctx, cudaStreamSynchronize(s));
   if (!(d->host[2] > 1e-28)) {  // correction vanished: nothing left to add
@@ -1230,8 +1219,8 @@ int su2_energy_check(su2_ctx* ctx, su2_dav* d, int32_t prec, double* rq, double*
   if (!rc) rc = su2_apply_heff(ctx, d->env, d->x, hx, prec);
   double xs[2] = {0.0, 0.0}, rr = 0.0;
   if (!rc) {
-    dav_multidot(s, d->x, n, 1, d->x, n, d->partial, d->scal, 1.0);   // <x|x>
-    dav_multidot(s, d->x, n, 1, hx, n, d->partial, d->scal + 1, 1.0);  // <x|Hx>
+    dav_multidot(s, d->x, n, 1, d->x, n, d->partial, d->scal);   // <x|x>
+    dav_multidot(s, d->x, n, 1, hx, n, d->partial, d->scal + 1);  // <x|Hx>
     if (cudaMemcpyAsync(xs, d->scal, 2 * sizeof(double), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess)
       rc = fail(ctx, SU2_ECUDA, "energy check: reading the dot products");
@@ -1246,7 +1235,7 @@ int su2_energy_check(su2_ctx* ctx, su2_dav* d, int32_t prec, double* rq, double*
         rc = fail(ctx, SU2_ECUDA, "energy check: upload");
       if (!rc) {
         dav_residual(s, d->x, hx, d->scal + 2, n, r);
-        dav_multidot(s, r, n, 1, r, n, d->partial, d->scal + 3, 1.0);
+        dav_multidot(s, r, n, 1, r, n, d->partial, d->scal + 3);
         if (cudaMemcpyAsync(&rr, d->scal + 3, sizeof(double), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
             cudaStreamSynchronize(s) != cudaSuccess)
           rc = fail(ctx, SU2_ECUDA, "energy check: reading the residual");
@@ -1279,7 +1268,7 @@ int su2_davidson_vector(su2_ctx* ctx, su2_dav* d, double* x_dev) {
   double xv = 0.0;
   CUDA_TRY(ctx, cudaMemcpy(&xv, d->x + pi[best], sizeof(double), cudaMemcpyDeviceToHost));
   // x has unit norm up to rounding; scale by +-1 / ||x||
-  dav_multidot(s, d->x, n, 1, d->x, n, d->partial, d->scal, 1.0);
+  dav_multidot(s, d->x, n, 1, d->x, n, d->partial, d->scal);
   double nrm2 = 0.0;
   CUDA_TRY(ctx, cudaMemcpyAsync(&nrm2, d->scal, sizeof(double), cudaMemcpyDeviceToHost, s));
   CUDA_TRY(ctx, cudaStreamSynchronize(s));

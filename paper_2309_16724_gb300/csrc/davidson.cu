@@ -18,7 +18,33 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-// partial[blockIdx.x * nvec + i] = sum over this CTA's slice of V_i . w
+// the CTA's sums of acc[0 .. nvec) into partial[i * gridDim.x + blockIdx.x]
+__device__ __forceinline__ void put_partials(const double (&acc)[kMaxSub], int nvec, double (*red)[kMaxSub],
+                                             double* __restrict__ partial) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+  for (int i = 0; i < kMaxSub; ++i) {
+    if (i >= nvec) break;
+    const double s = warp_sum(acc[i]);
+    if (lane == 0) red[wid][i] = s;
+  }
+  __syncthreads();
+  if (threadIdx.x < nvec) {
+    double s = 0.0;
+    for (int q = 0; q < kRedThreads / 32; ++q) s += red[q][threadIdx.x];
+    partial[int64_t(threadIdx.x) * gridDim.x + blockIdx.x] = s;
+  }
+}
+
+// sum of ng partials of one vector by a whole warp (lane-strided, then a fixed shuffle tree); valid in lane 0
+__device__ __forceinline__ double sum_partials(const double* __restrict__ p, int ng) {
+  double s = 0.0;
+#pragma unroll 8
+  for (int g = threadIdx.x & 31; g < ng; g += 32) s += p[g];
+  return warp_sum(s);
+}
+
+// partial[i * gridDim.x + blockIdx.x] = sum over this CTA's slice of V_i . w
 __global__ void __launch_bounds__(kRedThreads) multidot_kernel(const double* __restrict__ V, int64_t ldv, int nvec,
                                                                const double* __restrict__ w, int64_t n,
                                                                double* __restrict__ partial, const int* __restrict__ dn) {
@@ -34,31 +60,18 @@ __global__ void __launch_bounds__(kRedThreads) multidot_kernel(const double* __r
     for (int i = 0; i < kMaxSub; ++i)
       if (i < nvec) acc[i] = fma(V[i * ldv + x], wx, acc[i]);
   }
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-  for (int i = 0; i < kMaxSub; ++i) {
-    if (i >= nvec) break;
-    const double s = warp_sum(acc[i]);
-    if (lane == 0) red[wid][i] = s;
-  }
-  __syncthreads();
-  if (threadIdx.x < nvec) {
-    double s = 0.0;
-    for (int q = 0; q < kRedThreads / 32; ++q) s += red[q][threadIdx.x];
-    partial[int64_t(blockIdx.x) * nvec + threadIdx.x] = s;
-  }
+  put_partials(acc, nvec, red, partial);
 }
 
-// out[i] = scale * sum_g partial[g*nvec + i]  (fixed order)
-__global__ void reduce_partials_kernel(const double* __restrict__ partial, int ng, int nvec, double scale,
-                                       double* __restrict__ out, const int* __restrict__ dn) {
+// out[i] = sum_g partial[i * ng + g], one warp per vector (one thread walking
+// the 1216 partials of a vector took 80 us, six times per iteration)
+__global__ void __launch_bounds__(1024) reduce_partials_kernel(const double* __restrict__ partial, int ng, int nvec,
+                                                               double* __restrict__ out, const int* __restrict__ dn) {
   if (dn) nvec = *dn + nvec;
-  const int i = threadIdx.x;
-  if (i < nvec) {
-    double s = 0.0;
-    for (int g = 0; g < ng; ++g) s += partial[int64_t(g) * nvec + i];
-    out[i] = scale * s;
-  }
+  const int i = threadIdx.x >> 5;
+  if (i >= nvec) return;
+  const double s = sum_partials(partial + int64_t(i) * ng, ng);
+  if ((threadIdx.x & 31) == 0) out[i] = s;
 }
 
 // out = sum_i y[i] V_i    (and optionally out2 = sum_i y[i] W_i)
@@ -81,18 +94,74 @@ __global__ void combine_kernel(const double* __restrict__ V, const double* __res
   }
 }
 
-// t -= sum_i h[i] V_i
-__global__ void subtract_kernel(const double* __restrict__ V, int64_t ldv, int nvec, const double* __restrict__ h,
-                                int64_t n, double* __restrict__ t, const int* __restrict__ dn) {
+// t -= sum_i h[i] V_i, and in the same pass the partial sums of V_i . t (norm
+// = 0) or of t . t (norm = 1) of the new t: the second read of V hits L1
+__global__ void __launch_bounds__(kRedThreads) ortho_kernel(const double* __restrict__ V, int64_t ldv, int nvec,
+                                                            const double* __restrict__ h, int64_t n, int norm,
+                                                            double* __restrict__ t, double* __restrict__ partial,
+                                                            const int* __restrict__ dn) {
   if (dn) nvec = *dn + nvec;
-  __shared__ double sh[kMaxSub];
+  __shared__ double sh[kMaxSub], red[kRedThreads / 32][kMaxSub];
   if (threadIdx.x < nvec) sh[threadIdx.x] = h[threadIdx.x];
   __syncthreads();
+  double acc[kMaxSub];
+#pragma unroll
+  for (int i = 0; i < kMaxSub; ++i) acc[i] = 0.0;
   const int64_t stride = int64_t(gridDim.x) * blockDim.x;
   for (int64_t x = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; x < n; x += stride) {
     double a = t[x];
-    for (int i = 0; i < nvec; ++i) a = fma(-sh[i], V[i * ldv + x], a);
+#pragma unroll
+    for (int i = 0; i < kMaxSub; ++i)
+      if (i < nvec) a = fma(-sh[i], V[i * ldv + x], a);
     t[x] = a;
+    if (norm) {
+      acc[0] = fma(a, a, acc[0]);
+    } else {
+#pragma unroll
+      for (int i = 0; i < kMaxSub; ++i)
+        if (i < nvec) acc[i] = fma(V[i * ldv + x], a, acc[i]);
+    }
+  }
+  put_partials(acc, norm ? 1 : nvec, red, partial);
+}
+
+// Ritz pair, residual and correction in one pass: x = V y, r = AV y - theta x,
+// t = r / (diag - theta) with |diag - theta| clamped to >= 1e-12 (sign kept),
+// and the partial sums of r . r
+__global__ void __launch_bounds__(kRedThreads) ritz_kernel(const double* __restrict__ V, const double* __restrict__ W,
+                                                           int64_t ldv, int nvec, const double* __restrict__ y,
+                                                           const double* __restrict__ theta,
+                                                           const double* __restrict__ diag, int64_t n,
+                                                           double* __restrict__ xout, double* __restrict__ t,
+                                                           double* __restrict__ partial, const int* __restrict__ dn) {
+  if (dn) nvec = *dn + nvec;
+  __shared__ double sy[kMaxSub], red[kRedThreads / 32];
+  if (threadIdx.x < nvec) sy[threadIdx.x] = y[threadIdx.x];
+  __syncthreads();
+  const double th = *theta;
+  double acc = 0.0;
+  const int64_t stride = int64_t(gridDim.x) * blockDim.x;
+  for (int64_t x = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; x < n; x += stride) {
+    double a = 0.0, b = 0.0;
+#pragma unroll 8
+    for (int i = 0; i < nvec; ++i) {
+      a = fma(sy[i], V[i * ldv + x], a);
+      b = fma(sy[i], W[i * ldv + x], b);
+    }
+    const double r = fma(-th, a, b);
+    double d = diag[x] - th;
+    if (fabs(d) < 1e-12) d = d >= 0.0 ? 1e-12 : -1e-12;
+    xout[x] = a;
+    t[x] = r / d;
+    acc = fma(r, r, acc);
+  }
+  acc = warp_sum(acc);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double s = 0.0;
+    for (int q = 0; q < kRedThreads / 32; ++q) s += red[q];
+    partial[blockIdx.x] = s;
   }
 }
 
@@ -104,18 +173,6 @@ __global__ void residual_kernel(const double* __restrict__ x, const double* __re
   for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += stride) r[i] = fma(-th, x[i], ax[i]);
 }
 
-// t = r / (diag - theta), |diag - theta| clamped to >= 1e-12 (sign kept)
-__global__ void precond_kernel(const double* __restrict__ r, const double* __restrict__ diag,
-                               const double* __restrict__ theta, int64_t n, double* __restrict__ t) {
-  const double th = *theta;
-  const int64_t stride = int64_t(gridDim.x) * blockDim.x;
-  for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += stride) {
-    double d = diag[i] - th;
-    if (fabs(d) < 1e-12) d = d >= 0.0 ? 1e-12 : -1e-12;
-    t[i] = r[i] / d;
-  }
-}
-
 // y = x * s[0]^(-1/2) when s holds a squared norm
 __global__ void scale_kernel(double* __restrict__ y, const double* __restrict__ x, const double* __restrict__ nrm2,
                              int64_t n) {
@@ -124,85 +181,110 @@ __global__ void scale_kernel(double* __restrict__ y, const double* __restrict__ 
   for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += stride) y[i] = x[i] * s;
 }
 
-// cyclic Jacobi on the symmetrised nsub x nsub matrix H (leading dim ld);
-// outputs ascending eigenvalues w and eigenvectors Y (column j, ld rows)
-__global__ void jacobi_kernel(const double* __restrict__ H, int ld, int n, double* __restrict__ w,
-                              double* __restrict__ Y, int* __restrict__ status, const int* __restrict__ dn) {
+// Rayleigh-Ritz of the subspace: the new column of the projected matrix H
+// (leading dim ld) from the partial sums of V_i . A V_(n-1), then cyclic Jacobi
+// on its symmetrised n x n part; ascending eigenvalues w and eigenvectors Y
+// (column j, ld rows).  One CTA; the n / 2 rotations of a round (round-robin
+// order) act on disjoint rows and columns and run side by side, one warp each.
+// A rotation's tangent is taken in FP32 (from entries scaled to their common
+// exponent) and c = 1 / sqrt(1 + t^2), s = t c in FP64: orthogonal to FP64
+// accuracy, while the annihilated entry is left at 1e-7 of its size for the
+// next sweep.  One rotation after another, each with FP64 divisions and square
+// roots by one thread, took about 1.7 us a rotation, 2 to 3 ms at n = 24.
+__global__ void __launch_bounds__(1024) rayleigh_kernel(double* __restrict__ H, int ld, int n,
+                                                        const double* __restrict__ partial, int ng,
+                                                        double* __restrict__ w, double* __restrict__ Y,
+                                                        int* __restrict__ status, const int* __restrict__ dn) {
   if (dn) n = *dn + n;
   __shared__ double A[kMaxSub][kMaxSub + 1], V[kMaxSub][kMaxSub + 1];
-  __shared__ double cs[2];
+  __shared__ double soff[32], stot[32];
   __shared__ int done;
-  const int t = threadIdx.x;
-  for (int idx = t; idx < n * n; idx += blockDim.x) {
-    const int i = idx % n, j = idx / n;
-    A[i][j] = 0.5 * (H[i + j * ld] + H[j + i * ld]);
-    V[i][j] = (i == j) ? 1.0 : 0.0;
+  const int t = threadIdx.x & 31, k = threadIdx.x >> 5;
+  if (k < n) {
+    const double h = sum_partials(partial + int64_t(k) * ng, ng);
+    if (t == 0) {
+      H[k + (n - 1) * ld] = h;
+      H[(n - 1) + k * ld] = h;
+    }
   }
   __syncthreads();
+  if (k < n && t < n) {
+    A[k][t] = 0.5 * (H[k + t * ld] + H[t + k * ld]);
+    V[k][t] = (k == t) ? 1.0 : 0.0;
+  }
+  if (threadIdx.x == 0) done = 0;
+  __syncthreads();
+  const int m = n + (n & 1);  // (an odd n plays against a dummy)
   for (int sweep = 0; sweep < 60; ++sweep) {
+    const double v = (k < n && t < n) ? A[k][t] : 0.0;
+    const double o = warp_sum(k == t ? 0.0 : v * v), d = warp_sum(v * v);
     if (t == 0) {
-      double off = 0.0, tot = 0.0;
-      for (int i = 0; i < n; ++i)
-        for (int j = 0; j < n; ++j) {
-          tot += A[i][j] * A[i][j];
-          if (i != j) off += A[i][j] * A[i][j];
-        }
-      done = (off <= 1e-30 * tot) || tot == 0.0;
+      soff[k] = o;
+      stot[k] = d;
+    }
+    __syncthreads();
+    if (threadIdx.x < 32) {
+      const double off = warp_sum(soff[t]), tot = warp_sum(stot[t]);
+      if (t == 0) done = (off <= 1e-30 * tot) || tot == 0.0;
     }
     __syncthreads();
     if (done) break;
-    for (int p = 0; p < n - 1; ++p)
-      for (int q = p + 1; q < n; ++q) {
-        if (t == 0) {
-          const double apq = A[p][q];
-          double c = 1.0, s = 0.0;
-          if (apq != 0.0) {
-            const double tau = (A[q][q] - A[p][p]) / (2.0 * apq);
-            const double tt = (tau >= 0.0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
-            c = 1.0 / sqrt(1.0 + tt * tt);
-            s = tt * c;
-          }
-          cs[0] = c;
-          cs[1] = s;
+    for (int r = 0; r < m - 1; ++r) {
+      int p = 0, q = 0;
+      double c = 1.0, s = 0.0;
+      if (k < m / 2) {
+        p = k == 0 ? m - 1 : (r + k) % (m - 1);
+        q = k == 0 ? r : (r + m - 1 - k) % (m - 1);
+        if (p > q) {
+          const int x = p;
+          p = q;
+          q = x;
         }
-        __syncthreads();
-        const double c = cs[0], s = cs[1];
-        if (s != 0.0) {
-          if (t < n) {  // columns p, q
-            const double akp = A[t][p], akq = A[t][q];
-            A[t][p] = c * akp - s * akq;
-            A[t][q] = s * akp + c * akq;
-            const double vkp = V[t][p], vkq = V[t][q];
-            V[t][p] = c * vkp - s * vkq;
-            V[t][q] = s * vkp + c * vkq;
-          }
-          __syncthreads();
-          if (t < n) {  // rows p, q
-            const double apk = A[p][t], aqk = A[q][t];
-            A[p][t] = c * apk - s * aqk;
-            A[q][t] = s * apk + c * aqk;
+        if (q < n) {
+          const double apq = A[p][q], df = A[q][q] - A[p][p];
+          // common scale: the larger of the two gets exponent 0
+          const int be = max((__double2hiint(apq) >> 20) & 0x7FF, (__double2hiint(df) >> 20) & 0x7FF);
+          const double sc = __longlong_as_double((long long)min(2046, max(1, 2046 - be)) << 52);
+          const float fa = (float)(apq * sc), fd = (float)(df * sc);
+          if (fa != 0.f) {
+            const float tau = fd / (2.f * fa);
+            float tt = fabsf(tau) > 1e9f ? 0.5f / fabsf(tau) : 1.f / (fabsf(tau) + sqrtf(1.f + tau * tau));
+            if (tau < 0.f) tt = -tt;
+            const double td = tt, x = fma(td, td, 1.0);
+            double y = rsqrtf((float)x);
+            y = y * fma(-0.5 * x * y, y, 1.5);
+            y = y * fma(-0.5 * x * y, y, 1.5);
+            c = y;
+            s = td * y;
           }
         }
-        __syncthreads();
       }
-  }
-  if (t == 0) {
-    // selection sort of eigenpairs, ascending
-    int order[kMaxSub];
-    for (int i = 0; i < n; ++i) order[i] = i;
-    for (int i = 0; i < n; ++i)
-      for (int j = i + 1; j < n; ++j)
-        if (A[order[j]][order[j]] < A[order[i]][order[i]]) {
-          const int tmp = order[i];
-          order[i] = order[j];
-          order[j] = tmp;
-        }
-    for (int j = 0; j < n; ++j) {
-      w[j] = A[order[j]][order[j]];
-      for (int i = 0; i < n; ++i) Y[i + j * ld] = V[i][order[j]];
+      __syncthreads();
+      if (s != 0.0 && t < n) {  // columns p, q
+        const double akp = A[t][p], akq = A[t][q];
+        A[t][p] = c * akp - s * akq;
+        A[t][q] = s * akp + c * akq;
+        const double vkp = V[t][p], vkq = V[t][q];
+        V[t][p] = c * vkp - s * vkq;
+        V[t][q] = s * vkp + c * vkq;
+      }
+      __syncthreads();
+      if (s != 0.0 && t < n) {  // rows p, q
+        const double apk = A[p][t], aqk = A[q][t];
+        A[p][t] = c * apk - s * aqk;
+        A[q][t] = s * apk + c * aqk;
+      }
+      __syncthreads();
     }
-    if (!done) *status = 4;
   }
+  if (k < n) {  // eigenpair k to its place in ascending order (ties: by index)
+    int rank = 0;
+    const double e = A[k][k];
+    for (int j = 0; j < n; ++j) rank += A[j][j] < e || (A[j][j] == e && j < k);
+    if (t == 0) w[rank] = e;
+    if (t < n) Y[t + rank * ld] = V[t][k];
+  }
+  if (threadIdx.x == 0 && !done) *status = 4;
 }
 
 // partial max |x| and its index per CTA
@@ -241,19 +323,6 @@ __global__ void diag_set_kernel(double* __restrict__ H, int ld, int n, const dou
   for (int idx = threadIdx.x; idx < ld * ld; idx += blockDim.x) {
     const int i = idx % ld, j = idx / ld;
     H[idx] = (i == j && i < n) ? w[i] : 0.0;
-  }
-}
-
-__global__ void copy_col_kernel(double* __restrict__ H, int ld, int col, const double* __restrict__ h, int n,
-                                const int* __restrict__ dn) {
-  if (dn) {  // column nsub-1, n = nsub
-    n = *dn;
-    col = n - 1;
-  }
-  const int i = threadIdx.x;
-  if (i < n) {
-    H[i + col * ld] = h[i];
-    H[col + i * ld] = h[i];
   }
 }
 
@@ -329,31 +398,42 @@ int dav_grid(int64_t n) {
   return g < 1 ? 1 : (g > 152 * 8 ? 152 * 8 : g);
 }
 
+// partial sums of V_i . w; out (if given) gets the sums
 void dav_multidot(cudaStream_t s, const double* V, int64_t ldv, int nvec, const double* w, int64_t n,
-                  double* partial, double* out, double scale, const int* dn) {
+                  double* partial, double* out, const int* dn) {
   const int g = dav_grid(n);
   multidot_kernel<<<g, kRedThreads, 0, s>>>(V, ldv, nvec, w, n, partial, dn);
-  reduce_partials_kernel<<<1, 32, 0, s>>>(partial, g, nvec, scale, out, dn);
+  if (out) reduce_partials_kernel<<<1, 1024, 0, s>>>(partial, g, nvec, out, dn);
+}
+// t -= V h, then out = V^T t, or t . t with norm
+void dav_ortho(cudaStream_t s, const double* V, int64_t ldv, int nvec, const double* h, int64_t n, bool norm, double* t,
+               double* partial, double* out, const int* dn) {
+  const int g = dav_grid(n);
+  ortho_kernel<<<g, kRedThreads, 0, s>>>(V, ldv, nvec, h, n, norm ? 1 : 0, t, partial, dn);
+  reduce_partials_kernel<<<1, 1024, 0, s>>>(partial, g, norm ? 1 : nvec, out, norm ? nullptr : dn);
+}
+// x = V y, t = (AV y - theta x) / (diag - theta), out = || AV y - theta x ||^2
+void dav_ritz(cudaStream_t s, const double* V, const double* W, int64_t ldv, int nvec, const double* y,
+              const double* theta, const double* diag, int64_t n, double* x, double* t, double* partial, double* out,
+              const int* dn) {
+  const int g = dav_grid(n);
+  ritz_kernel<<<g, kRedThreads, 0, s>>>(V, W, ldv, nvec, y, theta, diag, n, x, t, partial, dn);
+  reduce_partials_kernel<<<1, 1024, 0, s>>>(partial, g, 1, out, nullptr);
+}
+// Rayleigh-Ritz from the partial sums of the last dav_multidot
+void dav_rayleigh(cudaStream_t s, double* H, int ld, int n, const double* partial, int64_t nvecs, double* w, double* Y,
+                  int* status, const int* dn) {
+  rayleigh_kernel<<<1, 1024, 0, s>>>(H, ld, n, partial, dav_grid(nvecs), w, Y, status, dn);
 }
 void dav_combine(cudaStream_t s, const double* V, const double* W, int64_t ldv, int nvec, const double* y, int64_t n,
                  double* out, double* out2, const int* dn) {
   combine_kernel<<<dav_grid(n), 256, 0, s>>>(V, W, ldv, nvec, y, n, out, out2, dn);
 }
-void dav_subtract(cudaStream_t s, const double* V, int64_t ldv, int nvec, const double* h, int64_t n, double* t,
-                  const int* dn) {
-  subtract_kernel<<<dav_grid(n), 256, 0, s>>>(V, ldv, nvec, h, n, t, dn);
-}
 void dav_residual(cudaStream_t s, const double* x, const double* ax, const double* theta, int64_t n, double* r) {
   residual_kernel<<<dav_grid(n), 256, 0, s>>>(x, ax, theta, n, r);
 }
-void dav_precond(cudaStream_t s, const double* r, const double* diag, const double* theta, int64_t n, double* t) {
-  precond_kernel<<<dav_grid(n), 256, 0, s>>>(r, diag, theta, n, t);
-}
 void dav_scale(cudaStream_t s, double* y, const double* x, const double* nrm2, int64_t n) {
   scale_kernel<<<dav_grid(n), 256, 0, s>>>(y, x, nrm2, n);
-}
-void dav_jacobi(cudaStream_t s, const double* H, int ld, int n, double* w, double* Y, int* status, const int* dn) {
-  jacobi_kernel<<<1, 32, 0, s>>>(H, ld, n, w, Y, status, dn);
 }
 void dav_absmax(cudaStream_t s, const double* x, int64_t n, double* pv, int64_t* pi, int* ng) {
   const int g = dav_grid(n);
@@ -362,9 +442,6 @@ void dav_absmax(cudaStream_t s, const double* x, int64_t n, double* pv, int64_t*
 }
 void dav_diag_set(cudaStream_t s, double* H, int ld, int n, const double* w) {
   diag_set_kernel<<<1, 256, 0, s>>>(H, ld, n, w);
-}
-void dav_copy_col(cudaStream_t s, double* H, int ld, int col, const double* h, int n, const int* dn) {
-  copy_col_kernel<<<1, 32, 0, s>>>(H, ld, col, h, n, dn);
 }
 void dav_newest(cudaStream_t s, double* V, int64_t n, const int* dn, double* w, int dir) {
   newest_copy_kernel<<<dav_grid(n), 256, 0, s>>>(V, n, dn, w, dir);

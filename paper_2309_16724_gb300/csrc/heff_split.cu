@@ -76,7 +76,7 @@ struct Unit { int32_t desc, tr, ks, pad; };
 // One product of the T' sum: T'(w, f) = sum over the tasks with left block w
 // and output block f of v_t T_u
 struct TPTask {
-  int64_t off;           // element (0, 0) of the task's T block in Th / Tl, or of its psi block
+  int64_t off;           // element (0, 0) of the task's block in T, or of its psi block
   int32_t ld;            // column stride, or row stride of a row-major T
   int32_t flags;         // kFromPsi, kRowMajor
   float vh, vl;          // v_t (float-float)
@@ -166,8 +166,10 @@ struct SplitState {
   int *d_ax = nullptr, *d_rho = nullptr, *d_zeta = nullptr, *d_eps = nullptr, *d_gamma = nullptr, *d_grp = nullptr;
   uint8_t *d_ascale = nullptr, *d_scale = nullptr;
   int64_t n_ax = 0, n_rho = 0, n_zeta = 0, n_eps = 0, n_gamma = 0, n_grp = 0;
-  // float-float buffers
-  float *dTh = nullptr, *dTl = nullptr, *dPh = nullptr, *dPl = nullptr;
+  // float-float buffers (leading part, trailing part): T of a chunk, psi.  Side
+  // by side, an 8-K piece is 64 contiguous bytes; in two arrays it was two
+  // 32-byte sectors, and the T' kernel read 30 % more from DRAM than it used
+  float2 *dT = nullptr, *dP = nullptr;
   int64_t t_elems = 0;
   // plan
   std::vector<SChunk> chunks;
@@ -362,7 +364,7 @@ __device__ __forceinline__ void cut_oct(float2 (&h)[4], float2 (&l)[4], int es, 
 // and runs in FP32 (an FP64 cut of the same slabs took 280 us instead of 60
 // at L = 32, D = 2048: GB300's FP64 rate is 1/64 of FP32's)
 __global__ void __launch_bounds__(256) psi_slab_kernel(const SlabDesc* __restrict__ descs, const Unit* __restrict__ units,
-                                                       const double* __restrict__ psi, float* Ph, float* Pl,
+                                                       const double* __restrict__ psi, float2* P,
                                                        int* __restrict__ eps, unsigned char* __restrict__ slab, int S) {
   __shared__ float sm[8][kRowTile];
   const Unit u = units[blockIdx.x];
@@ -376,8 +378,7 @@ __global__ void __launch_bounds__(256) psi_slab_kernel(const SlabDesc* __restric
       const int64_t i = d.src_off + r + int64_t(c) * d.ld;
       const double v = psi[i];
       const float a = (float)v;
-      Ph[i] = a;
-      Pl[i] = (float)(v - (double)a);
+      P[i] = make_float2(a, (float)(v - (double)a));
       m = fmaxf(m, fabsf(a));
     }
   }
@@ -398,45 +399,54 @@ __global__ void __launch_bounds__(256) psi_slab_kernel(const SlabDesc* __restric
     for (int q = 0; q < 8; ++q) {
       const int c = o * 8 + q;
       const int64_t i = d.src_off + r + int64_t(c) * d.ld;
-      hv[q] = c < d.cols ? Ph[i] : 0.f;
-      lv[q] = c < d.cols ? Pl[i] : 0.f;
+      const float2 v = c < d.cols ? P[i] : make_float2(0.f, 0.f);
+      hv[q] = v.x;
+      lv[q] = v.y;
     }
     cut_oct(h, l, sp::kLead - (e < -1000 ? 0 : e), tile + int64_t(o >> 1) * S * trows * 32 + (o & 1) * 128, trows * 32, S);
   }
 }
 
-// eight consecutive rows k.. of column c of a task's T (or psi) block; rows
-// past nk are zero.  Column-major T has 16-byte aligned pieces (row offsets
-// and strides are multiples of 4): rows past the block's end are read (they
-// lie inside the buffer) and dropped.  Row-major T: neighbouring lanes read
-// neighbouring columns.  psi blocks are unpadded.
-__device__ __forceinline__ void load_oct(const TPTask& t, const float* __restrict__ T, const float* __restrict__ P,
-                                         int k, int c, int nk, float (&x)[8]) {
+// eight consecutive rows k.. of column c of a task's T (or psi) block as four
+// packed pairs, leading (a) and trailing parts (b); rows past nk are zero.
+// Column-major T has 64-byte aligned pieces (row offsets and strides are
+// multiples of 8): a row past the block's end may be read with its pair (it
+// lies inside the buffer) and is dropped.  Row-major T: neighbouring lanes
+// read neighbouring columns.  psi blocks are unpadded.
+__device__ __forceinline__ void load_oct(const TPTask& t, const float2* __restrict__ T, const float2* __restrict__ P,
+                                         int k, int c, int nk, float2 (&a)[4], float2 (&b)[4]) {
   if (t.flags == 0) {
     const float4* p = reinterpret_cast<const float4*>(T + t.off + k + int64_t(c) * t.ld);
-    const float4 a = p[0], b = nk > 4 ? p[1] : make_float4(0.f, 0.f, 0.f, 0.f);
-    x[0] = a.x, x[1] = a.y, x[2] = a.z, x[3] = a.w, x[4] = b.x, x[5] = b.y, x[6] = b.z, x[7] = b.w;
 #pragma unroll
-    for (int q = 1; q < 8; ++q)
-      if (q >= nk) x[q] = 0.f;
+    for (int j = 0; j < 4; ++j) {
+      const float4 v = 2 * j < nk ? p[j] : make_float4(0.f, 0.f, 0.f, 0.f);
+      const bool two = 2 * j + 1 < nk;
+      a[j] = make_float2(v.x, two ? v.z : 0.f);
+      b[j] = make_float2(v.y, two ? v.w : 0.f);
+    }
   } else {
     const bool rm = (t.flags & kRowMajor) != 0;
-    const float* p = ((t.flags & kFromPsi) ? P : T) + t.off + (rm ? int64_t(k) * t.ld + c : k + int64_t(c) * t.ld);
+    const float2* p = ((t.flags & kFromPsi) ? P : T) + t.off + (rm ? int64_t(k) * t.ld + c : k + int64_t(c) * t.ld);
     const int64_t step = rm ? t.ld : 1;
 #pragma unroll
-    for (int q = 0; q < 8; ++q) x[q] = q < nk ? p[q * step] : 0.f;
+    for (int j = 0; j < 4; ++j) {
+      const float2 z = make_float2(0.f, 0.f);
+      const float2 u = 2 * j < nk ? p[2 * j * step] : z, v = 2 * j + 1 < nk ? p[(2 * j + 1) * step] : z;
+      a[j] = make_float2(u.x, v.x);
+      b[j] = make_float2(u.y, v.y);
+    }
   }
 }
 
 // h + l += v T of one task, eight K: (a + b) * (vh + vl) in float-float, added
 // with TwoSum
-__device__ __forceinline__ void add_task(const TPTask& t, const float (&av)[8], const float (&bv)[8], float2 (&h)[4],
+__device__ __forceinline__ void add_task(const TPTask& t, const float2 (&av)[4], const float2 (&bv)[4], float2 (&h)[4],
                                          float2 (&l)[4]) {
   const float2 m1 = make_float2(-1.f, -1.f);
   const float2 vh2 = make_float2(t.vh, t.vh), nvh = make_float2(-t.vh, -t.vh), vl2 = make_float2(t.vl, t.vl);
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
-    const float2 a = make_float2(av[2 * j], av[2 * j + 1]), b = make_float2(bv[2 * j], bv[2 * j + 1]);
+    const float2 a = av[j], b = bv[j];
     const float2 pn = __fmul2_rn(a, nvh);               // -RN(a vh)
     float2 e = __ffma2_rn(a, vh2, pn);
     e = __ffma2_rn(a, vl2, e);
@@ -463,8 +473,8 @@ constexpr int kTPWarps = kWinSteps;
 __global__ void __launch_bounds__(32 * kTPWarps, 2)
     tprime_kernel(const TPUnit* __restrict__ units, const Stack* __restrict__ stacks, const Col* __restrict__ cols,
                   const Oct* __restrict__ octs, const int32_t* __restrict__ tab, const TPTask* __restrict__ tasks,
-                  const float* __restrict__ Th, const float* __restrict__ Tl, const float* __restrict__ Ph,
-                  const float* __restrict__ Pl, int* __restrict__ grp, unsigned char* __restrict__ slab, int S) {
+                  const float2* __restrict__ T, const float2* __restrict__ P, int* __restrict__ grp,
+                  unsigned char* __restrict__ slab, int S) {
   __shared__ float sm[kTPWarps][32];
   const TPUnit u = units[blockIdx.x];
   const Stack& s = stacks[u.st];
@@ -486,9 +496,8 @@ __global__ void __launch_bounds__(32 * kTPWarps, 2)
       const int t1 = tb[int64_t(k.w) * nf + 1];
       for (int t = tb[int64_t(k.w) * nf]; t < t1; ++t) {
         const TPTask tk = tasks[t];
-        float av[8], bv[8];
-        load_oct(tk, Th, Ph, k.k, cm.c, k.nk, av);
-        load_oct(tk, Tl, Pl, k.k, cm.c, k.nk, bv);
+        float2 av[4], bv[4];
+        load_oct(tk, T, P, k.k, cm.c, k.nk, av, bv);
         add_task(tk, av, bv, h[i], l[i]);
       }
     }
@@ -766,7 +775,7 @@ double orient_cost(int Mr, int Nr, double steps, double chunks, int S) {
 
 // the stripe GEMM instantiated for each mode and slice count
 using GemmFn = void (*)(const sp::Job*, int, const unsigned char*, const unsigned char*, const int*, const int*, int,
-                        float*, float*, double*, double*, int*, int*, const uint8_t*, const uint8_t*, int, int);
+                        float2*, double*, double*, int*, int*, const uint8_t*, const uint8_t*, int, int);
 GemmFn gemm_fn(int mode, int S) {
   static const GemmFn t[2][sp::kMaxS - 1] = {
       {sp::split_gemm_kernel<sp::MODE_T, 2>, sp::split_gemm_kernel<sp::MODE_T, 3>, sp::split_gemm_kernel<sp::MODE_T, 4>,
@@ -784,8 +793,8 @@ void launch_gemm(int mode, cudaStream_t s, SplitState* st, const Job* jobs, int 
   // 17 % slower K2)
   const int smem = sp::stages_of(st->S, st->sk) * sp::stage_bytes_of(st->S, st->sk) + 1024;
   const int grid = std::min(njobs, st->n_sms);
-  gemm_fn(mode, st->S)<<<grid, sp::kThreads, smem, s>>>(jobs, njobs, A, B, rexp, cexp, 2 * sp::kLead, st->dTh, st->dTl,
-                                                        F, st->d_part, st->d_status, counter, st->d_ascale,
+  gemm_fn(mode, st->S)<<<grid, sp::kThreads, smem, s>>>(jobs, njobs, A, B, rexp, cexp, 2 * sp::kLead, st->dT, F,
+                                                        st->d_part, st->d_status, counter, st->d_ascale,
                                                         st->d_scale, st->sk, st->spin);
 }
 
@@ -1302,10 +1311,8 @@ int split_prepare(su2_env* env, int S, std::string& err) {
   if (!rc2) rc2 = dalloc(&st->dD, size_t(st->d_bytes), err);
   if (!rc2) rc2 = dalloc(&st->dE, size_t(st->e_bytes), err);
   if (!rc2) rc2 = dalloc(&st->dTP, size_t(std::max<int64_t>(st->tp_bytes, 16)), err);
-  if (!rc2) rc2 = dalloc(&st->dTh, size_t(st->t_elems + 16), err);
-  if (!rc2) rc2 = dalloc(&st->dTl, size_t(st->t_elems + 16), err);
-  if (!rc2) rc2 = dalloc(&st->dPh, size_t(env->psi_len), err);
-  if (!rc2) rc2 = dalloc(&st->dPl, size_t(env->psi_len), err);
+  if (!rc2) rc2 = dalloc(&st->dT, size_t(st->t_elems + 16), err);
+  if (!rc2) rc2 = dalloc(&st->dP, size_t(env->psi_len), err);
   if (!rc2) rc2 = dalloc(&st->d_rho, size_t(st->n_rho), err);
   if (!rc2) rc2 = dalloc(&st->d_ax, size_t(st->n_ax), err);
   if (!rc2) rc2 = dalloc(&st->d_ascale, size_t(st->n_ax), err);
@@ -1415,7 +1422,7 @@ int split_apply(su2_env* env, const double* psi, double* F, std::string& err) {
   if (any) {  // (an environment of small tasks only needs no slabs)
     pf.count(1);
     cudaMemsetAsync(st->d_counter, 0, 2 * st->chunks.size() * sizeof(int), s);
-    psi_slab_kernel<<<unsigned(st->erow.size()), 256, 0, s>>>(st->d_edesc, st->d_erow, psi, st->dPh, st->dPl, st->d_eps,
+    psi_slab_kernel<<<unsigned(st->erow.size()), 256, 0, s>>>(st->d_edesc, st->d_erow, psi, st->dP, st->d_eps,
                                                               st->dE, S);
   }
   pf.end(s, slot);
@@ -1450,7 +1457,7 @@ int split_apply(su2_env* env, const double* psi, double* F, std::string& err) {
     SPLIT_CHECK("K1 split GEMM");
     slot = pf.begin(s, 2, 0.0);
     tprime_kernel<<<unsigned(c.tpu1 - c.tpu0), 32 * kTPWarps, 0, s>>>(st->d_tpu + c.tpu0, st->d_stk + c.st0, st->d_col, st->d_oct,
-                                                            st->d_tab, st->d_tpt, st->dTh, st->dTl, st->dPh, st->dPl,
+                                                            st->d_tab, st->d_tpt, st->dT, st->dP,
                                                             st->d_grp, st->dTP, S);
     groupmax_kernel<<<unsigned(c.gu1 - c.gu0), 512, 0, s>>>(st->d_gu + c.gu0, st->d_grp, st->d_gamma, st->d_scale);
     pf.end(s, slot);
@@ -1588,7 +1595,7 @@ void split_free(su2_env* env) {
   if (!st) return;
   void* ps[] = {st->dA, st->dD, st->dE, st->dTP, st->d_adesc, st->d_ddesc, st->d_edesc, st->d_aunit, st->d_dunit,
                 st->d_drow, st->d_erow, st->d_axu, st->d_amu, st->d_gu, st->d_ax, st->d_ascale, st->d_rho, st->d_zeta,
-                st->d_eps, st->d_gamma, st->d_grp, st->dTh, st->dTl, st->dPh, st->dPl, st->d_k1j, st->d_k2j, st->d_tpt,
+                st->d_eps, st->d_gamma, st->d_grp, st->dT, st->dP, st->d_k1j, st->d_k2j, st->d_tpt,
                 st->d_tab, st->d_oct, st->d_stk, st->d_col, st->d_tpu, st->d_spt, st->d_part, st->d_counter,
                 st->d_scale, st->d_small, st->d_small_out, st->d_small_seg, st->d_small_part};
   for (void* p : ps) cudaFree(p);

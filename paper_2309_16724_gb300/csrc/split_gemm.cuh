@@ -312,7 +312,7 @@ template <int MODE, int S>
 __global__ void __launch_bounds__(kThreads, 1)
     split_gemm_kernel(const Job* __restrict__ jobs, int njobs, const unsigned char* __restrict__ Aslab,
                       const unsigned char* __restrict__ Bslab, const int* __restrict__ rexp,
-                      const int* __restrict__ cexp, int shift, float* __restrict__ Th, float* __restrict__ Tl,
+                      const int* __restrict__ cexp, int shift, float2* __restrict__ T,
                       double* __restrict__ F, double* __restrict__ part, int* __restrict__ status,
                       int* __restrict__ job_counter, const uint8_t* __restrict__ ascale,
                       const uint8_t* __restrict__ bscale, int sk, int spin) {
@@ -689,8 +689,7 @@ __global__ void __launch_bounds__(kThreads, 1)
               const float la = (c & 1) ? lo2[c >> 1].y : lo2[c >> 1].x;
               const float hs = __fadd_rn(ha, la), bb = __fsub_rn(hs, ha);
               const float ls = __fadd_rn(__fsub_rn(ha, __fsub_rn(hs, bb)), __fsub_rn(la, bb));
-              Th[o] = ldexp_f(hs, ex);
-              Tl[o] = ldexp_f(ls, ex);
+              T[o] = make_float2(ldexp_f(hs, ex), ldexp_f(ls, ex));
             } else {
               const double v = ldexp_d((double)((c & 1) ? hi2[c >> 1].y : hi2[c >> 1].x) +
                                            (double)((c & 1) ? lo2[c >> 1].y : lo2[c >> 1].x),

@@ -18,15 +18,32 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-// the CTA's sums of acc[0 .. nvec) into partial[i * gridDim.x + blockIdx.x]
-__device__ __forceinline__ void put_partials(const double (&acc)[kMaxSub], int nvec, double (*red)[kMaxSub],
-                                             double* __restrict__ partial) {
+// partial[i * gridDim.x + blockIdx.x] = sum over this CTA's slice of V_i . w,
+// eight vectors at a time (w is read again from L1 for the next eight): all 32
+// accumulators at once took 255 registers, one CTA per SM and 50 us for four
+// vectors that L2 holds
+constexpr int kDotGroup = 8;
+__device__ __forceinline__ void dot_slices(const double* V, int64_t ldv, int nvec, const double* w, int64_t n,
+                                           double (*red)[kMaxSub], double* __restrict__ partial) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int64_t stride = int64_t(gridDim.x) * blockDim.x;
+  for (int v0 = 0; v0 < nvec; v0 += kDotGroup) {
+    double acc[kDotGroup];
 #pragma unroll
-  for (int i = 0; i < kMaxSub; ++i) {
-    if (i >= nvec) break;
-    const double s = warp_sum(acc[i]);
-    if (lane == 0) red[wid][i] = s;
+    for (int i = 0; i < kDotGroup; ++i) acc[i] = 0.0;
+#pragma unroll 2
+    for (int64_t x = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; x < n; x += stride) {
+      const double wx = w[x];
+#pragma unroll
+      for (int i = 0; i < kDotGroup; ++i)
+        if (v0 + i < nvec) acc[i] = fma(V[(v0 + i) * ldv + x], wx, acc[i]);
+    }
+#pragma unroll
+    for (int i = 0; i < kDotGroup; ++i) {
+      if (v0 + i >= nvec) break;
+      const double s = warp_sum(acc[i]);
+      if (lane == 0) red[wid][v0 + i] = s;
+    }
   }
   __syncthreads();
   if (threadIdx.x < nvec) {
@@ -44,23 +61,12 @@ __device__ __forceinline__ double sum_partials(const double* __restrict__ p, int
   return warp_sum(s);
 }
 
-// partial[i * gridDim.x + blockIdx.x] = sum over this CTA's slice of V_i . w
 __global__ void __launch_bounds__(kRedThreads) multidot_kernel(const double* __restrict__ V, int64_t ldv, int nvec,
                                                                const double* __restrict__ w, int64_t n,
                                                                double* __restrict__ partial, const int* __restrict__ dn) {
   if (dn) nvec = *dn + nvec;
   __shared__ double red[kRedThreads / 32][kMaxSub];
-  double acc[kMaxSub];
-#pragma unroll
-  for (int i = 0; i < kMaxSub; ++i) acc[i] = 0.0;
-  const int64_t stride = int64_t(gridDim.x) * blockDim.x;
-  for (int64_t x = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; x < n; x += stride) {
-    const double wx = w[x];
-#pragma unroll
-    for (int i = 0; i < kMaxSub; ++i)
-      if (i < nvec) acc[i] = fma(V[i * ldv + x], wx, acc[i]);
-  }
-  put_partials(acc, nvec, red, partial);
+  dot_slices(V, ldv, nvec, w, n, red, partial);
 }
 
 // out[i] = sum_g partial[i * ng + g], one warp per vector (one thread walking
@@ -94,35 +100,27 @@ __global__ void combine_kernel(const double* __restrict__ V, const double* __res
   }
 }
 
-// t -= sum_i h[i] V_i, and in the same pass the partial sums of V_i . t (norm
-// = 0) or of t . t (norm = 1) of the new t: the second read of V hits L1
+// t -= sum_i h[i] V_i, then the partial sums of V_i . t (norm = 0) or of t . t
+// (norm = 1) of the new t (a thread reads back the elements it wrote; the
+// second read of V hits L2)
 __global__ void __launch_bounds__(kRedThreads) ortho_kernel(const double* __restrict__ V, int64_t ldv, int nvec,
                                                             const double* __restrict__ h, int64_t n, int norm,
-                                                            double* __restrict__ t, double* __restrict__ partial,
+                                                            double* t, double* __restrict__ partial,
                                                             const int* __restrict__ dn) {
   if (dn) nvec = *dn + nvec;
   __shared__ double sh[kMaxSub], red[kRedThreads / 32][kMaxSub];
   if (threadIdx.x < nvec) sh[threadIdx.x] = h[threadIdx.x];
   __syncthreads();
-  double acc[kMaxSub];
-#pragma unroll
-  for (int i = 0; i < kMaxSub; ++i) acc[i] = 0.0;
   const int64_t stride = int64_t(gridDim.x) * blockDim.x;
+#pragma unroll 2
   for (int64_t x = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; x < n; x += stride) {
     double a = t[x];
-#pragma unroll
-    for (int i = 0; i < kMaxSub; ++i)
-      if (i < nvec) a = fma(-sh[i], V[i * ldv + x], a);
+#pragma unroll 8
+    for (int i = 0; i < nvec; ++i) a = fma(-sh[i], V[i * ldv + x], a);
     t[x] = a;
-    if (norm) {
-      acc[0] = fma(a, a, acc[0]);
-    } else {
-#pragma unroll
-      for (int i = 0; i < kMaxSub; ++i)
-        if (i < nvec) acc[i] = fma(V[i * ldv + x], a, acc[i]);
-    }
   }
-  put_partials(acc, norm ? 1 : nvec, red, partial);
+  if (norm) dot_slices(t, 0, 1, t, n, red, partial);
+  else dot_slices(V, ldv, nvec, t, n, red, partial);
 }
 
 // Ritz pair, residual and correction in one pass: x = V y, r = AV y - theta x,
@@ -393,9 +391,11 @@ __global__ void append_count_kernel(int* __restrict__ dn, const double* __restri
 
 }  // namespace
 
+// CTAs of a vector kernel: about four elements per thread while that fills the
+// chip, at most four CTAs per SM (fewer partial sums to add up afterwards)
 int dav_grid(int64_t n) {
-  int g = int((n + 255) / 256);
-  return g < 1 ? 1 : (g > 152 * 8 ? 152 * 8 : g);
+  const int64_t g = (n + 1023) / 1024, most = 152 * 4, least = (n + 255) / 256;
+  return int(g >= 152 ? (g > most ? most : g) : least < 1 ? 1 : (least > 152 ? 152 : least));
 }
 
 // partial sums of V_i . w; out (if given) gets the sums

@@ -1208,11 +1208,12 @@ int split_prepare(su2_env* env, int S, std::string& err) {
       const int sid = int(st->stk.size() - ch.st0);
       st->stk.push_back(s);
       for (int tl = 0; tl < int(live.size()); ++tl)
-        if (live[tl]) {
-          st->gu.push_back(MaxUnit{s.grp_off, N, s.Npad, s.ngrp, s.col0, tl, 0});
-          for (int g = 0; g < (s.kst + kWinSteps - 1) / kWinSteps; ++g)
-            for (int q = 4 * tl; q < std::min(4 * tl + 4, (N + 31) / 32); ++q) st->tpu.push_back(TPUnit{sid, g, q, 0});
-        }
+        if (live[tl]) st->gu.push_back(MaxUnit{s.grp_off, N, s.Npad, s.ngrp, s.col0, tl, 0});
+      // T' units window by window: the output blocks that share a T block have
+      // neighbouring columns tiles of the same window, so its second read hits L2
+      for (int g = 0; g < (s.kst + kWinSteps - 1) / kWinSteps; ++g)
+        for (int q = 0; q < (N + 31) / 32; ++q)
+          if (live[q / 4]) st->tpu.push_back(TPUnit{sid, g, q, 0});
       for (int q = 0; q < s.mpad / 128; ++q) st->amu.push_back(MaxUnit{s.ax_off, m, s.mpad, s.ngrp, rho_off, q, 0});
       for (int g = 0; g < s.ngrp; ++g)
         for (int q = 0; q < (m + kRowTile - 1) / kRowTile; ++q) st->axu.push_back(TPUnit{int32_t(st->stk.size()) - 1, g, q, 0});

@@ -19,104 +19,6 @@ namespace {
 constexpr int TK = 16;
 constexpr int NT = 256;
 
-// acc += alpha * A(r0:r0+64, 0:K) . B(0:K, c0:c0+64); A column-major (lda),
-// B(kk, c) = BT ? B[c + kk*ldb] : B[kk + c*ldb].  Out-of-range entries are 0.
-template <bool BT>
-__device__ __forceinline__ void tile_gemm(double (&acc)[4][4], const double* __restrict__ A, int lda,
-                                          const double* __restrict__ B, int ldb, int M, int N, int K, int r0, int c0,
-                                          double alpha, double (*sA)[kTile], double (*sB)[kTile]) {
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  for (int k0 = 0; k0 < K; k0 += TK) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int idx = tid + NT * i;
-      const int r = idx & 63, kk = idx >> 6;
-      const int gr = r0 + r, gk = k0 + kk;
-      sA[kk][r] = (gr < M && gk < K) ? alpha * A[gr + int64_t(gk) * lda] : 0.0;
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int idx = tid + NT * i;
-      int kk, c;
-      if (BT) {
-        c = idx & 63;
-        kk = idx >> 6;
-      } else {
-        kk = idx & 15;
-        c = idx >> 4;
-      }
-      const int gc = c0 + c, gk = k0 + kk;
-      double v = 0.0;
-      if (gc < N && gk < K) v = BT ? B[gc + int64_t(gk) * ldb] : B[gk + int64_t(gc) * ldb];
-      sB[kk][c] = v;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < TK; ++kk) {
-      double a[4], b[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = sA[kk][ty + 16 * i];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = sB[kk][tx + 16 * j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
-    }
-    __syncthreads();
-  }
-}
-
-__global__ void __launch_bounds__(NT) k1_fp64(const K1Job* __restrict__ jobs, const double* __restrict__ psi,
-                                              const double* __restrict__ R, double* __restrict__ T) {
-  __shared__ double sA[TK][kTile], sB[TK][kTile];
-  const K1Job j = jobs[blockIdx.x];
-  double acc[4][4] = {};
-  const int r0 = j.tr * kTile, c0 = j.tc * kTile;
-  tile_gemm<true>(acc, psi + j.e_off, j.k1, R + j.d_off, j.n, j.k1, j.n, j.k2, r0, c0, 1.0, sA, sB);
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int jj = 0; jj < 4; ++jj) {
-      const int r = r0 + ty + 16 * i, c = c0 + tx + 16 * jj;
-      if (r < j.k1 && c < j.n) T[j.t_off + r + int64_t(c) * j.k1] = acc[i][jj];
-    }
-}
-
-__global__ void __launch_bounds__(NT) k2_fp64(const K2Job* __restrict__ jobs, const K2Task* __restrict__ tasks,
-                                              const double* __restrict__ L, const double* __restrict__ psi,
-                                              const double* __restrict__ T, double* __restrict__ F) {
-  __shared__ double sA[TK][kTile], sB[TK][kTile];
-  const K2Job j = jobs[blockIdx.x];
-  const int r0 = j.tr * kTile, c0 = j.tc * kTile;
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  double acc[4][4] = {};
-  for (int t = j.t0; t < j.t1; ++t) {
-    const K2Task task = tasks[t];
-    const double* B = ((task.flags & K2_B_FROM_PSI) ? psi : T) + task.b_off;
-    if (task.flags & K2_A_IDENTITY) {
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int jj = 0; jj < 4; ++jj) {
-          const int r = r0 + ty + 16 * i, c = c0 + tx + 16 * jj;
-          if (r < j.m && c < j.n) acc[i][jj] = fma(task.v, B[r + int64_t(c) * task.k1], acc[i][jj]);
-        }
-    } else {
-      tile_gemm<false>(acc, L + task.a_off, j.m, B, task.k1, j.m, j.n, task.k1, r0, c0, task.v, sA, sB);
-    }
-  }
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int jj = 0; jj < 4; ++jj) {
-      const int r = r0 + ty + 16 * i, c = c0 + tx + 16 * jj;
-      if (r < j.m && c < j.n) F[j.f_off + r + int64_t(c) * j.m] += acc[i][jj];
-    }
-}
-
-// ------------------------------------------------------------------ stacked H.psi
 // acc(row, col) += sum_kk A(kk, row) B(kk, col), thread (tx, ty) owning rows
 // ty + 16 i, i < NI, and columns tx + 16 j, j < NJ.  NI is uniform in a warp
 // (two rows of ty) and NJ in the CTA, and both are template parameters: a
@@ -156,6 +58,85 @@ __device__ __forceinline__ void fma_tile(double (&acc)[4][4], const double (*sA)
 // row slots of this warp below `rows` (its lower row is ty & ~1)
 __device__ __forceinline__ int row_slots(int ty, int rows) { return max(0, min(4, (rows - (ty & ~1) + 15) >> 4)); }
 
+// acc += alpha * A(r0:r0+64, 0:K) . B(0:K, c0:c0+64); A column-major (lda),
+// B(kk, c) = BT ? B[c + kk*ldb] : B[kk + c*ldb].  Out-of-range entries are 0.
+template <bool BT>
+__device__ __forceinline__ void tile_gemm(double (&acc)[4][4], const double* __restrict__ A, int lda,
+                                          const double* __restrict__ B, int ldb, int M, int N, int K, int r0, int c0,
+                                          double alpha, double (*sA)[kTile], double (*sB)[kTile]) {
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const int ni = row_slots(ty, M - r0), nj = (min(kTile, N - c0) + 15) / 16;
+  for (int k0 = 0; k0 < K; k0 += TK) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int idx = tid + NT * i;
+      const int r = idx & 63, kk = idx >> 6;
+      const int gr = r0 + r, gk = k0 + kk;
+      sA[kk][r] = (gr < M && gk < K) ? alpha * A[gr + int64_t(gk) * lda] : 0.0;
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int idx = tid + NT * i;
+      int kk, c;
+      if (BT) {
+        c = idx & 63;
+        kk = idx >> 6;
+      } else {
+        kk = idx & 15;
+        c = idx >> 4;
+      }
+      const int gc = c0 + c, gk = k0 + kk;
+      double v = 0.0;
+      if (gc < N && gk < K) v = BT ? B[gc + int64_t(gk) * ldb] : B[gk + int64_t(gc) * ldb];
+      sB[kk][c] = v;
+    }
+    __syncthreads();
+    fma_tile(acc, sA, sB, tx, ty, min(TK, K - k0), ni, nj);
+    __syncthreads();
+  }
+}
+
+__global__ void __launch_bounds__(NT) k1_fp64(const K1Job* __restrict__ jobs, const double* __restrict__ psi,
+                                              const double* __restrict__ R, double* __restrict__ T) {
+  __shared__ double sA[TK][kTile], sB[TK][kTile];
+  const K1Job j = jobs[blockIdx.x];
+  double acc[4][4] = {};
+  const int r0 = j.tr * kTile, c0 = j.tc * kTile;
+  tile_gemm<true>(acc, psi + j.e_off, j.k1, R + j.d_off, j.n, j.k1, j.n, j.k2, r0, c0, 1.0, sA, sB);
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int jj = 0; jj < 4; ++jj) {
+      const int r = r0 + ty + 16 * i, c = c0 + tx + 16 * jj;
+      if (r < j.k1 && c < j.n) T[j.t_off + r + int64_t(c) * j.k1] = acc[i][jj];
+    }
+}
+
+__global__ void __launch_bounds__(NT) k2_fp64(const K2Job* __restrict__ jobs, const K2Task* __restrict__ tasks,
+                                              const double* __restrict__ L, const double* __restrict__ T,
+                                              double* __restrict__ F, double* __restrict__ part) {
+  __shared__ double sA[TK][kTile], sB[TK][kTile];
+  const K2Job j = jobs[blockIdx.x];
+  const int r0 = j.tr * kTile, c0 = j.tc * kTile;
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  double acc[4][4] = {};
+  for (int t = j.t0; t < j.t1; ++t) {
+    const K2Task task = tasks[t];
+    tile_gemm<false>(acc, L + task.a_off, j.m, T + task.b_off, task.k1, j.m, j.n, task.k1, r0, c0, task.v, sA, sB);
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int jj = 0; jj < 4; ++jj) {
+      const int r = r0 + ty + 16 * i, c = c0 + tx + 16 * jj;
+      if (r >= j.m || c >= j.n) continue;
+      if (j.slot >= 0) part[(int64_t(j.slot) * kTile + (c - c0)) * kTile + (r - r0)] = acc[i][jj];
+      else F[j.f_off + r + int64_t(c) * j.m] += acc[i][jj];
+    }
+}
+
+// ------------------------------------------------------------------ stacked H.psi
 // the entry of [lo, hi) that holds column c (col0 ascending, col0[lo] <= c)
 __device__ __forceinline__ int find_ent(const P64Ent* __restrict__ ents, int lo, int hi, int c) {
   while (hi - lo > 1) {
@@ -388,20 +369,12 @@ __global__ void __launch_bounds__(NT, 2) diag_kernel(const DiagJob* __restrict__
 }  // namespace
 
 void launch_heff_fp64(cudaStream_t s, const double* L, const double* R, const double* psi, double* F, double* T,
-                      const K1Job* k1, const K2Job* k2, const K2Task* tasks, const Chunk& c, int64_t,
-                      Profiler* prof) {
-  const int64_t n1 = c.k1_end - c.k1_begin, n2 = c.k2_end - c.k2_begin;
-  prof->count(int(n1 > 0) + int(n2 > 0));
-  if (n1 > 0) {
-    const int slot = prof->begin(s, 0, c.k1_flops);
-    k1_fp64<<<unsigned(n1), NT, 0, s>>>(k1 + c.k1_begin, psi, R, T);
-    prof->end(s, slot);
-  }
-  if (n2 > 0) {
-    const int slot = prof->begin(s, 1, c.k2_flops);
-    k2_fp64<<<unsigned(n2), NT, 0, s>>>(k2 + c.k2_begin, tasks, L, psi, T, F);
-    prof->end(s, slot);
-  }
+                      const K1Job* k1, const K2Job* k2, const K2Task* tasks, const P64Tile* split, double* part,
+                      const Chunk& c) {
+  const int64_t n1 = c.k1_end - c.k1_begin, n2 = c.k2_end - c.k2_begin, n3 = c.sp_end - c.sp_begin;
+  if (n1 > 0) k1_fp64<<<unsigned(n1), NT, 0, s>>>(k1 + c.k1_begin, psi, R, T);
+  if (n2 > 0) k2_fp64<<<unsigned(n2), NT, 0, s>>>(k2 + c.k2_begin, tasks, L, T, F, part);
+  if (n3 > 0) part_sum<<<unsigned(n3), NT, 0, s>>>(split + c.sp_begin, part, F);
 }
 
 void launch_stack_fp64(cudaStream_t s, const Plan64& p, const Chunk64& c, const double* L, const double* R,

@@ -5,6 +5,7 @@
 // kernel that walks each destination range once; on the host the same work
 // runs as plain loops (host-only contexts).
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 #include <map>
 #include <tuple>
@@ -90,6 +91,8 @@ class DeviceBackend : public RenormBackend {
     K1Job* dk1 = nullptr;
     K2Job* dk2 = nullptr;
     K2Task* dk2t = nullptr;
+    P64Tile* dsp = nullptr;
+    double* part = nullptr;
     auto ck = [&](cudaError_t e, const char* what) {
       if (e != cudaSuccess && err.empty()) err = std::string("renormalisation: ") + what + ": " + cudaGetErrorString(e);
       return err.empty();
@@ -119,10 +122,13 @@ class DeviceBackend : public RenormBackend {
       std::vector<K2Job> k2;
       std::vector<K2Task> k2t;
       std::vector<Chunk> chunks;
-      int64_t max_t = 0;
+      std::vector<P64Tile> split;
+      int64_t max_t = 0, max_part = 0;
+      int n_sms = 148;
+      cudaDeviceGetAttribute(&n_sms, cudaDevAttrMultiProcessorCount, device_);
       size_t i = 0;
       while (i < ord.size()) {
-        Chunk c{int64_t(k1.size()), 0, int64_t(k2.size()), 0, 0.0, 0.0};
+        Chunk c{int64_t(k1.size()), 0, int64_t(k2.size()), 0, int64_t(split.size()), 0, 0.0, 0.0};
         std::map<std::tuple<int64_t, int64_t, int32_t, int32_t, int32_t>, int64_t> toff;
         int64_t tsz = 0;
         size_t j = i;
@@ -155,24 +161,49 @@ class DeviceBackend : public RenormBackend {
             kt.a_off = t.a;
             kt.b_off = it->second;
             kt.k1 = t.k1;
-            kt.flags = 0;
+            kt.pad = 0;
             kt.v = t.v;
             k2t.push_back(kt);
             c.k2_flops += 2.0 * t.m * t.k1 * t.n;
-            c2 += t.k1;
+            c2 += (t.k1 + 15) / 16;
           }
           const RTask& t0 = st.tasks[ord[j]];
           for (int tc = 0; tc < (t0.n + kTile - 1) / kTile; ++tc)
             for (int tr = 0; tr < (t0.m + kTile - 1) / kTile; ++tr) {
-              jobs.push_back(K2Job{f, t0.m, t0.n, tr, tc, tb, int32_t(k2t.size())});
-              cost.push_back(c2);
+              // modelled cycles of a 16-K step: DFMAs at two lanes per SM and
+              // clock, and about 2000 cycles to fill it
+              jobs.push_back(K2Job{f, t0.m, t0.n, tr, tc, tb, int32_t(k2t.size()), -1, 0});
+              cost.push_back(c2 * (8.0 * std::min(kTile, t0.m - tr * kTile) * ((std::min(kTile, t0.n - tc * kTile) + 15) / 16 * 16) + 2000.0));
             }
           j = e;
         }
-        std::vector<size_t> jo(jobs.size());
-        for (size_t x = 0; x < jo.size(); ++x) jo[x] = x;
-        std::stable_sort(jo.begin(), jo.end(), [&](size_t a, size_t b) { return cost[a] > cost[b]; });
-        for (size_t x : jo) k2.push_back(jobs[x]);
+        // tiles above a sixteenth of an SM's share run as several jobs of at
+        // least four tasks each, summed afterwards in task order: a grown
+        // block's tile can have thousands of small products
+        double total = 0.0;
+        for (double x : cost) total += x;
+        const double share = std::max(1.0, total / (16.0 * n_sms));
+        int64_t slots = 0;
+        std::vector<std::pair<double, K2Job>> runs;
+        for (size_t x = 0; x < jobs.size(); ++x) {
+          const K2Job& q = jobs[x];
+          const int nt = q.t1 - q.t0, parts = std::max(1, std::min(int(std::min(1e6, std::ceil(cost[x] / share))), nt / 4));
+          if (parts > 1)
+            split.push_back(P64Tile{q.f_off + q.tr * kTile + int64_t(q.tc) * kTile * q.m, std::min(kTile, q.m - q.tr * kTile),
+                                    std::min(kTile, q.n - q.tc * kTile), q.m, int32_t(slots), parts, 0});
+          for (int p = 0; p < parts; ++p) {
+            K2Job y = q;
+            y.t0 = q.t0 + int(int64_t(nt) * p / parts);
+            y.t1 = q.t0 + int(int64_t(nt) * (p + 1) / parts);
+            if (parts > 1) y.slot = int32_t(slots++);
+            runs.push_back({cost[x] * (y.t1 - y.t0) / std::max(1, nt), y});
+          }
+        }
+        max_part = std::max(max_part, slots);
+        std::stable_sort(runs.begin(), runs.end(),
+                         [](const std::pair<double, K2Job>& a, const std::pair<double, K2Job>& b) { return a.first > b.first; });
+        for (const auto& x : runs) k2.push_back(x.second);
+        c.sp_end = int64_t(split.size());
         c.k1_end = int64_t(k1.size());
         c.k2_end = int64_t(k2.size());
         chunks.push_back(c);
@@ -185,9 +216,10 @@ class DeviceBackend : public RenormBackend {
       if (err.empty()) ck(upload(&dk1, k1), "K1 jobs");
       if (err.empty()) ck(upload(&dk2, k2), "K2 jobs");
       if (err.empty()) ck(upload(&dk2t, k2t), "K2 tasks");
-      Profiler off;
+      if (err.empty()) ck(upload(&dsp, split), "split tiles");
+      if (err.empty() && max_part > 0) ck(cudaMalloc(&part, size_t(max_part) * kTile * kTile * sizeof(double)), "partial tiles");
       if (err.empty())
-        for (const Chunk& c : chunks) launch_heff_fp64(s_, q, q, src, dst, T, dk1, dk2, dk2t, c, 0, &off);
+        for (const Chunk& c : chunks) launch_heff_fp64(s_, q, q, src, dst, T, dk1, dk2, dk2t, dsp, part, c);
       if (err.empty()) ck(cudaGetLastError(), "launch");
     }
     const auto cp = pieces_of(st.copies);
@@ -195,7 +227,7 @@ class DeviceBackend : public RenormBackend {
       group_kernel<<<unsigned(cp.size()), 256, 0, s_>>>(dcp, dct, src, dst);
     if (err.empty()) ck(cudaGetLastError(), "launch");
     if (err.empty()) ck(cudaStreamSynchronize(s_), "step");
-    void* ps[] = {src, q, T, did, dtp, dcp, dtt, dct, dk1, dk2, dk2t};
+    void* ps[] = {src, q, T, did, dtp, dcp, dtt, dct, dk1, dk2, dk2t, dsp, part};
     for (void* p : ps) cudaFree(p);
     if (!err.empty()) {
       cudaFree(dst);

@@ -68,13 +68,13 @@ struct K1Job {
 struct K2Job {
   int64_t f_off;
   int32_t m, n, tr, tc, t0, t1;
+  int32_t slot, pad;  // slot >= 0: a run of the tile's tasks, stored as a partial tile
 };
-enum { K2_A_IDENTITY = 1, K2_B_FROM_PSI = 2 };
 struct K2Task {
-  int64_t a_off;  // left operator block in the left arena (m x k1), unused for identity
-  int64_t b_off;  // T in the chunk buffer (k1 x n) or the input block of psi
-  int32_t k1, flags;
-  double v;       // sector-value table entry
+  int64_t a_off;  // left operand (m x k1)
+  int64_t b_off;  // T in the chunk buffer (k1 x n)
+  int32_t k1, pad;
+  double v;       // coefficient
 };
 struct DiagJob {  // one 64 x 64 tile of a block of the diagonal, its diagonal tasks [t0, t1)
   int64_t f_off;
@@ -86,7 +86,7 @@ struct DiagTask {
   double v;
 };
 struct Chunk {
-  int64_t k1_begin, k1_end, k2_begin, k2_end;
+  int64_t k1_begin, k1_end, k2_begin, k2_end, sp_begin, sp_end;
   double k1_flops, k2_flops;
 };
 
@@ -145,9 +145,10 @@ struct Profiler {
 // cores in the split path (the small-task class)
 constexpr int kSmallDim = 16;
 
+// one chunk of the renormalisation's products (split: its tiles with several K2 jobs)
 void launch_heff_fp64(cudaStream_t s, const double* L, const double* R, const double* psi, double* F, double* T,
-                      const K1Job* k1, const K2Job* k2, const K2Task* tasks, const Chunk& c, int64_t psi_len,
-                      Profiler* prof);
+                      const K1Job* k1, const K2Job* k2, const K2Task* tasks, const P64Tile* split, double* part,
+                      const Chunk& c);
 // one term chunk of the FP64 H.psi: F += its terms (T: the chunk's intermediates)
 void launch_stack_fp64(cudaStream_t s, const Plan64& p, const Chunk64& c, const double* L, const double* R,
                        const double* psi, double* F, double* T, Profiler* prof);

@@ -735,66 +735,96 @@ double u1_counted_flops(const OpTable& t, const std::vector<Sector>& left, const
       for (int m = -q.twoS; m <= q.twoS; m += 2) d[{q.N, m}] += q.dim;
     return d;
   };
-  const auto dl = u1(left), dr = u1(right);
+  const auto dlm = u1(left), drm = u1(right);
+  // U(1) sectors as lists, with their indices by (N, M)
+  struct US { int N, M; int64_t dim; };
+  auto listed = [](const std::map<std::pair<int, int>, int64_t>& d, std::vector<US>& v) {
+    std::map<std::pair<int, int>, int> at;
+    for (const auto& [q, n] : d) {
+      at[q] = int(v.size());
+      v.push_back(US{q.first, q.second, n});
+    }
+    return at;
+  };
+  std::vector<US> dl, dr;
+  const auto lat = listed(dlm, dl), rat = listed(drm, dr);
+  // the sector reached by (dN, dM), -1 if there is none
+  auto reached = [](const std::vector<US>& v, const std::map<std::pair<int, int>, int>& at, int dN, int dM) {
+    std::vector<int> to(v.size(), -1);
+    for (size_t i = 0; i < v.size(); ++i) {
+      auto it = at.find({v[i].N + dN, v[i].M + dM});
+      if (it != at.end()) to[i] = it->second;
+    }
+    return to;
+  };
   struct MS { int s, m; };
   std::vector<MS> ms;
   for (int s = 0; s < int(sN.size()); ++s)
     for (int m = -sS[s]; m <= sS[s]; m += 2) ms.push_back({s, m});
-  struct UB { int Na, Ma, i1, i2, Nb, Mb; };
+  const int nm = int(ms.size()), nL = int(dl.size()), nR = int(dr.size());
+  struct UB { int a, i1, i2, b; };
   std::vector<UB> blocks;
-  std::map<std::tuple<int, int, int, int, int, int>, int> bidx;
-  for (const auto& [a, da] : dl)
-    for (int i1 = 0; i1 < int(ms.size()); ++i1)
-      for (int i2 = 0; i2 < int(ms.size()); ++i2)
-        for (const auto& [b, db] : dr) {
-          if (a.first + sN[ms[i1].s] + sN[ms[i2].s] + b.first != N) continue;
-          if (a.second + ms[i1].m + ms[i2].m + b.second != twoS) continue;
-          bidx[{a.first, a.second, i1, i2, b.first, b.second}] = int(blocks.size());
-          blocks.push_back({a.first, a.second, i1, i2, b.first, b.second});
+  std::vector<char> is_block(size_t(nL) * nm * nm * nR, 0);
+  auto place = [&](int a, int i1, int i2, int b) { return ((size_t(a) * nm + i1) * nm + i2) * nR + b; };
+  for (int a = 0; a < nL; ++a)
+    for (int i1 = 0; i1 < nm; ++i1)
+      for (int i2 = 0; i2 < nm; ++i2)
+        for (int b = 0; b < nR; ++b) {
+          if (dl[a].N + sN[ms[i1].s] + sN[ms[i2].s] + dr[b].N != N) continue;
+          if (dl[a].M + ms[i1].m + ms[i2].m + dr[b].M != twoS) continue;
+          is_block[place(a, i1, i2, b)] = 1;
+          blocks.push_back({a, i1, i2, b});
         }
-  // site transitions of one component of a site operator
-  auto site_next = [&](const SiteOp& op, int i, int q, std::vector<int>& out) {
-    out.clear();
-    for (int j = 0; j < int(ms.size()); ++j) {
-      if (ms[j].m != ms[i].m + q) continue;
-      if (op.red[ms[j].s][ms[i].s] == 0.0) continue;
-      if (cg_coef(sS[ms[i].s], ms[i].m, op.k, q, sS[ms[j].s], ms[j].m) == 0.0) continue;
-      out.push_back(j);
-    }
+  // site transitions of one component of a site operator, by initial state
+  auto site_next = [&](const SiteOp& op, int q, std::vector<std::vector<int>>& out) {
+    out.assign(size_t(nm), {});
+    for (int i = 0; i < nm; ++i)
+      for (int j = 0; j < nm; ++j) {
+        if (ms[j].m != ms[i].m + q) continue;
+        if (op.red[ms[j].s][ms[i].s] == 0.0) continue;
+        if (cg_coef(sS[ms[i].s], ms[i].m, op.k, q, sS[ms[j].s], ms[j].m) == 0.0) continue;
+        out[i].push_back(j);
+      }
   };
   double flops = 0.0;
-  std::set<std::tuple<int, int, int, int, int>> k1seen;
-  std::vector<int> n1, n2;
+  // K1 products seen: (right operator, component) -> one flag per block (the
+  // output sector follows from the component and the block's right sector)
+  std::map<std::pair<int, int>, std::vector<char>> k1seen;
+  std::vector<std::vector<int>> n1, n2;
   for (const Term& term : t.terms) {
     const BlockOp& A = t.lops[term.A];
     const BlockOp& D = t.rops[term.D];
     const bool aid = A.kind == OP_IDENTITY, did = D.kind == OP_IDENTITY;
     const int k = term.k;
     for (int q = -k; q <= k; q += 2) {
-      const double c0 = cg_coef(k, q, k, -q, 0, 0);
-      if (c0 == 0.0) continue;
+      if (cg_coef(k, q, k, -q, 0, 0) == 0.0) continue;
       for (int qA = -A.k; qA <= A.k; qA += 2) {
         const int qB = q - qA;
         if (std::abs(qB) > term.B.k || cg_coef(A.k, qA, term.B.k, qB, k, q) == 0.0) continue;
+        const std::vector<int> ato = reached(dl, lat, A.dN, qA);
+        site_next(term.B, qB, n1);
         for (int qC = -term.C.k; qC <= term.C.k; qC += 2) {
           const int qD = -q - qC;
           if (std::abs(qD) > D.k || cg_coef(term.C.k, qC, D.k, qD, k, -q) == 0.0) continue;
-          for (int e = 0; e < int(blocks.size()); ++e) {
+          const std::vector<int> bto = reached(dr, rat, D.dN, qD);
+          site_next(term.C, qC, n2);
+          std::vector<char>* seen = nullptr;
+          if (!did) {
+            seen = &k1seen[{term.D, qD}];
+            if (seen->empty()) seen->assign(blocks.size(), 0);
+          }
+          for (size_t e = 0; e < blocks.size(); ++e) {
             const UB& E = blocks[e];
-            const auto ao = std::make_pair(E.Na + A.dN, E.Ma + qA);
-            const auto bo = std::make_pair(E.Nb + D.dN, E.Mb + qD);
-            auto ia = dl.find(ao);
-            auto ib = dr.find(bo);
-            if (ia == dl.end() || ib == dr.end()) continue;
-            site_next(term.B, E.i1, qB, n1);
-            if (n1.empty()) continue;
-            site_next(term.C, E.i2, qC, n2);
-            if (n2.empty()) continue;
-            const int64_t k1 = dl.at({E.Na, E.Ma}), k2 = dr.at({E.Nb, E.Mb}), m = ia->second, n = ib->second;
-            for (int j1 : n1)
-              for (int j2 : n2) {
-                if (!bidx.count({ao.first, ao.second, j1, j2, bo.first, bo.second})) continue;
-                if (!did && k1seen.insert({term.D, qD, bo.first, bo.second, e}).second) flops += 2.0 * k1 * k2 * n;
+            const int ao = ato[E.a], bo = bto[E.b];
+            if (ao < 0 || bo < 0 || n1[E.i1].empty() || n2[E.i2].empty()) continue;
+            const int64_t k1 = dl[E.a].dim, k2 = dr[E.b].dim, m = dl[ao].dim, n = dr[bo].dim;
+            for (int j1 : n1[E.i1])
+              for (int j2 : n2[E.i2]) {
+                if (!is_block[place(ao, j1, j2, bo)]) continue;
+                if (!did && !(*seen)[e]) {
+                  (*seen)[e] = 1;
+                  flops += 2.0 * k1 * k2 * n;
+                }
                 if (!aid) flops += 2.0 * m * k1 * n;
               }
           }

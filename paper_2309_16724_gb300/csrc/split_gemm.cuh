@@ -161,6 +161,18 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
   return false;
 }
 
+// has the phase completed?  (does not suspend; what is read after a true
+// answer is ordered as after a wait)
+__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n.reg .pred p;\nmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+
 // bounded wait by every lane of a warp, then a warp vote: the warp leaves
 // converged (the .sync.aligned TMEM loads that follow need that) and agrees
 // on the outcome (polling by lane 0 alone measured slower)
@@ -169,16 +181,12 @@ __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatil
   return __all_sync(0xffffffffu, got);
 }
 
-__device__ __forceinline__ uint64_t make_desc(uint32_t saddr) {
-  // no swizzle, K-major: LBO = 128 B (next core matrix along K), SBO = 256 B
-  // (next 8-row group), descriptor version 1 (bit 46)
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr & 0x3FFFF) >> 4);
-  d |= (uint64_t)(128 >> 4) << 16;
-  d |= (uint64_t)(256 >> 4) << 32;
-  d |= (uint64_t)1 << 46;
-  return d;
-}
+// shared-memory descriptors: no swizzle, K-major, LBO = 128 B (next core
+// matrix along K), SBO = 256 B (next 8-row group), descriptor version 1 (bit
+// 46).  The address and LBO fill the low word, so stepping through slices is
+// 32-bit arithmetic
+constexpr uint32_t kDescHi = (256u >> 4) | (1u << 14);
+__device__ __forceinline__ uint32_t make_desc(uint32_t saddr) { return ((saddr & 0x3FFFF) >> 4) | ((128u >> 4) << 16); }
 
 // kind::f16, A = B = BF16, D = F32, both K-major, M = 128, N = n (multiple of 16)
 __device__ __forceinline__ uint32_t idesc_n(int n) {
@@ -191,17 +199,18 @@ __device__ __forceinline__ uint32_t idesc_n(int n) {
 // about 75 cycles at any N; from the converged warp 67 cycles at N = 128 and
 // 53 at N = 64, close to the tensor core's own 64 and 48.)
 template <bool ACC>
-__device__ __forceinline__ void mma_bf16(uint32_t tmem, uint64_t a, uint64_t b, uint32_t idesc) {
+__device__ __forceinline__ void mma_bf16(uint32_t tmem, uint32_t a, uint32_t b, uint32_t idesc) {
+  // a, b: the low words of the descriptors; the high word is the same for all
   if (ACC)
     asm volatile(
-        "{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\n"
-        "@p tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, 1;\n}\n" ::"r"(tmem),
-        "l"(a), "l"(b), "r"(idesc));
+        "{\n.reg .pred p;\n.reg .b64 da, db;\nmov.b64 da, {%1, %4};\nmov.b64 db, {%2, %4};\nelect.sync _|p, 0xffffffff;\n"
+        "@p tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %3, 1;\n}\n" ::"r"(tmem),
+        "r"(a), "r"(b), "r"(idesc), "n"(kDescHi));
   else
     asm volatile(
-        "{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\n"
-        "@p tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, 0;\n}\n" ::"r"(tmem),
-        "l"(a), "l"(b), "r"(idesc));
+        "{\n.reg .pred p;\n.reg .b64 da, db;\nmov.b64 da, {%1, %4};\nmov.b64 db, {%2, %4};\nelect.sync _|p, 0xffffffff;\n"
+        "@p tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %3, 0;\n}\n" ::"r"(tmem),
+        "r"(a), "r"(b), "r"(idesc), "n"(kDescHi));
 }
 
 // the S(S+1)/2 slice products of one 16-K step, unrolled: pair (i, j) goes to
@@ -212,15 +221,15 @@ __device__ __forceinline__ void mma_bf16(uint32_t tmem, uint64_t a, uint64_t b, 
 // the tile, whose outputs are never used).  In the first step of a chunk the
 // first product into each level, (0, level), overwrites it.
 template <int S, bool FIRST>
-__device__ __forceinline__ void issue_stage(uint32_t tbuf, uint64_t da, uint64_t db, uint32_t as16, uint32_t bs16,
+__device__ __forceinline__ void issue_stage(uint32_t tbuf, uint32_t da, uint32_t db, uint32_t as16, uint32_t bs16,
                                             uint32_t idesc) {
 #pragma unroll
   for (int i = 0; i < S; ++i)
 #pragma unroll
     for (int jj = 0; jj < S - i; ++jj) {
       const int lvl = (i + jj) < 3 ? (i + jj) : 3;
-      const uint64_t a = da + (uint64_t)(i * as16);
-      const uint64_t b = db + (uint64_t)(jj * bs16);
+      const uint32_t a = da + i * as16;
+      const uint32_t b = db + jj * bs16;
       if (FIRST && i == 0 && jj == lvl) mma_bf16<false>(tbuf + lvl * kCols, a, b, idesc);
       else mma_bf16<true>(tbuf + lvl * kCols, a, b, idesc);
     }
@@ -466,7 +475,11 @@ __global__ void __launch_bounds__(kThreads, 1)
       bool ok = true;
       const uint32_t sbase = smem_u32(smem);
       for (;;) {
-        if (!warp_wait(smem_u32(&full_bar[st]), ph, &abort_flag, spin)) {
+        // the stage is usually there: a test costs about 150 cycles less than a
+        // (potentially suspending) try_wait, and the tensor core queues little
+        // more than one MMA meanwhile
+        if (!__all_sync(0xffffffffu, mbar_test(smem_u32(&full_bar[st]), ph)) &&
+            !warp_wait(smem_u32(&full_bar[st]), ph, &abort_flag, spin)) {
           ok = false;
           break;
         }
@@ -485,13 +498,13 @@ __global__ void __launch_bounds__(kThreads, 1)
         const uint32_t idesc = idesc_n((int)n16 * 16);
         const uint32_t bs16 = n16 * 32, as16 = a16 * 32;  // sub-tile strides in 16-byte units (rows * 32 / 16)
         const uint32_t sa = sbase + st * stage_bytes;
-        const uint64_t da = make_desc(sa), db = make_desc(sa + sk * S * kSub);
+        const uint32_t da = make_desc(sa), db = make_desc(sa + sk * S * kSub);
         const uint32_t tb = tmem + buf * kBufCols;
         const int nk = (int)((m >> 4) & 0xf);
         if (m & kMetaFirst) issue_stage<S, true>(tb, da, db, as16, bs16, idesc);
         else issue_stage<S, false>(tb, da, db, as16, bs16, idesc);
         for (int kk = 1; kk < nk; ++kk)
-          issue_stage<S, false>(tb, da + (uint64_t)(kk * S * as16), db + (uint64_t)(kk * S * bs16), as16, bs16, idesc);
+          issue_stage<S, false>(tb, da + kk * S * as16, db + kk * S * bs16, as16, bs16, idesc);
         mma_commit(smem_u32(&empty_bar[st]));
         if (m & kMetaLast) {
           mma_commit(smem_u32(&accf_bar[buf]));

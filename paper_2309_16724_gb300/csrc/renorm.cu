@@ -126,6 +126,24 @@ class DeviceBackend : public RenormBackend {
       int64_t max_t = 0, max_part = 0;
       int n_sms = 148;
       cudaDeviceGetAttribute(&n_sms, cudaDevAttrMultiProcessorCount, device_);
+      // modelled cycles of a tile: per 16-K step of its tasks the DFMAs at two
+      // lanes per SM and clock, and about 2000 cycles to fill it
+      auto tile_cost = [&](const RTask& t, int tr, int tc, double steps) {
+        return steps * (8.0 * std::min(kTile, t.m - tr * kTile) * ((std::min(kTile, t.n - tc * kTile) + 15) / 16 * 16) + 2000.0);
+      };
+      // Tiles above a sixteenth of an SM's share of the step run as several jobs
+      // of at least four tasks each, summed afterwards in task order: a grown
+      // block's tile can have thousands of small products.  The share is the
+      // whole step's, so the operators do not depend on the chunk budget.
+      double total = 0.0;
+      for (size_t a = 0; a < ord.size();) {
+        const RTask& t0 = st.tasks[ord[a]];
+        double steps = 0.0;
+        for (; a < ord.size() && st.tasks[ord[a]].f == t0.f; ++a) steps += (st.tasks[ord[a]].k1 + 15) / 16;
+        for (int tc = 0; tc < (t0.n + kTile - 1) / kTile; ++tc)
+          for (int tr = 0; tr < (t0.m + kTile - 1) / kTile; ++tr) total += tile_cost(t0, tr, tc, steps);
+      }
+      const double share = std::max(1.0, total / (16.0 * n_sms));
       size_t i = 0;
       while (i < ord.size()) {
         Chunk c{int64_t(k1.size()), 0, int64_t(k2.size()), 0, int64_t(split.size()), 0, 0.0, 0.0};
@@ -170,19 +188,11 @@ class DeviceBackend : public RenormBackend {
           const RTask& t0 = st.tasks[ord[j]];
           for (int tc = 0; tc < (t0.n + kTile - 1) / kTile; ++tc)
             for (int tr = 0; tr < (t0.m + kTile - 1) / kTile; ++tr) {
-              // modelled cycles of a 16-K step: DFMAs at two lanes per SM and
-              // clock, and about 2000 cycles to fill it
               jobs.push_back(K2Job{f, t0.m, t0.n, tr, tc, tb, int32_t(k2t.size()), -1, 0});
-              cost.push_back(c2 * (8.0 * std::min(kTile, t0.m - tr * kTile) * ((std::min(kTile, t0.n - tc * kTile) + 15) / 16 * 16) + 2000.0));
+              cost.push_back(tile_cost(t0, tr, tc, c2));
             }
           j = e;
         }
-        // tiles above a sixteenth of an SM's share run as several jobs of at
-        // least four tasks each, summed afterwards in task order: a grown
-        // block's tile can have thousands of small products
-        double total = 0.0;
-        for (double x : cost) total += x;
-        const double share = std::max(1.0, total / (16.0 * n_sms));
         int64_t slots = 0;
         std::vector<std::pair<double, K2Job>> runs;
         for (size_t x = 0; x < jobs.size(); ++x) {

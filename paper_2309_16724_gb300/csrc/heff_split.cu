@@ -270,54 +270,6 @@ __global__ void __launch_bounds__(256) winexp_kernel(const TPUnit* __restrict__ 
   out[s.ax_off + int64_t(u.win) * s.mpad + r] = exp_of(m);
 }
 
-// slices of FP64 blocks into their stack's slab (compact layout,
-// split_gemm.cuh): one CTA of 128 threads per (block, 128-row tile, 16-K
-// step); thread = one block row, 16 K elements = two 16-byte pieces per
-// slice.  Any row offset and any K offset that is a multiple of 8 keeps the
-// pieces whole
-__global__ void slab_fp64_kernel(const SlabDesc* __restrict__ descs, const Unit* __restrict__ units,
-                                 const double* __restrict__ src, const int* __restrict__ rexp,
-                                 unsigned char* __restrict__ slab, int S) {
-  const Unit u = units[blockIdx.x];
-  const SlabDesc d = descs[u.desc];
-  const int r = u.tr * 128 + threadIdx.x;
-  if (r >= d.rows) return;
-  const int row = d.row0 + r, tr = row >> 7, t = row & 127;
-  const int trows = sp::tile_rows(d.R, tr);
-  unsigned char* tile = slab + d.slab_off + sp::slab_pos(d.R, d.kst, S, tr, 0, 0) + (t >> 3) * 256 + (t & 7) * 16;
-#pragma unroll
-  for (int kg = 0; kg < 2; ++kg) {
-    const int o = 2 * u.ks + kg;  // 8-K piece of the block
-    if (o >= d.noct) break;
-    const int ko = (d.k0 >> 3) + o;  // 8-K piece of the stack
-    int sigma = rexp[d.exp_off + r + (d.gst ? int64_t(ko / (2 * d.gst)) * d.exp_ld : 0)];
-    if (sigma < -1000) sigma = 0;
-    double y[8];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const int k = o * 8 + q;
-      double x = 0.0;
-      if (k < d.cols) {
-        if (d.src_off < 0) x = (r == k) ? 1.0 : 0.0;
-        else x = src[d.src_off + r + int64_t(k) * d.ld];
-      }
-      y[q] = scale2(x, sp::kLead - sigma);  // |y| < 2^kLead
-    }
-    unsigned char* base = tile + int64_t(ko >> 1) * S * trows * 32 + (ko & 1) * 128;
-    float si = 1.f;  // 2^-8i
-    for (int i = 0; i < S; ++i, si *= 0x1p-8f) {
-      __align__(16) __nv_bfloat16 v[8];
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        const double qi = rint(y[q]);
-        y[q] = (y[q] - qi) * 256.0;
-        v[q] = __float2bfloat16_rn((float)qi * si);
-      }
-      *(uint4*)(base + int64_t(i) * trows * 32) = *(const uint4*)v;
-    }
-  }
-}
-
 // eight float-float values (four packed pairs) scaled by 2^es to |x| <
 // 2^kLead and cut into S slices: 16 bytes each at base + i * stride.  rint by
 // the 1.5 * 2^23 shift (|x| <= 2^8 + 1 here); every difference is exact
@@ -354,6 +306,49 @@ __device__ __forceinline__ void cut_oct(float2 (&h)[4], float2 (&l)[4], int es, 
       wv[j] = *reinterpret_cast<const uint32_t*>(&v2);
     }
     *(uint4*)(base + int64_t(i) * stride) = w;
+  }
+}
+
+// slices of FP64 blocks into their stack's slab (compact layout,
+// split_gemm.cuh): one CTA of 128 threads per (block, 128-row tile, 16-K
+// step); thread = one block row, 16 K elements = two 16-byte pieces per
+// slice.  Any row offset and any K offset that is a multiple of 8 keeps the
+// pieces whole.  A value is scaled to |x| < 2^kLead in FP64 (any range) and cut
+// from its float-float form in FP32: the FP64 operations per element (4 instead
+// of 2 + 3 S) bound this kernel, which runs for every streamed block
+__global__ void slab_fp64_kernel(const SlabDesc* __restrict__ descs, const Unit* __restrict__ units,
+                                 const double* __restrict__ src, const int* __restrict__ rexp,
+                                 unsigned char* __restrict__ slab, int S) {
+  const Unit u = units[blockIdx.x];
+  const SlabDesc d = descs[u.desc];
+  const int r = u.tr * 128 + threadIdx.x;
+  if (r >= d.rows) return;
+  const int row = d.row0 + r, tr = row >> 7, t = row & 127;
+  const int trows = sp::tile_rows(d.R, tr);
+  unsigned char* tile = slab + d.slab_off + sp::slab_pos(d.R, d.kst, S, tr, 0, 0) + (t >> 3) * 256 + (t & 7) * 16;
+#pragma unroll
+  for (int kg = 0; kg < 2; ++kg) {
+    const int o = 2 * u.ks + kg;  // 8-K piece of the block
+    if (o >= d.noct) break;
+    const int ko = (d.k0 >> 3) + o;  // 8-K piece of the stack
+    int sigma = rexp[d.exp_off + r + (d.gst ? int64_t(ko / (2 * d.gst)) * d.exp_ld : 0)];
+    if (sigma < -1000) sigma = 0;
+    float2 h[4], l[4];
+    float* hv = &h[0].x;
+    float* lv = &l[0].x;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int k = o * 8 + q;
+      double x = 0.0;
+      if (k < d.cols) {
+        if (d.src_off < 0) x = (r == k) ? 1.0 : 0.0;
+        else x = src[d.src_off + r + int64_t(k) * d.ld];
+      }
+      x = scale2(x, sp::kLead - sigma);
+      hv[q] = (float)x;
+      lv[q] = (float)(x - (double)hv[q]);
+    }
+    cut_oct(h, l, 0, tile + int64_t(ko >> 1) * S * trows * 32 + (ko & 1) * 128, trows * 32, S);
   }
 }
 

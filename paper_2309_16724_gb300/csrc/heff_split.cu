@@ -53,7 +53,6 @@ namespace {
 using sp::Job;
 constexpr int kSentinel = -100000;
 constexpr int kSub = sp::kSub;
-constexpr int kGroupBlocks = 2;                  // left blocks of an exponent group (on average)
 constexpr int kWinSteps = sp::kChunkSteps;       // 16-K steps of one T' CTA (a whole number of exponent groups)
 constexpr int kWinOct = 2 * kWinSteps;           // 8-K pieces of it
 
@@ -1117,13 +1116,16 @@ int split_prepare(su2_env* env, int S, std::string& err) {
       for (int w = 0; w < nw; ++w) K8 += (a_cols(a_of[a][w]) + 7) / 8;
       s.kst = (K8 + 1) / 2;
       s.noct = 2 * s.kst;
-      // exponent groups (drain chunks) of about two blocks, at most 192 K:
-      // the blocks of a group share one exponent per row, and a group of a
-      // dozen small blocks was measured to double the error of H.psi (L = 12,
-      // D = 100)
+      // exponent groups (drain chunks) of about one and a half blocks, at most
+      // 192 K: the blocks of a group share one exponent per row.  Error of H.psi
+      // against FP64 at L = 12, D = 100 with groups of 192 K 5.5e-12, of three
+      // blocks 2.6e-12, of one and a half 1.9e-12 (2.8e-12 with one exponent set
+      // per task); at L = 12, D = 397 with two blocks 5.9e-12, with one and a
+      // half 4.0e-12 (4.8e-12).  The shorter chunks cost 1 % at L = 16, D = 512 and
+      // nothing where sectors pass 128
       s.gst = kWinSteps;
       for (int g : {2, 3, 4, 6})
-        if (16 * g * nw >= kGroupBlocks * 8 * K8) {
+        if (32 * g * nw >= 3 * 8 * K8) {
           s.gst = g;
           break;
         }

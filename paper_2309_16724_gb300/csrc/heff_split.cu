@@ -461,10 +461,13 @@ __device__ __forceinline__ void add_task(const TPTask& t, const float2 (&av)[4],
 // sum_t v_t T_t), so K2 runs once per (left block, output block) instead of
 // once per task (1.7 to 3 times fewer flops).  The float-float sums stay in
 // registers until the group's column exponents are known (one exchange
-// through shared memory), so T is read once, in whole 32-byte sectors (row
-// offsets and strides are multiples of 8).
+// through shared memory), so T is read once, in whole 64-byte pieces (row
+// offsets and strides are multiples of 8).  Bound by the latency of its loads
+// (unit, pieces, task list, task, T): three CTAs per SM at 56 registers with a
+// few spills take 27.1 ms at L = 32, D = 2048, two at 80 registers 31.0; lists
+// with the first task inline (one load fewer) gained nothing.
 constexpr int kTPWarps = kWinSteps;
-__global__ void __launch_bounds__(32 * kTPWarps, 2)
+__global__ void __launch_bounds__(32 * kTPWarps, 3)
     tprime_kernel(const TPUnit* __restrict__ units, const Stack* __restrict__ stacks, const Col* __restrict__ cols,
                   const Oct* __restrict__ octs, const int32_t* __restrict__ tab, const TPTask* __restrict__ tasks,
                   const float2* __restrict__ T, const float2* __restrict__ P, int* __restrict__ grp,

@@ -3,32 +3,28 @@
 // scales, the sector GEMMs run on tcgen05 tensor cores (split_gemm.cuh) and
 // are recombined in float-float and finally in FP64.
 //
+// Products are stacked (split_prepare): K1 is one product per right sector, K2
+// one per left output sector, and the tasks that share a left block and an
+// output block are summed on the way (T').
+//
 // Scales:
-//  * left operator blocks A (K2): a common row exponent rho(a', r) per row of
-//    each left sector (max over every operator block with that output sector,
-//    identity included) so that all tasks of one output tile share it; each
-//    block is additionally shifted up by delta_b = min_r (rho - e_b(r)) >= 0
-//    and the shift is folded into its tasks' coefficient (v * 2^-delta).
-//  * T'_t = v_t 2^-delta T_u (K2 B operand): the task's own column exponents
-//    phi_t + cexp_u(c), so every task keeps all S*8 bits of its own
-//    magnitude in every column; chunks of the K2 stripe end at task
-//    boundaries and the drain multiplies each chunk by the exact power of
-//    two 2^(own - gamma(f, c)), gamma the output block's column exponent (the
-//    max over its tasks).  A common column exponent for all tasks of a tile
-//    was measured to lose ~4 bits: each task's truncation error then scales
-//    with the largest task of the column, and thousands of tasks add up.
+//  * K2 operands: every drain chunk (a group of 2 to 12 16-K steps, about one
+//    and a half left blocks) has its own exponent per row of the A stack and
+//    per output column of T'; the drain multiplies the chunk by the exact power
+//    of two 2^(own - maximum over the groups) on both sides, so every chunk
+//    keeps all S*8 bits of its own magnitude.
 //  * K1 (T = E D^T): per-row exponents of the psi blocks and of the right
 //    operator blocks.
 //
-// Per H.psi: psi is copied to float-float and sliced (psi slabs); per term
-// chunk (whose intermediates fit the T budget): K1 writes T in float-float
-// (column-major with columns padded to a multiple of 4, or row-major where
-// K1 computes the block transposed), column exponents of T and of psi
-// blocks, gamma and the 8-bit drain exponents, T' slabs, then K2 adds into
-// F.  Tasks whose four dimensions are all <= kSmallDim run afterwards in
-// FP64 on CUDA cores (small-task class).  The operator slabs are built once
-// per site by split_prepare; split_autotune picks the slice count and the
-// stage depth.
+// Per H.psi: psi is copied to float-float and sliced (psi_slab_kernel); per
+// term chunk (whose intermediates fit the T budget): K1 writes T in float-float
+// (column-major, or row-major where K1 computes the product transposed),
+// tprime_kernel sums and cuts the T' slabs with their exponents,
+// groupmax_kernel makes the drain exponents, then K2 adds into F (split tiles
+// through partial tiles).  Tasks whose four dimensions are all <= kSmallDim run
+// afterwards in FP64 on CUDA cores (small-task class).  The operator slabs are
+// built once per site by split_prepare; split_autotune picks the slice count
+// and the stage depth.
 #include <algorithm>
 #include <climits>
 #include <cmath>

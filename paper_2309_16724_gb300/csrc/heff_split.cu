@@ -141,6 +141,7 @@ struct SplitState {
   SmallOut* d_small_out = nullptr;
   SmallSeg* d_small_seg = nullptr;
   double* d_small_part = nullptr;  // kSmallDim^2 doubles per segment
+  int small_max = 0;               // largest dimension of a small task
   int sk = 2;  // 16-K steps per pipeline stage (a tile-shape parameter of the split GEMM)
   // stacked operand slabs
   unsigned char *dA = nullptr, *dD = nullptr, *dE = nullptr, *dTP = nullptr;
@@ -572,14 +573,17 @@ __global__ void __launch_bounds__(256) part_reduce_kernel(const SplitTile* __res
 // the same left block, then A T (m x n); the partial goes to part[w *
 // kSmallDim^2 ...].  Lane l owns the elements l, l + 32, ..., eight
 // independent DFMA chains, and loads the next task's operands into registers
-// while it computes
-constexpr int kSmallElems = kSmallDim * kSmallDim / 32;  // elements of a lane
+// while it computes.  kDim: the largest dimension of any task, 8 or 16: the
+// registers of eight elements a lane (127) leave 16 warps per SM, those of two
+// twice as many, which tiny tasks need (L = 31, D = 16, 322,782 tasks of at most
+// 5: 244 us with kDim = 16)
+template <int kDim>
 __global__ void __launch_bounds__(128) small_tasks_kernel(const SmallSeg* __restrict__ segs, int nseg,
                                                           const SmallTask* __restrict__ tasks,
                                                           const double* __restrict__ psi,
                                                           const double* __restrict__ Lop,
                                                           const double* __restrict__ Rop, double* __restrict__ part) {
-  constexpr int kD = kSmallDim * kSmallDim, kQ = kSmallElems;
+  constexpr int kD = kDim * kDim, kQ = kD / 32;  // elements of a block, of a lane
   __shared__ double sm[4][4][kD];  // per warp: E, D, A, T
   const int wl = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int w = blockIdx.x * 4 + wl;
@@ -680,7 +684,7 @@ __global__ void __launch_bounds__(128) small_tasks_kernel(const SmallSeg* __rest
     __syncwarp();
   }
 #pragma unroll
-  for (int q = 0; q < kQ; ++q) part[int64_t(w) * kD + lane + 32 * q] = acc[q];
+  for (int q = 0; q < kQ; ++q) part[int64_t(w) * (kSmallDim * kSmallDim) + lane + 32 * q] = acc[q];
 }
 
 // F += the partials of each output block's segments: one CTA per output block,
@@ -860,6 +864,7 @@ int split_prepare(su2_env* env, int S, std::string& err) {
     const Task& t = env->tasks[i];
     const Block& Fb = B[t.f];
     const Block& Eb = B[t.e];
+    st->small_max = std::max(st->small_max, std::max(std::max(Fb.rows, Fb.cols), std::max(Eb.rows, Eb.cols)));
     const int32_t ti = int32_t(st->small.size());
     if (st->small_out.empty() || st->small_out.back().f_off != Fb.offset) {
       const int32_t sg = int32_t(st->small_seg.size());
@@ -1473,8 +1478,8 @@ int split_apply(su2_env* env, const double* psi, double* F, std::string& err) {
     pf.count(2);
     slot = pf.begin(s, 2, 0.0);
     const int nseg = int(st->small_seg.size()), nout = int(st->small_out.size());
-    small_tasks_kernel<<<unsigned((nseg + 3) / 4), 128, 0, s>>>(st->d_small_seg, nseg, st->d_small, psi, env->dL,
-                                                                 env->dR, st->d_small_part);
+    const auto fn = st->small_max <= kSmallDim / 2 ? small_tasks_kernel<kSmallDim / 2> : small_tasks_kernel<kSmallDim>;
+    fn<<<unsigned((nseg + 3) / 4), 128, 0, s>>>(st->d_small_seg, nseg, st->d_small, psi, env->dL, env->dR, st->d_small_part);
     small_reduce_kernel<<<unsigned(nout), 4 * kSmallDim * kSmallDim, 0, s>>>(st->d_small_out, st->d_small_part, F);
     pf.end(s, slot);
     SPLIT_CHECK("small tasks");

@@ -470,7 +470,9 @@ def main():
                            "median of 2 timed H.psi after one untimed" if n_sh > 1 else
                            "the whole H.psi, median of 2 timed after one untimed"),
                 "split_over_fp64": value / world / fv,
-                "frac_of_nominal_fp64": fv / FP64_PEAK_TFLOPS}
+                "frac_of_nominal_fp64": fv / FP64_PEAK_TFLOPS,
+                "flops_note": "rates count the flops of the sector-task-table; tasks that share their left and "
+                              "output block are merged before K2, so fewer flops are executed on either path"}
         if senv is not env:
             senv.close()
 

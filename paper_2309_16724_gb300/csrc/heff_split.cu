@@ -13,6 +13,14 @@
 //    per output column of T'; the drain multiplies the chunk by the exact power
 //    of two 2^(own - maximum over the groups) on both sides, so every chunk
 //    keeps all S*8 bits of its own magnitude.
+//  * The left blocks of a stack are brought to one magnitude first: A_w 2^-d
+//    and T'_w 2^d with d = exponent of max |A_w| less the stack's largest (d <=
+//    0, exact).  Where blocks of different magnitude share a group, a large A
+//    with a small T' beside a small A with a large T' (H_L beside the identity,
+//    complementary beside bare operators) would otherwise leave an error of
+//    2^-8S max |A| max |T'|, far above 2^-8S |A T'|: integrals in a unit 1e5
+//    times smaller cost four digits.  H_L and the identity, whose rows
+//    differ most, have groups of their own besides.
 //  * K1 (T = E D^T): per-row exponents of the psi blocks and of the right
 //    operator blocks.
 //
@@ -60,7 +68,7 @@ struct SlabDesc {
   int32_t rows, cols, ld;
   int32_t row0, k0;      // place in the stack (k0 a multiple of 8)
   int32_t R, kst;        // the stack's rows and 16-K steps
-  int32_t noct;          // 8-K pieces to write (the last block of a stack also fills up to 16)
+  int32_t noct;          // 8-K pieces to write (up to the next block of the stack, or its end)
   int32_t exp_off;       // offset of the row exponents of the block's rows ...
   int32_t exp_ld;        // ... of the stack's first exponent group; stride to the next
   int32_t gst;           // K steps of an exponent group (0: one group)
@@ -92,6 +100,7 @@ struct Stack {
   int32_t gst;           // 16-K steps of a group (divides kWinSteps)
   int32_t desc0;         // slab descriptor of its first left block
   int32_t m, mpad;       // rows of the left blocks, padded to whole 128-row tiles
+  int32_t nw, pad;       // left blocks
   int64_t ax_off;        // offset of its per-(group, row) exponents
 };
 struct Col { int32_t f, c; };            // stack column -> output block (within the sector), its column
@@ -129,6 +138,7 @@ struct SChunk {
   int64_t st0, st1, tpu0, tpu1, gu0, gu1, sp0, sp1;  // stacks, T' units, gamma units, split tiles
   int64_t au0, au1, du0, du1;      // their slicing units
   int64_t ax0, ax1, dr0, dr1;      // exponent units: (stack, group, rows) of A, (block, rows) of D
+  int64_t ad0, ad1;                // slab descriptors of A
   double k1_flops, k2_flops;
 };
 
@@ -159,6 +169,7 @@ struct SplitState {
   // exponents
   // A: per (group, row) exponents, their maxima rho per (stack, row) and the
   // drain exponents; T': the same of one chunk (grp, gamma, scale); E, D: eps, zeta
+  int* d_delta = nullptr;        // per left block (slab descriptor): its exponent, then its shift d
   int *d_ax = nullptr, *d_rho = nullptr, *d_zeta = nullptr, *d_eps = nullptr, *d_gamma = nullptr, *d_grp = nullptr;
   uint8_t *d_ascale = nullptr, *d_scale = nullptr;
   int64_t n_ax = 0, n_rho = 0, n_zeta = 0, n_eps = 0, n_gamma = 0, n_grp = 0;
@@ -237,6 +248,54 @@ __global__ void __launch_bounds__(256) rowexp_kernel(const SlabDesc* __restrict_
   out[d.exp_off + r] = exp_of(m);
 }
 
+// exponent of the largest entry of each left block of a stack; one CTA per block
+__global__ void __launch_bounds__(256) blockexp_kernel(const SlabDesc* __restrict__ descs, const double* __restrict__ src,
+                                                       int* __restrict__ out) {
+  __shared__ double sm[8];
+  const SlabDesc d = descs[blockIdx.x];
+  double m = d.src_off < 0 ? 1.0 : 0.0;
+  if (d.src_off >= 0) {
+    const int64_t n = int64_t(d.rows) * d.cols;  // (blocks are stored without gaps: ld = rows)
+    for (int64_t i = threadIdx.x; i < n; i += 256) m = fmax(m, fabs(src[d.src_off + i]));
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = m;
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  for (int q = 1; q < 8; ++q) m = fmax(m, sm[q]);
+  out[blockIdx.x] = exp_of(m);
+}
+
+// the shifts d of a stack's left blocks from their exponents (in place), and
+// 2^d into the coefficients of their tasks; one CTA per stack.  d >= kMinShift:
+// T' stays far from the ends of the FP32 range
+constexpr int kMinShift = -60;
+__global__ void __launch_bounds__(256) shift_kernel(const Stack* __restrict__ stacks, const int32_t* __restrict__ tab,
+                                                    int* __restrict__ delta, TPTask* __restrict__ tasks) {
+  __shared__ int sm[256];
+  const Stack s = stacks[blockIdx.x];
+  int m = kSentinel;
+  for (int w = threadIdx.x; w < s.nw; w += 256) m = max(m, delta[s.desc0 + w]);
+  sm[threadIdx.x] = m;
+  __syncthreads();
+  for (int o = 128; o > 0; o >>= 1) {
+    if (threadIdx.x < o) sm[threadIdx.x] = max(sm[threadIdx.x], sm[threadIdx.x + o]);
+    __syncthreads();
+  }
+  m = sm[0];
+  for (int w = 0; w < s.nw; ++w) {
+    const int e = delta[s.desc0 + w], d = e < -1000 ? 0 : max(kMinShift, e - m);
+    __syncthreads();
+    if (threadIdx.x == 0) delta[s.desc0 + w] = d;
+    const float f = __int_as_float((127 + d) << 23);
+    for (int t = tab[s.tab_off + int64_t(w) * s.nf] + threadIdx.x; t < tab[s.tab_off + int64_t(w + 1) * s.nf]; t += 256) {
+      tasks[t].vh *= f;
+      tasks[t].vl *= f;
+    }
+  }
+}
+
 // row exponents of the stacked left blocks, one per (group, row): one
 // CTA of 32 x 8 threads per (stack, group, kRowTile rows), one thread row per
 // K of an 8-K piece.  (One exponent per row for all blocks of a sector was
@@ -244,7 +303,8 @@ __global__ void __launch_bounds__(256) rowexp_kernel(const SlabDesc* __restrict_
 // sets it for most rows.)
 __global__ void __launch_bounds__(256) winexp_kernel(const TPUnit* __restrict__ units, const Stack* __restrict__ stacks,
                                                      const Oct* __restrict__ octs, const SlabDesc* __restrict__ descs,
-                                                     const double* __restrict__ src, int* __restrict__ out) {
+                                                     const double* __restrict__ src, const int* __restrict__ delta,
+                                                     int* __restrict__ out) {
   __shared__ double sm[8][kRowTile];
   const TPUnit u = units[blockIdx.x];
   const Stack s = stacks[u.st];
@@ -256,7 +316,8 @@ __global__ void __launch_bounds__(256) winexp_kernel(const TPUnit* __restrict__ 
       const Oct k = octs[s.oct_off + o];
       if (k.w < 0 || ty >= k.nk) continue;
       const SlabDesc d = descs[s.desc0 + k.w];
-      m = fmax(m, d.src_off < 0 ? (r == k.k + ty ? 1.0 : 0.0) : fabs(src[d.src_off + r + int64_t(k.k + ty) * d.ld]));
+      const double x = d.src_off < 0 ? (r == k.k + ty ? 1.0 : 0.0) : fabs(src[d.src_off + r + int64_t(k.k + ty) * d.ld]);
+      m = fmax(m, scale2(x, -delta[s.desc0 + k.w]));
     }
   sm[ty][lane] = m;
   __syncthreads();
@@ -314,11 +375,12 @@ __device__ __forceinline__ void cut_oct(float2 (&h)[4], float2 (&l)[4], int es, 
 // of 2 + 3 S) bound this kernel, which runs for every streamed block
 __global__ void slab_fp64_kernel(const SlabDesc* __restrict__ descs, const Unit* __restrict__ units,
                                  const double* __restrict__ src, const int* __restrict__ rexp,
-                                 unsigned char* __restrict__ slab, int S) {
+                                 const int* __restrict__ delta, unsigned char* __restrict__ slab, int S) {
   const Unit u = units[blockIdx.x];
   const SlabDesc d = descs[u.desc];
   const int r = u.tr * 128 + threadIdx.x;
   if (r >= d.rows) return;
+  const int shift = delta ? delta[u.desc] : 0;  // left blocks: the block's shift
   const int row = d.row0 + r, tr = row >> 7, t = row & 127;
   const int trows = sp::tile_rows(d.R, tr);
   unsigned char* tile = slab + d.slab_off + sp::slab_pos(d.R, d.kst, S, tr, 0, 0) + (t >> 3) * 256 + (t & 7) * 16;
@@ -340,7 +402,7 @@ __global__ void slab_fp64_kernel(const SlabDesc* __restrict__ descs, const Unit*
         if (d.src_off < 0) x = (r == k) ? 1.0 : 0.0;
         else x = src[d.src_off + r + int64_t(k) * d.ld];
       }
-      x = scale2(x, sp::kLead - sigma);
+      x = scale2(x, sp::kLead - sigma - shift);
       hv[q] = (float)x;
       lv[q] = (float)(x - (double)hv[q]);
     }
@@ -923,10 +985,24 @@ int split_prepare(su2_env* env, int S, std::string& err) {
     err = "exponent tables too large";
     return SU2_EINVAL;
   }
+  // the block Hamiltonian: the left operator of the terms that act on nothing else
+  auto site_identity = [&](const SiteOp& x) {
+    const SiteOp id = site_op(env->table.site_kind, "I");
+    bool same = x.k == 0 && x.dN == 0;
+    for (int i = 0; i < x.n; ++i)
+      for (int j = 0; j < x.n; ++j) same = same && std::fabs(x.red[i][j] - id.red[i][j]) <= 1e-12;
+    return same;
+  };
+  std::vector<char> is_ham(env->table.lops.size(), 0);
+  for (const Term& t : env->table.terms)
+    if (env->table.rops[t.D].kind == OP_IDENTITY && env->table.lops[t.A].kind != OP_IDENTITY && site_identity(t.B) &&
+        site_identity(t.C))
+      is_ham[t.A] = 1;
   // the identity of left sector a is left block nLb + a
   auto a_id = [&](const Task& t) { return t.ablk >= 0 ? t.ablk : nLb + B[t.e].a; };
   auto a_out = [&](int id) { return id < nLb ? L.blocks[id].qo : id - nLb; };
   auto a_cols = [&](int id) { return id < nLb ? L.blocks[id].cols : ls[id - nLb].dim; };
+  auto a_own = [&](int id) { return id >= nLb || is_ham[L.blocks[id].op]; };  // has exponent groups of its own
   auto d_in = [&](int d) { return R.blocks[d].qi; };
   // ---------------------------------------------------------- term chunks
   // consecutive terms in the order of their left operators' first use (the
@@ -1007,6 +1083,7 @@ int split_prepare(su2_env* env, int S, std::string& err) {
     ch.du0 = int64_t(st->dunit.size());
     ch.ax0 = int64_t(st->axu.size());
     ch.dr0 = int64_t(st->drow.size());
+    ch.ad0 = int64_t(st->adesc.size());
     int64_t a_pos = ooc ? 0 : st->a_bytes, d_pos = ooc ? 0 : st->d_bytes, tsz = 0, tpsz = 0, grpsz = 0;
     // the chunk's left blocks by output sector and right blocks by input sector
     std::vector<std::vector<int>> a_of(static_cast<size_t>(nl)), d_of(static_cast<size_t>(nr));
@@ -1118,8 +1195,6 @@ int split_prepare(su2_env* env, int S, std::string& err) {
       s.oct_off = int32_t(st->oct.size());
       int K8 = 0;
       for (int w = 0; w < nw; ++w) K8 += (a_cols(a_of[a][w]) + 7) / 8;
-      s.kst = (K8 + 1) / 2;
-      s.noct = 2 * s.kst;
       // exponent groups (drain chunks) of about one and a half blocks, at most
       // 192 K: the blocks of a group share one exponent per row.  Error of H.psi
       // against FP64 at L = 12, D = 100 with groups of 192 K 5.5e-12, of three
@@ -1133,28 +1208,38 @@ int split_prepare(su2_env* env, int S, std::string& err) {
           s.gst = g;
           break;
         }
+      // K places of the left blocks: H_L and the identity begin and end a group (1
+      // to 2 % more K; without it the errors below are a third larger and twice
+      // as large where the two are the only blocks of a chunk)
+      std::vector<int> at(size_t(nw) + 1, 0);
+      for (int w = 0; w < nw; ++w) {
+        const int g8 = 2 * s.gst;
+        if (a_own(a_of[a][w]) || (w > 0 && a_own(a_of[a][w - 1]))) at[w] = (at[w] + g8 - 1) / g8 * g8;
+        at[w + 1] = at[w] + (a_cols(a_of[a][w]) + 7) / 8;
+      }
+      s.kst = (at[nw] + 1) / 2;
+      s.noct = 2 * s.kst;
       s.ngrp = (s.kst + s.gst - 1) / s.gst;
       s.m = m;
+      s.nw = nw;
       s.mpad = (m + 127) & ~127;
       s.desc0 = int32_t(st->adesc.size());
       s.ax_off = st->n_ax;
       st->n_ax += int64_t(s.ngrp) * s.mpad;
       const int32_t rho_off = int32_t(st->n_rho);
       st->n_rho += m;
-      int ko = 0;
       const int64_t aslab = a_pos;
       for (int w = 0; w < nw; ++w) {
-        const int id = a_of[a][w], k = a_cols(id), no = (k + 7) / 8;
+        const int id = a_of[a][w], k = a_cols(id), next = w + 1 < nw ? at[w + 1] : s.noct;
         a_w[id] = w;
         const int64_t src = id >= nLb ? -1 : ooc ? env->os.dev_off(L.blocks[id].off, c) : L.blocks[id].off;
         const int did = int(st->adesc.size());
-        st->adesc.push_back(SlabDesc{src, aslab, m, k, m, 0, 8 * ko, m, s.kst, no + (w + 1 == nw ? s.noct - K8 : 0),
+        st->adesc.push_back(SlabDesc{src, aslab, m, k, m, 0, 8 * at[w], m, s.kst, next - at[w],
                                      int32_t(s.ax_off), s.mpad, s.gst, 0});
         add_units(st->aunit, did, st->adesc.back());
-        for (int q = 0; q < no; ++q) st->oct.push_back(Oct{w, 8 * q, std::min(8, k - 8 * q), 0});
-        ko += no;
+        for (int q = 0; q < next - at[w]; ++q)
+          st->oct.push_back(8 * q < k ? Oct{w, 8 * q, std::min(8, k - 8 * q), 0} : Oct{-1, 0, 0, 0});
       }
-      if (K8 < s.noct) st->oct.push_back(Oct{-1, 0, 0, 0});
       a_pos += slab_bytes(m, s.kst, S);
       s.tp_off = tpsz;
       tpsz += slab_bytes(N, s.kst, S);
@@ -1284,6 +1369,7 @@ int split_prepare(su2_env* env, int S, std::string& err) {
     ch.du1 = int64_t(st->dunit.size());
     ch.ax1 = int64_t(st->axu.size());
     ch.dr1 = int64_t(st->drow.size());
+    ch.ad1 = int64_t(st->adesc.size());
     st->chunks.push_back(ch);
     if (ooc) {
       max_as = std::max(max_as, a_pos);
@@ -1316,6 +1402,7 @@ int split_prepare(su2_env* env, int S, std::string& err) {
   if (!rc2) rc2 = dalloc(&st->dT, size_t(st->t_elems + 16), err);
   if (!rc2) rc2 = dalloc(&st->dP, size_t(env->psi_len), err);
   if (!rc2) rc2 = dalloc(&st->d_rho, size_t(st->n_rho), err);
+  if (!rc2) rc2 = dalloc(&st->d_delta, st->adesc.size(), err);
   if (!rc2) rc2 = dalloc(&st->d_ax, size_t(st->n_ax), err);
   if (!rc2) rc2 = dalloc(&st->d_ascale, size_t(st->n_ax), err);
   if (!rc2) rc2 = dalloc(&st->d_zeta, size_t(st->n_zeta), err);
@@ -1366,9 +1453,12 @@ int split_prepare(su2_env* env, int S, std::string& err) {
       rc2 = SU2_ECUDA;
       break;
     }
-    if (ch.ax1 > ch.ax0)
+    if (ch.ax1 > ch.ax0) {
+      blockexp_kernel<<<unsigned(ch.ad1 - ch.ad0), 256, 0, s>>>(st->d_adesc + ch.ad0, env->dL, st->d_delta + ch.ad0);
+      shift_kernel<<<unsigned(ch.st1 - ch.st0), 256, 0, s>>>(st->d_stk + ch.st0, st->d_tab, st->d_delta, st->d_tpt);
       winexp_kernel<<<unsigned(ch.ax1 - ch.ax0), 256, 0, s>>>(st->d_axu + ch.ax0, st->d_stk, st->d_oct, st->d_adesc,
-                                                               env->dL, st->d_ax);
+                                                               env->dL, st->d_delta, st->d_ax);
+    }
     if (ch.dr1 > ch.dr0)
       rowexp_kernel<<<unsigned(ch.dr1 - ch.dr0), 256, 0, s>>>(st->d_ddesc, st->d_drow + ch.dr0, env->dR, st->d_zeta);
   }
@@ -1377,10 +1467,10 @@ int split_prepare(su2_env* env, int S, std::string& err) {
   if (!ooc) {
     if (!st->aunit.empty())
       slab_fp64_kernel<<<unsigned(st->aunit.size()), 128, 0, s>>>(st->d_adesc, st->d_aunit, env->dL, st->d_ax,
-                                                                   st->dA, S);
+                                                                   st->d_delta, st->dA, S);
     if (!st->dunit.empty())
       slab_fp64_kernel<<<unsigned(st->dunit.size()), 128, 0, s>>>(st->d_ddesc, st->d_dunit, env->dR, st->d_zeta,
-                                                                   st->dD, S);
+                                                                   nullptr, st->dD, S);
   }
   {
     const cudaError_t e1 = cudaGetLastError();
@@ -1442,10 +1532,10 @@ int split_apply(su2_env* env, const double* psi, double* F, std::string& err) {
       slot = pf.begin(s, 2, 0.0);
       if (c.au1 > c.au0)
         slab_fp64_kernel<<<unsigned(c.au1 - c.au0), 128, 0, s>>>(st->d_adesc, st->d_aunit + c.au0, env->os.dbuf,
-                                                                  st->d_ax, st->dA, S);
+                                                                  st->d_ax, st->d_delta, st->dA, S);
       if (c.du1 > c.du0)
         slab_fp64_kernel<<<unsigned(c.du1 - c.du0), 128, 0, s>>>(st->d_ddesc, st->d_dunit + c.du0, env->os.dbuf,
-                                                                  st->d_zeta, st->dD, S);
+                                                                  st->d_zeta, nullptr, st->dD, S);
       pf.end(s, slot);
       stream_release(env->os, int(ci), s);
       SPLIT_CHECK("operator slabs of the chunk");
@@ -1596,7 +1686,7 @@ void split_free(su2_env* env) {
   auto* st = static_cast<SplitState*>(env->split);
   if (!st) return;
   void* ps[] = {st->dA, st->dD, st->dE, st->dTP, st->d_adesc, st->d_ddesc, st->d_edesc, st->d_aunit, st->d_dunit,
-                st->d_drow, st->d_erow, st->d_axu, st->d_amu, st->d_gu, st->d_ax, st->d_ascale, st->d_rho, st->d_zeta,
+                st->d_drow, st->d_erow, st->d_axu, st->d_amu, st->d_gu, st->d_delta, st->d_ax, st->d_ascale, st->d_rho, st->d_zeta,
                 st->d_eps, st->d_gamma, st->d_grp, st->dT, st->dP, st->d_k1j, st->d_k2j, st->d_tpt,
                 st->d_tab, st->d_oct, st->d_stk, st->d_col, st->d_tpu, st->d_spt, st->d_part, st->d_counter,
                 st->d_scale, st->d_small, st->d_small_out, st->d_small_seg, st->d_small_part};

@@ -1,0 +1,58 @@
+"""The split path on operators of different magnitude.
+
+H.psi is linear in the integrals, so neither a change of their unit nor a
+constant on the diagonal of h may cost relative accuracy: the first makes the
+complementary operators (which carry integrals) large beside the bare ones, the
+second the block Hamiltonian beside the identity.  Neighbouring left blocks
+share exponents in the split path, and which ones are neighbours depends on the
+term chunks, hence the budgets: from one term a chunk to all in one.
+
+Bound: five slices hold an operand to 2^-40 of its largest entry, 1e-12; the
+same windows with integrals of order 1 and one exponent set per task give
+1.3e-12 from K2 alone (the same slices in NumPy on these operators).  Four times
+that for both products.
+"""
+import numpy as np
+import pytest
+
+import synth
+
+from gpu_common import rel_err
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+TOL = 5e-12
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2309_16724_gb300 as P
+    return P.Context(0, stream=torch.cuda.current_stream())
+
+
+@pytest.mark.parametrize("unit,shift", [(1.0, 0.0), (1.0, -10.0), (1.0, -50.0), (1e5, 0.0), (1e-4, 0.0)])
+@pytest.mark.parametrize("resident", [0, 1])
+def test_split_accuracy_does_not_depend_on_unit_or_shift(ctx, unit, shift, resident):
+    import paper_2309_16724_gb300 as P
+    from paper_2309_16724_gb300 import workload
+    cfg = synth.Config("mag", synth.SPATIAL_ORBITAL, 10, 10, 0, 220, 1002)
+    h, eri = synth.integrals(cfg.L, cfg.seed)
+    h[np.diag_indices(cfg.L)] += shift
+    kw = dict(model=P.SU2_MODEL_AB_INITIO, h=unit * h, eri=unit * eri, prepare_split=True, n_slices=5,
+              resident_bytes=resident)
+    F, worst = None, {}
+    for budget in [0] + [3 << k for k in range(14, 24)]:
+        sec, env = workload.build(ctx, cfg, t_budget_bytes=budget, **kw)
+        x = torch.from_numpy(synth.gaussian_psi(sec.psi_len, 3)).cuda()
+        y, z = torch.full_like(x, float("nan")), torch.full_like(x, float("nan"))
+        P.apply_heff(ctx, env, x, y, P.SU2_SPLIT_BF16)
+        if F is None:
+            P.apply_heff(ctx, env, x, z, P.SU2_FP64)
+            F = z.cpu().numpy()
+        assert ctx.status() == 0
+        worst[budget] = rel_err(y.cpu().numpy(), F)
+        env.close()
+    assert max(worst.values()) <= TOL, worst

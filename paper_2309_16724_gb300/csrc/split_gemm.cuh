@@ -27,8 +27,7 @@
 // keeps its own S*8 bits), and the first MMA of the next chunk into each level overwrites
 // it.  The chunk enters as the pair (s, (y1 - (s - x0)) + y2 + y3) with
 // s = RN(x0 + y1), exact in levels 0 and 1.  The job's first chunk becomes
-// the accumulator; later ones are added with TwoSum, the pair renormalised
-// every fourth chunk.  At the end of the job they write the tile (K1:
+// the accumulator; later ones are added with TwoSum and renormalised.  At the end of the job they write the tile (K1:
 // normalised float-float T; K2: F += FP64).
 //
 // Warp roles (576 threads): warp 0, one lane: job fetcher (dynamic schedule:
@@ -558,7 +557,6 @@ __global__ void __launch_bounds__(kThreads, 1)
         lo2[c] = make_float2(0.f, 0.f);
       }
       bool first = true;
-      uint32_t nren = 0;  // chunks folded into this job's accumulator
       // the 16 drain warps split the job's nmma columns evenly: nmma / 4 (a
       // multiple of 4, at most kDrainCols) per lane-quarter warp, so a narrow
       // tile drains in proportionally less time
@@ -594,11 +592,6 @@ __global__ void __launch_bounds__(kThreads, 1)
             break;
           }
           asm volatile("tcgen05.fence::after_thread_sync;");
-          // every fourth chunk the pair is renormalised (|lo| <= ulp(hi) / 2):
-          // in between lo gathers at most four chunks' remainders, whose own
-          // rounding stays below 2^-45 of the leading part
-          const bool renorm = (nren & 3u) == 3u;
-          ++nren;
 #pragma unroll
           for (int g = 0; g < kNG; ++g) {
             if (g >= ng) break;
@@ -654,14 +647,9 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const float2 eb = MODE == MODE_F ? __ffma2_rn(sc, f2, nb) : add2(sc, nb);
                 const float2 lt = MODE == MODE_F ? __ffma2_rn(t, f2, lo2[k >> 1]) : add2(t, lo2[k >> 1]);
                 const float2 l = add2(lt, add2(ea, eb));
-                if (renorm) {
-                  const float2 hs = add2(h, l);
-                  lo2[k >> 1] = sub2(l, sub2(hs, h));
-                  hi2[k >> 1] = hs;
-                } else {
-                  hi2[k >> 1] = h;
-                  lo2[k >> 1] = l;
-                }
+                const float2 hs = add2(h, l);
+                lo2[k >> 1] = sub2(l, sub2(hs, h));
+                hi2[k >> 1] = hs;
               }
             }
           }

@@ -56,3 +56,21 @@ def test_split_accuracy_does_not_depend_on_unit_or_shift(ctx, unit, shift, resid
         worst[budget] = rel_err(y.cpu().numpy(), F)
         env.close()
     assert max(worst.values()) <= TOL, worst
+
+
+def test_six_slices_lose_nothing_in_the_accumulator(ctx):
+    """With six slices the rounding of a chunk's tail (2^-38 of the chunk) is
+    what is left of the error; the tile accumulator must not add to it over the
+    chunks of a long K axis.  The same slices and drain in NumPy give 1.01e-12
+    for K2 and 0.81e-12 for K1, 1.29e-12 together; a pair that is normalised
+    every fourth chunk 1.60e-12.  The bound is the geometric mean of the two."""
+    import paper_2309_16724_gb300 as P
+    from paper_2309_16724_gb300 import workload
+    cfg = synth.Config("six", synth.SPATIAL_ORBITAL, 12, 12, 0, 300, 1002)
+    sec, env = workload.build(ctx, cfg, model=P.SU2_MODEL_AB_INITIO, prepare_split=True, n_slices=6)
+    x = torch.from_numpy(synth.gaussian_psi(sec.psi_len, 3)).cuda()
+    y, z = torch.empty_like(x), torch.empty_like(x)
+    P.apply_heff(ctx, env, x, y, P.SU2_SPLIT_BF16)
+    P.apply_heff(ctx, env, x, z, P.SU2_FP64)
+    assert ctx.status() == 0
+    assert rel_err(y.cpu().numpy(), z.cpu().numpy()) <= 1.44e-12

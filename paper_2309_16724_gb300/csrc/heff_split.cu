@@ -327,29 +327,14 @@ __global__ void __launch_bounds__(256) winexp_kernel(const TPUnit* __restrict__ 
   out[s.ax_off + int64_t(u.win) * s.mpad + r] = exp_of(m);
 }
 
-// eight float-float values (four packed pairs) scaled by 2^es to |x| <
-// 2^kLead and cut into S slices: 16 bytes each at base + i * stride.  rint by
-// the 1.5 * 2^23 shift (|x| <= 2^8 + 1 here); every difference is exact
-__device__ __forceinline__ void cut_oct(float2 (&h)[4], float2 (&l)[4], int es, unsigned char* base, int64_t stride,
-                                        int S) {
+// slices i0 .. S - 1 of eight float-float values (four packed pairs, |x| <=
+// 2^kLead): 16 bytes each at base + i * stride.  rint by the 1.5 * 2^23 shift
+// (|x| <= 2^8 + 1 here); every difference is exact
+__device__ __forceinline__ void cut_slices(float2 (&h)[4], float2 (&l)[4], int i0, unsigned char* base, int64_t stride,
+                                           int S) {
   const float2 m1 = make_float2(-1.f, -1.f), mg = make_float2(12582912.f, 12582912.f), c256 = make_float2(256.f, 256.f);
-  if (es >= -126 && es <= 127) {
-    const float fac = __int_as_float((127 + es) << 23);
-    const float2 f2 = make_float2(fac, fac);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      h[j] = __fmul2_rn(h[j], f2);
-      l[j] = __fmul2_rn(l[j], f2);
-    }
-  } else {
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      h[j] = make_float2(ldexpf(h[j].x, es), ldexpf(h[j].y, es));
-      l[j] = make_float2(ldexpf(l[j].x, es), ldexpf(l[j].y, es));
-    }
-  }
-  float2 si = make_float2(1.f, 1.f);  // 2^-8i
-  for (int i = 0; i < S; ++i, si = __fmul2_rn(si, make_float2(0x1p-8f, 0x1p-8f))) {
+  float2 si = i0 ? make_float2(0x1p-8f, 0x1p-8f) : make_float2(1.f, 1.f);  // 2^-8i (i0: 0 or 1)
+  for (int i = i0; i < S; ++i, si = __fmul2_rn(si, make_float2(0x1p-8f, 0x1p-8f))) {
     uint4 w;
     uint32_t* wv = &w.x;
 #pragma unroll
@@ -366,13 +351,72 @@ __device__ __forceinline__ void cut_oct(float2 (&h)[4], float2 (&l)[4], int es, 
   }
 }
 
+// eight float-float values scaled by 2^es to |x| < 2^kLead and cut into S slices
+__device__ __forceinline__ void cut_oct(float2 (&h)[4], float2 (&l)[4], int es, unsigned char* base, int64_t stride,
+                                        int S) {
+  if (es >= -126 && es <= 127) {
+    const float fac = __int_as_float((127 + es) << 23);
+    const float2 f2 = make_float2(fac, fac);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      h[j] = __fmul2_rn(h[j], f2);
+      l[j] = __fmul2_rn(l[j], f2);
+    }
+  } else {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      h[j] = make_float2(ldexpf(h[j].x, es), ldexpf(h[j].y, es));
+      l[j] = make_float2(ldexpf(l[j].x, es), ldexpf(l[j].y, es));
+    }
+  }
+  cut_slices(h, l, 0, base, stride, S);
+}
+
+// the float whose value is the double x truncated to 24 bits (0 below 2^-126),
+// |x| < 2: by integer operations, since a conversion costs as much as an FP64
+// operation (2 a clock and SM)
+__device__ __forceinline__ float top24(double x) {
+  const unsigned hi = unsigned(__double2hiint(x)), lo = unsigned(__double2loint(x));
+  const unsigned u = __funnelshift_l(lo, hi, 3) - (896u << 23);  // exponent bias 1023 -> 127
+  return __uint_as_float((hi & 0x7FFFFFFFu) < (897u << 20) ? 0u : (hi & 0x80000000u) | (u & 0x7FFFFFFFu));
+}
+
+// S slices of eight FP64 values |x| <= 2^kLead: the leading one is cut in FP64
+// (rint by the 1.5 * 2^52 shift), what is left (|r| <= 1/2, at most 45 bits below
+// a leading slice) is held exactly by a float-float pair and cut in FP32.  From
+// the float-float form of x itself the sixth slice was off by up to 1.4 times
+// its rounding.  A NaN or an infinity gives a NaN
+__device__ __forceinline__ void cut_fp64(const double (&x)[8], unsigned char* base, int64_t stride, int S) {
+  float2 h[4], l[4];
+  uint4 w;
+  uint32_t* wv = &w.x;
+  float q[8];
+  float* hv = &h[0].x;
+  float* lv = &l[0].x;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const double mg = 6755399441055744.0, m = x[i] + mg, r = x[i] - (m - mg);
+    const double rh = __hiloint2double(__double2hiint(r), __double2loint(r) & int(0xE0000000u));
+    hv[i] = 256.f * top24(rh);
+    lv[i] = 256.f * top24(r - rh);
+    q[i] = (__double2hiint(x[i]) & 0x7FF00000) == 0x7FF00000 ? __int_as_float(0x7FC00000) : float(__double2loint(m));
+  }
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const __nv_bfloat162 v2 = __float22bfloat162_rn(make_float2(q[2 * j], q[2 * j + 1]));
+    wv[j] = *reinterpret_cast<const uint32_t*>(&v2);
+  }
+  *(uint4*)base = w;
+  cut_slices(h, l, 1, base, stride, S);
+}
+
 // slices of FP64 blocks into their stack's slab (compact layout,
 // split_gemm.cuh): one CTA of 128 threads per (block, 128-row tile, 16-K
 // step); thread = one block row, 16 K elements = two 16-byte pieces per
 // slice.  Any row offset and any K offset that is a multiple of 8 keeps the
-// pieces whole.  A value is scaled to |x| < 2^kLead in FP64 (any range) and cut
-// from its float-float form in FP32: the FP64 operations per element (4 instead
-// of 2 + 3 S) bound this kernel, which runs for every streamed block
+// pieces whole.  A value is scaled to |x| < 2^kLead in FP64 (any range); the
+// slices after the first are cut in FP32: the FP64 operations per element (5
+// instead of 2 + 3 S) bound this kernel, which runs for every streamed block
 __global__ void slab_fp64_kernel(const SlabDesc* __restrict__ descs, const Unit* __restrict__ units,
                                  const double* __restrict__ src, const int* __restrict__ rexp,
                                  const int* __restrict__ delta, unsigned char* __restrict__ slab, int S) {
@@ -391,9 +435,7 @@ __global__ void slab_fp64_kernel(const SlabDesc* __restrict__ descs, const Unit*
     const int ko = (d.k0 >> 3) + o;  // 8-K piece of the stack
     int sigma = rexp[d.exp_off + r + (d.gst ? int64_t(ko / (2 * d.gst)) * d.exp_ld : 0)];
     if (sigma < -1000) sigma = 0;
-    float2 h[4], l[4];
-    float* hv = &h[0].x;
-    float* lv = &l[0].x;
+    double y[8];
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
       const int k = o * 8 + q;
@@ -402,29 +444,27 @@ __global__ void slab_fp64_kernel(const SlabDesc* __restrict__ descs, const Unit*
         if (d.src_off < 0) x = (r == k) ? 1.0 : 0.0;
         else x = src[d.src_off + r + int64_t(k) * d.ld];
       }
-      x = scale2(x, sp::kLead - sigma - shift);
-      hv[q] = (float)x;
-      lv[q] = (float)(x - (double)hv[q]);
+      y[q] = scale2(x, sp::kLead - sigma - shift);
     }
-    cut_oct(h, l, 0, tile + int64_t(ko >> 1) * S * trows * 32 + (ko & 1) * 128, trows * 32, S);
+    cut_fp64(y, tile + int64_t(ko >> 1) * S * trows * 32 + (ko & 1) * 128, trows * 32, S);
   }
 }
 
 // psi, once per H.psi: the float-float copy (read by T' for tasks without a
 // right operator), the row exponents and the slabs of its stacks in one
-// kernel; one CTA of 32 x 8 threads per (block, kRowTile rows).  psi is read
-// once in FP64; the cut reads the CTA's own float-float values back from L2
-// and runs in FP32 (an FP64 cut of the same slabs took 280 us instead of 60
-// at L = 32, D = 2048: GB300's FP64 rate is 1/64 of FP32's)
+// kernel; one CTA of 32 x 8 threads per (block, kRowTile rows).  The slabs are
+// cut from psi in FP64 (its second read hits L2), after the leading slice in
+// FP32 (an FP64 cut of all slices took 280 us at L = 32, D = 2048: GB300's FP64
+// rate is 1/64 of FP32's)
 __global__ void __launch_bounds__(256) psi_slab_kernel(const SlabDesc* __restrict__ descs, const Unit* __restrict__ units,
-                                                       const double* __restrict__ psi, float2* P,
+                                                       const double* __restrict__ psi, float2* __restrict__ P,
                                                        int* __restrict__ eps, unsigned char* __restrict__ slab, int S) {
-  __shared__ float sm[8][kRowTile];
+  __shared__ int sm[8][kRowTile];
   const Unit u = units[blockIdx.x];
   const SlabDesc d = descs[u.desc];
   const int lane = threadIdx.x & 31, ty = threadIdx.x >> 5;
   const int r = u.tr * kRowTile + lane;
-  float m = 0.f;
+  int m = 0;  // largest upper word of |psi|: the exponent without FP64 operations
   if (r < d.rows) {
 #pragma unroll 4
     for (int c = ty; c < d.cols; c += 8) {
@@ -432,31 +472,28 @@ __global__ void __launch_bounds__(256) psi_slab_kernel(const SlabDesc* __restric
       const double v = psi[i];
       const float a = (float)v;
       P[i] = make_float2(a, (float)(v - (double)a));
-      m = fmaxf(m, fabsf(a));
+      m = max(m, __double2hiint(v) & 0x7FFFFFFF);
     }
   }
   sm[ty][lane] = m;
-  __syncthreads();  // (also orders the float-float copy before its reads below)
+  __syncthreads();
   if (r >= d.rows) return;
 #pragma unroll
-  for (int q = 0; q < 8; ++q) m = fmaxf(m, sm[q][lane]);
-  const int e = exp_of_f(m);
+  for (int q = 0; q < 8; ++q) m = max(m, sm[q][lane]);
+  const int e = m < (1 << 20) ? kSentinel : (m >> 20) - 1022;  // |psi| < 2^e; below 2^-1022: zero
   if (ty == 0) eps[d.exp_off + r] = e;
   const int row = d.row0 + r, tr = row >> 7, tt = row & 127, trows = sp::tile_rows(d.R, tr);
   unsigned char* tile = slab + d.slab_off + sp::slab_pos(d.R, d.kst, S, tr, 0, 0) + (tt >> 3) * 256 + (tt & 7) * 16;
+  // 2^(kLead - e): the exponent is between -1017 and 1008, a normal number
+  const double fac = __longlong_as_double((long long)(1023 + sp::kLead - (e < -1000 ? 0 : e)) << 52);
   for (int o = ty; o < d.noct; o += 8) {
-    float2 h[4], l[4];
-    float* hv = &h[0].x;
-    float* lv = &l[0].x;
+    double y[8];
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
       const int c = o * 8 + q;
-      const int64_t i = d.src_off + r + int64_t(c) * d.ld;
-      const float2 v = c < d.cols ? P[i] : make_float2(0.f, 0.f);
-      hv[q] = v.x;
-      lv[q] = v.y;
+      y[q] = c < d.cols ? psi[d.src_off + r + int64_t(c) * d.ld] * fac : 0.0;
     }
-    cut_oct(h, l, sp::kLead - (e < -1000 ? 0 : e), tile + int64_t(o >> 1) * S * trows * 32 + (o & 1) * 128, trows * 32, S);
+    cut_fp64(y, tile + int64_t(o >> 1) * S * trows * 32 + (o & 1) * 128, trows * 32, S);
   }
 }
 

@@ -74,3 +74,35 @@ def test_six_slices_lose_nothing_in_the_accumulator(ctx):
     P.apply_heff(ctx, env, x, z, P.SU2_FP64)
     assert ctx.status() == 0
     assert rel_err(y.cpu().numpy(), z.cpu().numpy()) <= 1.44e-12
+
+
+@pytest.mark.parametrize("power", [-60, 60])
+def test_split_is_homogeneous_in_psi(ctx, power):
+    """A power of two on psi passes through every cut and scale exactly."""
+    import paper_2309_16724_gb300 as P
+    from paper_2309_16724_gb300 import workload
+    cfg = synth.Config("pow", synth.SPATIAL_ORBITAL, 12, 11, 1, 150, 23)
+    sec, env = workload.build(ctx, cfg, prepare_split=True)
+    x = torch.from_numpy(synth.gaussian_psi(sec.psi_len, 3)).cuda()
+    y, z = torch.empty_like(x), torch.empty_like(x)
+    P.apply_heff(ctx, env, x, y, P.SU2_SPLIT_BF16)
+    P.apply_heff(ctx, env, x * 2.0 ** power, z, P.SU2_SPLIT_BF16)
+    assert torch.equal(z, y * 2.0 ** power)
+
+
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+def test_a_nan_or_infinity_in_psi_reaches_the_result(ctx, bad):
+    """Where the FP64 path returns something that is not finite, so does the split path."""
+    import paper_2309_16724_gb300 as P
+    from paper_2309_16724_gb300 import workload
+    cfg = synth.Config("nan", synth.SPATIAL_ORBITAL, 12, 11, 1, 150, 23)
+    sec, env = workload.build(ctx, cfg, prepare_split=True)
+    x = torch.from_numpy(synth.gaussian_psi(sec.psi_len, 3)).cuda()
+    big = max(sec.blocks, key=lambda b: b[6] * b[7])
+    x[big[8] + big[6] * (big[7] // 2) + big[6] // 3] = bad
+    y, z = torch.empty_like(x), torch.empty_like(x)
+    P.apply_heff(ctx, env, x, y, P.SU2_SPLIT_BF16)
+    P.apply_heff(ctx, env, x, z, P.SU2_FP64)
+    assert ctx.status() == 0
+    lost = ~torch.isfinite(z)
+    assert bool(lost.any()) and not bool(torch.isfinite(y[lost]).any())

@@ -10,6 +10,7 @@
 #include <thread>
 #include <chrono>
 #include <unordered_map>
+#include <unordered_set>
 
 #include "su2_device.h"
 
@@ -239,27 +240,30 @@ static int build_plan(su2_env* env, const su2_sectors* S, int64_t budget) {
   if (env->os.on) {
     starts = env->os.starts;
   } else {
-    std::unordered_map<uint64_t, int64_t> seen;
+    std::unordered_set<uint64_t> seen, mine;
     int64_t bytes = 0;
     starts.push_back(0);
     for (int ti = 0; ti < nterms; ++ti) {
-      int64_t add = 0;
-      std::unordered_map<uint64_t, int64_t> mine;
-      for (int64_t i : by_term[ti]) {
-        const Task& t = tasks[i];
-        if (t.dblk < 0) continue;
-        const uint64_t key = (uint64_t(uint32_t(t.dblk)) << 32) | uint32_t(t.e);
-        if (seen.count(key) || mine.count(key)) continue;
-        const int64_t sz = int64_t(blocks[t.e].rows) * env->R.blocks[t.dblk].rows * 8;
-        mine[key] = sz;
-        add += sz;
-      }
+      auto add_of = [&]() {  // bytes of T that the term adds to the chunk
+        int64_t add = 0;
+        mine.clear();
+        for (int64_t i : by_term[ti]) {
+          const Task& t = tasks[i];
+          if (t.dblk < 0) continue;
+          const uint64_t key = (uint64_t(uint32_t(t.dblk)) << 32) | uint32_t(t.e);
+          if (!seen.count(key) && mine.insert(key).second)
+            add += ((int64_t(blocks[t.e].rows) * env->R.blocks[t.dblk].rows + 1) & ~int64_t(1)) * 8;
+        }
+        return add;
+      };
+      int64_t add = add_of();
       if (bytes > 0 && bytes + add > budget) {
         starts.push_back(ti);
         seen.clear();
         bytes = 0;
+        add = add_of();  // what it shared with the closed chunk is its own now
       }
-      for (auto& kv : mine) seen.insert(kv);
+      seen.insert(mine.begin(), mine.end());
       bytes += add;
     }
     starts.push_back(nterms);

@@ -110,29 +110,37 @@ std::string stream_plan(su2_env* env, int64_t budget, int64_t resident_bytes, st
     for (int ti = 0; ti < nterms; ++ti) {
       int64_t add_t = 0, add_o = 0;
       std::unordered_set<uint64_t> mine_t, mine_o, mine_p;
-      for (int64_t i : by_term[size_t(ti)]) {
-        const Task& t = tasks[size_t(i)];
-        const Block& E = B[t.e];
-        const Block& F = B[t.f];
-        const uint64_t pair = (uint64_t(uint32_t(t.ablk + 1)) << 32) | uint32_t(t.f);
-        if (!seen_p.count(pair) && mine_p.insert(pair).second) add_t += 12 * int64_t(F.cols) * E.rows;
-        if (t.dblk >= 0) {
-          const uint64_t key = (uint64_t(uint32_t(t.dblk)) << 32) | uint32_t(t.e);
-          if (!seen_t.count(key) && mine_t.insert(key).second) add_t += 16 * int64_t(E.rows) * env->R.blocks[t.dblk].rows;
+      auto count = [&]() {  // what the term adds to the chunk
+        add_t = add_o = 0;
+        mine_t.clear();
+        mine_o.clear();
+        mine_p.clear();
+        for (int64_t i : by_term[size_t(ti)]) {
+          const Task& t = tasks[size_t(i)];
+          const Block& E = B[t.e];
+          const Block& F = B[t.f];
+          const uint64_t pair = (uint64_t(uint32_t(t.ablk + 1)) << 32) | uint32_t(t.f);
+          if (!seen_p.count(pair) && mine_p.insert(pair).second) add_t += 12 * int64_t(F.cols) * E.rows;
+          if (t.dblk >= 0) {
+            const uint64_t key = (uint64_t(uint32_t(t.dblk)) << 32) | uint32_t(t.e);
+            if (!seen_t.count(key) && mine_t.insert(key).second) add_t += 16 * int64_t(E.rows) * env->R.blocks[t.dblk].rows;
+          }
+          for (int sd = 0; sd < 2; ++sd) {
+            const int b = sd == 0 ? t.ablk : t.dblk;
+            if (b < 0) continue;
+            const uint64_t key = (uint64_t(sd) << 32) | uint32_t(b);
+            if (!seen_o.count(key) && mine_o.insert(key).second) add_o += 8 * padded(side[sd]->blocks[size_t(b)]);
+          }
         }
-        for (int sd = 0; sd < 2; ++sd) {
-          const int b = sd == 0 ? t.ablk : t.dblk;
-          if (b < 0) continue;
-          const uint64_t key = (uint64_t(sd) << 32) | uint32_t(b);
-          if (!seen_o.count(key) && mine_o.insert(key).second) add_o += 8 * padded(side[sd]->blocks[size_t(b)]);
-        }
-      }
+      };
+      count();
       if ((tbytes > 0 || obytes > 0) && (tbytes + add_t > budget || obytes + add_o > budget)) {
         starts.push_back(ti);
         seen_t.clear();
         seen_o.clear();
         seen_p.clear();
         tbytes = obytes = 0;
+        count();  // what it shared with the closed chunk is its own now
       }
       seen_t.insert(mine_t.begin(), mine_t.end());
       seen_o.insert(mine_o.begin(), mine_o.end());

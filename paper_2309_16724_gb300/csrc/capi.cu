@@ -646,7 +646,9 @@ static int finish_env(su2_ctx* ctx, su2_env* env, const su2_sectors* S, const su
         }
       }
     }
-    if (!rc) rc = dev_alloc(ctx, &env->dT, size_t(std::max<int64_t>(env->t_elems, 2)));
+    // out of core with the split path: its chunk buffer too
+    const bool split = opts && (opts->prepare_split || opts->autotune);
+    if (!rc) rc = dev_alloc(ctx, &env->dT, size_t(std::max<int64_t>({env->t_elems, env->os.on && split ? env->os.work / 8 + 1 : 0, 2})));
     Plan64& p = env->p64;
     if (!rc) rc = upload(ctx, &p.d_ent, p.ent);
     if (!rc) rc = upload(ctx, &p.d_in, p.in);
@@ -662,7 +664,7 @@ static int finish_env(su2_ctx* ctx, su2_env* env, const su2_sectors* S, const su
     if (!rc) rc = dev_alloc(ctx, &p.d_part, size_t(std::max<int64_t>(p.n_part, 1)) * kTile * kTile);
     if (!rc) rc = upload(ctx, &env->ddj, env->dj);
     if (!rc) rc = upload(ctx, &env->ddt, env->dt);
-    if (!rc && opts && (opts->prepare_split || opts->autotune)) {
+    if (!rc && split) {
       std::string err;
       if (opts->autotune) rc = split_autotune(env, opts->split_tol > 0 ? opts->split_tol : 3e-11, err);
       else rc = split_prepare(env, opts->n_slices > 0 ? opts->n_slices : 5, err);

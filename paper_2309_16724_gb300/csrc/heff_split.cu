@@ -85,6 +85,8 @@ struct TPTask {
   float vh, vl;          // v_t (float-float)
 };
 constexpr int32_t kFromPsi = 1, kRowMajor = 2;
+constexpr int64_t kWorkAlign = 256;  // the T' slabs of the chunk buffer begin at a multiple of it
+static_assert(kMaxSlices == sp::kMaxS);
 // the K axis of one left sector's operand: 8-K piece -> (left block w, first row k within it, valid rows)
 struct Oct { int32_t w, k, nk, pad; };
 // one left output sector of a term chunk: F_a (all psi blocks with left
@@ -139,6 +141,7 @@ struct SChunk {
   int64_t au0, au1, du0, du1;      // their slicing units
   int64_t ax0, ax1, dr0, dr1;      // exponent units: (stack, group, rows) of A, (block, rows) of D
   int64_t ad0, ad1;                // slab descriptors of A
+  int64_t tp_base;                 // byte offset of the T' slabs in the chunk buffer
   double k1_flops, k2_flops;
 };
 
@@ -154,8 +157,13 @@ struct SplitState {
   int small_max = 0;               // largest dimension of a small task
   int sk = 2;  // 16-K steps per pipeline stage (a tile-shape parameter of the split GEMM)
   // stacked operand slabs
-  unsigned char *dA = nullptr, *dD = nullptr, *dE = nullptr, *dTP = nullptr;
-  int64_t a_bytes = 0, d_bytes = 0, e_bytes = 0, tp_bytes = 0;
+  unsigned char *dA = nullptr, *dD = nullptr, *dE = nullptr;
+  int64_t a_bytes = 0, d_bytes = 0, e_bytes = 0;
+  // intermediates of a chunk: T (float-float), then the T' slabs (SChunk::tp_base);
+  // out of core the environment's buffer of both paths
+  unsigned char* dW = nullptr;
+  bool own_w = false;
+  int64_t w_bytes = 0;
   std::vector<SlabDesc> adesc, ddesc, edesc;
   std::vector<Unit> aunit, dunit;  // slicing units: (block, 128-row tile, 16-K step)
   std::vector<Unit> drow, erow;           // row units: (block, kRowTile rows)
@@ -173,11 +181,10 @@ struct SplitState {
   int *d_ax = nullptr, *d_rho = nullptr, *d_zeta = nullptr, *d_eps = nullptr, *d_gamma = nullptr, *d_grp = nullptr;
   uint8_t *d_ascale = nullptr, *d_scale = nullptr;
   int64_t n_ax = 0, n_rho = 0, n_zeta = 0, n_eps = 0, n_gamma = 0, n_grp = 0;
-  // float-float buffers (leading part, trailing part): T of a chunk, psi.  Side
-  // by side, an 8-K piece is 64 contiguous bytes; in two arrays it was two
-  // 32-byte sectors, and the T' kernel read 30 % more from DRAM than it used
-  float2 *dT = nullptr, *dP = nullptr;
-  int64_t t_elems = 0;
+  // psi in float-float (as T: leading and trailing parts side by side, an 8-K
+  // piece is 64 contiguous bytes; in two arrays it was two 32-byte sectors, and
+  // the T' kernel read 30 % more from DRAM than it used)
+  float2* dP = nullptr;
   // plan
   std::vector<SChunk> chunks;
   std::vector<Job> k1j, k2j;
@@ -889,13 +896,125 @@ void launch_gemm(int mode, cudaStream_t s, SplitState* st, const Job* jobs, int 
   // 17 % slower K2)
   const int smem = sp::stages_of(st->S, st->sk) * sp::stage_bytes_of(st->S, st->sk) + 1024;
   const int grid = std::min(njobs, st->n_sms);
-  gemm_fn(mode, st->S)<<<grid, sp::kThreads, smem, s>>>(jobs, njobs, A, B, rexp, cexp, 2 * sp::kLead, st->dT, F,
+  gemm_fn(mode, st->S)<<<grid, sp::kThreads, smem, s>>>(jobs, njobs, A, B, rexp, cexp, 2 * sp::kLead, (float2*)st->dW, F,
                                                         st->d_part, st->d_status, counter, st->d_ascale,
                                                         st->d_scale, st->sk, st->spin);
 }
 
 }  // namespace
 
+
+std::vector<char> left_hamiltonians(const OpTable& t) {
+  const SiteOp id = site_op(t.site_kind, "I");
+  auto site_identity = [&](const SiteOp& x) {
+    bool same = x.k == 0 && x.dN == 0;
+    for (int i = 0; i < x.n; ++i)
+      for (int j = 0; j < x.n; ++j) same = same && std::fabs(x.red[i][j] - id.red[i][j]) <= 1e-12;
+    return same;
+  };
+  std::vector<char> ham(t.lops.size(), 0);
+  for (const Term& x : t.terms)
+    if (t.rops[x.D].kind == OP_IDENTITY && t.lops[x.A].kind != OP_IDENTITY && site_identity(x.B) && site_identity(x.C))
+      ham[x.A] = 1;
+  return ham;
+}
+
+// Exponent groups (drain chunks) of about one and a half blocks, at most 192 K:
+// the blocks of a group share one exponent per row.  Error of H.psi against
+// FP64 at L = 12, D = 100 with groups of 192 K 5.5e-12, of three blocks 2.6e-12,
+// of one and a half 1.9e-12 (2.8e-12 with one exponent set per task); at L = 12,
+// D = 397 with two blocks 5.9e-12, with one and a half 4.0e-12 (4.8e-12); all
+// before the blocks were brought to one magnitude, now 1.4e-12 at L = 12, D =
+// 100.  The shorter chunks cost 1 % at L = 16, D = 512 and nothing where sectors
+// pass 128.  H_L and the identity (own) have groups to themselves: 1 to 2 % more
+// K; without it errors are a third larger, and twice as large where the two are
+// the only blocks of a chunk
+StackK stack_k(const std::vector<int>& cols, const std::vector<char>& own) {
+  const int nw = int(cols.size());
+  StackK s;
+  int K8 = 0;
+  for (int k : cols) K8 += (k + 7) / 8;
+  s.gst = kWinSteps;
+  for (int g : {2, 3, 4, 6})
+    if (32 * g * nw >= 3 * 8 * K8) {
+      s.gst = g;
+      break;
+    }
+  const int g8 = 2 * s.gst;
+  s.at.assign(size_t(nw) + 1, 0);
+  for (int w = 0; w < nw; ++w) {
+    if (own[w] || (w > 0 && own[w - 1])) s.at[w] = (s.at[w] + g8 - 1) / g8 * g8;
+    s.at[w + 1] = s.at[w] + (cols[w] + 7) / 8;
+  }
+  s.kst = (s.at[nw] + 1) / 2;
+  return s;
+}
+
+static bool small_task(const su2_env& env, const Task& t) {
+  const Block& F = env.blocks[t.f];
+  const Block& E = env.blocks[t.e];
+  return std::max(std::max(F.rows, F.cols), std::max(E.rows, E.cols)) <= kSmallDim;
+}
+
+SplitBytes::SplitBytes(const su2_env& env, int S)
+    : env_(env), S_(S), ham_(left_hamiltonians(env.table)), f_cols_(env.lsec.size(), 0), e_rows_(env.rsec.size(), 0),
+      d_rows_(env.rsec.size(), 0), a_seen_(env.L.blocks.size() + env.lsec.size(), -1),
+      d_seen_(env.R.blocks.size(), -1), a_of_(env.lsec.size()), tp_(env.lsec.size(), 0), t_(env.rsec.size(), 0) {
+  for (const Block& b : env.blocks) {
+    f_cols_[b.a] += b.cols;
+    e_rows_[b.b] += (b.rows + 7) & ~7;
+  }
+}
+
+void SplitBytes::clear() {
+  stamp_ += 1;
+  bytes_ = 0;
+  std::fill(d_rows_.begin(), d_rows_.end(), 0);
+  for (auto& v : a_of_) v.clear();
+  std::fill(tp_.begin(), tp_.end(), 0);
+  std::fill(t_.begin(), t_.end(), 0);
+}
+
+int64_t SplitBytes::add(const std::vector<int64_t>& tasks) {
+  const int nLb = int(env_.L.blocks.size());
+  std::vector<int> as, bs;  // sectors that grow
+  for (int64_t i : tasks) {
+    const Task& t = env_.tasks[size_t(i)];
+    if (small_task(env_, t)) continue;
+    const int a = env_.blocks[t.f].a, id = t.ablk >= 0 ? t.ablk : nLb + a;
+    if (a_seen_[id] != stamp_) {
+      a_seen_[id] = stamp_;
+      a_of_[a].insert(std::lower_bound(a_of_[a].begin(), a_of_[a].end(), id), id);
+      as.push_back(a);
+    }
+    if (t.dblk >= 0 && d_seen_[t.dblk] != stamp_) {
+      d_seen_[t.dblk] = stamp_;
+      d_rows_[env_.R.blocks[t.dblk].qi] += env_.R.blocks[t.dblk].rows;
+      bs.push_back(env_.R.blocks[t.dblk].qi);
+    }
+  }
+  for (auto* v : {&as, &bs}) {
+    std::sort(v->begin(), v->end());
+    v->erase(std::unique(v->begin(), v->end()), v->end());
+  }
+  for (int a : as) {
+    std::vector<int> cols;
+    std::vector<char> own;
+    for (int id : a_of_[a]) {
+      cols.push_back(id < nLb ? env_.L.blocks[id].cols : env_.lsec[a].dim);
+      own.push_back(id >= nLb || ham_[env_.L.blocks[id].op]);
+    }
+    const int64_t n = slab_bytes(f_cols_[a], stack_k(cols, own).kst, S_);
+    bytes_ += n - tp_[a];
+    tp_[a] = n;
+  }
+  for (int b : bs) {  // (either orientation: the row-major one pads the right blocks' rows to 8)
+    const int64_t n = int64_t(sizeof(float2)) * ((d_rows_[b] + 7) & ~7) * e_rows_[b];
+    bytes_ += n - t_[b];
+    t_[b] = n;
+  }
+  return bytes_ > 0 ? bytes_ + kWorkAlign : 0;
+}
 
 // Plan of the split path.  Every product of a term chunk is one tile of a
 // large "stacked" product:
@@ -946,14 +1065,9 @@ int split_prepare(su2_env* env, int S, std::string& err) {
   const int nterms = int(env->table.terms.size());
   const int64_t nt = int64_t(env->tasks.size());
   const bool ooc = env->os.on;  // out-of-core operators: the slabs of a chunk are cut per H.psi into a workspace
-  auto is_small = [&](const Task& t) {
-    const Block& Fb = B[t.f];
-    const Block& Eb = B[t.e];
-    return std::max(std::max(Fb.rows, Fb.cols), std::max(Eb.rows, Eb.cols)) <= kSmallDim;
-  };
   // ---------------------------------------------------------- small-task class, by output block and left block
   std::vector<int64_t> big, few;  // the other tasks; the small ones
-  for (int64_t i = 0; i < nt; ++i) (is_small(env->tasks[i]) ? few : big).push_back(i);
+  for (int64_t i = 0; i < nt; ++i) (small_task(*env, env->tasks[i]) ? few : big).push_back(i);
   std::stable_sort(few.begin(), few.end(), [&](int64_t x, int64_t y) {
     const Task &p = env->tasks[x], &q = env->tasks[y];
     return p.f != q.f ? p.f < q.f : p.ablk < q.ablk;
@@ -1022,19 +1136,7 @@ int split_prepare(su2_env* env, int S, std::string& err) {
     err = "exponent tables too large";
     return SU2_EINVAL;
   }
-  // the block Hamiltonian: the left operator of the terms that act on nothing else
-  auto site_identity = [&](const SiteOp& x) {
-    const SiteOp id = site_op(env->table.site_kind, "I");
-    bool same = x.k == 0 && x.dN == 0;
-    for (int i = 0; i < x.n; ++i)
-      for (int j = 0; j < x.n; ++j) same = same && std::fabs(x.red[i][j] - id.red[i][j]) <= 1e-12;
-    return same;
-  };
-  std::vector<char> is_ham(env->table.lops.size(), 0);
-  for (const Term& t : env->table.terms)
-    if (env->table.rops[t.D].kind == OP_IDENTITY && env->table.lops[t.A].kind != OP_IDENTITY && site_identity(t.B) &&
-        site_identity(t.C))
-      is_ham[t.A] = 1;
+  const std::vector<char> is_ham = left_hamiltonians(env->table);
   // the identity of left sector a is left block nLb + a
   auto a_id = [&](const Task& t) { return t.ablk >= 0 ? t.ablk : nLb + B[t.e].a; };
   auto a_out = [&](int id) { return id < nLb ? L.blocks[id].qo : id - nLb; };
@@ -1070,41 +1172,25 @@ int split_prepare(su2_env* env, int S, std::string& err) {
     }
     std::vector<std::vector<int64_t>> by_term(static_cast<size_t>(nterms));
     for (int64_t i : big) by_term[env->tasks[i].term].push_back(i);
-    std::vector<int> a_seen(size_t(nLb) + nl, -1), d_seen(size_t(std::max(nRb, 1)), -1);
+    SplitBytes size(*env, S);
     int cur = 0;
-    int64_t bytes = 0;
+    bool open = false;  // the chunk holds something
     for (int ti : order) {
-      auto add_of = [&]() {
-        int64_t add = 0;
-        for (int64_t i : by_term[ti]) {
-          const Task& t = env->tasks[i];
-          const int id = a_id(t);
-          if (a_seen[id] != cur) {
-            a_seen[id] = cur;
-            add += int64_t((a_cols(id) + 7) & ~7) * f_cols[a_out(id)] * 2 * S;
-          }
-          if (t.dblk >= 0 && d_seen[t.dblk] != cur) {
-            d_seen[t.dblk] = cur;
-            add += 8 * int64_t(R.blocks[t.dblk].rows) * e_rows[d_in(t.dblk)];
-          }
-        }
-        return add;
-      };
-      int64_t add = add_of();
-      if (bytes > 0 && bytes + add > budget) {
+      int64_t bytes = size.add(by_term[ti]);
+      if (open && bytes > budget) {
         cur += 1;
-        bytes = 0;
-        add = add_of();
+        size.clear();
+        bytes = size.add(by_term[ti]);
       }
       chunk_of[ti] = cur;
-      bytes += add;
+      open = bytes > 0;
     }
     nch = cur + 1;
   }
   std::vector<std::vector<int64_t>> chunk_tasks(static_cast<size_t>(nch));
   for (int64_t i : big) chunk_tasks[chunk_of[env->tasks[i].term]].push_back(i);
   // ---------------------------------------------------------- per chunk
-  int64_t max_t = 0, max_tp = 0, max_as = 0, max_ds = 0;
+  int64_t max_as = 0, max_ds = 0;
   std::vector<int> a_w(size_t(nLb) + nl, -1), a_stamp(size_t(nLb) + nl, -1), d_row(size_t(std::max(nRb, 1)), 0),
       d_stamp(size_t(std::max(nRb, 1)), -1), d_loc(size_t(std::max(nRb, 1)), 0);
   for (int c = 0; c < nch; ++c) {
@@ -1230,31 +1316,16 @@ int split_prepare(su2_env* env, int S, std::string& err) {
       s.Npad = (N + 127) & ~127;
       s.col0 = f_col0[a];
       s.oct_off = int32_t(st->oct.size());
-      int K8 = 0;
-      for (int w = 0; w < nw; ++w) K8 += (a_cols(a_of[a][w]) + 7) / 8;
-      // exponent groups (drain chunks) of about one and a half blocks, at most
-      // 192 K: the blocks of a group share one exponent per row.  Error of H.psi
-      // against FP64 at L = 12, D = 100 with groups of 192 K 5.5e-12, of three
-      // blocks 2.6e-12, of one and a half 1.9e-12 (2.8e-12 with one exponent set
-      // per task); at L = 12, D = 397 with two blocks 5.9e-12, with one and a
-      // half 4.0e-12 (4.8e-12).  The shorter chunks cost 1 % at L = 16, D = 512 and
-      // nothing where sectors pass 128
-      s.gst = kWinSteps;
-      for (int g : {2, 3, 4, 6})
-        if (32 * g * nw >= 3 * 8 * K8) {
-          s.gst = g;
-          break;
-        }
-      // K places of the left blocks: H_L and the identity begin and end a group (1
-      // to 2 % more K; without it the errors below are a third larger and twice
-      // as large where the two are the only blocks of a chunk)
-      std::vector<int> at(size_t(nw) + 1, 0);
-      for (int w = 0; w < nw; ++w) {
-        const int g8 = 2 * s.gst;
-        if (a_own(a_of[a][w]) || (w > 0 && a_own(a_of[a][w - 1]))) at[w] = (at[w] + g8 - 1) / g8 * g8;
-        at[w + 1] = at[w] + (a_cols(a_of[a][w]) + 7) / 8;
+      std::vector<int> kw;
+      std::vector<char> own;
+      for (int id : a_of[a]) {
+        kw.push_back(a_cols(id));
+        own.push_back(a_own(id));
       }
-      s.kst = (at[nw] + 1) / 2;
+      const StackK sh = stack_k(kw, own);
+      const std::vector<int>& at = sh.at;
+      s.gst = sh.gst;
+      s.kst = sh.kst;
       s.noct = 2 * s.kst;
       s.ngrp = (s.kst + s.gst - 1) / s.gst;
       s.m = m;
@@ -1407,6 +1478,7 @@ int split_prepare(su2_env* env, int S, std::string& err) {
     ch.ax1 = int64_t(st->axu.size());
     ch.dr1 = int64_t(st->drow.size());
     ch.ad1 = int64_t(st->adesc.size());
+    ch.tp_base = (tsz * int64_t(sizeof(float2)) + kWorkAlign - 1) / kWorkAlign * kWorkAlign;
     st->chunks.push_back(ch);
     if (ooc) {
       max_as = std::max(max_as, a_pos);
@@ -1415,8 +1487,7 @@ int split_prepare(su2_env* env, int S, std::string& err) {
       st->a_bytes = a_pos;
       st->d_bytes = d_pos;
     }
-    max_t = std::max(max_t, tsz);
-    max_tp = std::max(max_tp, tpsz);
+    st->w_bytes = std::max(st->w_bytes, ch.tp_base + tpsz);
     st->n_grp = std::max(st->n_grp, grpsz);
   }
   if (st->n_zeta >= INT32_MAX || st->n_ax >= INT32_MAX || int64_t(st->oct.size()) >= INT32_MAX || int64_t(st->adesc.size()) >= INT32_MAX ||
@@ -1424,8 +1495,6 @@ int split_prepare(su2_env* env, int S, std::string& err) {
     err = "split plan too large";
     return SU2_EINVAL;
   }
-  st->t_elems = max_t;
-  st->tp_bytes = max_tp;
   if (ooc) {
     st->a_bytes = max_as;
     st->d_bytes = max_ds;
@@ -1435,8 +1504,12 @@ int split_prepare(su2_env* env, int S, std::string& err) {
   if (!rc2) rc2 = dalloc(&st->dA, size_t(st->a_bytes), err);
   if (!rc2) rc2 = dalloc(&st->dD, size_t(st->d_bytes), err);
   if (!rc2) rc2 = dalloc(&st->dE, size_t(st->e_bytes), err);
-  if (!rc2) rc2 = dalloc(&st->dTP, size_t(std::max<int64_t>(st->tp_bytes, 16)), err);
-  if (!rc2) rc2 = dalloc(&st->dT, size_t(st->t_elems + 16), err);
+  if (ooc && st->w_bytes <= env->os.work) {
+    st->dW = (unsigned char*)env->dT;
+  } else {
+    st->own_w = true;
+    if (!rc2) rc2 = dalloc(&st->dW, size_t(st->w_bytes), err);
+  }
   if (!rc2) rc2 = dalloc(&st->dP, size_t(env->psi_len), err);
   if (!rc2) rc2 = dalloc(&st->d_rho, size_t(st->n_rho), err);
   if (!rc2) rc2 = dalloc(&st->d_delta, st->adesc.size(), err);
@@ -1586,14 +1659,14 @@ int split_apply(su2_env* env, const double* psi, double* F, std::string& err) {
     SPLIT_CHECK("K1 split GEMM");
     slot = pf.begin(s, 2, 0.0);
     tprime_kernel<<<unsigned(c.tpu1 - c.tpu0), 32 * kTPWarps, 0, s>>>(st->d_tpu + c.tpu0, st->d_stk + c.st0, st->d_col, st->d_oct,
-                                                            st->d_tab, st->d_tpt, st->dT, st->dP,
-                                                            st->d_grp, st->dTP, S);
+                                                            st->d_tab, st->d_tpt, (const float2*)st->dW, st->dP,
+                                                            st->d_grp, st->dW + c.tp_base, S);
     groupmax_kernel<<<unsigned(c.gu1 - c.gu0), 512, 0, s>>>(st->d_gu + c.gu0, st->d_grp, st->d_gamma, st->d_scale);
     pf.end(s, slot);
     SPLIT_CHECK("T' slabs");
     slot = pf.begin(s, 4, c.k2_flops * npairs);
     launch_gemm(sp::MODE_F, s, st, st->d_k2j + c.k2_j0, int(c.k2_j1 - c.k2_j0), st->d_counter + 2 * ci + 1, st->dA,
-                st->dTP, st->d_rho, st->d_gamma, F);
+                st->dW + c.tp_base, st->d_rho, st->d_gamma, F);
     if (c.sp1 > c.sp0)
       part_reduce_kernel<<<dim3(unsigned(c.sp1 - c.sp0), sp::kCols / 16), 256, 0, s>>>(st->d_spt + c.sp0, st->d_part, F);
     pf.end(s, slot);
@@ -1722,9 +1795,9 @@ int split_autotune(su2_env* env, double tol, std::string& err) {
 void split_free(su2_env* env) {
   auto* st = static_cast<SplitState*>(env->split);
   if (!st) return;
-  void* ps[] = {st->dA, st->dD, st->dE, st->dTP, st->d_adesc, st->d_ddesc, st->d_edesc, st->d_aunit, st->d_dunit,
+  void* ps[] = {st->dA, st->dD, st->dE, st->own_w ? st->dW : nullptr, st->d_adesc, st->d_ddesc, st->d_edesc, st->d_aunit, st->d_dunit,
                 st->d_drow, st->d_erow, st->d_axu, st->d_amu, st->d_gu, st->d_delta, st->d_ax, st->d_ascale, st->d_rho, st->d_zeta,
-                st->d_eps, st->d_gamma, st->d_grp, st->dT, st->dP, st->d_k1j, st->d_k2j, st->d_tpt,
+                st->d_eps, st->d_gamma, st->d_grp, st->dP, st->d_k1j, st->d_k2j, st->d_tpt,
                 st->d_tab, st->d_oct, st->d_stk, st->d_col, st->d_tpu, st->d_spt, st->d_part, st->d_counter,
                 st->d_scale, st->d_small, st->d_small_out, st->d_small_seg, st->d_small_part};
   for (void* p : ps) cudaFree(p);

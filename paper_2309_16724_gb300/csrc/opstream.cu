@@ -100,30 +100,30 @@ std::string stream_plan(su2_env* env, int64_t budget, int64_t resident_bytes, st
   };
   std::vector<std::vector<int64_t>> by_term(size_t(std::max(nterms, 1)));
   for (int64_t i = 0; i < int64_t(tasks.size()); ++i) by_term[size_t(tasks[i].term)].push_back(i);
-  // chunk boundaries: the intermediates of both paths (FP64 T, float-float
-  // T, T' slabs of up to six BF16 slices, one per left block and output block)
-  // and the operator blocks a chunk reads each stay within the budget
+  // chunk boundaries: the operator blocks a chunk reads stay within the budget,
+  // and so do its intermediates on either path (FP64: T; split: T in float-float
+  // and the T' slabs of up to six slices, dense stacks).  The two paths share
+  // one buffer: they share the slots too, so they never run at once
   std::vector<int> starts{0};
+  os.work = 0;
   {
     int64_t tbytes = 0, obytes = 0;
-    std::unordered_set<uint64_t> seen_t, seen_o, seen_p;
+    bool open = false;  // the chunk holds tasks
+    std::unordered_set<uint64_t> seen_t, seen_o;
+    SplitBytes split(*env, kMaxSlices);
     for (int ti = 0; ti < nterms; ++ti) {
       int64_t add_t = 0, add_o = 0;
-      std::unordered_set<uint64_t> mine_t, mine_o, mine_p;
+      std::unordered_set<uint64_t> mine_t, mine_o;
       auto count = [&]() {  // what the term adds to the chunk
         add_t = add_o = 0;
         mine_t.clear();
         mine_o.clear();
-        mine_p.clear();
         for (int64_t i : by_term[size_t(ti)]) {
           const Task& t = tasks[size_t(i)];
-          const Block& E = B[t.e];
-          const Block& F = B[t.f];
-          const uint64_t pair = (uint64_t(uint32_t(t.ablk + 1)) << 32) | uint32_t(t.f);
-          if (!seen_p.count(pair) && mine_p.insert(pair).second) add_t += 12 * int64_t(F.cols) * E.rows;
           if (t.dblk >= 0) {
             const uint64_t key = (uint64_t(uint32_t(t.dblk)) << 32) | uint32_t(t.e);
-            if (!seen_t.count(key) && mine_t.insert(key).second) add_t += 16 * int64_t(E.rows) * env->R.blocks[t.dblk].rows;
+            if (!seen_t.count(key) && mine_t.insert(key).second)
+              add_t += 8 * ((int64_t(B[t.e].rows) * env->R.blocks[t.dblk].rows + 1) & ~int64_t(1));
           }
           for (int sd = 0; sd < 2; ++sd) {
             const int b = sd == 0 ? t.ablk : t.dblk;
@@ -134,19 +134,23 @@ std::string stream_plan(su2_env* env, int64_t budget, int64_t resident_bytes, st
         }
       };
       count();
-      if ((tbytes > 0 || obytes > 0) && (tbytes + add_t > budget || obytes + add_o > budget)) {
+      int64_t now = split.add(by_term[size_t(ti)]);
+      if (open && (tbytes + add_t > budget || obytes + add_o > budget || now > budget)) {
         starts.push_back(ti);
         seen_t.clear();
         seen_o.clear();
-        seen_p.clear();
+        split.clear();
         tbytes = obytes = 0;
+        open = false;
         count();  // what it shared with the closed chunk is its own now
+        now = split.add(by_term[size_t(ti)]);
       }
       seen_t.insert(mine_t.begin(), mine_t.end());
       seen_o.insert(mine_o.begin(), mine_o.end());
-      seen_p.insert(mine_p.begin(), mine_p.end());
       tbytes += add_t;
       obytes += add_o;
+      open = open || !by_term[size_t(ti)].empty();
+      os.work = std::max(os.work, std::max(tbytes, now));
     }
     starts.push_back(nterms);
   }

@@ -173,6 +173,7 @@ struct OpStream {
   int64_t total = 0;             // doubles of the logical arena
   std::vector<int64_t> hs, he;   // streamed range of each chunk (logical offsets)
   int64_t slot = 0;              // doubles per device slot
+  int64_t work = 0;              // bytes of the intermediates of the largest chunk (either path, up to kMaxSlices slices)
   double* dbuf = nullptr;        // device: [0, prefix) resident, then the two slots
   double* host = nullptr;        // pinned host memory: logical [prefix, total)
   cudaStream_t io = nullptr;
@@ -189,6 +190,19 @@ struct OpStream {
     return off < prefix ? off : prefix + int64_t(c & 1) * slot + (off - hs[size_t(c)]);
   }
 };
+}  // namespace su2
+
+namespace su2 {
+// ---- sizes of the split path's stacks (heff_split.cu), shared with the out-of-core planner
+constexpr int kMaxSlices = 6;
+// left blocks that are the block Hamiltonian: the left operators of the terms
+// that act on nothing else
+std::vector<char> left_hamiltonians(const OpTable& t);
+// K axis of the stacked left blocks of one output sector: 16-K steps of an
+// exponent group, steps of the whole, first 8-K piece of each block (and the
+// end).  own: the block begins and ends a group
+struct StackK { int gst = 0, kst = 0; std::vector<int> at; };
+StackK stack_k(const std::vector<int>& cols, const std::vector<char>& own);
 }  // namespace su2
 
 struct su2_ctx {
@@ -234,3 +248,25 @@ struct su2_env {
   su2::OpStream os;       // out-of-core operator arenas (os.on)
   su2::Profiler prof;
 };
+
+namespace su2 {
+// Bytes of the split path's intermediates (T in float-float, the T' slabs) of a
+// growing set of tasks, as split_prepare lays them out: the stacks are dense (all
+// left blocks of a sector times all its output columns, all psi rows of a
+// right sector times all its right blocks)
+class SplitBytes {
+ public:
+  SplitBytes(const su2_env& env, int S);
+  void clear();
+  int64_t add(const std::vector<int64_t>& tasks);  // the bytes with these tasks too
+
+ private:
+  const su2_env& env_;
+  int S_, stamp_ = 0;
+  int64_t bytes_ = 0;
+  std::vector<char> ham_;
+  std::vector<int> f_cols_, e_rows_, d_rows_, a_seen_, d_seen_;
+  std::vector<std::vector<int>> a_of_;  // the left blocks of each output sector, ascending
+  std::vector<int64_t> tp_, t_;         // bytes of T' by left sector, of T by right sector
+};
+}  // namespace su2

@@ -131,8 +131,12 @@ typedef struct {
 } su2_hamiltonian;
 
 typedef struct {
-  int64_t t_budget_bytes;  /* device bytes for the intermediate T = E D^T of
-                              one term chunk (0: library default)           */
+  int64_t t_budget_bytes;  /* device bytes for the intermediates of one term
+                              chunk: T = E D^T and the partial tiles of the
+                              native-FP64 path, and as many again for T, T'
+                              and the partial tiles of the split path (0:
+                              library default).  A chunk holds at least one
+                              term, whatever that takes                     */
   int32_t n_slices;        /* BF16 slices per operand, 2..6 (0: default 5)  */
   int32_t prepare_split;   /* 1: also build the split-precision arenas      */
   int32_t autotune;        /* 1: build the split arenas with the slice count
@@ -177,7 +181,8 @@ typedef struct {
                               the compute of other chunks (one
                               cudaMemcpyAsync per chunk).  The chunk
                               boundaries then bound both the intermediates
-                              and the operator bytes of a chunk by
+                              (one buffer for both paths) and the operator
+                              bytes of a chunk by
                               t_budget_bytes (0: a quarter of the free
                               device memory beside resident_bytes, at most
                               16 GiB; 4 GiB on a host context).  With a host
@@ -310,7 +315,8 @@ int su2_apply_heff_host(su2_ctx* ctx, const su2_env* env, const double* psi_in_h
  * a deployment variant of the native-FP64 su2_apply_heff.  It calls no
  * cudaMalloc, cudaFree or allocating library routine: the intermediate
  * T = E D^T of each term chunk lives in a fixed 64 MiB device array that
- * every GPU loading the library holds until the process exits.  The caller
+ * every GPU loading the library holds until the process exits; the partial
+ * tiles of a split K2 lie in the environment's own buffer.  The caller
  * passes psi_in / psi_out (device, 8-byte aligned, psi_len doubles, not
  * overlapping) and an environment built on the same context; an
  * environment whose largest term chunk needs more than 64 MiB of T is

@@ -235,10 +235,15 @@ static int build_plan(su2_env* env, const su2_sectors* S, int64_t budget) {
   // uniques of K1 per term (first appearance order)
   std::vector<std::vector<int64_t>> by_term(nterms);
   for (int64_t i = 0; i < int64_t(tasks.size()); ++i) by_term[tasks[i].term].push_back(i);
-  // chunk boundaries over terms (out-of-core: the planner's)
+  // chunk boundaries over terms (out-of-core: the planner's).  T and the partial
+  // tiles of K2 share the budget: at most an eighth of it, and never more than
+  // the K split can ask for (32 tiles of 32 KiB an SM), is kept back for these
   std::vector<int> starts;
+  int64_t t_max = 0, limit = budget - std::min<int64_t>(budget / 8, int64_t(152) << 20);  // bytes
   if (env->os.on) {
     starts = env->os.starts;
+    t_max = env->os.t64;
+    budget = env->split_budget;
   } else {
     std::unordered_set<uint64_t> seen, mine;
     int64_t bytes = 0;
@@ -257,7 +262,7 @@ static int build_plan(su2_env* env, const su2_sectors* S, int64_t budget) {
         return add;
       };
       int64_t add = add_of();
-      if (bytes > 0 && bytes + add > budget) {
+      if (bytes > 0 && bytes + add > limit) {
         starts.push_back(ti);
         seen.clear();
         bytes = 0;
@@ -265,6 +270,7 @@ static int build_plan(su2_env* env, const su2_sectors* S, int64_t budget) {
       }
       seen.insert(mine.begin(), mine.end());
       bytes += add;
+      t_max = std::max(t_max, bytes);
     }
     starts.push_back(nterms);
   }
@@ -432,12 +438,20 @@ static int build_plan(su2_env* env, const su2_sectors* S, int64_t budget) {
     }
     // K split: tiles above a sixteenth of an SM's share run as several jobs of at
     // least four K steps, summed afterwards in K order (two or three CTAs share
-    // an SM, so a job takes a sixth of the whole)
-    const double share = std::max(1.0, total / (16.0 * n_sms));
+    // an SM, so a job takes a sixth of the whole).  The share grows until the
+    // partial tiles fit what T leaves of the budget
+    double share = std::max(1.0, total / (16.0 * n_sms));
+    auto parts_of = [&](const Tile& t) { return std::max(1, std::min(int(std::min(1e6, std::ceil(t.cost / share))), t.steps / 4)); };
+    auto slots_of = [&]() {
+      int64_t n = 0;
+      for (const Tile& t : tiles) n += parts_of(t) > 1 ? parts_of(t) : 0;
+      return n;
+    };
+    while (slots_of() * kTile * kTile * int64_t(sizeof(double)) > std::max<int64_t>(0, budget - t_max)) share *= 1.25;
     std::vector<std::pair<double, P64K2>> jobs;
     int64_t slots = 0;
     for (const Tile& t : tiles) {
-      const int parts = std::max(1, std::min(int(std::min(1e6, std::ceil(t.cost / share))), t.steps / 4));
+      const int parts = parts_of(t);
       const P64Stack& s = P.stack[t.j.st];
       if (parts > 1)
         P.tile.push_back(P64Tile{s.f_off + t.j.tr * kTile + int64_t(t.j.tc) * kTile * s.m, std::min(kTile, s.m - t.j.tr * kTile),
@@ -505,7 +519,7 @@ static void env_free_device(su2_env* e) {
   cudaFree(e->dR);
   cudaFree(e->dT);
   const Plan64& p = e->p64;
-  void* pd[] = {p.d_ent, p.d_in, p.d_k1, p.d_left, p.d_step, p.d_tab, p.d_task, p.d_col, p.d_stack, p.d_k2, p.d_tile, p.d_part};
+  void* pd[] = {p.d_ent, p.d_in, p.d_k1, p.d_left, p.d_step, p.d_tab, p.d_task, p.d_col, p.d_stack, p.d_k2, p.d_tile};
   for (void* x : pd) cudaFree(x);
   cudaFree(e->ddj);
   cudaFree(e->ddt);
@@ -646,10 +660,12 @@ static int finish_env(su2_ctx* ctx, su2_env* env, const su2_sectors* S, const su
         }
       }
     }
-    // out of core with the split path: its chunk buffer too
+    // T, then the partial tiles; out of core with the split path: its chunk buffer too
     const bool split = opts && (opts->prepare_split || opts->autotune);
-    if (!rc) rc = dev_alloc(ctx, &env->dT, size_t(std::max<int64_t>({env->t_elems, env->os.on && split ? env->os.work / 8 + 1 : 0, 2})));
     Plan64& p = env->p64;
+    const int64_t own = env->t_elems + p.n_part * kTile * kTile, both = env->os.on && split ? env->os.work / 8 + 1 : 0;
+    if (!rc) rc = dev_alloc(ctx, &env->dT, size_t(std::max<int64_t>({own, both, 2})));
+    if (!rc) p.d_part = env->dT + env->t_elems;
     if (!rc) rc = upload(ctx, &p.d_ent, p.ent);
     if (!rc) rc = upload(ctx, &p.d_in, p.in);
     if (!rc) rc = upload(ctx, &p.d_k1, p.k1);
@@ -661,7 +677,6 @@ static int finish_env(su2_ctx* ctx, su2_env* env, const su2_sectors* S, const su
     if (!rc) rc = upload(ctx, &p.d_stack, p.stack);
     if (!rc) rc = upload(ctx, &p.d_k2, p.k2);
     if (!rc) rc = upload(ctx, &p.d_tile, p.tile);
-    if (!rc) rc = dev_alloc(ctx, &p.d_part, size_t(std::max<int64_t>(p.n_part, 1)) * kTile * kTile);
     if (!rc) rc = upload(ctx, &env->ddj, env->dj);
     if (!rc) rc = upload(ctx, &env->ddt, env->dt);
     if (!rc && split) {

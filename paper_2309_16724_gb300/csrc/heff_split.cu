@@ -159,8 +159,9 @@ struct SplitState {
   // stacked operand slabs
   unsigned char *dA = nullptr, *dD = nullptr, *dE = nullptr;
   int64_t a_bytes = 0, d_bytes = 0, e_bytes = 0;
-  // intermediates of a chunk: T (float-float), then the T' slabs (SChunk::tp_base);
-  // out of core the environment's buffer of both paths
+  // intermediates of a chunk: T (float-float), over it the partial tiles of K2
+  // (kRows x kCols doubles each; T has been read by then), after it the T' slabs
+  // (SChunk::tp_base); out of core the environment's buffer of both paths
   unsigned char* dW = nullptr;
   bool own_w = false;
   int64_t w_bytes = 0;
@@ -203,8 +204,6 @@ struct SplitState {
   Col* d_col = nullptr;
   TPUnit* d_tpu = nullptr;
   SplitTile* d_spt = nullptr;
-  double* d_part = nullptr;      // partial tiles of the split K2 jobs (kRows x kCols doubles each)
-  int64_t n_part = 0;
   int* d_status = nullptr;
   int* d_counter = nullptr;      // job counters: two per term chunk
   int n_sms = 148;
@@ -897,7 +896,7 @@ void launch_gemm(int mode, cudaStream_t s, SplitState* st, const Job* jobs, int 
   const int smem = sp::stages_of(st->S, st->sk) * sp::stage_bytes_of(st->S, st->sk) + 1024;
   const int grid = std::min(njobs, st->n_sms);
   gemm_fn(mode, st->S)<<<grid, sp::kThreads, smem, s>>>(jobs, njobs, A, B, rexp, cexp, 2 * sp::kLead, (float2*)st->dW, F,
-                                                        st->d_part, st->d_status, counter, st->d_ascale,
+                                                        (double*)st->dW, st->d_status, counter, st->d_ascale,
                                                         st->d_scale, st->sk, st->spin);
 }
 
@@ -1150,6 +1149,7 @@ int split_prepare(su2_env* env, int S, std::string& err) {
   // budget; out-of-core: the planner's ranges of terms
   std::vector<int> chunk_of(size_t(std::max(nterms, 1)), 0);
   int nch = 1;
+  int64_t whole = env->os.work;  // bytes that a chunk's intermediates may take
   if (ooc) {
     nch = int(env->os.starts.size()) - 1;
     for (int c = 0; c < nch; ++c)
@@ -1161,6 +1161,7 @@ int split_prepare(su2_env* env, int S, std::string& err) {
       cudaMemGetInfo(&fr, &tot);
       budget = std::min<int64_t>(int64_t(16) << 30, std::max<int64_t>(int64_t(fr) / 4, int64_t(1) << 30));
     }
+    whole = budget;
     std::vector<int> order;
     {
       std::unordered_map<int, int> rank;
@@ -1428,13 +1429,24 @@ int split_prepare(su2_env* env, int S, std::string& err) {
     // K split: F_a's K axis runs over every left block of the sector, so one
     // tile can hold most of a small window's work.  Tiles above a quarter of
     // an SM's share are cut into runs of whole groups (at least 24 steps), whose
-    // partial tiles a second kernel adds in K order.
+    // partial tiles a second kernel adds in K order.  The partial tiles lie over T,
+    // or reach past it as far as the budget allows; the share grows until they fit
+    constexpr int64_t kPartBytes = int64_t(sp::kRows) * sp::kCols * sizeof(double);
+    const int64_t t_bytes = tsz * int64_t(sizeof(float2));
+    const int64_t room = std::max(t_bytes, whole - tpsz - kWorkAlign);
     double total = 0.0;
     for (const Tile& t : tiles) total += t.cost;
-    const double share = total / (4.0 * st->n_sms);
+    double share = std::max(1.0, total / (4.0 * st->n_sms));
+    auto parts_of = [&](const Tile& t) { return std::max(1, std::min(int(std::min(1e6, std::ceil(t.cost / share))), t.j.nst / 24)); };
+    auto slots_of = [&]() {
+      int64_t n = 0;
+      for (const Tile& t : tiles) n += parts_of(t) > 1 ? parts_of(t) : 0;
+      return n;
+    };
+    while (slots_of() * kPartBytes > room) share *= 1.25;
     int64_t slots = 0;
     for (const Tile& t : tiles) {
-      const int parts = std::max(1, std::min(int(std::ceil(t.cost / std::max(share, 1.0))), t.j.nst / 24));
+      const int parts = parts_of(t);
       const int arows = sp::tile_rows(t.m_rows, t.j.tr);
       if (parts > 1)
         st->spt.push_back(SplitTile{t.j.out_off + (t.trans ? int64_t(t.j.tr) * 128 * t.j.ld + t.j.tc * 128
@@ -1457,7 +1469,6 @@ int split_prepare(su2_env* env, int S, std::string& err) {
         k2cost.push_back(t.cost * (g1 - g0) / t.ngrp);
       }
     }
-    st->n_part = std::max(st->n_part, slots);
     // LPT order
     auto lpt = [](std::vector<Job>& jobs, const std::vector<double>& cost, std::vector<Job>& out) {
       std::vector<int> o(jobs.size());
@@ -1478,7 +1489,7 @@ int split_prepare(su2_env* env, int S, std::string& err) {
     ch.ax1 = int64_t(st->axu.size());
     ch.dr1 = int64_t(st->drow.size());
     ch.ad1 = int64_t(st->adesc.size());
-    ch.tp_base = (tsz * int64_t(sizeof(float2)) + kWorkAlign - 1) / kWorkAlign * kWorkAlign;
+    ch.tp_base = (std::max(t_bytes, slots * kPartBytes) + kWorkAlign - 1) / kWorkAlign * kWorkAlign;
     st->chunks.push_back(ch);
     if (ooc) {
       max_as = std::max(max_as, a_pos);
@@ -1520,7 +1531,6 @@ int split_prepare(su2_env* env, int S, std::string& err) {
   if (!rc2) rc2 = dalloc(&st->d_gamma, size_t(st->n_gamma), err);
   if (!rc2) rc2 = dalloc(&st->d_grp, size_t(st->n_grp), err);
   if (!rc2) rc2 = dalloc(&st->d_scale, size_t(st->n_grp), err);
-  if (!rc2) rc2 = dalloc(&st->d_part, size_t(st->n_part) * sp::kRows * sp::kCols, err);
   if (!rc2) rc2 = dalloc(&st->d_counter, 2 * st->chunks.size(), err);
   if (!rc2) rc2 = dput(&st->d_adesc, st->adesc, err);
   if (!rc2) rc2 = dput(&st->d_ddesc, st->ddesc, err);
@@ -1668,7 +1678,7 @@ int split_apply(su2_env* env, const double* psi, double* F, std::string& err) {
     launch_gemm(sp::MODE_F, s, st, st->d_k2j + c.k2_j0, int(c.k2_j1 - c.k2_j0), st->d_counter + 2 * ci + 1, st->dA,
                 st->dW + c.tp_base, st->d_rho, st->d_gamma, F);
     if (c.sp1 > c.sp0)
-      part_reduce_kernel<<<dim3(unsigned(c.sp1 - c.sp0), sp::kCols / 16), 256, 0, s>>>(st->d_spt + c.sp0, st->d_part, F);
+      part_reduce_kernel<<<dim3(unsigned(c.sp1 - c.sp0), sp::kCols / 16), 256, 0, s>>>(st->d_spt + c.sp0, (const double*)st->dW, F);
     pf.end(s, slot);
     SPLIT_CHECK("K2 split GEMM");
   }
@@ -1798,7 +1808,7 @@ void split_free(su2_env* env) {
   void* ps[] = {st->dA, st->dD, st->dE, st->own_w ? st->dW : nullptr, st->d_adesc, st->d_ddesc, st->d_edesc, st->d_aunit, st->d_dunit,
                 st->d_drow, st->d_erow, st->d_axu, st->d_amu, st->d_gu, st->d_delta, st->d_ax, st->d_ascale, st->d_rho, st->d_zeta,
                 st->d_eps, st->d_gamma, st->d_grp, st->dP, st->d_k1j, st->d_k2j, st->d_tpt,
-                st->d_tab, st->d_oct, st->d_stk, st->d_col, st->d_tpu, st->d_spt, st->d_part, st->d_counter,
+                st->d_tab, st->d_oct, st->d_stk, st->d_col, st->d_tpu, st->d_spt, st->d_counter,
                 st->d_scale, st->d_small, st->d_small_out, st->d_small_seg, st->d_small_part};
   for (void* p : ps) cudaFree(p);
   delete st;

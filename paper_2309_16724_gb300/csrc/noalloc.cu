@@ -6,7 +6,8 @@
 // fail, and host code that must not touch the CUDA allocator after start-up.
 // For them su2_apply_heff_static_scratch runs the native-FP64 H.psi with its
 // intermediate T = E D^T in the fixed device array below instead of the
-// environment's workspace.  The caller still passes psi in and out.
+// environment's workspace (the partial tiles of a K2 whose K is split stay in the
+// latter, allocated with the environment).  The caller still passes psi in and out.
 #include <cuda_runtime.h>
 
 #include <mutex>

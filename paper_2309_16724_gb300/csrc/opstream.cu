@@ -105,7 +105,7 @@ std::string stream_plan(su2_env* env, int64_t budget, int64_t resident_bytes, st
   // and the T' slabs of up to six slices, dense stacks).  The two paths share
   // one buffer: they share the slots too, so they never run at once
   std::vector<int> starts{0};
-  os.work = 0;
+  os.work = os.t64 = 0;
   {
     int64_t tbytes = 0, obytes = 0;
     bool open = false;  // the chunk holds tasks
@@ -150,6 +150,7 @@ std::string stream_plan(su2_env* env, int64_t budget, int64_t resident_bytes, st
       tbytes += add_t;
       obytes += add_o;
       open = open || !by_term[size_t(ti)].empty();
+      os.t64 = std::max(os.t64, tbytes);
       os.work = std::max(os.work, std::max(tbytes, now));
     }
     starts.push_back(nterms);

@@ -113,7 +113,7 @@ class DeviceBackend : public RenormBackend {
     if (err.empty()) ck(upload(&q, st.q), "Q arena");
     if (err.empty() && ck(cudaMalloc(&dst, size_t(dstn) * sizeof(double)), "destination arena"))
       ck(cudaMemsetAsync(dst, 0, size_t(dstn) * sizeof(double), s_), "memset");
-    // the products, in chunks whose intermediates T fit the budget
+    // the products, in chunks whose intermediates (T, partial tiles) fit the budget
     if (err.empty() && !st.tasks.empty()) {
       std::vector<int64_t> ord(st.tasks.size());
       for (size_t i = 0; i < ord.size(); ++i) ord[i] = int64_t(i);
@@ -144,23 +144,36 @@ class DeviceBackend : public RenormBackend {
           for (int tr = 0; tr < (t0.m + kTile - 1) / kTile; ++tr) total += tile_cost(t0, tr, tc, steps);
       }
       const double share = std::max(1.0, total / (16.0 * n_sms));
+      constexpr int64_t kPartBytes = int64_t(kTile) * kTile * sizeof(double);
+      auto parts_of = [&](double cost, int64_t ntasks) {
+        return int(std::max<int64_t>(1, std::min(int64_t(std::min(1e6, std::ceil(cost / share))), ntasks / 4)));
+      };
       size_t i = 0;
       while (i < ord.size()) {
         Chunk c{int64_t(k1.size()), 0, int64_t(k2.size()), 0, int64_t(split.size()), 0, 0.0, 0.0};
         std::map<std::tuple<int64_t, int64_t, int32_t, int32_t, int32_t>, int64_t> toff;
-        int64_t tsz = 0;
+        int64_t tsz = 0, psz = 0;  // doubles of T; bytes of the partial tiles
         size_t j = i;
         std::vector<K2Job> jobs;
         std::vector<double> cost;
         while (j < ord.size()) {
           const int64_t f = st.tasks[ord[j]].f;
           size_t e = j;
-          int64_t add = 0;
+          int64_t add = 0, addp = 0;
+          double steps = 0.0;
           for (; e < ord.size() && st.tasks[ord[e]].f == f; ++e) {
             const RTask& t = st.tasks[ord[e]];
+            steps += (t.k1 + 15) / 16;
             if (!toff.count({t.e, t.d, t.k1, t.k2, t.n})) add += (int64_t(t.k1) * t.n + 1) & ~int64_t(1);
           }
-          if (j > i && (tsz + add) * int64_t(sizeof(double)) > budget_) break;
+          const RTask& t0 = st.tasks[ord[j]];
+          for (int tc = 0; tc < (t0.n + kTile - 1) / kTile; ++tc)
+            for (int tr = 0; tr < (t0.m + kTile - 1) / kTile; ++tr) {
+              const int n = parts_of(tile_cost(t0, tr, tc, steps), int64_t(e - j));
+              if (n > 1) addp += n * kPartBytes;
+            }
+          if (j > i && (tsz + add) * int64_t(sizeof(double)) + psz + addp > budget_) break;
+          psz += addp;
           const int32_t tb = int32_t(k2t.size());
           double c2 = 0.0;
           for (size_t x = j; x < e; ++x) {
@@ -185,7 +198,6 @@ class DeviceBackend : public RenormBackend {
             c.k2_flops += 2.0 * t.m * t.k1 * t.n;
             c2 += (t.k1 + 15) / 16;
           }
-          const RTask& t0 = st.tasks[ord[j]];
           for (int tc = 0; tc < (t0.n + kTile - 1) / kTile; ++tc)
             for (int tr = 0; tr < (t0.m + kTile - 1) / kTile; ++tr) {
               jobs.push_back(K2Job{f, t0.m, t0.n, tr, tc, tb, int32_t(k2t.size()), -1, 0});
@@ -197,7 +209,7 @@ class DeviceBackend : public RenormBackend {
         std::vector<std::pair<double, K2Job>> runs;
         for (size_t x = 0; x < jobs.size(); ++x) {
           const K2Job& q = jobs[x];
-          const int nt = q.t1 - q.t0, parts = std::max(1, std::min(int(std::min(1e6, std::ceil(cost[x] / share))), nt / 4));
+          const int nt = q.t1 - q.t0, parts = parts_of(cost[x], nt);
           if (parts > 1)
             split.push_back(P64Tile{q.f_off + q.tr * kTile + int64_t(q.tc) * kTile * q.m, std::min(kTile, q.m - q.tr * kTile),
                                     std::min(kTile, q.n - q.tc * kTile), q.m, int32_t(slots), parts, 0});

@@ -42,7 +42,7 @@ struct Plan64 {
   std::vector<P64Stack> stack;
   std::vector<P64K2> k2;
   std::vector<P64Tile> tile;
-  int64_t n_part = 0;  // partial tiles of a chunk (the most of any chunk)
+  int64_t n_part = 0;  // partial tiles of a chunk (the most of any chunk; behind T in the environment's dT)
   P64Ent* d_ent = nullptr;
   P64In* d_in = nullptr;
   P64K1* d_k1 = nullptr;
@@ -173,6 +173,7 @@ struct OpStream {
   int64_t total = 0;             // doubles of the logical arena
   std::vector<int64_t> hs, he;   // streamed range of each chunk (logical offsets)
   int64_t slot = 0;              // doubles per device slot
+  int64_t t64 = 0;               // bytes of the largest chunk's T on the FP64 path
   int64_t work = 0;              // bytes of the intermediates of the largest chunk (either path, up to kMaxSlices slices)
   double* dbuf = nullptr;        // device: [0, prefix) resident, then the two slots
   double* host = nullptr;        // pinned host memory: logical [prefix, total)

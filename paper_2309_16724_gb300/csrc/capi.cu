@@ -236,10 +236,12 @@ static int build_plan(su2_env* env, const su2_sectors* S, int64_t budget) {
   std::vector<std::vector<int64_t>> by_term(nterms);
   for (int64_t i = 0; i < int64_t(tasks.size()); ++i) by_term[tasks[i].term].push_back(i);
   // chunk boundaries over terms (out-of-core: the planner's).  T and the partial
-  // tiles of K2 share the budget: at most an eighth of it, and never more than
-  // the K split can ask for (32 tiles of 32 KiB an SM), is kept back for these
+  // tiles of K2 share the budget: at most a half of it, and never more than the K
+  // split can ask for (32 tiles of 32 KiB an SM), is kept back for these (L = 16, D
+  // = 512: 30.4, 29.6 and 28.4 ms with budgets of 64, 128 and 256 MB, 27.0 with 2
+  // GiB; with a quarter 32.6, 31.2 and 28.0: fewer chunks, but a coarser split)
   std::vector<int> starts;
-  int64_t t_max = 0, limit = budget - std::min<int64_t>(budget / 8, int64_t(152) << 20);  // bytes
+  int64_t t_max = 0, limit = budget - std::min<int64_t>(budget / 2, int64_t(152) << 20);  // bytes
   if (env->os.on) {
     starts = env->os.starts;
     t_max = env->os.t64;
@@ -430,7 +432,7 @@ static int build_plan(su2_env* env, const su2_sectors* S, int64_t budget) {
         for (int tr = 0; tr < (s.m + kTile - 1) / kTile; ++tr) {
           const double rows = std::min(kTile, s.m - tr * kTile), cls = (std::min(kTile, s.N - tc * kTile) + 15) / 16 * 16;
           const double cost = nsteps * (8.0 * rows * cls + 1500.0);
-          tiles.push_back(Tile{P64K2{int32_t(P.stack.size()), tr, tc, 0, nsteps, -1}, cost, nsteps});
+          tiles.push_back(Tile{P64K2{-1, int32_t(P.stack.size()), tr, tc, 0, nsteps, 0}, cost, nsteps});
           total += cost;
         }
       }
@@ -442,29 +444,36 @@ static int build_plan(su2_env* env, const su2_sectors* S, int64_t budget) {
     // partial tiles fit what T leaves of the budget
     double share = std::max(1.0, total / (16.0 * n_sms));
     auto parts_of = [&](const Tile& t) { return std::max(1, std::min(int(std::min(1e6, std::ceil(t.cost / share))), t.steps / 4)); };
-    auto slots_of = [&]() {
+    auto area = [&](const Tile& t) {
+      const P64Stack& s = P.stack[t.j.st];
+      return int64_t(std::min(kTile, s.m - t.j.tr * kTile)) * std::min(kTile, s.N - t.j.tc * kTile);
+    };
+    auto doubles_of = [&]() {
       int64_t n = 0;
-      for (const Tile& t : tiles) n += parts_of(t) > 1 ? parts_of(t) : 0;
+      for (const Tile& t : tiles) n += parts_of(t) > 1 ? parts_of(t) * area(t) : 0;
       return n;
     };
-    while (slots_of() * kTile * kTile * int64_t(sizeof(double)) > std::max<int64_t>(0, budget - t_max)) share *= 1.25;
+    while (doubles_of() * int64_t(sizeof(double)) > std::max<int64_t>(0, budget - t_max)) share *= 1.1;
     std::vector<std::pair<double, P64K2>> jobs;
-    int64_t slots = 0;
+    int64_t used = 0;
     for (const Tile& t : tiles) {
       const int parts = parts_of(t);
       const P64Stack& s = P.stack[t.j.st];
       if (parts > 1)
-        P.tile.push_back(P64Tile{s.f_off + t.j.tr * kTile + int64_t(t.j.tc) * kTile * s.m, std::min(kTile, s.m - t.j.tr * kTile),
-                                 std::min(kTile, s.N - t.j.tc * kTile), s.m, int32_t(slots), parts, 0});
+        P.tile.push_back(P64Tile{s.f_off + t.j.tr * kTile + int64_t(t.j.tc) * kTile * s.m, used, std::min(kTile, s.m - t.j.tr * kTile),
+                                 std::min(kTile, s.N - t.j.tc * kTile), s.m, parts});
       for (int q = 0; q < parts; ++q) {
         P64K2 j = t.j;
         j.s0 = int(int64_t(t.steps) * q / parts);
         j.s1 = int(int64_t(t.steps) * (q + 1) / parts);
-        if (parts > 1) j.slot = int32_t(slots++);
+        if (parts > 1) {
+          j.part = used;
+          used += area(t);
+        }
         jobs.push_back({t.cost * (j.s1 - j.s0) / t.steps, j});
       }
     }
-    P.n_part = std::max(P.n_part, slots);
+    P.n_part = std::max(P.n_part, used);
     std::stable_sort(jobs.begin(), jobs.end(), [](const std::pair<double, P64K2>& x, const std::pair<double, P64K2>& y) { return x.first > y.first; });
     for (const auto& q : jobs) P.k2.push_back(q.second);
     ch.k2_end = int64_t(P.k2.size());
@@ -663,7 +672,7 @@ static int finish_env(su2_ctx* ctx, su2_env* env, const su2_sectors* S, const su
     // T, then the partial tiles; out of core with the split path: its chunk buffer too
     const bool split = opts && (opts->prepare_split || opts->autotune);
     Plan64& p = env->p64;
-    const int64_t own = env->t_elems + p.n_part * kTile * kTile, both = env->os.on && split ? env->os.work / 8 + 1 : 0;
+    const int64_t own = env->t_elems + p.n_part, both = env->os.on && split ? env->os.work / 8 + 1 : 0;
     if (!rc) rc = dev_alloc(ctx, &env->dT, size_t(std::max<int64_t>({own, both, 2})));
     if (!rc) p.d_part = env->dT + env->t_elems;
     if (!rc) rc = upload(ctx, &p.d_ent, p.ent);

@@ -131,7 +131,7 @@ __global__ void __launch_bounds__(NT) k2_fp64(const K2Job* __restrict__ jobs, co
     for (int jj = 0; jj < 4; ++jj) {
       const int r = r0 + ty + 16 * i, c = c0 + tx + 16 * jj;
       if (r >= j.m || c >= j.n) continue;
-      if (j.slot >= 0) part[(int64_t(j.slot) * kTile + (c - c0)) * kTile + (r - r0)] = acc[i][jj];
+      if (j.part >= 0) part[j.part + (c - c0) * min(kTile, j.m - r0) + (r - r0)] = acc[i][jj];
       else F[j.f_off + r + int64_t(c) * j.m] += acc[i][jj];
     }
 }
@@ -296,7 +296,7 @@ __global__ void __launch_bounds__(NT, 2) k2_stack(const P64K2* __restrict__ jobs
     for (int jj = 0; jj < 4; ++jj) {
       const int r = ty + 16 * i, c = tx + 16 * jj;
       if (!on[i] || c0 + c >= s.N) continue;
-      if (j.slot >= 0) part[(int64_t(j.slot) * kTile + c) * kTile + r] = acc[i][jj];
+      if (j.part >= 0) part[j.part + c * min(kTile, s.m - r0) + r] = acc[i][jj];
       else F[s.f_off + r0 + r + int64_t(c0 + c) * s.m] += acc[i][jj];
     }
 }
@@ -310,7 +310,7 @@ __global__ void __launch_bounds__(NT) part_sum(const P64Tile* __restrict__ tiles
   for (int c = threadIdx.x >> 6; c < t.cols; c += NT / 64) {
     double x = 0.0;
 #pragma unroll 4
-    for (int i = 0; i < t.nslot; ++i) x += part[(int64_t(t.slot0 + i) * kTile + c) * kTile + r];
+    for (int i = 0; i < t.npart; ++i) x += part[t.part0 + int64_t(i) * t.rows * t.cols + c * t.rows + r];
     F[t.f_off + r + int64_t(c) * t.ld] += x;
   }
 }

@@ -144,7 +144,9 @@ class DeviceBackend : public RenormBackend {
           for (int tr = 0; tr < (t0.m + kTile - 1) / kTile; ++tr) total += tile_cost(t0, tr, tc, steps);
       }
       const double share = std::max(1.0, total / (16.0 * n_sms));
-      constexpr int64_t kPartBytes = int64_t(kTile) * kTile * sizeof(double);
+      auto area = [&](int m, int n, int tr, int tc) {
+        return int64_t(std::min(kTile, m - tr * kTile)) * std::min(kTile, n - tc * kTile);
+      };
       auto parts_of = [&](double cost, int64_t ntasks) {
         return int(std::max<int64_t>(1, std::min(int64_t(std::min(1e6, std::ceil(cost / share))), ntasks / 4)));
       };
@@ -170,7 +172,7 @@ class DeviceBackend : public RenormBackend {
           for (int tc = 0; tc < (t0.n + kTile - 1) / kTile; ++tc)
             for (int tr = 0; tr < (t0.m + kTile - 1) / kTile; ++tr) {
               const int n = parts_of(tile_cost(t0, tr, tc, steps), int64_t(e - j));
-              if (n > 1) addp += n * kPartBytes;
+              if (n > 1) addp += n * area(t0.m, t0.n, tr, tc) * int64_t(sizeof(double));
             }
           if (j > i && (tsz + add) * int64_t(sizeof(double)) + psz + addp > budget_) break;
           psz += addp;
@@ -200,28 +202,31 @@ class DeviceBackend : public RenormBackend {
           }
           for (int tc = 0; tc < (t0.n + kTile - 1) / kTile; ++tc)
             for (int tr = 0; tr < (t0.m + kTile - 1) / kTile; ++tr) {
-              jobs.push_back(K2Job{f, t0.m, t0.n, tr, tc, tb, int32_t(k2t.size()), -1, 0});
+              jobs.push_back(K2Job{f, t0.m, t0.n, tr, tc, tb, int32_t(k2t.size()), -1});
               cost.push_back(tile_cost(t0, tr, tc, c2));
             }
           j = e;
         }
-        int64_t slots = 0;
+        int64_t used = 0;
         std::vector<std::pair<double, K2Job>> runs;
         for (size_t x = 0; x < jobs.size(); ++x) {
           const K2Job& q = jobs[x];
           const int nt = q.t1 - q.t0, parts = parts_of(cost[x], nt);
           if (parts > 1)
-            split.push_back(P64Tile{q.f_off + q.tr * kTile + int64_t(q.tc) * kTile * q.m, std::min(kTile, q.m - q.tr * kTile),
-                                    std::min(kTile, q.n - q.tc * kTile), q.m, int32_t(slots), parts, 0});
+            split.push_back(P64Tile{q.f_off + q.tr * kTile + int64_t(q.tc) * kTile * q.m, used, std::min(kTile, q.m - q.tr * kTile),
+                                    std::min(kTile, q.n - q.tc * kTile), q.m, parts});
           for (int p = 0; p < parts; ++p) {
             K2Job y = q;
             y.t0 = q.t0 + int(int64_t(nt) * p / parts);
             y.t1 = q.t0 + int(int64_t(nt) * (p + 1) / parts);
-            if (parts > 1) y.slot = int32_t(slots++);
+            if (parts > 1) {
+              y.part = used;
+              used += area(q.m, q.n, q.tr, q.tc);
+            }
             runs.push_back({cost[x] * (y.t1 - y.t0) / std::max(1, nt), y});
           }
         }
-        max_part = std::max(max_part, slots);
+        max_part = std::max(max_part, used);
         std::stable_sort(runs.begin(), runs.end(),
                          [](const std::pair<double, K2Job>& a, const std::pair<double, K2Job>& b) { return a.first > b.first; });
         for (const auto& x : runs) k2.push_back(x.second);
@@ -239,7 +244,7 @@ class DeviceBackend : public RenormBackend {
       if (err.empty()) ck(upload(&dk2, k2), "K2 jobs");
       if (err.empty()) ck(upload(&dk2t, k2t), "K2 tasks");
       if (err.empty()) ck(upload(&dsp, split), "split tiles");
-      if (err.empty() && max_part > 0) ck(cudaMalloc(&part, size_t(max_part) * kTile * kTile * sizeof(double)), "partial tiles");
+      if (err.empty() && max_part > 0) ck(cudaMalloc(&part, size_t(max_part) * sizeof(double)), "partial tiles");
       if (err.empty())
         for (const Chunk& c : chunks) launch_heff_fp64(s_, q, q, src, dst, T, dk1, dk2, dk2t, dsp, part, c);
       if (err.empty()) ck(cudaGetLastError(), "launch");

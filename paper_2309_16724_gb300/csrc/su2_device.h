@@ -24,8 +24,8 @@ struct P64Left { int64_t a_off; int32_t k0, pad; };        // A block (-1: ident
 struct P64Task { int64_t off; double v; int32_t ld, psi; };
 struct P64Col { int32_t f, c; };
 struct P64Stack { int64_t f_off, tab_off; int32_t left0, step0, nf, N, m, K, col0, pad; };
-struct P64K2 { int32_t st, tr, tc, s0, s1, slot; };        // K steps [s0, s1) of one tile; slot >= 0: a partial tile
-struct P64Tile { int64_t f_off; int32_t rows, cols, ld, slot0, nslot, pad; };
+struct P64K2 { int64_t part; int32_t st, tr, tc, s0, s1, pad; };  // K steps [s0, s1) of one tile; part >= 0: a partial tile, stored there
+struct P64Tile { int64_t f_off, part0; int32_t rows, cols, ld, npart; };  // npart partial tiles (rows x cols, no padding) from part0
 struct Chunk64 {
   int64_t k1_begin, k1_end, k2_begin, k2_end, sp_begin, sp_end;
   double k1_flops, k2_flops;
@@ -42,7 +42,7 @@ struct Plan64 {
   std::vector<P64Stack> stack;
   std::vector<P64K2> k2;
   std::vector<P64Tile> tile;
-  int64_t n_part = 0;  // partial tiles of a chunk (the most of any chunk; behind T in the environment's dT)
+  int64_t n_part = 0;  // doubles of a chunk's partial tiles (the most of any chunk; behind T in the environment's dT)
   P64Ent* d_ent = nullptr;
   P64In* d_in = nullptr;
   P64K1* d_k1 = nullptr;
@@ -68,7 +68,7 @@ struct K1Job {
 struct K2Job {
   int64_t f_off;
   int32_t m, n, tr, tc, t0, t1;
-  int32_t slot, pad;  // slot >= 0: a run of the tile's tasks, stored as a partial tile
+  int64_t part;  // >= 0: a run of the tile's tasks, stored there as a partial tile
 };
 struct K2Task {
   int64_t a_off;  // left operand (m x k1)

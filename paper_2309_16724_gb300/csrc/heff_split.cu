@@ -121,7 +121,9 @@ struct SplitTile {
 // second pass adds each block's partials into F in a fixed order
 // (deterministic).  A segment's length makes one wave of kSmallWarps warps per
 // SM out of all tasks, between 4 and 32: 32 for all left two CTAs per SM at L =
-// 12, D = 100 and took 335 us there
+// 12, D = 100 and took 335 us there.  (The same length for the variant of tasks
+// of at most 8, whose registers would allow twice the warps: it has more of
+// them only where the 32 cap gives more segments than one wave)
 constexpr int kSmallWarps = 16;
 struct SmallTask {
   int64_t e_off, a_off, d_off;  // psi block, left / right operator block (-1: identity)

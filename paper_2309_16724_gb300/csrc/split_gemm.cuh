@@ -63,7 +63,7 @@ constexpr int kSub = kRows * kKS * 2;  // bytes of one 128 x 16 BF16 sub-tile (s
 constexpr int kSubB = kCols * kKS * 2;  // bytes of the B part of a stage slice (kCols rows)
 constexpr int kBufCols = 4 * kCols;  // TMEM columns of one accumulator buffer (4 levels)
 constexpr int kDrainCols = kCols / 4;  // most columns per drain thread (16 drain warps: 4 lane quarters x 4 groups)
-constexpr int kGroup = kDrainCols >= 32 ? 4 : 8;  // columns per TMEM load group
+constexpr int kGroup = 4;  // columns per TMEM load group (eight spilled more registers)
 constexpr int kMaxS = 6;
 constexpr int kChunkSteps = 12;      // 16-K steps per exact drain chunk (192 K)
 constexpr int kLead = 8;             // leading slice |q_0| <= 2^kLead, the others |q_i| <= 128
@@ -242,10 +242,12 @@ __device__ __forceinline__ void mma_commit(uint32_t bar) {
       : "memory");
 }
 
-// four 32x32b.x4 TMEM loads (four columns of each accumulator level) and
-// the wait in one asm statement (see below)
-__device__ __forceinline__ void tmem_ld4x4_wait(uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
-                                                float (&v)[16]) {
+// four columns of each accumulator level (level l at column offset l * kCols):
+// four 32x32b.x4 TMEM loads and the wait in one asm statement.  tcgen05.ld
+// writes its destination registers asynchronously, so they must not exist as
+// values in the program before tcgen05.wait::ld (a separate wait statement
+// would let the compiler reuse or read them early)
+__device__ __forceinline__ void tmem_ld_levels(uint32_t a, float (&v)[4 * kGroup]) {
   uint32_t r[16];
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%16];\n"
@@ -255,46 +257,10 @@ __device__ __forceinline__ void tmem_ld4x4_wait(uint32_t a0, uint32_t a1, uint32
       "tcgen05.wait::ld.sync.aligned;\n"
       : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
         "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(a0), "r"(a1), "r"(a2), "r"(a3)
+      : "r"(a), "r"(a + kCols), "r"(a + 2 * kCols), "r"(a + 3 * kCols)
       : "memory");
 #pragma unroll
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
-}
-
-// four 32x32b.x8 TMEM loads (eight columns of each accumulator level) and
-// the wait in one asm statement: tcgen05.ld writes its destination registers
-// asynchronously, so they must not exist as values in the program before
-// tcgen05.wait::ld (a separate wait statement would let the compiler reuse or
-// read them early)
-__device__ __forceinline__ void tmem_ld8x4_wait(uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
-                                                float (&v)[32]) {
-  uint32_t r[32];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%32];\n"
-      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%8,%9,%10,%11,%12,%13,%14,%15}, [%33];\n"
-      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%16,%17,%18,%19,%20,%21,%22,%23}, [%34];\n"
-      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%24,%25,%26,%27,%28,%29,%30,%31}, [%35];\n"
-      "tcgen05.wait::ld.sync.aligned;\n"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-        "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-        "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(a0), "r"(a1), "r"(a2), "r"(a3)
-      : "memory");
-#pragma unroll
-  for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
-}
-
-// kG columns of all four accumulator levels (level l at column offset l * kCols)
-template <int kG>
-__device__ __forceinline__ void tmem_ld_levels(uint32_t a, float (&x)[4 * kG]);
-template <>
-__device__ __forceinline__ void tmem_ld_levels<4>(uint32_t a, float (&x)[16]) {
-  tmem_ld4x4_wait(a, a + kCols, a + 2 * kCols, a + 3 * kCols, x);
-}
-template <>
-__device__ __forceinline__ void tmem_ld_levels<8>(uint32_t a, float (&x)[32]) {
-  tmem_ld8x4_wait(a, a + kCols, a + 2 * kCols, a + 3 * kCols, x);
 }
 
 // packed FP32 pairs (two drain columns per instruction); every step is the
@@ -563,7 +529,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       constexpr int kNG = kDrainCols / kGroup;
       static_assert(kGroup == 4, "the drain exponent of column 4g + c is byte c of word g");
       const int w = jb.nmma >> 2;
-      const int ng = w / kGroup;  // column groups of this warp
+      const int ng = w / kGroup;  // column groups of this warp (at least one: nmma >= 16)
       const int c0 = jb.tc * kCols + cgrp * w;
       const uint32_t lane_addr = lane_base + cgrp * w;
       const bool trans = (jb.flags & kJobTrans) != 0;
@@ -597,7 +563,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (g >= ng) break;
             const uint32_t a = lane_addr + buf * kBufCols + g * kGroup;
             float x[4 * kGroup];  // levels 0..3, kGroup columns each
-            tmem_ld_levels<kGroup>(a, x);
+            tmem_ld_levels(a, x);
             const uint32_t dxg = MODE == MODE_F ? __shfl_sync(0xffffffffu, dxl, g) : 0u;
             if (g == ng - 1) {
               // the warp's last TMEM read of this chunk has completed: hand
@@ -652,11 +618,6 @@ __global__ void __launch_bounds__(kThreads, 1)
                 hi2[k >> 1] = hs;
               }
             }
-          }
-          if (ng <= 0) {  // (nmma >= 16 gives ng >= 1; kept so that the barrier always completes)
-            __syncwarp();
-            if (lane == 0)
-              asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&acce_bar[buf])) : "memory");
           }
           first = false;
           chunk += 1;

@@ -39,9 +39,10 @@ DEFAULT_CONFIG = "qc48"   # L = N = 48, D = 4096: the batching configuration the
 FP64_PEAK_TFLOPS = 1.25   # 152 SMs x 2 DFMA/clk x 2 flop x 2.07 GHz (nominal FP64 rate)
 
 
-def k2_traffic(workload, slices, stage_k):
-    """DRAM bytes per K2 launch from the committed ncu capture, or None when the
-    split sources changed since it was taken or the workload differs."""
+def split_traffic(kernel, workload, slices, stage_k):
+    """DRAM bytes per launch of a split GEMM ("k1_split" or "k2_split") from the
+    committed ncu capture, or None when the split sources changed since it was
+    taken or the workload differs."""
     import hashlib
     root = os.path.dirname(os.path.abspath(__file__))
     src = os.path.join(root, "paper_2309_16724_gb300", "csrc")
@@ -57,7 +58,8 @@ def k2_traffic(workload, slices, stage_k):
         return None
     if (kv.get("workload"), kv.get("slices"), kv.get("stage_k16")) != (workload, str(slices), str(stage_k)):
         return None
-    return float(kv["k2_split_traffic_bytes_per_launch"])
+    v = kv.get(f"{kernel}_traffic_bytes_per_launch")
+    return None if v is None else float(v)
 
 
 def workload_config(cfg):
@@ -665,8 +667,7 @@ def main():
                     "steps": e2e_steps},
             "roofline": {"bound": bound, "achieved": achieved, "peak": peak, "unit": unit,
                          "frac": achieved / peak if peak else None,
-                         "traffic": (k2_traffic(cfg.name, info["split_slices"], info["split_stage_k"])
-                                     if name == "k2_split" else None),
+                         "traffic": split_traffic(name, cfg.name, info["split_slices"], info["split_stage_k"]),
                          "kernel": name, "peak_source": peak_note},
             "kernels": {k: {"launches": v[0], "ms": v[1], "flops": v[2]} for k, v in prof.items() if v[0]},
             "gpu_launches": gpu_launches,

@@ -462,8 +462,9 @@ __global__ void slab_fp64_kernel(const SlabDesc* __restrict__ descs, const Unit*
 // right operator), the row exponents and the slabs of its stacks in one
 // kernel; one CTA of 32 x 8 threads per (block, kRowTile rows).  The slabs are
 // cut from psi in FP64 (its second read hits L2), after the leading slice in
-// FP32 (an FP64 cut of all slices took 280 us at L = 32, D = 2048: GB300's FP64
-// rate is 1/64 of FP32's)
+// FP32: 116 us of 101 ms at L = 32, D = 2048 (all slices in FP64 280, GB300's
+// FP64 rate being 1/64 of FP32's; from the rounded float-float copy 60, with fewer
+// bits)
 __global__ void __launch_bounds__(256) psi_slab_kernel(const SlabDesc* __restrict__ descs, const Unit* __restrict__ units,
                                                        const double* __restrict__ psi, float2* __restrict__ P,
                                                        int* __restrict__ eps, unsigned char* __restrict__ slab, int S) {
@@ -568,7 +569,7 @@ __device__ __forceinline__ void add_task(const TPTask& t, const float2 (&av)[4],
 // through shared memory), so T is read once, in whole 64-byte pieces (row
 // offsets and strides are multiples of 8).  Bound by the latency of its loads
 // (unit, pieces, task list, task, T): three CTAs per SM at 56 registers with a
-// few spills take 27.1 ms at L = 32, D = 2048, two at 80 registers 31.0; lists
+// few spills take 26.5 ms at L = 32, D = 2048, two at 80 registers 31.0; lists
 // with the first task inline (one load fewer) gained nothing.
 constexpr int kTPWarps = kWinSteps;
 __global__ void __launch_bounds__(32 * kTPWarps, 3)
